@@ -307,7 +307,7 @@ int32_t gq_objective_noalloc(const float *W, const float *W_hat, int64_t d_in, i
  *   codebook   fp32 [d_out, m], 1 <= m <= 16 (need not be sorted)
  *   H          fp32 [g, d_in, d_in], FULL symmetric matrices (after gq_hessian_finalize), 16-byte aligned.
  *              A coordinate with H_k[i][i] <= 0 is rounded to the codebook value nearest to W[j][i].
- *   cycles     >= 0 (0 only transposes W_hat through the workspace and back; Q is then all zero)
+ *   cycles     >= 0 (0 leaves W_hat as it is; Q is then all zero)
  *   workspace  device scratch of at least gq_cd_workspace_bytes(d_in, d_out, g) bytes, 1024-byte aligned
  * Same shape rules as gq_objective.
  * Arithmetic: coordinates are processed in blocks of 256.  The contributions of the coordinates outside

@@ -16,21 +16,27 @@
 // Work arrays are coordinate-major ([d_in][d_out], the paper's orientation) so that one coordinate of all
 // channels is contiguous; W, What and the codes are transposed on the way in and out.
 #pragma once
+#include <cuda.h>
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 #include <math_constants.h>
 #include <stdint.h>
 
+#include "gq_pipeline.cuh"
+
 namespace gq {
 
 constexpr int CD_BLOCK = 256;           // coordinates per block
-constexpr int CD_CH = 32;               // channels per CTA of the block kernel
-constexpr int CD_LANES = 8;             // threads per channel
-constexpr int CD_THREADS = CD_CH * CD_LANES;
+constexpr int CD_BAND = 32;             // coordinates whose running sums one chain thread holds
+constexpr int CD_BANDS = CD_BLOCK / CD_BAND;
+constexpr int CD_CH = 32;               // channels per CTA of the block kernel: one lane of the chain warp each
+constexpr int CD_THREADS = 256;
 constexpr int CD_MAX_LEVELS = 16;       // codebook entries per channel (m = 2^b, b <= 4)
-constexpr int CD_TILE_LD = CD_CH + 1;   // padded row of the [CD_BLOCK][CD_CH] shared-memory tiles
-constexpr int CD_HCHUNK = 32;           // rows of the block's Hessian staged at a time
-constexpr int CD_SMEM_BYTES = (3 * CD_BLOCK * CD_TILE_LD + 2 * CD_HCHUNK * CD_BLOCK + CD_BLOCK + 2 * CD_CH * CD_MAX_LEVELS) * 4;
+constexpr int CD_LEVEL_LD = CD_MAX_LEVELS + 1;   // padded per-channel rows of the level tables
+constexpr int CD_H_BUFS = 3;
+constexpr int CD_TILE_FLOATS = CD_BLOCK * CD_CH;         // one [256][32] tile: 32 KB
+constexpr int CD_PARTS = 6;             // pieces of the contraction range of a band's pulled sums: one per product warp
+constexpr int CD_SMEM_BYTES = ((3 + CD_H_BUFS) * CD_TILE_FLOATS + CD_PARTS * CD_BAND * CD_CH + CD_BLOCK + 3 * CD_CH * CD_LEVEL_LD) * 4 + 1024;
 
 __device__ __forceinline__ void split_bf16(float v, __nv_bfloat16 &hi, __nv_bfloat16 &lo)
 {
@@ -38,10 +44,10 @@ __device__ __forceinline__ void split_bf16(float v, __nv_bfloat16 &hi, __nv_bflo
     lo = __float2bfloat16_rn(v - __bfloat162float(hi));
 }
 
-// Wt = W^T, Wht = What^T, E = Wht - Wt (fp32 and as bf16 hi + lo), all [d_in][d_out].  32 x 32 tiles.
+// Wt = W^T, E = (What - W)^T (fp32 and as bf16 hi + lo), all [d_in][d_out].  32 x 32 tiles.
 __global__ void __launch_bounds__(256)
 cd_prepare_kernel(const float *__restrict__ W, const float *__restrict__ What, int d_in, int d_out,
-                  float *__restrict__ Wt, float *__restrict__ Wht, float *__restrict__ Et,
+                  float *__restrict__ Wt, float *__restrict__ Et,
                   __nv_bfloat16 *__restrict__ Ehi, __nv_bfloat16 *__restrict__ Elo)
 {
     __shared__ float tw[32][33], th[32][33];
@@ -60,7 +66,6 @@ cd_prepare_kernel(const float *__restrict__ W, const float *__restrict__ What, i
             const float w = tw[tx][r], h = th[tx][r], e = h - w;
             const size_t o = static_cast<size_t>(i) * d_out + j;
             Wt[o] = w;
-            Wht[o] = h;
             Et[o] = e;
             __nv_bfloat16 hi, lo;
             split_bf16(e, hi, lo);
@@ -70,56 +75,58 @@ cd_prepare_kernel(const float *__restrict__ W, const float *__restrict__ What, i
     }
 }
 
-// H -> bf16 hi + lo (operands of the panel product) and rdiag[k][i] = 1 / H_k[i][i] (0 where H_ii <= 0).
+// H -> bf16 hi + lo (operands of the panel product) and rdiag[k][i] = 1 / H_k[i][i] (0 where H_ii <= 0).  One block
+// per row of a group's matrix, 16-byte loads (d_in is a multiple of 8): bound by the 8 bytes per entry it moves.  With
+// one entry per thread and a 64-bit modulo each to find the diagonal it took 342 us for four 4096 x 4096 matrices, now 79.
 __global__ void __launch_bounds__(256)
-cd_split_h_kernel(const float *__restrict__ H, long long count, int d_in, __nv_bfloat16 *__restrict__ Hhi,
-                  __nv_bfloat16 *__restrict__ Hlo, float *__restrict__ rdiag)
+cd_split_h_kernel(const float *__restrict__ H, int d_in, __nv_bfloat16 *__restrict__ Hhi, __nv_bfloat16 *__restrict__ Hlo,
+                  float *__restrict__ rdiag)
 {
-    const long long stride = static_cast<long long>(gridDim.x) * blockDim.x;
-    for (long long idx = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x; idx < count; idx += stride) {
-        const float v = H[idx];
-        __nv_bfloat16 hi, lo;
-        split_bf16(v, hi, lo);
-        Hhi[idx] = hi;
-        Hlo[idx] = lo;
-        const long long within = idx % (static_cast<long long>(d_in) * d_in);
-        const int r = static_cast<int>(within / d_in), c = static_cast<int>(within - static_cast<long long>(r) * d_in);
-        if (r == c) rdiag[idx / (static_cast<long long>(d_in) * d_in) * d_in + r] = v > 0.0f ? 1.0f / v : 0.0f;
+    const int i = static_cast<int>(blockIdx.x);
+    const size_t row = static_cast<size_t>(blockIdx.y) * d_in + i;
+    const float4 *src = reinterpret_cast<const float4 *>(H + row * d_in);
+    uint2 *hi = reinterpret_cast<uint2 *>(Hhi + row * d_in), *lo = reinterpret_cast<uint2 *>(Hlo + row * d_in);
+    for (int c = threadIdx.x; c < d_in / 4; c += 256) {
+        const float4 v = src[c];
+        const float f[4] = {v.x, v.y, v.z, v.w};
+        __align__(8) __nv_bfloat16 h[4], l[4];
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            split_bf16(f[e], h[e], l[e]);
+            if (4 * c + e == i) rdiag[row] = f[e] > 0.0f ? 1.0f / f[e] : 0.0f;
+        }
+        hi[c] = *reinterpret_cast<uint2 *>(h);
+        lo[c] = *reinterpret_cast<uint2 *>(l);
     }
 }
 
-// What = Wht^T, Q = Qt^T back to [d_out][d_in].
+// Q = Qt^T back to [d_out][d_in] and What = codebook[Q].
 __global__ void __launch_bounds__(256)
-cd_finish_kernel(const float *__restrict__ Wht, const uint8_t *__restrict__ Qt, int d_in, int d_out,
+cd_finish_kernel(const float *__restrict__ codebook, const uint8_t *__restrict__ Qt, int d_in, int d_out, int m,
                  float *__restrict__ What, uint8_t *__restrict__ Q)
 {
-    __shared__ float th[32][33];
     __shared__ uint8_t tq[32][33];
     const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
     const int i0 = blockIdx.x * 32, j0 = blockIdx.y * 32;
     for (int r = ty; r < 32; r += 8) {
         const int i = i0 + r, j = j0 + tx;
-        const bool ok = i < d_in && j < d_out;
-        th[r][tx] = ok ? Wht[static_cast<size_t>(i) * d_out + j] : 0.0f;
-        tq[r][tx] = ok ? Qt[static_cast<size_t>(i) * d_out + j] : 0;
+        tq[r][tx] = (i < d_in && j < d_out) ? Qt[static_cast<size_t>(i) * d_out + j] : 0;
     }
     __syncthreads();
     for (int r = ty; r < 32; r += 8) {
         const int j = j0 + r, i = i0 + tx;
         if (j < d_out && i < d_in) {
-            What[static_cast<size_t>(j) * d_in + i] = th[tx][r];
-            Q[static_cast<size_t>(j) * d_in + i] = tq[tx][r];
+            const uint8_t code = tq[tx][r];
+            What[static_cast<size_t>(j) * d_in + i] = codebook[static_cast<size_t>(j) * m + code];
+            Q[static_cast<size_t>(j) * d_in + i] = code;
         }
     }
 }
 
 struct CdBlockParams {
-    const float *H;          // [g][d_in][d_in] full symmetric
     const float *rdiag;      // [g][d_in]
-    const float *P;          // [CD_BLOCK][d_out]: contributions of the coordinates outside the block
-    const float *Wt;         // [d_in][d_out]
     const float *codebook;   // [d_out][m]
-    float *Wht;              // [d_in][d_out]
+    float *P;                // [CD_BLOCK][d_out] pulled sums; zeroed again once read
     float *Et;               // [d_in][d_out]
     __nv_bfloat16 *Ehi, *Elo;
     uint8_t *Qt;             // [d_in][d_out]
@@ -127,90 +134,166 @@ struct CdBlockParams {
     int s0;                  // first coordinate of the block
     int rows;                // coordinates in the block (<= CD_BLOCK)
     int slices;              // ceil(mk / CD_CH): CTAs per group
+    bool last_cycle;         // write the codes
+    uint32_t *status;
+    unsigned long long wait_budget_ns;
 };
 
-// One block of coordinates for CD_CH channels of one group.  Eight threads share a channel; thread l of
-// them owns the rows 32 t + 4 l + e (band t < 8, e < 4) of the running sums
-//     Bu[r] = sum_{c != r} H[r][c] * E_c      (current E: this cycle's values for c < r, last cycle's for c > r).
-// Pass 1 adds the in-block part of last cycle's values (c > r).  Pass 2 walks the rows in order; per row i:
-//   * the owner hands the rounding target W_i - Bu[i] / H_ii to the channel's threads (one shuffle);
-//   * Round_j: the channel's levels are kept sorted, thread l holding the thresholds between the sorted levels
-//     2l, 2l+1 and 2l+1, 2l+2 (their midpoints, lowered by one ulp where the upper level has the smaller
-//     original index, so that an exact tie goes to the smaller index); the nearest level is at sorted position
-//     #{q : target > thr_q}: two compares and two warp votes per thread, one table read;
-//   * every thread adds H[i][r] * E_i to those of its rows that come after i.
-// H[i][.] rows come through shared memory in chunks of 32 (= one band).  The codes are recovered at the end as
-// the first level, in the codebook's given order, that equals the chosen value.
-__global__ void __launch_bounds__(CD_THREADS, 1)
-cd_block_kernel(const CdBlockParams p)
+__device__ __forceinline__ void bar_sync_named(int id, int threads)
 {
-    extern __shared__ float smem_f[];
-    float *Ws = smem_f;                                  // [CD_BLOCK][CD_TILE_LD]  W of the block
-    float *Es = Ws + CD_BLOCK * CD_TILE_LD;              // E of the block, updated in place
-    float *Xs = Es + CD_BLOCK * CD_TILE_LD;              // first P (pulled sums), then What of the block
-    float *Hs = Xs + CD_BLOCK * CD_TILE_LD;              // [2][CD_HCHUNK][CD_BLOCK]
-    float *rds = Hs + 2 * CD_HCHUNK * CD_BLOCK;          // [CD_BLOCK]
-    float *cbs = rds + CD_BLOCK;                         // [CD_CH][CD_MAX_LEVELS] codebooks in their given order
-    float *srt = cbs + CD_CH * CD_MAX_LEVELS;            // [CD_CH][CD_MAX_LEVELS] the same, sorted
+    asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(threads) : "memory");
+}
+__device__ __forceinline__ void bar_arrive_named(int id, int threads)
+{
+    asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(threads) : "memory");
+}
 
-    const int tid = threadIdx.x;
+// The nearest of LEV sorted levels, ties already decided by the thresholds between neighbours: the number of thresholds
+// below the target is the position of the level.  A tree of compares and selects: no table read, no exchange between lanes.
+template <int LEV>
+__device__ __forceinline__ float nearest_level(float target, const float (&lev)[LEV], const float (&thr)[LEV])
+{
+    float v[LEV];
+#pragma unroll
+    for (int q = 0; q < LEV; ++q) v[q] = lev[q];
+#pragma unroll
+    for (int width = 1; width < LEV; width *= 2)
+#pragma unroll
+        for (int k = 0; k < LEV / (2 * width); ++k)
+            v[k] = target > thr[2 * width * k + width - 1] ? v[2 * k + 1] : v[2 * k];
+    return v[0];
+}
+
+// What step I of a band reads from shared memory: H[I][rows after I], W_I of the lane's channel, 1 / H_II.
+struct ChainOperands {
+    float4 h[CD_BAND / 4];
+    float w, rd;
+    template <int I>
+    __device__ __forceinline__ void load(const float *hd, const float *wb, const float *rb)
+    {
+#pragma unroll
+        for (int q = (I + 1) / 4; q < CD_BAND / 4; ++q) h[q] = *reinterpret_cast<const float4 *>(hd + I * CD_BAND + 4 * q);
+        w = wb[I * CD_CH];
+        rd = rb[I];
+    }
+};
+
+// Steps I .. CD_BAND - 1 of a band.  Operands are read two steps ahead (the product warps keep the shared-memory pipe
+// busy, so a read takes longer than a step).  Written as a recursion because the compiler does not unroll the loop, and
+// the sums have to stay in registers.
+template <int LEV, int I>
+__device__ __forceinline__ void chain_steps(const ChainOperands &cur, const ChainOperands &nxt, const float *hd, const float *rb,
+                                            float *wb, float *eb, float (&Bu)[CD_BAND], const float (&lev)[LEV],
+                                            const float (&thr)[LEV])
+{
+    ChainOperands after;
+    if constexpr (I + 2 < CD_BAND) after.load<I + 2>(hd, wb, rb);
+    const float val = nearest_level<LEV>(cur.w - cur.rd * Bu[I], lev, thr);
+    const float e_new = val - cur.w;
+#pragma unroll
+    for (int r = I + 1; r < CD_BAND; ++r) {
+        const float4 hq = cur.h[r >> 2];
+        Bu[r] = fmaf((r & 3) == 0 ? hq.x : (r & 3) == 1 ? hq.y : (r & 3) == 2 ? hq.z : hq.w, e_new, Bu[r]);
+    }
+    eb[I * CD_CH] = e_new;
+    wb[I * CD_CH] = val;                                 // W_i is not needed any more: What of the block takes its place
+    if constexpr (I + 1 < CD_BAND) chain_steps<LEV, I + 1>(nxt, after, hd, rb, wb, eb, Bu, lev, thr);
+}
+
+// Where four rows (quad rq of a band) of channel ch stand in a part of the pulled sums, in floats: the swizzle keeps both
+// the products' stores (a quarter warp: channels 4 j + b, one quad) and the chain's loads (one quad of 32 channels) free
+// of bank conflicts.
+__device__ __forceinline__ int sums_at(int ch, int rq)
+{
+    return ch * CD_BAND + ((rq ^ (ch >> 2) ^ ch) & 7) * 4;
+}
+
+// One block of coordinates for CD_CH channels of one group.
+//
+// The running sums  Bu[r] = sum_{c != r} H[r][c] E_c  (current E: this cycle's values for c < r, last cycle's for c > r)
+// are needed one coordinate after the other, each after a rounding decision on the one before it: 256 dependent steps.
+// What bounds the kernel is the length of one step, so everything that is not part of it is moved to other warps:
+//   chain warp (0)       one lane per channel.  A band of 32 coordinates at a time, its 32 running sums in registers: round
+//                        (nearest_level: compares and selects only), E_i = val - W_i, add H[i][r] E_i to the sums of the
+//                        rows after i inside the band.  No shuffle, vote or table read lies on the path.
+//   product warps (6)    while the chain works on band t they form the sums of band t + 1 over every coordinate of the block
+//                        outside bands t and t + 1, plus last cycle's values of band t + 1 above its diagonal; when the chain
+//                        is through with band t they add its new values (32 x 32 x 32) and hand the sums over.  Every warp
+//                        forms the whole 32 x 32 sums, 8 rows x 4 channels per thread, over a share of the contraction;
+//                        all of them on the three schedulers that the chain warp does not use.  A value loaded from shared
+//                        memory costs a lane-register write whether or not lanes share it (measured: a 16-byte load takes
+//                        4 clocks of the SM's load pipe, 2 if all lanes read the same address), hence 12 loaded values
+//                        per 32 multiply-adds.
+//   loader warp (4)      TMA: the tiles of W, E and P (256 coordinates x 32 channels), and H[all 256][band] (32 KB) per
+//                        band into one of three buffers, two bands ahead.
+// Two named barriers per band: sums ready (products -> chain), band done (chain -> products, loader).
+// Measured for one block of 4096 channels, 16 levels: 42 us (8 levels, 1408 channels: 38); with eight threads per channel
+// that did all updates themselves and two votes and a table read per step it was 81 us (78).
+template <int LEV>
+__global__ void __launch_bounds__(CD_THREADS, 1)
+cd_block_kernel(const __grid_constant__ CUtensorMap mapH, const __grid_constant__ CUtensorMap mapW,
+                const __grid_constant__ CUtensorMap mapE, const __grid_constant__ CUtensorMap mapP, const CdBlockParams p)
+{
+    extern __shared__ uint8_t smem_raw[];
+    __shared__ __align__(8) uint64_t bar_tiles;
+    __shared__ __align__(8) uint64_t bar_h[CD_H_BUFS];
+    __shared__ volatile uint32_t abort_flag;
+    float *Ws = reinterpret_cast<float *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
+    float *Es = Ws + CD_TILE_FLOATS;                     // [256][32] E of the block, updated in place
+    float *Ps = Es + CD_TILE_FLOATS;                     // [256][32] P
+    float *Hs = Ps + CD_TILE_FLOATS;                     // [CD_H_BUFS][256][32] H[c][rows of a band]
+    float *Ss = Hs + CD_H_BUFS * CD_TILE_FLOATS;         // [CD_PARTS][32 ch][32 rows] pulled sums of a band (sums_at)
+    float *rds = Ss + CD_PARTS * CD_BAND * CD_CH;        // [256]
+    float *srt = rds + CD_BLOCK;                         // [32][CD_LEVEL_LD] sorted levels
+    float *thr_s = srt + CD_CH * CD_LEVEL_LD;            // [32][CD_LEVEL_LD] thresholds between neighbours
+    int *sidx = reinterpret_cast<int *>(thr_s + CD_CH * CD_LEVEL_LD);   // [32][CD_LEVEL_LD] given index by sorted position
+
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int k = blockIdx.x / p.slices;
     const int ch0 = k * p.mk + (blockIdx.x % p.slices) * CD_CH;          // first channel of this CTA
-    const int ch_n = min(CD_CH, (k + 1) * p.mk - ch0);                   // valid channels
-    const int cidx = tid / CD_LANES, l = tid % CD_LANES;
-    const int group_shift = 8 * ((tid >> 3) & 3);                       // where this channel's eight threads sit in a warp vote
-    const float *Hk = p.H + static_cast<size_t>(k) * p.d_in * p.d_in;
+    const int ch_n = min(CD_CH, (k + 1) * p.mk - ch0);                   // valid channels (a multiple of 8)
+    const WaitCtx wc{&abort_flag, p.status, p.wait_budget_ns};
 
-    // ---- tiles in: 32 channels x 256 coordinates, coalesced over channels
-    for (int idx = tid; idx < CD_BLOCK * CD_CH; idx += CD_THREADS) {
-        const int r = idx / CD_CH, c = idx % CD_CH;
-        const bool ok = r < p.rows && c < ch_n;
-        const size_t o = static_cast<size_t>(p.s0 + r) * p.d_out + ch0 + c;
-        Ws[r * CD_TILE_LD + c] = ok ? p.Wt[o] : 0.0f;
-        Es[r * CD_TILE_LD + c] = ok ? p.Et[o] : 0.0f;
-        Xs[r * CD_TILE_LD + c] = ok ? p.P[static_cast<size_t>(r) * p.d_out + ch0 + c] : 0.0f;
-    }
-    for (int r = tid; r < CD_BLOCK; r += CD_THREADS)
-        rds[r] = r < p.rows ? p.rdiag[static_cast<size_t>(k) * p.d_in + p.s0 + r] : 0.0f;
-
-    // rows [c0, c0 + CD_HCHUNK) of the block's H (columns of the block only) into buffer b, zero outside the
-    // block; asynchronous copies (cp.async), completed by h_chunk_wait() before the next __syncthreads
-    auto load_h_chunk = [&](int c0, int b) {
-        float *dst = Hs + b * CD_HCHUNK * CD_BLOCK;
-        for (int idx = tid; idx < CD_HCHUNK * CD_BLOCK / 4; idx += CD_THREADS) {
-            const int rr = idx / (CD_BLOCK / 4), cc = (idx % (CD_BLOCK / 4)) * 4;
-            float *d = dst + rr * CD_BLOCK + cc;
-            if (c0 + rr < p.rows && cc < p.rows) {    // rows is a multiple of 8 (d_in % 8 == 0): whole float4 in range
-                const float *src = Hk + static_cast<size_t>(p.s0 + c0 + rr) * p.d_in + p.s0 + cc;
-                asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(static_cast<uint32_t>(
-                                 __cvta_generic_to_shared(d))), "l"(src) : "memory");
-            } else {
-                *reinterpret_cast<float4 *>(d) = make_float4(0.f, 0.f, 0.f, 0.f);
-            }
-        }
-        asm volatile("cp.async.commit_group;" ::: "memory");
+    auto load_band = [&](int t) {                        // H[block coordinates][band t] (zero outside the matrix)
+        const uint32_t bar = smem_u32(&bar_h[t % CD_H_BUFS]);
+        mbar_arrive_expect_tx(bar, CD_TILE_FLOATS * 4);
+        tma_load_3d(smem_u32(Hs + (t % CD_H_BUFS) * CD_TILE_FLOATS), &mapH, bar, p.s0 + t * CD_BAND, p.s0, k);
     };
-    auto h_chunk_wait = [&]() { asm volatile("cp.async.wait_group 0;" ::: "memory"); };
-
-    // ---- the channel's levels: given order (cbs), sorted (srt), this thread's two thresholds
-    static_assert(CD_MAX_LEVELS == 2 * CD_LANES, "two codebook levels per thread");
-    float thr_a = CUDART_INF_F, thr_b = CUDART_INF_F;
+    // A wait that ran out is recorded; the warps go on (with wrong values) so that every barrier completes.
+    auto wait_band = [&](int t) {
+        (void)bounded_wait(smem_u32(&bar_h[t % CD_H_BUFS]), static_cast<uint32_t>(t / CD_H_BUFS) & 1u, wc, 21u, blockIdx.x);
+    };
+    if (tid == 128) {
+        mbar_init(smem_u32(&bar_tiles), 1);
+        for (int b = 0; b < CD_H_BUFS; ++b) mbar_init(smem_u32(&bar_h[b]), 1);
+        abort_flag = 0u;
+        fence_mbar_init();
+        fence_proxy_async_smem();
+        load_band(0);
+        const uint32_t bar = smem_u32(&bar_tiles);
+        mbar_arrive_expect_tx(bar, 3 * CD_TILE_FLOATS * 4);
+        tma_load_3d(smem_u32(Es), &mapE, bar, ch0, p.s0, 0);
+        tma_load_3d(smem_u32(Ps), &mapP, bar, ch0, 0, 0);
+        tma_load_3d(smem_u32(Ws), &mapW, bar, ch0, p.s0, 0);
+        for (int b = 1; b < CD_H_BUFS; ++b) load_band(b);
+    }
+    rds[tid] = tid < p.rows ? p.rdiag[static_cast<size_t>(k) * p.d_in + p.s0 + tid] : 0.0f;
+    // ---- the channel's levels, sorted (eight threads per channel), and the thresholds between neighbours: their midpoints,
+    // lowered by one ulp where the upper level has the smaller given index, so that a tie goes to the smaller index
     {
+        const int cidx = tid >> 3, l = tid & 7;
         const bool chan = cidx < ch_n;
         const float v0 = (l < p.m && chan) ? p.codebook[static_cast<size_t>(ch0 + cidx) * p.m + l] : CUDART_INF_F;
         const float v1 = (l + 8 < p.m && chan) ? p.codebook[static_cast<size_t>(ch0 + cidx) * p.m + l + 8] : CUDART_INF_F;
         int rank0 = 0, rank1 = 0;                        // positions of (v0, l) and (v1, l + 8) among the 16 pairs
 #pragma unroll
         for (int r = 0; r < CD_MAX_LEVELS; ++r) {
-            const float vr = __shfl_sync(0xffffffffu, r < 8 ? v0 : v1, r & 7, CD_LANES);
+            const float vr = __shfl_sync(0xffffffffu, r < 8 ? v0 : v1, r & 7, 8);
             rank0 += (vr < v0 || (vr == v0 && r < l)) ? 1 : 0;
             rank1 += (vr < v1 || (vr == v1 && r < l + 8)) ? 1 : 0;
         }
-        int *sidx = reinterpret_cast<int *>(Hs);         // [CD_CH][CD_MAX_LEVELS] original index by sorted position
-        float *mc = cbs + cidx * CD_MAX_LEVELS, *ms = srt + cidx * CD_MAX_LEVELS;
-        int *mi = sidx + cidx * CD_MAX_LEVELS;
-        mc[l] = v0;
-        mc[l + 8] = v1;
+        float *ms = srt + cidx * CD_LEVEL_LD;
+        int *mi = sidx + cidx * CD_LEVEL_LD;
         ms[rank0] = v0;
         mi[rank0] = l;
         ms[rank1] = v1;
@@ -220,123 +303,169 @@ cd_block_kernel(const CdBlockParams p)
             const float mid = 0.5f * (ms[q] + ms[q + 1]);
             return (mi[q] < mi[q + 1] || !(fabsf(mid) < CUDART_INF_F)) ? mid : nextafterf(mid, -CUDART_INF_F);
         };
-        thr_a = threshold(2 * l);
-        if (2 * l + 2 < CD_MAX_LEVELS) thr_b = threshold(2 * l + 1);
+        thr_s[cidx * CD_LEVEL_LD + 2 * l] = threshold(2 * l);
+        thr_s[cidx * CD_LEVEL_LD + 2 * l + 1] = 2 * l + 2 < CD_MAX_LEVELS ? threshold(2 * l + 1) : CUDART_INF_F;
     }
-    const float *my_levels = srt + cidx * CD_MAX_LEVELS;
-    __syncthreads();                                     // sidx (in the H buffer) has been read by everybody
+    __syncthreads();
+    (void)bounded_wait(smem_u32(&bar_tiles), 0u, wc, 20u, blockIdx.x);
 
-    load_h_chunk(0, 0);
-    h_chunk_wait();
+    constexpr int BAR_SUMS = 1, BAR_BAND = 2;
+    constexpr int SUMS_THREADS = 7 * 32, BAND_THREADS = CD_THREADS;
+    if (warp == 0) {
+        // ------------------------------------------------------------------ chain: the coordinates in order
+        float lev[LEV], thr[LEV];
+#pragma unroll
+        for (int q = 0; q < LEV; ++q) {
+            lev[q] = srt[lane * CD_LEVEL_LD + q];
+            thr[q] = thr_s[lane * CD_LEVEL_LD + q];
+        }
+#pragma unroll 1
+        for (int t = 0; t < CD_BANDS; ++t) {
+            wait_band(t);
+            const float *hd = Hs + (t % CD_H_BUFS) * CD_TILE_FLOATS + t * CD_BAND * CD_BAND;      // H[band][band]
+            float *wb = Ws + t * CD_BAND * CD_CH + lane, *eb = Es + t * CD_BAND * CD_CH + lane;
+            const float *rb = rds + t * CD_BAND;
+            ChainOperands first, second;                 // not written by the products: read while the sums are awaited
+            first.load<0>(hd, wb, rb);
+            second.load<1>(hd, wb, rb);
+            bar_sync_named(BAR_SUMS, SUMS_THREADS);
+            float Bu[CD_BAND];
+#pragma unroll
+            for (int q = 0; q < CD_BAND / 4; ++q) {
+                const float *sp = Ss + sums_at(lane, q);
+                float4 v[CD_PARTS];
+#pragma unroll
+                for (int n = 0; n < CD_PARTS; ++n) v[n] = *reinterpret_cast<const float4 *>(sp + n * CD_BAND * CD_CH);
+                Bu[4 * q + 0] = ((v[0].x + v[1].x) + (v[2].x + v[3].x)) + (v[4].x + v[5].x);
+                Bu[4 * q + 1] = ((v[0].y + v[1].y) + (v[2].y + v[3].y)) + (v[4].y + v[5].y);
+                Bu[4 * q + 2] = ((v[0].z + v[1].z) + (v[2].z + v[3].z)) + (v[4].z + v[5].z);
+                Bu[4 * q + 3] = ((v[0].w + v[1].w) + (v[2].w + v[3].w)) + (v[4].w + v[5].w);
+            }
+            chain_steps<LEV, 0>(first, second, hd, rb, wb, eb, Bu, lev, thr);
+            if (t + 1 < CD_BANDS) bar_arrive_named(BAR_BAND, BAND_THREADS);
+        }
+    } else if (warp == 4) {
+        // ------------------------------------------------------------------ loader
+        for (int t = 0; t + 1 < CD_BANDS; ++t) {
+            bar_sync_named(BAR_BAND, BAND_THREADS);      // band t's buffer is free
+            if (lane == 0 && t + CD_H_BUFS < CD_BANDS) load_band(t + CD_H_BUFS);
+        }
+    } else {
+        // ------------------------------------------------------------------ products: sums of band t
+        const int part = warp < 4 ? warp - 1 : warp - 2;                       // 0..5
+        const int r0 = (lane >> 3) * 8, c0 = (lane & 7) * 4;                   // 8 rows x 4 channels
+#pragma unroll 1
+        for (int t = 0; t < CD_BANDS; ++t) {
+            wait_band(t);
+            const float *hb = Hs + (t % CD_H_BUFS) * CD_TILE_FLOATS + r0;
+            const float *eb = Es + c0;
+            float acc[8][4];
+#pragma unroll
+            for (int a = 0; a < 8; ++a) {
+                const float4 v = part == 0 ? *reinterpret_cast<const float4 *>(Ps + (t * CD_BAND + r0 + a) * CD_CH + c0)
+                                           : make_float4(0.f, 0.f, 0.f, 0.f);
+                acc[a][0] = v.x; acc[a][1] = v.y; acc[a][2] = v.z; acc[a][3] = v.w;
+            }
+            auto add = [&](const float (&h)[8], const float4 &e) {
+#pragma unroll
+                for (int a = 0; a < 8; ++a) {
+                    acc[a][0] = fmaf(h[a], e.x, acc[a][0]);
+                    acc[a][1] = fmaf(h[a], e.y, acc[a][1]);
+                    acc[a][2] = fmaf(h[a], e.z, acc[a][2]);
+                    acc[a][3] = fmaf(h[a], e.w, acc[a][3]);
+                }
+            };
+            auto load_h = [&](int c, float (&h)[8]) {
+                const float4 lo = *reinterpret_cast<const float4 *>(hb + c * CD_BAND);
+                const float4 hi = *reinterpret_cast<const float4 *>(hb + c * CD_BAND + 4);
+                h[0] = lo.x; h[1] = lo.y; h[2] = lo.z; h[3] = lo.w;
+                h[4] = hi.x; h[5] = hi.y; h[6] = hi.z; h[7] = hi.w;
+            };
+            auto load_e = [&](int c) { return *reinterpret_cast<const float4 *>(eb + c * CD_CH); };
+            // `count` (even) coordinates of the block from `first` on, the next one's operands read ahead.  One copy of
+            // this loop serves every use: the chain's unrolled steps already fill most of the instruction cache.
+            auto add_rows = [&](int first, int count) {
+                float ha[8], hb2[8];
+                load_h(first, ha);
+                float4 ea = load_e(first), eb2;
+#pragma unroll 1
+                for (int c = first; c < first + count; c += 2) {
+                    load_h(c + 1, hb2);
+                    eb2 = load_e(c + 1);
+                    add(ha, ea);
+                    const int n = c + 2 < first + count ? c + 2 : first;
+                    load_h(n, ha);
+                    ea = load_e(n);
+                    add(hb2, eb2);
+                }
+            };
+            // n = 0: one band for each warp, neither the one the chain is working on (t - 1) nor this one; n = 1 (t = 0
+            // only): the one left over, shared by four warps; n = 2: band t - 1 once the chain is through with it, ditto
+#pragma unroll 1
+            for (int n = 0; n < 3; ++n) {
+                int first = (t == 0 ? part + 1 : part >= t - 1 ? part + 2 : part) * CD_BAND, count = CD_BAND;
+                if (n == 1) {
+                    first = 7 * CD_BAND + part * (CD_BAND / 4);
+                    count = t == 0 && part < 4 ? CD_BAND / 4 : 0;
+                    if (part >= 4) {
+                        // last cycle's values inside the band, coordinates after the row only: half a band each
+                        const int k0 = (part - 4) * (CD_BAND / 2);
+#pragma unroll 2
+                        for (int c = k0; c < k0 + CD_BAND / 2; ++c) {
+                            float h[8];
+                            load_h(t * CD_BAND + c, h);
+#pragma unroll
+                            for (int a = 0; a < 8; ++a) h[a] = r0 + a < c ? h[a] : 0.0f;
+                            add(h, load_e(t * CD_BAND + c));
+                        }
+                    }
+                } else if (n == 2) {
+                    if (t > 0) bar_sync_named(BAR_BAND, BAND_THREADS);
+                    first = (t - 1) * CD_BAND + part * (CD_BAND / 4);
+                    count = t > 0 && part < 4 ? CD_BAND / 4 : 0;
+                }
+                if (count > 0) add_rows(first, count);
+            }
+#pragma unroll
+            for (int b = 0; b < 4; ++b)
+#pragma unroll
+                for (int q = 0; q < 2; ++q)
+                    *reinterpret_cast<float4 *>(Ss + part * CD_BAND * CD_CH + sums_at(c0 + b, r0 / 4 + q)) =
+                        make_float4(acc[4 * q][b], acc[4 * q + 1][b], acc[4 * q + 2][b], acc[4 * q + 3][b]);
+            bar_arrive_named(BAR_SUMS, SUMS_THREADS);
+        }
+    }
     __syncthreads();
 
-    float Bu[8][4];
+    // ---- tiles out, four channels per thread; P is left zero for the next block's panel product
+    for (int idx = tid; idx < CD_BLOCK * CD_CH / 4; idx += CD_THREADS) {
+        const int r = idx >> 3, c = (idx & 7) * 4;
+        if (c >= ch_n) continue;
+        *reinterpret_cast<float4 *>(p.P + static_cast<size_t>(r) * p.d_out + ch0 + c) = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (r >= p.rows) continue;
+        const size_t o = static_cast<size_t>(p.s0 + r) * p.d_out + ch0 + c;
+        const float4 e4 = *reinterpret_cast<const float4 *>(Es + r * CD_CH + c);
+        const float e[4] = {e4.x, e4.y, e4.z, e4.w};
+        __align__(8) __nv_bfloat16 hi[4], lo[4];
 #pragma unroll
-    for (int t = 0; t < 8; ++t)
+        for (int b = 0; b < 4; ++b) split_bf16(e[b], hi[b], lo[b]);
+        *reinterpret_cast<float4 *>(p.Et + o) = e4;
+        *reinterpret_cast<uint2 *>(p.Ehi + o) = *reinterpret_cast<uint2 *>(hi);
+        *reinterpret_cast<uint2 *>(p.Elo + o) = *reinterpret_cast<uint2 *>(lo);
+        if (!p.last_cycle) continue;                     // the codes of earlier cycles are never read
+        const float4 v4 = *reinterpret_cast<const float4 *>(Ws + r * CD_CH + c);
+        const float v[4] = {v4.x, v4.y, v4.z, v4.w};
+        uint32_t codes = 0;
 #pragma unroll
-        for (int e = 0; e < 4; ++e) Bu[t][e] = Xs[(32 * t + 4 * l + e) * CD_TILE_LD + cidx];
-
-    // ---- pass 1: Bu[r] += sum_{c in block, c > r} H[c][r] * E_old[c]
-    // (The 32-row bands t are unrolled so that Bu is indexed statically; the rows inside a band are a real
-    // loop - unrolling all 256 steps makes the code larger than the instruction cache and ten times slower.)
+        for (int b = 0; b < 4; ++b) {
+            const float *ms = srt + (c + b) * CD_LEVEL_LD;
+            int pos = 0;                                 // first sorted level that is not below val: among equal ones the
 #pragma unroll
-    for (int t = 0; t < 8; ++t) {
-        if (t + 1 < 8) load_h_chunk((t + 1) * CD_HCHUNK, (t + 1) & 1);
-        const float *hc = Hs + (t & 1) * CD_HCHUNK * CD_BLOCK;
-#pragma unroll 1
-        for (int ii = 0; ii < 32; ++ii) {
-            const float ec = Es[(32 * t + ii) * CD_TILE_LD + cidx];
-#pragma unroll
-            for (int tp = 0; tp <= t; ++tp) {
-                const float4 h = *reinterpret_cast<const float4 *>(hc + ii * CD_BLOCK + 32 * tp + 4 * l);
-                if (tp < t) {
-                    Bu[tp][0] = fmaf(h.x, ec, Bu[tp][0]);
-                    Bu[tp][1] = fmaf(h.y, ec, Bu[tp][1]);
-                    Bu[tp][2] = fmaf(h.z, ec, Bu[tp][2]);
-                    Bu[tp][3] = fmaf(h.w, ec, Bu[tp][3]);
-                } else {                                  // same 32-row band: only rows before c
-                    if (4 * l + 0 < ii) Bu[tp][0] = fmaf(h.x, ec, Bu[tp][0]);
-                    if (4 * l + 1 < ii) Bu[tp][1] = fmaf(h.y, ec, Bu[tp][1]);
-                    if (4 * l + 2 < ii) Bu[tp][2] = fmaf(h.z, ec, Bu[tp][2]);
-                    if (4 * l + 3 < ii) Bu[tp][3] = fmaf(h.w, ec, Bu[tp][3]);
-                }
-            }
+            for (int step = LEV / 2; step > 0; step >>= 1)      // one with the smallest given index
+                if (ms[pos + step - 1] < v[b]) pos += step;
+            codes |= static_cast<uint32_t>(sidx[(c + b) * CD_LEVEL_LD + pos]) << (8 * b);
         }
-        h_chunk_wait();
-        __syncthreads();
-    }
-
-    // ---- pass 2: the coordinates in order
-    load_h_chunk(0, 0);
-    h_chunk_wait();
-    __syncthreads();
-#pragma unroll
-    for (int t = 0; t < 8; ++t) {
-        if (t + 1 < 8) load_h_chunk((t + 1) * CD_HCHUNK, (t + 1) & 1);
-        const float *hc = Hs + (t & 1) * CD_HCHUNK * CD_BLOCK;
-#pragma unroll 1
-        for (int i4 = 0; i4 < 32; i4 += 4) {
-            const int owner = i4 >> 2;                    // the thread that owns rows 32 t + i4 .. + 3
-            const bool after = l > owner, mine = l == owner;
-            const float4 h4[4] = {*reinterpret_cast<const float4 *>(hc + (i4 + 0) * CD_BLOCK + 32 * t + 4 * l),
-                                  *reinterpret_cast<const float4 *>(hc + (i4 + 1) * CD_BLOCK + 32 * t + 4 * l),
-                                  *reinterpret_cast<const float4 *>(hc + (i4 + 2) * CD_BLOCK + 32 * t + 4 * l),
-                                  *reinterpret_cast<const float4 *>(hc + (i4 + 3) * CD_BLOCK + 32 * t + 4 * l)};
-#pragma unroll
-            for (int oe = 0; oe < 4; ++oe) {
-                const int i = 32 * t + i4 + oe;
-                const float w = Ws[i * CD_TILE_LD + cidx];
-                const float target = __shfl_sync(0xffffffffu, w - rds[i] * Bu[t][oe], owner, CD_LANES);
-                // the thresholds ascend, so the number of thresholds below the target is the level's position
-                const unsigned below_a = __ballot_sync(0xffffffffu, target > thr_a);
-                const unsigned below_b = __ballot_sync(0xffffffffu, target > thr_b);
-                const int pos = __popc((below_a >> group_shift) & 0xffu) + __popc((below_b >> group_shift) & 0xffu);
-                const float val = my_levels[pos];
-                const float e_new = val - w;
-                if (mine) {
-                    Es[i * CD_TILE_LD + cidx] = e_new;
-                    Xs[i * CD_TILE_LD + cidx] = val;
-                }
-                // same band: only rows after i (a zero factor instead of a branch)
-                const float4 h = h4[oe];
-                const float e_after = after ? e_new : 0.0f, e_from = (after || mine) ? e_new : 0.0f;
-                Bu[t][0] = fmaf(h.x, 0 > oe ? e_from : e_after, Bu[t][0]);
-                Bu[t][1] = fmaf(h.y, 1 > oe ? e_from : e_after, Bu[t][1]);
-                Bu[t][2] = fmaf(h.z, 2 > oe ? e_from : e_after, Bu[t][2]);
-                Bu[t][3] = fmaf(h.w, 3 > oe ? e_from : e_after, Bu[t][3]);
-#pragma unroll
-                for (int tp = t + 1; tp < 8; ++tp) {      // later bands: all rows
-                    const float4 hh = *reinterpret_cast<const float4 *>(hc + (i4 + oe) * CD_BLOCK + 32 * tp + 4 * l);
-                    Bu[tp][0] = fmaf(hh.x, e_new, Bu[tp][0]);
-                    Bu[tp][1] = fmaf(hh.y, e_new, Bu[tp][1]);
-                    Bu[tp][2] = fmaf(hh.z, e_new, Bu[tp][2]);
-                    Bu[tp][3] = fmaf(hh.w, e_new, Bu[tp][3]);
-                }
-            }
-        }
-        h_chunk_wait();
-        __syncthreads();
-    }
-
-    // ---- tiles out
-    for (int idx = tid; idx < CD_BLOCK * CD_CH; idx += CD_THREADS) {
-        const int r = idx / CD_CH, c = idx % CD_CH;
-        if (r < p.rows && c < ch_n) {
-            const size_t o = static_cast<size_t>(p.s0 + r) * p.d_out + ch0 + c;
-            const float e = Es[r * CD_TILE_LD + c];
-            const float val = Xs[r * CD_TILE_LD + c];
-            int code = 0;                                 // first level, in the given order, with this value
-#pragma unroll
-            for (int q = CD_MAX_LEVELS - 1; q >= 0; --q)
-                if (cbs[c * CD_MAX_LEVELS + q] == val) code = q;
-            p.Et[o] = e;
-            p.Wht[o] = val;
-            p.Qt[o] = static_cast<uint8_t>(code);
-            __nv_bfloat16 hi, lo;
-            split_bf16(e, hi, lo);
-            p.Ehi[o] = hi;
-            p.Elo[o] = lo;
-        }
+        *reinterpret_cast<uint32_t *>(p.Qt + o) = codes;
     }
 }
 

@@ -140,8 +140,9 @@ int32_t device_info(DeviceInfo **out)
                                      cudaFuncAttributeMaxDynamicSharedMemorySize, gq::OBJ_SMEM_BYTES));
         GQ_CUDA(cudaFuncSetAttribute(gq::wide_gemm_kernel<gq::WG_FULL>, cudaFuncAttributeMaxDynamicSharedMemorySize, gq::WG_SMEM_BYTES));
         GQ_CUDA(cudaFuncSetAttribute(gq::gram_dot_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, gq::GD_SMEM_BYTES));
-        GQ_CUDA(cudaFuncSetAttribute(gq::cd_block_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     gq::CD_SMEM_BYTES));
+        GQ_CUDA(cudaFuncSetAttribute(gq::cd_block_kernel<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, gq::CD_SMEM_BYTES));
+        GQ_CUDA(cudaFuncSetAttribute(gq::cd_block_kernel<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, gq::CD_SMEM_BYTES));
+        GQ_CUDA(cudaFuncSetAttribute(gq::cd_block_kernel<16>, cudaFuncAttributeMaxDynamicSharedMemorySize, gq::CD_SMEM_BYTES));
         GQ_CUDA(cudaFuncSetAttribute(gq::hessian_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                      gq::HS_SMEM_BYTES));
         {
@@ -214,21 +215,28 @@ int32_t make_map(CUtensorMap *map, const void *base, int64_t features, int64_t r
     return GQ_OK;
 }
 
-// fp32 tensor [groups][d][d] as a TMA map with 32 x 32 boxes and the 128-byte swizzle (reduce-add target).
-int32_t make_map_h(CUtensorMap *map, float *H, int64_t d, int64_t groups)
+// fp32 tensor [groups][rows][cols] as a TMA map with boxes of 32 columns x `box_rows` rows.
+int32_t make_map_f32(CUtensorMap *map, const float *base, int64_t cols, int64_t rows, int64_t groups, int box_rows,
+                     CUtensorMapSwizzle swizzle)
 {
-    cuuint64_t dims[3] = {static_cast<cuuint64_t>(d), static_cast<cuuint64_t>(d), static_cast<cuuint64_t>(groups)};
-    cuuint64_t strides[2] = {static_cast<cuuint64_t>(d) * 4, static_cast<cuuint64_t>(d) * static_cast<cuuint64_t>(d) * 4};
-    cuuint32_t box[3] = {32, 32, 1};
+    cuuint64_t dims[3] = {static_cast<cuuint64_t>(cols), static_cast<cuuint64_t>(rows), static_cast<cuuint64_t>(groups)};
+    cuuint64_t strides[2] = {static_cast<cuuint64_t>(cols) * 4, static_cast<cuuint64_t>(cols) * static_cast<cuuint64_t>(rows) * 4};
+    cuuint32_t box[3] = {32, static_cast<cuuint32_t>(box_rows), 1};
     cuuint32_t estr[3] = {1, 1, 1};
-    CUresult r = g_encode(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, H, dims, strides, box, estr,
-                          CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_NONE,
+    CUresult r = g_encode(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, const_cast<float *>(base), dims, strides, box, estr,
+                          CU_TENSOR_MAP_INTERLEAVE_NONE, swizzle, CU_TENSOR_MAP_L2_PROMOTION_NONE,
                           CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     if (r != CUDA_SUCCESS) {
         tl_last_cuda_error = static_cast<int32_t>(cudaErrorInvalidValue);
         return GQ_ERR_CUDA;
     }
     return GQ_OK;
+}
+
+// H [groups][d][d] with 32 x 32 boxes and the 128-byte swizzle (reduce-add target).
+int32_t make_map_h(CUtensorMap *map, float *H, int64_t d, int64_t groups)
+{
+    return make_map_f32(map, H, d, d, groups, 32, CU_TENSOR_MAP_SWIZZLE_128B);
 }
 
 int grid_for(long long work_items, int threads, int sm_count, int blocks_per_sm)
@@ -361,7 +369,7 @@ CodebookLayout codebook_layout(int64_t d_in, int64_t d_out, int32_t g, int32_t m
 }
 
 struct CdLayout {
-    size_t wt, wht, et, ehi, elo, hhi, hlo, rdiag, p, qt, total;
+    size_t wt, et, ehi, elo, hhi, hlo, rdiag, p, qt, total;
 };
 CdLayout cd_layout(int64_t d_in, int64_t d_out, int32_t g)
 {
@@ -371,7 +379,6 @@ CdLayout cd_layout(int64_t d_in, int64_t d_out, int32_t g)
     const size_t h2 = round_up(static_cast<size_t>(g) * d_in * d_in * 2, 1024);
     size_t o = 0;
     L.wt = o; o += mat4;
-    L.wht = o; o += mat4;
     L.et = o; o += mat4;
     L.ehi = o; o += mat2;
     L.elo = o; o += mat2;
@@ -940,9 +947,12 @@ int32_t gq_cd_cycles(const float *W, float *W_hat, uint8_t *Q, const float *code
     DeviceInfo *di;
     if (int32_t rc = device_info(&di)) return rc;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
+    if (cycles == 0) {                                   // W_hat stays as it is, no code has been chosen
+        GQ_CUDA(cudaMemsetAsync(Q, 0, static_cast<size_t>(d_out) * d_in, st));
+        return GQ_OK;
+    }
     uint8_t *ws = static_cast<uint8_t *>(workspace);
     float *Wt = reinterpret_cast<float *>(ws + L.wt);
-    float *Wht = reinterpret_cast<float *>(ws + L.wht);
     float *Et = reinterpret_cast<float *>(ws + L.et);
     __nv_bfloat16 *Ehi = reinterpret_cast<__nv_bfloat16 *>(ws + L.ehi);
     __nv_bfloat16 *Elo = reinterpret_cast<__nv_bfloat16 *>(ws + L.elo);
@@ -955,15 +965,14 @@ int32_t gq_cd_cycles(const float *W, float *W_hat, uint8_t *Q, const float *code
     const dim3 tgrid(static_cast<unsigned>((d_in + 31) / 32), static_cast<unsigned>((d_out + 31) / 32));
     {
         LaunchScope scope(GQ_KERNEL_CD_AUX, st);
-        gq::cd_prepare_kernel<<<tgrid, 256, 0, st>>>(W, W_hat, static_cast<int>(d_in), static_cast<int>(d_out), Wt, Wht,
+        gq::cd_prepare_kernel<<<tgrid, 256, 0, st>>>(W, W_hat, static_cast<int>(d_in), static_cast<int>(d_out), Wt,
                                                      Et, Ehi, Elo);
     }
     GQ_CUDA(cudaGetLastError());
     {
-        const long long count = static_cast<long long>(g) * d_in * d_in;
+        const dim3 hgrid(static_cast<unsigned>(d_in), static_cast<unsigned>(g));
         LaunchScope scope(GQ_KERNEL_CD_AUX, st);
-        gq::cd_split_h_kernel<<<grid_for(count, 256, di->sm_count, 8), 256, 0, st>>>(H, count, static_cast<int>(d_in), Hhi,
-                                                                                 Hlo, rdiag);
+        gq::cd_split_h_kernel<<<hgrid, 256, 0, st>>>(H, static_cast<int>(d_in), Hhi, Hlo, rdiag);
     }
     GQ_CUDA(cudaGetLastError());
 
@@ -972,6 +981,12 @@ int32_t gq_cd_cycles(const float *W, float *W_hat, uint8_t *Q, const float *code
     if (int32_t rc = make_map(&mapHlo, Hlo, d_in, d_in, g, d_in, d_in * d_in)) return rc;
     if (int32_t rc = make_map(&mapEhi, Ehi, d_out, d_in, 1, d_out, d_in * d_out)) return rc;
     if (int32_t rc = make_map(&mapElo, Elo, d_out, d_in, 1, d_out, d_in * d_out)) return rc;
+    CUtensorMap mapHb, mapWb, mapEb, mapPb;              // fp32 tiles of the block kernel
+    if (int32_t rc = make_map_f32(&mapHb, H, d_in, d_in, g, gq::CD_BLOCK, CU_TENSOR_MAP_SWIZZLE_NONE)) return rc;
+    if (int32_t rc = make_map_f32(&mapWb, Wt, d_out, d_in, 1, gq::CD_BLOCK, CU_TENSOR_MAP_SWIZZLE_NONE)) return rc;
+    if (int32_t rc = make_map_f32(&mapEb, Et, d_out, d_in, 1, gq::CD_BLOCK, CU_TENSOR_MAP_SWIZZLE_NONE)) return rc;
+    if (int32_t rc = make_map_f32(&mapPb, P, d_out, gq::CD_BLOCK, 1, gq::CD_BLOCK, CU_TENSOR_MAP_SWIZZLE_NONE)) return rc;
+    GQ_CUDA(cudaMemsetAsync(P, 0, static_cast<size_t>(gq::CD_BLOCK) * d_out * sizeof(float), st));   // the block kernel leaves it zero
     const int kblocks = static_cast<int>((d_in + gq::TILE_K - 1) / gq::TILE_K);
     const int ch_tiles = static_cast<int>((mk + gq::TILE_N - 1) / gq::TILE_N);
     const int slices = static_cast<int>((mk + gq::CD_CH - 1) / gq::CD_CH);
@@ -981,7 +996,6 @@ int32_t gq_cd_cycles(const float *W, float *W_hat, uint8_t *Q, const float *code
             const int rows = static_cast<int>(d_in - s0 < gq::CD_BLOCK ? d_in - s0 : gq::CD_BLOCK);
             const int blk_ksteps = (rows + gq::TILE_K - 1) / gq::TILE_K;
             const int nk = kblocks - blk_ksteps;
-            GQ_CUDA(cudaMemsetAsync(P, 0, static_cast<size_t>(gq::CD_BLOCK) * d_out * sizeof(float), st));
             if (nk > 0) {
                 gq::PairGemmParams pp{};
                 pp.d = static_cast<int>(d_in);
@@ -1016,20 +1030,25 @@ int32_t gq_cd_cycles(const float *W, float *W_hat, uint8_t *Q, const float *code
                 GQ_CUDA(cudaGetLastError());
             }
             gq::CdBlockParams bp{};
-            bp.H = H; bp.rdiag = rdiag; bp.P = P; bp.Wt = Wt; bp.codebook = codebook; bp.Wht = Wht; bp.Et = Et;
+            bp.rdiag = rdiag; bp.P = P; bp.codebook = codebook; bp.Et = Et;
             bp.Ehi = Ehi; bp.Elo = Elo; bp.Qt = Qt;
             bp.d_in = static_cast<int>(d_in); bp.d_out = static_cast<int>(d_out); bp.g = g; bp.mk = static_cast<int>(mk);
             bp.m = m; bp.s0 = static_cast<int>(s0); bp.rows = rows; bp.slices = slices;
+            bp.last_cycle = cyc + 1 == cycles;
+            bp.status = di->status_ptr;
+            bp.wait_budget_ns = wait_budget_ns();
             {
                 LaunchScope scope(GQ_KERNEL_CD_BLOCK, st);
-                gq::cd_block_kernel<<<g * slices, gq::CD_THREADS, gq::CD_SMEM_BYTES, st>>>(bp);
+                // fewer levels, fewer compares and selects per coordinate
+                const auto kernel = m <= 4 ? gq::cd_block_kernel<4> : m <= 8 ? gq::cd_block_kernel<8> : gq::cd_block_kernel<16>;
+                kernel<<<g * slices, gq::CD_THREADS, gq::CD_SMEM_BYTES, st>>>(mapHb, mapWb, mapEb, mapPb, bp);
             }
             GQ_CUDA(cudaGetLastError());
         }
     }
     {
         LaunchScope scope(GQ_KERNEL_CD_AUX, st);
-        gq::cd_finish_kernel<<<tgrid, 256, 0, st>>>(Wht, Qt, static_cast<int>(d_in), static_cast<int>(d_out), W_hat, Q);
+        gq::cd_finish_kernel<<<tgrid, 256, 0, st>>>(codebook, Qt, static_cast<int>(d_in), static_cast<int>(d_out), m, W_hat, Q);
     }
     GQ_CUDA(cudaGetLastError());
     return GQ_OK;

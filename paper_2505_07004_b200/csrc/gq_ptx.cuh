@@ -135,6 +135,15 @@ __device__ __forceinline__ void tma_load_3d_pair(uint32_t smem_dst, const void *
         : "memory");
 }
 
+// 3-D tiled load global -> this CTA's shared memory, bytes counted on this CTA's mbarrier `bar` (no CTA pair involved).
+__device__ __forceinline__ void tma_load_3d(uint32_t smem_dst, const void *map, uint32_t bar, int32_t c0, int32_t c1, int32_t c2)
+{
+    asm volatile(
+        "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5}], [%2];"
+        ::"r"(smem_dst), "l"(reinterpret_cast<uint64_t>(map)), "r"(bar), "r"(c0), "r"(c1), "r"(c2)
+        : "memory");
+}
+
 // 3-D tiled reduce-add shared memory -> global: every element of the box is added to the tensor in
 // global memory by the memory system.  Part of the calling thread's current bulk async-group.
 // c0 times the element size must be a multiple of 16 bytes and no coordinate may be negative.
