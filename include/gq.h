@@ -352,8 +352,8 @@ int32_t gq_check(void *stream, uint32_t *detail /* HOST, may be NULL */);
  * Same shape rules as gq_objective.
  * Arithmetic: H_k W_k^T and H_k [P^(j) ...] are formed on the tensor cores, fp32 accumulation, from bf16
  * hi + lo splits of H and W (16 significant bits per factor; what is dropped is of the size of the fp32
- * accumulation error; the one-hot columns are exact).  The sums over the rows of each level and the m x m
- * Cholesky solves are fp64.
+ * accumulation error; the one-hot columns are exact).  The sums over the rows of each level are fp32 over 128
+ * rows and fp64 beyond (atomic adds: runs agree to the last bits), the m x m Cholesky solves fp64.
  * Together with gq_cd_cycles and gq_objective this is Algorithm 2: repeat { gq_codebook_update (with W_hat);
  * gq_cd_cycles } T times, then gq_codebook_update once more.
  */

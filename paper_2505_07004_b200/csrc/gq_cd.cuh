@@ -75,11 +75,12 @@ cd_prepare_kernel(const float *__restrict__ W, const float *__restrict__ What, i
     }
 }
 
-// H -> bf16 hi + lo (operands of the panel product) and rdiag[k][i] = 1 / H_k[i][i] (0 where H_ii <= 0).  One block
-// per row of a group's matrix, 16-byte loads (d_in is a multiple of 8): bound by the 8 bytes per entry it moves.  With
-// one entry per thread and a 64-bit modulo each to find the diagonal it took 342 us for four 4096 x 4096 matrices, now 79.
+// H -> bf16 hi + lo and rdiag[k][i] = 1 / H_k[i][i] (0 where H_ii <= 0), for the panel products here and for the codebook
+// step (gq_codebook_gemm.cuh).  One block per row of a group's matrix, 16-byte loads (d_in is a multiple of 8): bound by the
+// 8 bytes per entry it moves.  With one entry per thread and a 64-bit modulo each to find the diagonal it took 342 us for
+// four 4096 x 4096 matrices, now 79.
 __global__ void __launch_bounds__(256)
-cd_split_h_kernel(const float *__restrict__ H, int d_in, __nv_bfloat16 *__restrict__ Hhi, __nv_bfloat16 *__restrict__ Hlo,
+split_h_kernel(const float *__restrict__ H, int d_in, __nv_bfloat16 *__restrict__ Hhi, __nv_bfloat16 *__restrict__ Hlo,
                   float *__restrict__ rdiag)
 {
     const int i = static_cast<int>(blockIdx.x);

@@ -3,17 +3,8 @@
 //
 //     c^(j) = (P^T H_k P + lambda I)^-1  P^T H_k w_j .
 //
-// The two d_in^2-sized contractions run on the tensor cores (pair_gemm_kernel<MODE_FULL>):
-//     HW = H_k W_k^T                      [d_in x channels]
-//     HP = H_k [P^(j0) ... P^(j0+c-1)]    [d_in x (channels * m)]   for a slab of channels at a time
-// with H and W as bf16 hi + lo pairs (16 significant bits, what is dropped is below 2^-16 of each entry: the
-// size of the fp32 accumulation error of these 4096-long sums); accumulation is fp32.  HW takes
-// hi hi + hi lo + lo hi; HP, where the one-hot columns are exact in bf16, the two terms of H.  (Three-way
-// splits that reproduce the fp32 values exactly were measured to change the codebooks by less than the
-// difference to the fp64 oracle that remains either way.)
-// The kernels here prepare those operands, fold HP and HW over the rows of each level (fp64),
-//     G^(j)[q][q'] = sum_{i : Q_ij = q} HP[i][j m + q'],      r^(j)[q] = sum_{i : Q_ij = q} HW[i][j],
-// and solve the m x m systems by Cholesky in fp64.
+// The d_in^2-sized contractions and their sums by level are one tensor-core kernel (gq_codebook_gemm.cuh).  The kernels
+// here prepare its W operand, solve the m x m systems by Cholesky in fp64 and write W_hat.
 #pragma once
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
@@ -22,271 +13,93 @@
 namespace gq {
 
 constexpr int CB_MAX_LEVELS = 16;
-constexpr int CB_SLAB_CHANNELS = 1024;      // channels whose one-hot columns are multiplied at a time
 
-// v = t0 + t1 up to 2^-17 |v|: round to bf16, round the remainder to bf16.
-__device__ __forceinline__ void split2_bf16(float v, __nv_bfloat16 &t0, __nv_bfloat16 &t1)
-{
-    t0 = __float2bfloat16_rn(v);
-    t1 = __float2bfloat16_rn(v - __bfloat162float(t0));
-}
-
+// W [d_out][d_in] -> bf16 hi + lo of W^T [d_in][d_out] (lo = what hi leaves, 2^-17 |w| is dropped).  Tiles of 32
+// coordinates x 64 channels, so that both sides move whole 128-byte segments (one bf16 per lane and 64-byte segments took
+// 57 us for 4096 x 4096 where the bytes need 20).
 __global__ void __launch_bounds__(256)
-cb_split2_kernel(const float *__restrict__ src, long long count, __nv_bfloat16 *__restrict__ d0,
-                 __nv_bfloat16 *__restrict__ d1)
+cb_transpose_kernel(const float *__restrict__ W, int d_in, int d_out, __nv_bfloat16 *__restrict__ W0, __nv_bfloat16 *__restrict__ W1)
 {
-    const long long stride = static_cast<long long>(gridDim.x) * blockDim.x;
-    for (long long idx = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x; idx < count; idx += stride) {
-        __nv_bfloat16 a, b;
-        split2_bf16(src[idx], a, b);
-        d0[idx] = a;
-        d1[idx] = b;
-    }
-}
-
-// W [d_out][d_in] -> bf16 hi + lo of W^T [d_in][d_out]; Q [d_out][d_in] -> Qt [d_in][d_out].  32 x 32 tiles.
-__global__ void __launch_bounds__(256)
-cb_transpose_kernel(const float *__restrict__ W, const uint8_t *__restrict__ Q, int d_in, int d_out,
-                    __nv_bfloat16 *__restrict__ W0, __nv_bfloat16 *__restrict__ W1, uint8_t *__restrict__ Qt)
-{
-    __shared__ float tw[32][33];
-    __shared__ uint8_t tq[32][33];
+    __shared__ float tw[64][33];
     const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
-    const int i0 = blockIdx.x * 32, j0 = blockIdx.y * 32;
-    for (int r = ty; r < 32; r += 8) {
-        const int j = j0 + r, i = i0 + tx;
-        const bool ok = j < d_out && i < d_in;
-        tw[r][tx] = ok ? W[static_cast<size_t>(j) * d_in + i] : 0.0f;
-        tq[r][tx] = ok ? Q[static_cast<size_t>(j) * d_in + i] : 0;
+    const int i0 = blockIdx.x * 32, j0 = blockIdx.y * 64;
+#pragma unroll
+    for (int r = 0; r < 64; r += 8) {
+        const int j = j0 + r + ty, i = i0 + tx;
+        tw[r + ty][tx] = (j < d_out && i < d_in) ? W[static_cast<size_t>(j) * d_in + i] : 0.0f;
     }
     __syncthreads();
-    for (int r = ty; r < 32; r += 8) {
-        const int i = i0 + r, j = j0 + tx;
+#pragma unroll
+    for (int r = 0; r < 32; r += 8) {
+        const int i = i0 + r + ty, j = j0 + 2 * tx;          // d_out is a multiple of 8: pairs are inside or outside
         if (i < d_in && j < d_out) {
+            const float a = tw[2 * tx][r + ty], b = tw[2 * tx + 1][r + ty];
+            const __nv_bfloat162 hi = __floats2bfloat162_rn(a, b);
+            const __nv_bfloat162 lo = __floats2bfloat162_rn(a - __low2float(hi), b - __high2float(hi));
             const size_t o = static_cast<size_t>(i) * d_out + j;
-            __nv_bfloat16 a, b;
-            split2_bf16(tw[tx][r], a, b);
-            W0[o] = a;
-            W1[o] = b;
-            Qt[o] = tq[tx][r];
+            *reinterpret_cast<__nv_bfloat162 *>(W0 + o) = hi;
+            *reinterpret_cast<__nv_bfloat162 *>(W1 + o) = lo;
         }
     }
 }
 
-// One-hot columns of channels [j0, j0 + nch): Pm[i][jj * m + q] = (Qt[i][j0 + jj] == q), bf16, row stride ld.
-// One thread writes the m columns of one (row, channel); with m = 16 and ld a multiple of 8 that is two
-// 16-byte stores, and consecutive threads write consecutive 32-byte pieces.
-__global__ void __launch_bounds__(256)
-cb_onehot_kernel(const uint8_t *__restrict__ Qt, int d_in, int d_out, int j0, int nch, int m,
-                 __nv_bfloat16 *__restrict__ Pm, long long ld)
-{
-    const long long total = static_cast<long long>(d_in) * nch;
-    const long long stride = static_cast<long long>(gridDim.x) * blockDim.x;
-    const bool wide = m == 16 && (ld & 7) == 0;
-    for (long long idx = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x; idx < total; idx += stride) {
-        const int i = static_cast<int>(idx / nch);
-        const int jj = static_cast<int>(idx - static_cast<long long>(i) * nch);
-        int code = Qt[static_cast<size_t>(i) * d_out + j0 + jj];
-        code = code < m ? code : m - 1;
-        __nv_bfloat16 *dst = Pm + static_cast<size_t>(i) * ld + static_cast<size_t>(jj) * m;
-        if (wide) {
-            uint32_t w[8];
-#pragma unroll
-            for (int t = 0; t < 8; ++t)            // bf16 1.0 = 0x3F80 in the low or the high half of word t
-                w[t] = (code >> 1) == t ? ((code & 1) ? 0x3F800000u : 0x00003F80u) : 0u;
-            uint4 *d4 = reinterpret_cast<uint4 *>(dst);
-            d4[0] = make_uint4(w[0], w[1], w[2], w[3]);
-            d4[1] = make_uint4(w[4], w[5], w[6], w[7]);
-        } else {
-            for (int q = 0; q < m; ++q) dst[q] = __float2bfloat16_rn(q == code ? 1.0f : 0.0f);
-        }
-    }
-}
-
-// Fold over the rows of each level.  One CTA = CB_FOLD_CH channels of the slab x 16 threads x one of gridDim.y
-// row ranges; thread (ch, q') owns column q' of G^(ch) in shared memory, so no two threads of a CTA ever add
-// to the same word; thread q' = 0 also owns r.  Within a row range (a few hundred rows, a few dozen per level)
-// the sums are fp32 and use shared-memory reductions whose results are not read back, so that nothing in the
-// row loop waits for an addition; the row ranges are combined in fp64 with atomic adds (the order of at most
-// gridDim.y fp64 partial sums is the only thing that can vary from run to run).
-constexpr int CB_FOLD_CH = 16;
-__global__ void __launch_bounds__(CB_FOLD_CH * 16)
-cb_fold_kernel(const float *__restrict__ HP, long long ld_hp, const float *__restrict__ HW, const uint8_t *__restrict__ Qt,
-               int d_in, int d_out, int j0, int nch, int m, double *__restrict__ G, double *__restrict__ R)
-{
-    __shared__ float Gs[CB_FOLD_CH][CB_MAX_LEVELS][CB_MAX_LEVELS + 1];
-    __shared__ float Rs[CB_FOLD_CH][CB_MAX_LEVELS];
-    const int ch = threadIdx.x >> 4, qp = threadIdx.x & 15;
-    const int jj = blockIdx.x * CB_FOLD_CH + ch;
-    for (int q = 0; q < CB_MAX_LEVELS; ++q) Gs[ch][q][qp] = 0.0f;
-    Rs[ch][qp] = 0.0f;
-    __syncthreads();
-    if (jj < nch && qp < m) {
-        const int j = j0 + jj;
-        const float *hp = HP + static_cast<size_t>(jj) * m + qp;
-        constexpr int BATCH = 8;                         // independent loads in flight per thread
-        const int rows_per = (d_in + static_cast<int>(gridDim.y) - 1) / static_cast<int>(gridDim.y);
-        const int i_begin = static_cast<int>(blockIdx.y) * rows_per;
-        const int i_end = i_begin + rows_per < d_in ? i_begin + rows_per : d_in;
-        for (int i0 = i_begin; i0 < i_end; i0 += BATCH) {
-            int q[BATCH];
-            float v[BATCH], w[BATCH];
-#pragma unroll
-            for (int t = 0; t < BATCH; ++t) {
-                const int i = i0 + t;
-                const bool ok = i < i_end;
-                q[t] = ok ? Qt[static_cast<size_t>(i) * d_out + j] : 0;
-                v[t] = ok ? hp[static_cast<size_t>(i) * ld_hp] : 0.0f;
-                w[t] = (ok && qp == 0) ? HW[static_cast<size_t>(i) * d_out + j] : 0.0f;
-            }
-#pragma unroll
-            for (int t = 0; t < BATCH; ++t) {
-                const int qq = q[t] < m ? q[t] : m - 1;  // codes are expected to be < m
-                atomicAdd(&Gs[ch][qq][qp], v[t]);
-                if (qp == 0) atomicAdd(&Rs[ch][qq], w[t]);
-            }
-        }
-    }
-    __syncthreads();
-    if (jj < nch && qp < m) {                        // G and R were zeroed by the host; row ranges add up
-        const int j = j0 + jj;
-        for (int q = 0; q < m; ++q)
-            atomicAdd(&G[(static_cast<size_t>(j) * CB_MAX_LEVELS + q) * CB_MAX_LEVELS + qp], static_cast<double>(Gs[ch][q][qp]));
-        atomicAdd(&R[static_cast<size_t>(j) * CB_MAX_LEVELS + qp], static_cast<double>(Rs[ch][qp]));
-    }
-}
-
-// The same fold for m a multiple of 4 (the usual 2-, 3- and 4-bit codebooks have m = 4, 8, 16): a thread takes
-// four neighbouring columns q' of one channel with one 16-byte load per row, so the row loop spends its
-// instructions on the data rather than on addresses (the one-column form above is issue-bound).  One CTA =
-// CB_FOLD4_CH channels x 4 threads.
-constexpr int CB_FOLD4_CH = 32;
-__global__ void __launch_bounds__(CB_FOLD4_CH * 4)
-cb_fold4_kernel(const float *__restrict__ HP, long long ld_hp, const float *__restrict__ HW, const uint8_t *__restrict__ Qt,
-                int d_in, int d_out, int j0, int nch, int m, double *__restrict__ G, double *__restrict__ R)
-{
-    __shared__ float Gs[CB_FOLD4_CH][CB_MAX_LEVELS][CB_MAX_LEVELS + 1];
-    __shared__ float Rs[CB_FOLD4_CH][CB_MAX_LEVELS];
-    const int ch = threadIdx.x >> 2, q4 = (threadIdx.x & 3) * 4;
-    const int jj = blockIdx.x * CB_FOLD4_CH + ch;
-    for (int q = 0; q < CB_MAX_LEVELS; ++q)
-        for (int e = 0; e < 4; ++e) Gs[ch][q][q4 + e] = 0.0f;
-    for (int e = 0; e < 4; ++e) Rs[ch][q4 + e] = 0.0f;
-    __syncthreads();
-    const bool active = jj < nch && q4 < m;
-    if (active) {
-        const int j = j0 + jj;
-        constexpr int BATCH = 8;                         // independent loads in flight per thread
-        const int rows_per = (d_in + static_cast<int>(gridDim.y) - 1) / static_cast<int>(gridDim.y);
-        const int i_begin = static_cast<int>(blockIdx.y) * rows_per;
-        const int i_end = i_begin + rows_per < d_in ? i_begin + rows_per : d_in;
-        const float *hp = HP + static_cast<size_t>(i_begin) * ld_hp + static_cast<size_t>(jj) * m + q4;
-        const uint8_t *qt = Qt + static_cast<size_t>(i_begin) * d_out + j;
-        const float *hw = HW + static_cast<size_t>(i_begin) * d_out + j;
-        float *gbase = &Gs[ch][0][q4];
-        int i0 = i_begin;
-        for (; i0 + BATCH <= i_end; i0 += BATCH) {       // whole batches: no row predicates
-            int q[BATCH];
-            float4 v[BATCH];
-            float w[BATCH];
-#pragma unroll
-            for (int t = 0; t < BATCH; ++t) {
-                q[t] = qt[static_cast<size_t>(t) * d_out];
-                v[t] = *reinterpret_cast<const float4 *>(hp + static_cast<size_t>(t) * ld_hp);
-                w[t] = q4 == 0 ? hw[static_cast<size_t>(t) * d_out] : 0.0f;
-            }
-#pragma unroll
-            for (int t = 0; t < BATCH; ++t) {
-                const int qq = q[t] < m ? q[t] : m - 1;  // codes are expected to be < m
-                float *gp = gbase + qq * (CB_MAX_LEVELS + 1);
-                atomicAdd(gp + 0, v[t].x);
-                atomicAdd(gp + 1, v[t].y);
-                atomicAdd(gp + 2, v[t].z);
-                atomicAdd(gp + 3, v[t].w);
-                if (q4 == 0) atomicAdd(&Rs[ch][qq], w[t]);
-            }
-            hp += static_cast<size_t>(BATCH) * ld_hp;
-            qt += static_cast<size_t>(BATCH) * d_out;
-            hw += static_cast<size_t>(BATCH) * d_out;
-        }
-        for (; i0 < i_end; ++i0) {                       // ragged end of the row range
-            const int qr = *qt;
-            const int qq = qr < m ? qr : m - 1;
-            const float4 v = *reinterpret_cast<const float4 *>(hp);
-            float *gp = gbase + qq * (CB_MAX_LEVELS + 1);
-            atomicAdd(gp + 0, v.x);
-            atomicAdd(gp + 1, v.y);
-            atomicAdd(gp + 2, v.z);
-            atomicAdd(gp + 3, v.w);
-            if (q4 == 0) atomicAdd(&Rs[ch][qq], *hw);
-            hp += ld_hp;
-            qt += d_out;
-            hw += d_out;
-        }
-    }
-    __syncthreads();
-    if (active) {                                    // G and R were zeroed by the host; row ranges add up
-        const int j = j0 + jj;
-        for (int q = 0; q < m; ++q)
-            for (int e = 0; e < 4; ++e)
-                atomicAdd(&G[(static_cast<size_t>(j) * CB_MAX_LEVELS + q) * CB_MAX_LEVELS + q4 + e],
-                          static_cast<double>(Gs[ch][q][q4 + e]));
-        for (int e = 0; e < 4; ++e)
-            atomicAdd(&R[static_cast<size_t>(j) * CB_MAX_LEVELS + q4 + e], static_cast<double>(Rs[ch][q4 + e]));
-    }
-}
-
-// (G + lambda I) c = r by Cholesky, one thread per channel, fp64; G is symmetrised first (its two triangles
-// come from different sums).  A pivot that is not positive (possible only through rounding) is replaced by
-// lambda-sized regularisation so that the solve always completes.
+// (G + lambda I) c = r by Cholesky in fp64; G is symmetrised first (its two triangles come from different sums).  Sixteen lanes per channel, lane q holds row q (rows from m on
+// are those of the identity).  A pivot that is not positive (possible only through rounding) is replaced by lambda-sized
+// regularisation so that the solve always completes.  With one thread per channel and its matrix in local memory 4096
+// channels took 89 us.
 __global__ void __launch_bounds__(128)
 cb_solve_kernel(const double *__restrict__ G, const double *__restrict__ R, int d_out, int m, double lambda,
                 float *__restrict__ codebook)
 {
-    const int j = blockIdx.x * blockDim.x + threadIdx.x;
-    if (j >= d_out) return;
-    double A[CB_MAX_LEVELS][CB_MAX_LEVELS];
-    double b[CB_MAX_LEVELS];
-    const double *g = G + static_cast<size_t>(j) * CB_MAX_LEVELS * CB_MAX_LEVELS;
-    for (int q = 0; q < m; ++q) {
-        for (int p = 0; p <= q; ++p) A[q][p] = 0.5 * (g[q * CB_MAX_LEVELS + p] + g[p * CB_MAX_LEVELS + q]);
-        A[q][q] += lambda;
-        b[q] = R[static_cast<size_t>(j) * CB_MAX_LEVELS + q];
+    constexpr int M = CB_MAX_LEVELS;
+    const int q = threadIdx.x & 15;
+    const int jj = blockIdx.x * 8 + (threadIdx.x >> 4);
+    const int j = jj < d_out ? jj : d_out - 1;           // all lanes take part in the shuffles
+    const double *g = G + static_cast<size_t>(j) * M * M;
+    double a[M], b = q < m ? R[static_cast<size_t>(j) * M + q] : 0.0, diag = 1.0;
+#pragma unroll
+    for (int t = 0; t < M; ++t) {
+        a[t] = (q < m && t < m) ? 0.5 * (g[q * M + t] + g[t * M + q]) : 0.0;
+        if (t == q) a[t] = q < m ? a[t] + lambda : 1.0;
     }
-    for (int q = 0; q < m; ++q) {                 // A = L L^T, L stored in the lower triangle
-        for (int p = 0; p < q; ++p) {
-            double v = A[q][p];
-            for (int t = 0; t < p; ++t) v -= A[q][t] * A[p][t];
-            A[q][p] = v / A[p][p];
-        }
-        double d = A[q][q];
-        for (int t = 0; t < q; ++t) d -= A[q][t] * A[q][t];
+    auto from = [](double v, int lane) { return __shfl_sync(0xffffffffu, v, lane, 16); };
+#pragma unroll
+    for (int t = 0; t < M; ++t) {                        // column t of L; a[t] of lane q > t becomes L[q][t]
+        double d = from(a[t], t);
         if (!(d > 0.0)) d = lambda > 0.0 ? lambda : 1e-300;
-        A[q][q] = sqrt(d);
+        const double root = sqrt(d);
+        if (q == t) diag = root;
+        const double l = q > t ? a[t] / root : 0.0;
+        a[t] = l;
+#pragma unroll
+        for (int s = t + 1; s < M; ++s) a[s] -= l * from(l, s);
+        const double y = from(b, t) / root;              // L y = r alongside
+        b = q == t ? y : b - l * y;
     }
-    for (int q = 0; q < m; ++q) {                 // L y = b
-        double v = b[q];
-        for (int t = 0; t < q; ++t) v -= A[q][t] * b[t];
-        b[q] = v / A[q][q];
+#pragma unroll
+    for (int t = M - 1; t >= 0; --t) {                   // L^T c = y
+        double sum = q > t ? a[t] * b : 0.0;             // lanes above t hold their c already
+#pragma unroll
+        for (int off = 8; off > 0; off >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, off, 16);
+        if (q == t) b = (b - sum) / diag;
     }
-    for (int q = m - 1; q >= 0; --q) {            // L^T c = y
-        double v = b[q];
-        for (int t = q + 1; t < m; ++t) v -= A[t][q] * b[t];
-        b[q] = v / A[q][q];
-    }
-    for (int q = 0; q < m; ++q) codebook[static_cast<size_t>(j) * m + q] = static_cast<float>(b[q]);
+    if (jj < d_out && q < m) codebook[static_cast<size_t>(j) * m + q] = static_cast<float>(b);
 }
 
-// What[j][i] = codebook[j][Q[j][i]]
+// What[j][i] = codebook[j][Q[j][i]], one block per channel, four codes per thread.  Q 4-byte aligned.
 __global__ void __launch_bounds__(256)
-cb_apply_kernel(const float *__restrict__ codebook, const uint8_t *__restrict__ Q, long long count, int d_in, int m,
-                float *__restrict__ What)
+cb_apply_kernel(const float *__restrict__ codebook, const uint8_t *__restrict__ Q, int d_in, int m, float *__restrict__ What)
 {
-    const long long stride = static_cast<long long>(gridDim.x) * blockDim.x;
-    for (long long idx = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x; idx < count; idx += stride) {
-        const long long j = idx / d_in;
-        const int q = Q[idx];
-        What[idx] = codebook[j * m + (q < m ? q : m - 1)];
+    __shared__ float cb[CB_MAX_LEVELS];
+    const size_t j = blockIdx.x;
+    if (threadIdx.x < m) cb[threadIdx.x] = codebook[j * m + threadIdx.x];
+    __syncthreads();
+    const uchar4 *src = reinterpret_cast<const uchar4 *>(Q + j * d_in);
+    float4 *dst = reinterpret_cast<float4 *>(What + j * d_in);
+    for (int c = threadIdx.x; c < d_in / 4; c += 256) {
+        const uchar4 q = src[c];
+        dst[c] = make_float4(cb[min(static_cast<int>(q.x), m - 1)], cb[min(static_cast<int>(q.y), m - 1)],
+                             cb[min(static_cast<int>(q.z), m - 1)], cb[min(static_cast<int>(q.w), m - 1)]);
     }
 }
 

@@ -18,7 +18,7 @@
 #include "gq_cd.cuh"
 #include "gq_codebook.cuh"
 #include "gq_exchange.cuh"
-#include "gq_wide_gemm.cuh"
+#include "gq_codebook_gemm.cuh"
 #include "gq_gram_dot.cuh"
 #include "gq_kernels.cuh"
 
@@ -136,9 +136,9 @@ int32_t device_info(DeviceInfo **out)
                                      cudaFuncAttributeMaxDynamicSharedMemorySize, gq::OBJ_SMEM_BYTES));
         GQ_CUDA(cudaFuncSetAttribute(gq::pair_gemm_kernel<gq::MODE_PANEL>,
                                      cudaFuncAttributeMaxDynamicSharedMemorySize, gq::OBJ_SMEM_BYTES));
-        GQ_CUDA(cudaFuncSetAttribute(gq::pair_gemm_kernel<gq::MODE_FULL>,
-                                     cudaFuncAttributeMaxDynamicSharedMemorySize, gq::OBJ_SMEM_BYTES));
-        GQ_CUDA(cudaFuncSetAttribute(gq::wide_gemm_kernel<gq::WG_FULL>, cudaFuncAttributeMaxDynamicSharedMemorySize, gq::WG_SMEM_BYTES));
+        GQ_CUDA(cudaFuncSetAttribute(gq::codebook_gemm_kernel<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, gq::CG_SMEM_BYTES));
+        GQ_CUDA(cudaFuncSetAttribute(gq::codebook_gemm_kernel<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, gq::CG_SMEM_BYTES));
+        GQ_CUDA(cudaFuncSetAttribute(gq::codebook_gemm_kernel<16>, cudaFuncAttributeMaxDynamicSharedMemorySize, gq::CG_SMEM_BYTES));
         GQ_CUDA(cudaFuncSetAttribute(gq::gram_dot_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, gq::GD_SMEM_BYTES));
         GQ_CUDA(cudaFuncSetAttribute(gq::cd_block_kernel<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, gq::CD_SMEM_BYTES));
         GQ_CUDA(cudaFuncSetAttribute(gq::cd_block_kernel<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, gq::CD_SMEM_BYTES));
@@ -341,50 +341,52 @@ ObjectiveLayout objective_layout(int64_t d_in, int64_t d_out, int32_t g)
     return L;
 }
 
-struct CodebookLayout {
-    size_t h0, h1, w0, w1, qt, hw, pm, hp, gmat, rvec, total;
-    int64_t slab_channels, slab_ld;
+// Scratch of the quantiser's two steps.  Both start with the split of H (gq_cd.cuh), so that gq_lnq forms it once; what
+// a step needs beside it follows from `at` on.
+struct SplitLayout {
+    size_t h0, h1, rdiag, total;
 };
-CodebookLayout codebook_layout(int64_t d_in, int64_t d_out, int32_t g, int32_t m)
+SplitLayout split_layout(int64_t d_in, int32_t g)
+{
+    SplitLayout L;
+    const size_t h2 = round_up(static_cast<size_t>(g) * d_in * d_in * 2, 1024);
+    L.h0 = 0;
+    L.h1 = h2;
+    L.rdiag = 2 * h2;
+    L.total = L.rdiag + round_up(static_cast<size_t>(g) * d_in * 4, 1024);
+    return L;
+}
+
+struct CodebookLayout {
+    size_t w0, w1, gmat, rvec, q, total;
+};
+CodebookLayout codebook_layout(int64_t d_in, int64_t d_out, size_t at)
 {
     CodebookLayout L;
-    const int64_t mk = d_out / g;
-    L.slab_channels = mk < gq::CB_SLAB_CHANNELS ? mk : gq::CB_SLAB_CHANNELS;
-    L.slab_ld = (L.slab_channels * m + 7) / 8 * 8;
-    const size_t h2 = round_up(static_cast<size_t>(g) * d_in * d_in * 2, 1024);
     const size_t w2 = round_up(static_cast<size_t>(d_in) * d_out * 2, 1024);
-    size_t o = 0;
-    L.h0 = o; o += h2;
-    L.h1 = o; o += h2;
+    size_t o = at;
     L.w0 = o; o += w2;
     L.w1 = o; o += w2;
-    L.qt = o; o += round_up(static_cast<size_t>(d_in) * d_out, 1024);
-    L.hw = o; o += round_up(static_cast<size_t>(d_in) * d_out * 4, 1024);
-    L.pm = o; o += round_up(static_cast<size_t>(d_in) * L.slab_ld * 2, 1024);
-    L.hp = o; o += round_up(static_cast<size_t>(d_in) * L.slab_ld * 4, 1024);
-    L.gmat = o; o += round_up(static_cast<size_t>(d_out) * gq::CB_MAX_LEVELS * gq::CB_MAX_LEVELS * 8, 1024);
-    L.rvec = o; o += round_up(static_cast<size_t>(d_out) * gq::CB_MAX_LEVELS * 8, 1024);
+    L.gmat = o; o += static_cast<size_t>(d_out) * gq::CB_MAX_LEVELS * gq::CB_MAX_LEVELS * 8;      // G and R in one piece:
+    L.rvec = o; o += round_up(static_cast<size_t>(d_out) * gq::CB_MAX_LEVELS * 8, 1024);          // zeroed together
+    L.q = o; o += round_up(static_cast<size_t>(d_in) * d_out, 1024);
     L.total = o;
     return L;
 }
 
 struct CdLayout {
-    size_t wt, et, ehi, elo, hhi, hlo, rdiag, p, qt, total;
+    size_t wt, et, ehi, elo, p, qt, total;
 };
-CdLayout cd_layout(int64_t d_in, int64_t d_out, int32_t g)
+CdLayout cd_layout(int64_t d_in, int64_t d_out, size_t at)
 {
     CdLayout L;
     const size_t mat4 = round_up(static_cast<size_t>(d_in) * d_out * 4, 1024);
     const size_t mat2 = round_up(static_cast<size_t>(d_in) * d_out * 2, 1024);
-    const size_t h2 = round_up(static_cast<size_t>(g) * d_in * d_in * 2, 1024);
-    size_t o = 0;
+    size_t o = at;
     L.wt = o; o += mat4;
     L.et = o; o += mat4;
     L.ehi = o; o += mat2;
     L.elo = o; o += mat2;
-    L.hhi = o; o += h2;
-    L.hlo = o; o += h2;
-    L.rdiag = o; o += round_up(static_cast<size_t>(g) * d_in * 4, 1024);
     L.p = o; o += round_up(static_cast<size_t>(gq::CD_BLOCK) * d_out * 4, 1024);
     L.qt = o; o += round_up(static_cast<size_t>(d_in) * d_out, 1024);
     L.total = o;
@@ -920,45 +922,60 @@ int32_t gq_objective_noalloc(const float *W, const float *W_hat, int64_t d_in, i
     return GQ_OK;
 }
 
+// H into two bf16 terms and the reciprocals of its diagonal, at the start of the workspace of both quantiser steps.
+static int32_t split_h(const float *H, int64_t d_in, int32_t g, uint8_t *ws, cudaStream_t st)
+{
+    const SplitLayout S = split_layout(d_in, g);
+    const dim3 grid(static_cast<unsigned>(d_in), static_cast<unsigned>(g));
+    {
+        LaunchScope scope(GQ_KERNEL_CD_AUX, st);
+        gq::split_h_kernel<<<grid, 256, 0, st>>>(H, static_cast<int>(d_in), reinterpret_cast<__nv_bfloat16 *>(ws + S.h0),
+                                                 reinterpret_cast<__nv_bfloat16 *>(ws + S.h1), reinterpret_cast<float *>(ws + S.rdiag));
+    }
+    GQ_CUDA(cudaGetLastError());
+    return GQ_OK;
+}
+
 size_t gq_cd_workspace_bytes(int64_t d_in, int64_t d_out, int32_t g)
 {
     if (check_layer_shape(d_in, d_out, g, true) != GQ_OK) return 0;
-    return cd_layout(d_in, d_out, g).total;
+    return cd_layout(d_in, d_out, split_layout(d_in, g).total).total;
 }
 
-int32_t gq_cd_cycles(const float *W, float *W_hat, uint8_t *Q, const float *codebook, int32_t m, int64_t d_in,
-                     int64_t d_out, const float *H, int32_t g, int32_t cycles, void *workspace,
-                     size_t workspace_bytes, void *stream)
+// Arguments of coordinate descent; `need` = bytes of workspace the caller's layout takes.
+static int32_t check_cd_args(const float *W, const float *W_hat, const uint8_t *Q, const float *codebook, int32_t m, int64_t d_in,
+                             int64_t d_out, const float *H, int32_t g, int32_t cycles, const void *workspace,
+                             size_t workspace_bytes, size_t need)
 {
     if (!W || !W_hat || !Q || !codebook || !H || cycles < 0 || m < 1) return GQ_ERR_INVALID_ARG;
     if (int32_t rc = check_layer_shape(d_in, d_out, g, true)) return rc;
     if (m > gq::CD_MAX_LEVELS) return GQ_ERR_UNSUPPORTED_SHAPE;
     if (!aligned(W, 16) || !aligned(W_hat, 16) || !aligned(H, 16) || !aligned(codebook, 4)) return GQ_ERR_ALIGNMENT;
-    const CdLayout L = cd_layout(d_in, d_out, g);
-    if (!workspace || workspace_bytes < L.total) return GQ_ERR_WORKSPACE;
+    if (!workspace || workspace_bytes < need) return GQ_ERR_WORKSPACE;
     if (!aligned(workspace, 1024)) return GQ_ERR_ALIGNMENT;
-    {
-        const size_t w4 = static_cast<size_t>(d_out) * d_in * 4;
-        const ByteRange wr[3] = {{W_hat, w4}, {Q, static_cast<size_t>(d_out) * d_in}, {workspace, L.total}};
-        const ByteRange ro[3] = {{W, w4}, {codebook, static_cast<size_t>(d_out) * m * 4},
-                                 {H, static_cast<size_t>(g) * d_in * d_in * 4}};
-        if (int32_t rc = check_disjoint(wr, ro)) return rc;
-    }
+    const size_t w4 = static_cast<size_t>(d_out) * d_in * 4;
+    const ByteRange wr[3] = {{W_hat, w4}, {Q, static_cast<size_t>(d_out) * d_in}, {workspace, need}};
+    const ByteRange ro[3] = {{W, w4}, {codebook, static_cast<size_t>(d_out) * m * 4},
+                             {H, static_cast<size_t>(g) * d_in * d_in * 4}};
+    return check_disjoint(wr, ro);
+}
+
+// `L`: where coordinate descent's own arrays lie in `workspace`; the split of H at its start has been formed.
+static int32_t cd_cycles_impl(const float *W, float *W_hat, uint8_t *Q, const float *codebook, int32_t m, int64_t d_in,
+                              int64_t d_out, const float *H, int32_t g, int32_t cycles, void *workspace, const CdLayout &L,
+                              cudaStream_t st)
+{
     DeviceInfo *di;
     if (int32_t rc = device_info(&di)) return rc;
-    cudaStream_t st = static_cast<cudaStream_t>(stream);
-    if (cycles == 0) {                                   // W_hat stays as it is, no code has been chosen
-        GQ_CUDA(cudaMemsetAsync(Q, 0, static_cast<size_t>(d_out) * d_in, st));
-        return GQ_OK;
-    }
     uint8_t *ws = static_cast<uint8_t *>(workspace);
+    const SplitLayout S = split_layout(d_in, g);
     float *Wt = reinterpret_cast<float *>(ws + L.wt);
     float *Et = reinterpret_cast<float *>(ws + L.et);
     __nv_bfloat16 *Ehi = reinterpret_cast<__nv_bfloat16 *>(ws + L.ehi);
     __nv_bfloat16 *Elo = reinterpret_cast<__nv_bfloat16 *>(ws + L.elo);
-    __nv_bfloat16 *Hhi = reinterpret_cast<__nv_bfloat16 *>(ws + L.hhi);
-    __nv_bfloat16 *Hlo = reinterpret_cast<__nv_bfloat16 *>(ws + L.hlo);
-    float *rdiag = reinterpret_cast<float *>(ws + L.rdiag);
+    const __nv_bfloat16 *Hhi = reinterpret_cast<const __nv_bfloat16 *>(ws + S.h0);
+    const __nv_bfloat16 *Hlo = reinterpret_cast<const __nv_bfloat16 *>(ws + S.h1);
+    const float *rdiag = reinterpret_cast<const float *>(ws + S.rdiag);
     float *P = reinterpret_cast<float *>(ws + L.p);
     uint8_t *Qt = ws + L.qt;
     const int64_t mk = d_out / g;
@@ -967,12 +984,6 @@ int32_t gq_cd_cycles(const float *W, float *W_hat, uint8_t *Q, const float *code
         LaunchScope scope(GQ_KERNEL_CD_AUX, st);
         gq::cd_prepare_kernel<<<tgrid, 256, 0, st>>>(W, W_hat, static_cast<int>(d_in), static_cast<int>(d_out), Wt,
                                                      Et, Ehi, Elo);
-    }
-    GQ_CUDA(cudaGetLastError());
-    {
-        const dim3 hgrid(static_cast<unsigned>(d_in), static_cast<unsigned>(g));
-        LaunchScope scope(GQ_KERNEL_CD_AUX, st);
-        gq::cd_split_h_kernel<<<hgrid, 256, 0, st>>>(H, static_cast<int>(d_in), Hhi, Hlo, rdiag);
     }
     GQ_CUDA(cudaGetLastError());
 
@@ -1054,156 +1065,147 @@ int32_t gq_cd_cycles(const float *W, float *W_hat, uint8_t *Q, const float *code
     return GQ_OK;
 }
 
+int32_t gq_cd_cycles(const float *W, float *W_hat, uint8_t *Q, const float *codebook, int32_t m, int64_t d_in,
+                     int64_t d_out, const float *H, int32_t g, int32_t cycles, void *workspace,
+                     size_t workspace_bytes, void *stream)
+{
+    if (int32_t rc = check_cd_args(W, W_hat, Q, codebook, m, d_in, d_out, H, g, cycles, workspace, workspace_bytes,
+                                   gq_cd_workspace_bytes(d_in, d_out, g)))
+        return rc;
+    DeviceInfo *di;
+    if (int32_t rc = device_info(&di)) return rc;
+    cudaStream_t st = static_cast<cudaStream_t>(stream);
+    if (cycles == 0) {                                   // W_hat stays as it is, no code has been chosen
+        GQ_CUDA(cudaMemsetAsync(Q, 0, static_cast<size_t>(d_out) * d_in, st));
+        return GQ_OK;
+    }
+    if (int32_t rc = split_h(H, d_in, g, static_cast<uint8_t *>(workspace), st)) return rc;
+    return cd_cycles_impl(W, W_hat, Q, codebook, m, d_in, d_out, H, g, cycles, workspace,
+                          cd_layout(d_in, d_out, split_layout(d_in, g).total), st);
+}
+
 size_t gq_codebook_workspace_bytes(int64_t d_in, int64_t d_out, int32_t g, int32_t m)
 {
     if (m < 1 || m > gq::CB_MAX_LEVELS || check_layer_shape(d_in, d_out, g, true) != GQ_OK) return 0;
-    return codebook_layout(d_in, d_out, g, m).total;
+    return codebook_layout(d_in, d_out, split_layout(d_in, g).total).total;
+}
+
+static int32_t check_codebook_args(const float *W, const uint8_t *Q, int32_t m, int64_t d_in, int64_t d_out, const float *H,
+                                   int32_t g, double lambda, const float *codebook, const float *W_hat, const void *workspace,
+                                   size_t workspace_bytes, size_t need)
+{
+    if (!W || !Q || !H || !codebook || m < 1 || !(lambda >= 0.0)) return GQ_ERR_INVALID_ARG;
+    if (int32_t rc = check_layer_shape(d_in, d_out, g, true)) return rc;
+    if (m > gq::CB_MAX_LEVELS) return GQ_ERR_UNSUPPORTED_SHAPE;
+    if (!aligned(W, 16) || !aligned(H, 16) || !aligned(codebook, 4) || (W_hat && !aligned(W_hat, 16))) return GQ_ERR_ALIGNMENT;
+    if (!workspace || workspace_bytes < need) return GQ_ERR_WORKSPACE;
+    if (!aligned(workspace, 1024)) return GQ_ERR_ALIGNMENT;
+    const size_t w4 = static_cast<size_t>(d_out) * d_in * 4;
+    const ByteRange wr[3] = {{codebook, static_cast<size_t>(d_out) * m * 4}, {W_hat, W_hat ? w4 : 0}, {workspace, need}};
+    const ByteRange ro[3] = {{W, w4}, {Q, static_cast<size_t>(d_out) * d_in}, {H, static_cast<size_t>(g) * d_in * d_in * 4}};
+    return check_disjoint(wr, ro);
+}
+
+// W^T into two bf16 terms.
+static int32_t split_w(const float *W, int64_t d_in, int64_t d_out, uint8_t *ws, const CodebookLayout &L, cudaStream_t st)
+{
+    const dim3 grid(static_cast<unsigned>((d_in + 31) / 32), static_cast<unsigned>((d_out + 63) / 64));
+    {
+        LaunchScope scope(GQ_KERNEL_CB_AUX, st);
+        gq::cb_transpose_kernel<<<grid, 256, 0, st>>>(W, static_cast<int>(d_in), static_cast<int>(d_out),
+                                                      reinterpret_cast<__nv_bfloat16 *>(ws + L.w0),
+                                                      reinterpret_cast<__nv_bfloat16 *>(ws + L.w1));
+    }
+    GQ_CUDA(cudaGetLastError());
+    return GQ_OK;
+}
+
+// The split of H has been formed.
+static int32_t codebook_update_impl(const float *W, const uint8_t *Q, int32_t m, int64_t d_in, int64_t d_out, int32_t g,
+                                    double lambda, float *codebook, float *W_hat, void *workspace, const CodebookLayout &L,
+                                    cudaStream_t st)
+{
+    DeviceInfo *di;
+    if (int32_t rc = device_info(&di)) return rc;
+    uint8_t *ws = static_cast<uint8_t *>(workspace);
+    const SplitLayout S = split_layout(d_in, g);
+    double *Gm = reinterpret_cast<double *>(ws + L.gmat);
+    double *Rv = reinterpret_cast<double *>(ws + L.rvec);
+    const int64_t mk = d_out / g;
+    if (int32_t rc = split_w(W, d_in, d_out, ws, L, st)) return rc;
+    if (!aligned(Q, 8)) {                                // the kernels below read several codes at a time
+        GQ_CUDA(cudaMemcpyAsync(ws + L.q, Q, static_cast<size_t>(d_in) * d_out, cudaMemcpyDeviceToDevice, st));
+        Q = ws + L.q;
+    }
+    GQ_CUDA(cudaMemsetAsync(Gm, 0, static_cast<size_t>(d_out) * (gq::CB_MAX_LEVELS + 1) * gq::CB_MAX_LEVELS * sizeof(double), st));
+    CUtensorMap mH0, mH1, mW0, mW1;
+    if (int32_t rc = make_map(&mH0, ws + S.h0, d_in, d_in, g, d_in, d_in * d_in)) return rc;
+    if (int32_t rc = make_map(&mH1, ws + S.h1, d_in, d_in, g, d_in, d_in * d_in)) return rc;
+    if (int32_t rc = make_map(&mW0, ws + L.w0, d_out, d_in, 1, d_out, d_in * d_out)) return rc;
+    if (int32_t rc = make_map(&mW1, ws + L.w1, d_out, d_in, 1, d_out, d_in * d_out)) return rc;
+    // one-hot columns per channel: the next of 4, 8, 16, so that a channel's columns never straddle 16 accumulator rows
+    const int mp = m <= 4 ? 4 : m <= 8 ? 8 : 16;
+    gq::CodebookGemmParams p{};
+    p.Q = Q;
+    p.G = Gm;
+    p.R = Rv;
+    p.d = static_cast<int>(d_in);
+    p.d_out = static_cast<int>(d_out);
+    p.g = g;
+    p.mk = static_cast<int>(mk);
+    p.m = m;
+    p.row_blocks = static_cast<int>((d_in + gq::TILE_N - 1) / gq::TILE_N);
+    p.w_tiles = static_cast<int>((mk + gq::TILE_M - 1) / gq::TILE_M);
+    p.hot_tiles = static_cast<int>((mk * mp + gq::TILE_M - 1) / gq::TILE_M);
+    const int64_t units = static_cast<int64_t>(p.row_blocks) * g * (static_cast<int64_t>(p.w_tiles) + p.hot_tiles);
+    if (units >= (1ll << 30)) return GQ_ERR_UNSUPPORTED_SHAPE;
+    p.w_units = p.row_blocks * g * p.w_tiles;
+    p.units = static_cast<int>(units);
+    p.pairs = p.units < di->max_pairs ? p.units : di->max_pairs;
+    p.status = di->status_ptr;
+    p.wait_budget_ns = wait_budget_ns();
+    {
+        LaunchScope scope(GQ_KERNEL_CB_GEMM, st);
+        const auto kernel = mp == 4 ? gq::codebook_gemm_kernel<4> : mp == 8 ? gq::codebook_gemm_kernel<8> : gq::codebook_gemm_kernel<16>;
+        kernel<<<2 * p.pairs, gq::CG_THREADS, gq::CG_SMEM_BYTES, st>>>(mH0, mH1, mW0, mW1, p);
+    }
+    GQ_CUDA(cudaGetLastError());
+    {
+        LaunchScope scope(GQ_KERNEL_CB_FOLD, st);
+        gq::cb_solve_kernel<<<static_cast<unsigned>((d_out + 7) / 8), 128, 0, st>>>(Gm, Rv, static_cast<int>(d_out), m,
+                                                                                    lambda, codebook);
+    }
+    GQ_CUDA(cudaGetLastError());
+    if (W_hat) {
+        LaunchScope scope(GQ_KERNEL_CB_AUX, st);
+        gq::cb_apply_kernel<<<static_cast<unsigned>(d_out), 256, 0, st>>>(codebook, Q, static_cast<int>(d_in), m, W_hat);
+        GQ_CUDA(cudaGetLastError());
+    }
+    return GQ_OK;
 }
 
 int32_t gq_codebook_update(const float *W, const uint8_t *Q, int32_t m, int64_t d_in, int64_t d_out, const float *H,
                            int32_t g, double lambda, float *codebook, float *W_hat, void *workspace,
                            size_t workspace_bytes, void *stream)
 {
-    if (!W || !Q || !H || !codebook || m < 1 || !(lambda >= 0.0)) return GQ_ERR_INVALID_ARG;
-    if (int32_t rc = check_layer_shape(d_in, d_out, g, true)) return rc;
-    if (m > gq::CB_MAX_LEVELS) return GQ_ERR_UNSUPPORTED_SHAPE;
-    if (!aligned(W, 16) || !aligned(H, 16) || !aligned(codebook, 4) || (W_hat && !aligned(W_hat, 16))) return GQ_ERR_ALIGNMENT;
-    const CodebookLayout L = codebook_layout(d_in, d_out, g, m);
-    if (!workspace || workspace_bytes < L.total) return GQ_ERR_WORKSPACE;
-    if (!aligned(workspace, 1024)) return GQ_ERR_ALIGNMENT;
-    {
-        const size_t w4 = static_cast<size_t>(d_out) * d_in * 4;
-        const ByteRange wr[3] = {{codebook, static_cast<size_t>(d_out) * m * 4}, {W_hat, W_hat ? w4 : 0}, {workspace, L.total}};
-        const ByteRange ro[3] = {{W, w4}, {Q, static_cast<size_t>(d_out) * d_in}, {H, static_cast<size_t>(g) * d_in * d_in * 4}};
-        if (int32_t rc = check_disjoint(wr, ro)) return rc;
-    }
+    if (int32_t rc = check_codebook_args(W, Q, m, d_in, d_out, H, g, lambda, codebook, W_hat, workspace, workspace_bytes,
+                                         gq_codebook_workspace_bytes(d_in, d_out, g, m)))
+        return rc;
     DeviceInfo *di;
     if (int32_t rc = device_info(&di)) return rc;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     uint8_t *ws = static_cast<uint8_t *>(workspace);
-    __nv_bfloat16 *H0 = reinterpret_cast<__nv_bfloat16 *>(ws + L.h0), *H1 = reinterpret_cast<__nv_bfloat16 *>(ws + L.h1);
-    __nv_bfloat16 *W0 = reinterpret_cast<__nv_bfloat16 *>(ws + L.w0), *W1 = reinterpret_cast<__nv_bfloat16 *>(ws + L.w1);
-    uint8_t *Qt = ws + L.qt;
-    float *HW = reinterpret_cast<float *>(ws + L.hw);
-    __nv_bfloat16 *Pm = reinterpret_cast<__nv_bfloat16 *>(ws + L.pm);
-    float *HP = reinterpret_cast<float *>(ws + L.hp);
-    double *Gm = reinterpret_cast<double *>(ws + L.gmat);
-    double *Rv = reinterpret_cast<double *>(ws + L.rvec);
-    const int64_t mk = d_out / g;
-    const long long hcount = static_cast<long long>(g) * d_in * d_in;
-    {
-        LaunchScope scope(GQ_KERNEL_CB_AUX, st);
-        gq::cb_split2_kernel<<<grid_for(hcount, 256, di->sm_count, 8), 256, 0, st>>>(H, hcount, H0, H1);
-    }
-    GQ_CUDA(cudaGetLastError());
-    {
-        const dim3 tgrid(static_cast<unsigned>((d_in + 31) / 32), static_cast<unsigned>((d_out + 31) / 32));
-        LaunchScope scope(GQ_KERNEL_CB_AUX, st);
-        gq::cb_transpose_kernel<<<tgrid, 256, 0, st>>>(W, Q, static_cast<int>(d_in), static_cast<int>(d_out), W0, W1, Qt);
-    }
-    GQ_CUDA(cudaGetLastError());
-    CUtensorMap mH0, mH1, mW0, mW1, mPm;
-    if (int32_t rc = make_map(&mH0, H0, d_in, d_in, g, d_in, d_in * d_in)) return rc;
-    if (int32_t rc = make_map(&mH1, H1, d_in, d_in, g, d_in, d_in * d_in)) return rc;
-    if (int32_t rc = make_map(&mW0, W0, d_out, d_in, 1, d_out, d_in * d_out)) return rc;
-    if (int32_t rc = make_map(&mW1, W1, d_out, d_in, 1, d_out, d_in * d_out)) return rc;
-    if (int32_t rc = make_map(&mPm, Pm, L.slab_ld, d_in, 1, L.slab_ld, d_in * L.slab_ld)) return rc;
-
-    auto launch_full = [&](gq::PairGemmParams &pp, const CUtensorMap &b0, const CUtensorMap &b1, const CUtensorMap &b2,
-                           int kernel_id, bool wide) -> int32_t {
-        pp.d = static_cast<int>(d_in);
-        pp.rows = static_cast<int>(d_in);
-        pp.g = g;
-        pp.map_grouped[0] = pp.map_grouped[1] = pp.map_grouped[2] = 1;
-        pp.map_grouped[3] = pp.map_grouped[4] = pp.map_grouped[5] = 0;
-        pp.col_tiles = (pp.cols + gq::TILE_N - 1) / gq::TILE_N;
-        const int row_blocks = static_cast<int>((d_in + gq::TILE_M - 1) / gq::TILE_M);
-        // wide: a unit is a row block times two neighbouring column tiles (gq_wide_gemm.cuh)
-        const int units = row_blocks * (wide ? (pp.col_tiles + 1) / 2 : pp.col_tiles);
-        const int ksteps = pp.n_terms * static_cast<int>((d_in + gq::TILE_K - 1) / gq::TILE_K);
-        pp.sched = gq::plan_schedule(units, ksteps, units < di->max_pairs ? units : di->max_pairs, false);
-        pp.status = di->status_ptr;
-        pp.wait_budget_ns = wait_budget_ns();
-        {
-            LaunchScope scope(kernel_id, st);
-            if (wide)
-                gq::wide_gemm_kernel<gq::WG_FULL><<<2 * pp.sched.pairs, gq::WG_THREADS, gq::WG_SMEM_BYTES, st>>>(mH0, mH1, mH1, b0, b1, b2, pp);
-            else
-                gq::pair_gemm_kernel<gq::MODE_FULL><<<2 * pp.sched.pairs, gq::OBJ_THREADS, gq::OBJ_SMEM_BYTES, st>>>(
-                    mH0, mH1, mH1, b0, b1, b2, pp);
-        }
-        GQ_CUDA(cudaGetLastError());
-        return GQ_OK;
-    };
-
-    GQ_CUDA(cudaMemsetAsync(Gm, 0, static_cast<size_t>(d_out) * gq::CB_MAX_LEVELS * gq::CB_MAX_LEVELS * sizeof(double), st));
-    GQ_CUDA(cudaMemsetAsync(Rv, 0, static_cast<size_t>(d_out) * gq::CB_MAX_LEVELS * sizeof(double), st));
-    for (int32_t k = 0; k < g; ++k) {
-        // HW[:, group k] = H_k W_k^T: H0 W0 + H0 W1 + H1 W0 (hi + lo splits, 16 significant bits per factor)
-        gq::PairGemmParams pp{};
-        pp.n_terms = 3;
-        const int ta[3] = {0, 0, 1}, tb[3] = {3, 4, 3};
-        for (int t = 0; t < 3; ++t) { pp.term_a[t] = ta[t]; pp.term_b[t] = tb[t]; }
-        pp.full_k = k;
-        pp.col0 = static_cast<int>(k * mk);
-        pp.cols = static_cast<int>(mk);
-        pp.C = HW + k * mk;
-        pp.ldc = d_out;
-        if (int32_t rc = launch_full(pp, mW0, mW1, mW1, GQ_KERNEL_CB_GEMM, false)) return rc;
-        for (int64_t j0 = k * mk; j0 < (k + 1) * mk; j0 += L.slab_channels) {
-            const int nch = static_cast<int>((k + 1) * mk - j0 < L.slab_channels ? (k + 1) * mk - j0 : L.slab_channels);
-            {
-                const long long total = static_cast<long long>(d_in) * nch;
-                LaunchScope scope(GQ_KERNEL_CB_AUX, st);
-                gq::cb_onehot_kernel<<<grid_for(total, 256, di->sm_count, 8), 256, 0, st>>>(
-                    Qt, static_cast<int>(d_in), static_cast<int>(d_out), static_cast<int>(j0), nch, m, Pm, L.slab_ld);
-            }
-            GQ_CUDA(cudaGetLastError());
-            // HP = H_k Pm: the one-hot columns are exact in bf16; the two leading terms of H carry 16 mantissa bits
-            gq::PairGemmParams pq{};
-            pq.n_terms = 2;
-            pq.term_a[0] = 0; pq.term_b[0] = 3;
-            pq.term_a[1] = 1; pq.term_b[1] = 3;
-            pq.full_k = k;
-            pq.col0 = 0;
-            pq.cols = nch * m;
-            pq.C = HP;
-            pq.ldc = L.slab_ld;
-            if (int32_t rc = launch_full(pq, mPm, mPm, mPm, GQ_KERNEL_CB_GEMM, pq.cols > 2 * gq::TILE_N)) return rc;
-            {
-                LaunchScope scope(GQ_KERNEL_CB_FOLD, st);
-                if (m % 4 == 0)
-                    gq::cb_fold4_kernel<<<dim3((nch + gq::CB_FOLD4_CH - 1) / gq::CB_FOLD4_CH, 16), gq::CB_FOLD4_CH * 4, 0, st>>>(
-                        HP, L.slab_ld, HW, Qt, static_cast<int>(d_in), static_cast<int>(d_out), static_cast<int>(j0), nch, m, Gm, Rv);
-                else
-                    gq::cb_fold_kernel<<<dim3((nch + gq::CB_FOLD_CH - 1) / gq::CB_FOLD_CH, 16), gq::CB_FOLD_CH * 16, 0, st>>>(
-                        HP, L.slab_ld, HW, Qt, static_cast<int>(d_in), static_cast<int>(d_out), static_cast<int>(j0), nch, m, Gm, Rv);
-            }
-            GQ_CUDA(cudaGetLastError());
-        }
-    }
-    {
-        LaunchScope scope(GQ_KERNEL_CB_FOLD, st);
-        gq::cb_solve_kernel<<<static_cast<unsigned>((d_out + 127) / 128), 128, 0, st>>>(Gm, Rv, static_cast<int>(d_out), m,
-                                                                                      lambda, codebook);
-    }
-    GQ_CUDA(cudaGetLastError());
-    if (W_hat) {
-        const long long count = static_cast<long long>(d_out) * d_in;
-        LaunchScope scope(GQ_KERNEL_CB_AUX, st);
-        gq::cb_apply_kernel<<<grid_for(count, 256, di->sm_count, 8), 256, 0, st>>>(codebook, Q, count, static_cast<int>(d_in),
-                                                                                 m, W_hat);
-        GQ_CUDA(cudaGetLastError());
-    }
-    return GQ_OK;
+    const CodebookLayout L = codebook_layout(d_in, d_out, split_layout(d_in, g).total);
+    if (int32_t rc = split_h(H, d_in, g, ws, st)) return rc;
+    return codebook_update_impl(W, Q, m, d_in, d_out, g, lambda, codebook, W_hat, workspace, L, st);
 }
 
 size_t gq_lnq_workspace_bytes(int64_t d_in, int64_t d_out, int32_t g, int32_t m)
 {
-    const size_t cb = gq_codebook_workspace_bytes(d_in, d_out, g, m);
-    const size_t cd = gq_cd_workspace_bytes(d_in, d_out, g);
-    if (cb == 0 || cd == 0) return 0;
-    return cb > cd ? cb : cd;                     // the two steps alternate: one region serves both
+    if (gq_codebook_workspace_bytes(d_in, d_out, g, m) == 0) return 0;
+    // the steps alternate: one region serves both, and the split of H at its start serves all of them
+    const size_t cb = gq_codebook_workspace_bytes(d_in, d_out, g, m), cd = gq_cd_workspace_bytes(d_in, d_out, g);
+    return cb > cd ? cb : cd;
 }
 
 int32_t gq_lnq(const float *W, uint8_t *Q, int32_t m, int64_t d_in, int64_t d_out, const float *H, int32_t g,
@@ -1224,15 +1226,21 @@ int32_t gq_lnq(const float *W, uint8_t *Q, int32_t m, int64_t d_in, int64_t d_ou
         const ByteRange ro[2] = {{W, w4}, {H, static_cast<size_t>(g) * d_in * d_in * 4}};
         if (int32_t rc = check_disjoint(wr, ro)) return rc;
     }
+    if (int32_t rc = check_codebook_args(W, Q, m, d_in, d_out, H, g, lambda, codebook, W_hat, workspace, workspace_bytes, need))
+        return rc;
+    DeviceInfo *di;
+    if (int32_t rc = device_info(&di)) return rc;
+    cudaStream_t st = static_cast<cudaStream_t>(stream);
+    uint8_t *ws = static_cast<uint8_t *>(workspace);
+    const CodebookLayout Lb = codebook_layout(d_in, d_out, split_layout(d_in, g).total);
+    const CdLayout Lc = cd_layout(d_in, d_out, split_layout(d_in, g).total);
+    if (int32_t rc = split_h(H, d_in, g, ws, st)) return rc;
     for (int32_t t = 0; t < T; ++t) {
-        if (int32_t rc = gq_codebook_update(W, Q, m, d_in, d_out, H, g, lambda, codebook, W_hat, workspace,
-                                            workspace_bytes, stream))
-            return rc;
+        if (int32_t rc = codebook_update_impl(W, Q, m, d_in, d_out, g, lambda, codebook, W_hat, workspace, Lb, st)) return rc;
         if (K == 0) continue;
-        if (int32_t rc = gq_cd_cycles(W, W_hat, Q, codebook, m, d_in, d_out, H, g, K, workspace, workspace_bytes, stream))
-            return rc;
+        if (int32_t rc = cd_cycles_impl(W, W_hat, Q, codebook, m, d_in, d_out, H, g, K, workspace, Lc, st)) return rc;
     }
-    return gq_codebook_update(W, Q, m, d_in, d_out, H, g, lambda, codebook, W_hat, workspace, workspace_bytes, stream);
+    return codebook_update_impl(W, Q, m, d_in, d_out, g, lambda, codebook, W_hat, workspace, Lb, st);
 }
 
 int32_t gq_selftest_wait_timeout(int32_t budget_ms, void *stream)

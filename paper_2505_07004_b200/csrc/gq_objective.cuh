@@ -23,9 +23,6 @@
 //                  B = E = (What - W)^T (rows = input coordinates c, columns = output channels); work unit =
 //                  (group, tile of 256 channels, piece of the contraction range); the pieces of a tile are
 //                  added into P with red.global.add.
-// MODE_FULL        C[r][col] = sum_c A[c][r] * B[c][col], a plain product of MN-major operands (used by the
-//                  LNQ codebook step: A = H_k split three ways, B = W^T or one-hot assignment columns); work
-//                  unit = (256-row block, 256-column tile), each unit stores its tile.
 #pragma once
 #include <cuda.h>
 #include <cuda_runtime.h>
@@ -47,7 +44,6 @@ constexpr int PARTIALS_PER_UNIT = 8;                   // one fp64 per (CTA of t
 
 constexpr int MODE_OBJECTIVE = 0;
 constexpr int MODE_PANEL = 1;
-constexpr int MODE_FULL = 2;
 
 struct PairGemmParams {
     int d;                   // number of features (d_in)
@@ -72,12 +68,6 @@ struct PairGemmParams {
     int mk;                  // channels per group
     int d_out;
     float *P;                // [256][d_out]
-    // MODE_FULL: C[r][col - col0] = sum over all `rows` contraction rows, r < d, col0 <= col < col0 + cols
-    int full_k;              // group index given to the grouped maps
-    int col0, cols;          // B columns of this launch
-    int col_tiles;           // ceil(cols / 256)
-    float *C;                // output, row stride ldc (floats), written (not added)
-    long long ldc;
     uint32_t *status;        // device status word (4 x u32)
     unsigned long long wait_budget_ns;
 };
@@ -98,16 +88,6 @@ __device__ __forceinline__ bool item_geom(const PairGemmParams &p, const WorkIte
         ge.k = w.unit % p.g;
         ge.a0 = ge.ti * TILE_M + static_cast<int>(rank) * CTA_ROWS;
         ge.b0 = ge.tj * TILE_N + static_cast<int>(rank) * CTA_ROWS;
-        ge.ks0 = w.ks0;
-        ge.ks1 = w.ks1;
-        return true;
-    }
-    if (MODE == MODE_FULL) {
-        ge.ti = w.unit / p.col_tiles;
-        ge.tj = w.unit % p.col_tiles;
-        ge.k = p.full_k;
-        ge.a0 = ge.ti * TILE_M + static_cast<int>(rank) * CTA_ROWS;
-        ge.b0 = p.col0 + ge.tj * TILE_N + static_cast<int>(rank) * CTA_ROWS;
         ge.ks0 = w.ks0;
         ge.ks1 = w.ks1;
         return true;
@@ -353,57 +333,30 @@ pair_gemm_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant
             ok = __all_sync(0xffffffffu, ok);
             if (!ok) break;
             tc_fence_after_sync();
-            if (MODE == MODE_OBJECTIVE) {
-            } else if (MODE == MODE_FULL) {
-                const int row0 = ge.ti * TILE_M + static_cast<int>(rank) * CTA_ROWS + q * 32;
-                const int row = row0 + lane;
-                float *crow = p.C + static_cast<size_t>(row < p.d ? row : 0) * p.ldc;
+            const int rl = static_cast<int>(rank) * CTA_ROWS + q * 32 + lane;      // row inside the block
+            const bool row_ok = p.s0 + rl < p.d;
+            const int ch_end = (ge.k + 1) * p.mk;                                  // channels of this group only
+            float *prow = p.P + static_cast<size_t>(rl) * p.d_out;
 #pragma unroll 1
-                for (int cc = 0; cc < TILE_N / 32; ++cc) {
-                    const int c0 = ge.tj * TILE_N + cc * 32;                           // column relative to col0
-                    if (c0 >= p.cols || row0 >= p.d) break;
-                    uint32_t r[32];
-                    tmem_ld_32x32(tmem_base + (static_cast<uint32_t>(q * 32) << 16) +
-                                      static_cast<uint32_t>(buf * TILE_N + cc * 32), r);
-                    tmem_ld_wait();
-                    if (row >= p.d) continue;
+            for (int cc = 0; cc < TILE_N / 32; ++cc) {
+                const int ch0 = ge.k * p.mk + ge.tj * TILE_N + cc * 32;
+                if (ch0 >= ch_end) break;
+                if (p.s0 + static_cast<int>(rank) * CTA_ROWS + q * 32 >= p.d) break;
+                uint32_t r[32];
+                tmem_ld_32x32(tmem_base + (static_cast<uint32_t>(q * 32) << 16) +
+                                  static_cast<uint32_t>(buf * TILE_N + cc * 32), r);
+                tmem_ld_wait();
+                if (!row_ok) continue;
 #pragma unroll
-                    for (int v = 0; v < 8; ++v) {
-                        if (c0 + v * 4 < p.cols)
-                            *reinterpret_cast<float4 *>(crow + c0 + v * 4) =
-                                make_float4(__uint_as_float(r[v * 4 + 0]), __uint_as_float(r[v * 4 + 1]),
-                                            __uint_as_float(r[v * 4 + 2]), __uint_as_float(r[v * 4 + 3]));
-                    }
+                for (int v = 0; v < 8; ++v) {
+                    if (ch0 + v * 4 < ch_end)
+                        red_add_f32x4(prow + ch0 + v * 4, __uint_as_float(r[v * 4 + 0]), __uint_as_float(r[v * 4 + 1]),
+                                      __uint_as_float(r[v * 4 + 2]), __uint_as_float(r[v * 4 + 3]));
                 }
-                tc_fence_before_sync();
-                __syncwarp();
-                if (lane == 0) mbar_arrive_cluster(map_to_cta(smem_u32(&bar_acc_empty[buf]), 0));
-            } else {
-                const int rl = static_cast<int>(rank) * CTA_ROWS + q * 32 + lane;      // row inside the block
-                const bool row_ok = p.s0 + rl < p.d;
-                const int ch_end = (ge.k + 1) * p.mk;                                  // channels of this group only
-                float *prow = p.P + static_cast<size_t>(rl) * p.d_out;
-#pragma unroll 1
-                for (int cc = 0; cc < TILE_N / 32; ++cc) {
-                    const int ch0 = ge.k * p.mk + ge.tj * TILE_N + cc * 32;
-                    if (ch0 >= ch_end) break;
-                    if (p.s0 + static_cast<int>(rank) * CTA_ROWS + q * 32 >= p.d) break;
-                    uint32_t r[32];
-                    tmem_ld_32x32(tmem_base + (static_cast<uint32_t>(q * 32) << 16) +
-                                      static_cast<uint32_t>(buf * TILE_N + cc * 32), r);
-                    tmem_ld_wait();
-                    if (!row_ok) continue;
-#pragma unroll
-                    for (int v = 0; v < 8; ++v) {
-                        if (ch0 + v * 4 < ch_end)
-                            red_add_f32x4(prow + ch0 + v * 4, __uint_as_float(r[v * 4 + 0]), __uint_as_float(r[v * 4 + 1]),
-                                          __uint_as_float(r[v * 4 + 2]), __uint_as_float(r[v * 4 + 3]));
-                    }
-                }
-                tc_fence_before_sync();
-                __syncwarp();
-                if (lane == 0) mbar_arrive_cluster(map_to_cta(smem_u32(&bar_acc_empty[buf]), 0));
             }
+            tc_fence_before_sync();
+            __syncwarp();
+            if (lane == 0) mbar_arrive_cluster(map_to_cta(smem_u32(&bar_acc_empty[buf]), 0));
             buf ^= 1;
             if (buf == 0) acc_ph ^= 1u;
         }

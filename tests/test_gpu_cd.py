@@ -121,6 +121,23 @@ def test_cd_llama_shaped_group(dev):
     print("channels on a different (near-tie) path: %d of %d" % (n_diff, W.shape[0]))
 
 
+@pytest.mark.parametrize("seed,d_in,d_out,g,m", [
+    (20, 296, 88, 1, 3),        # channel slices of 32, 32 and 24; second block of 40 coordinates: a band and a quarter
+    (21, 512, 40, 1, 5),        # whole blocks
+    (22, 264, 72, 3, 13),       # second block of 8 coordinates
+])
+def test_cd_block_edges(dev, seed, d_in, d_out, g, m):
+    """Level counts between the block kernel's 4, 8 and 16, in no order and with a level given twice (the codes name the
+    first of the two), ragged bands and channel slices."""
+    W, W0, cb, H = make_problem(seed, d_in, d_out, g, m)
+    cb = cb[:, np.random.default_rng(seed).permutation(m)].copy()
+    cb[:, m - 1] = cb[:, 0]
+    W0 = cdo.round_to_codebook(W, cb)[0].astype(np.float32)
+    What_g, Q_g = run_gpu(dev, W, W0, cb, H, 1)
+    check_against_oracle(W, W0, cb, H, What_g, Q_g, 1, certify_ties=True)
+    assert Q_g.max() < m - 1
+
+
 def test_cd_errors_and_zero_cycles(dev):
     W, W0, cb, H = make_problem(3, 64, 16, 1, 4)
     Wd, Whd = torch.from_numpy(W).to(dev), torch.from_numpy(W0.copy()).to(dev)
