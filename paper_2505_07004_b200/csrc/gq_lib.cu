@@ -691,8 +691,8 @@ int32_t gq_hessian_finalize(float *H, int64_t d_in, int32_t g, void *stream)
     if (!H) return GQ_ERR_INVALID_ARG;
     if (int32_t rc = check_layer_shape(d_in, 0, g, false)) return rc;
     if (!aligned(H, 128)) return GQ_ERR_ALIGNMENT;
-    const unsigned nb = static_cast<unsigned>((d_in + 31) / 32);
-    dim3 grid(nb, nb, static_cast<unsigned>(g));
+    const unsigned nb = static_cast<unsigned>((d_in + gq::MIRROR_TILE - 1) / gq::MIRROR_TILE);
+    dim3 grid(nb * (nb + 1) / 2, static_cast<unsigned>(g));
     {
         LaunchScope scope(GQ_KERNEL_MIRROR, static_cast<cudaStream_t>(stream));
         gq::mirror_kernel<<<grid, 256, 0, static_cast<cudaStream_t>(stream)>>>(H, static_cast<int>(d_in));
