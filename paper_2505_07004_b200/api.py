@@ -111,9 +111,16 @@ def lib() -> ctypes.CDLL:
     return _lib
 
 
-def _stream_ptr(stream: Optional[torch.cuda.Stream], device=None) -> int:
-    st = stream if stream is not None else torch.cuda.current_stream(device)
-    return int(st.cuda_stream)
+# The current stream of a device as a plain handle; building a torch.cuda.Stream for it costs several microseconds a call.
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+
+
+def _stream_ptr(stream: Optional[torch.cuda.Stream], device_index: int) -> int:
+    if stream is not None:
+        return int(stream.cuda_stream)
+    if _raw_stream is not None:
+        return _raw_stream(device_index)
+    return int(torch.cuda.current_stream(device_index).cuda_stream)
 
 
 def _same_device(*named):
@@ -140,18 +147,24 @@ def _same_device(*named):
 class _on:
     """Context: make `device` current for a library call and resolve the stream on that device."""
 
+    __slots__ = ("device", "stream", "guard")
+
     def __init__(self, device, stream):
         if stream is not None and getattr(stream, "device", device) != device:
             raise ValueError("stream belongs to %s, the tensors to %s" % (stream.device, device))
-        self.guard = torch.cuda.device(device)
-        self.device, self.stream = device, stream
+        self.device, self.stream, self.guard = device, stream, None
 
     def __enter__(self) -> int:
-        self.guard.__enter__()
-        return _stream_ptr(self.stream, self.device)
+        current, index = torch.cuda.current_device(), self.device.index
+        if index is None:
+            index = current
+        elif index != current:               # the guard is only paid for when there is something to switch
+            self.guard = torch.cuda.device(index)
+            self.guard.__enter__()
+        return _stream_ptr(self.stream, index)
 
     def __exit__(self, *exc):
-        return self.guard.__exit__(*exc)
+        return self.guard.__exit__(*exc) if self.guard is not None else None
 
 
 def _dev(t: torch.Tensor, dtype, name: str) -> torch.Tensor:
@@ -164,9 +177,12 @@ def _dev(t: torch.Tensor, dtype, name: str) -> torch.Tensor:
 
 def _rows(t: torch.Tensor, name: str):
     """(n, width, leading dimension) of a 2-D tensor whose last dimension is contiguous."""
-    if t.dim() != 2 or (t.shape[1] > 1 and t.stride(1) != 1):
+    if t.dim() != 2:
         raise ValueError("%s must be 2-D with a contiguous last dimension" % name)
-    return t.shape[0], t.shape[1], (t.stride(0) if t.shape[0] > 1 else max(t.shape[1], t.stride(0)))
+    (rows, width), (ld, step) = t.shape, t.stride()
+    if width > 1 and step != 1:
+        raise ValueError("%s must be 2-D with a contiguous last dimension" % name)
+    return rows, width, (ld if rows > 1 else max(width, ld))
 
 
 def alloc_workspace(nbytes: int, device) -> torch.Tensor:
@@ -234,9 +250,11 @@ def gq_saliency_strided(grad: torch.Tensor, g: int, grad_scale: float = 1.0, s: 
     pass a view ``s_all[:, offset:offset + batch * seq]`` to fill a slice of a calibration-wide buffer in place."""
     if not grad.is_cuda or grad.dtype not in _DTYPE_CODES:
         raise ValueError("grad must be a CUDA tensor of dtype bfloat16, float16 or float32")
-    if grad.dim() != 3 or (grad.shape[2] > 1 and grad.stride(2) != 1):
+    if grad.dim() != 3:
         raise ValueError("grad must be [batch, seq, d_out] with a contiguous last dimension")
-    batch, seq, d_out = grad.shape
+    (batch, seq, d_out), (by_batch, by_token, by_channel) = grad.shape, grad.stride()
+    if d_out > 1 and by_channel != 1:
+        raise ValueError("grad must be [batch, seq, d_out] with a contiguous last dimension")
     n = batch * seq
     if s is None:
         s = torch.empty((g, n), dtype=torch.float32, device=grad.device)
@@ -244,8 +262,8 @@ def gq_saliency_strided(grad: torch.Tensor, g: int, grad_scale: float = 1.0, s: 
     _, s_n, ld_s = _rows(s, "s")
     if s.shape[0] != g or s_n < n:
         raise ValueError("s must be [g, >= batch * seq]")
-    stride_b = grad.stride(0) if batch > 1 else max(grad.stride(0), seq * grad.stride(1))
-    stride_t = grad.stride(1) if seq > 1 else max(grad.stride(1), d_out)
+    stride_b = by_batch if batch > 1 else max(by_batch, seq * by_token)
+    stride_t = by_token if seq > 1 else max(by_token, d_out)
     with _on(_same_device(("grad", grad), ("s", s)), stream) as st:
         rc = lib().gq_saliency_strided(grad.data_ptr(), _DTYPE_CODES[grad.dtype], batch, seq, d_out, stride_b, stride_t, g,
                                        float(grad_scale), s.data_ptr(), ld_s, st)
