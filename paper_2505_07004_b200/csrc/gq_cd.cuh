@@ -46,11 +46,13 @@ __device__ __forceinline__ void split_bf16(float v, __nv_bfloat16 &hi, __nv_bflo
 
 // Wt = W^T, E = (What - W)^T (fp32 and as bf16 hi + lo), all [d_in][d_out].  32 x 32 tiles.
 __global__ void __launch_bounds__(256)
-cd_prepare_kernel(const float *__restrict__ W, const float *__restrict__ What, int d_in, int d_out,
-                  float *__restrict__ Wt, float *__restrict__ Et,
-                  __nv_bfloat16 *__restrict__ Ehi, __nv_bfloat16 *__restrict__ Elo)
+cd_prepare_kernel(const float *W, const float *What, int d_in, int d_out,
+                  float *Wt, float *Et,
+                  __nv_bfloat16 *Ehi, __nv_bfloat16 *Elo)
 {
     __shared__ float tw[32][33], th[32][33];
+    griddep_launch();
+    griddep_wait();
     const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
     const int i0 = blockIdx.x * 32, j0 = blockIdx.y * 32;          // coordinate / channel origin
     for (int r = ty; r < 32; r += 8) {
@@ -80,9 +82,11 @@ cd_prepare_kernel(const float *__restrict__ W, const float *__restrict__ What, i
 // 8 bytes per entry it moves.  With one entry per thread and a 64-bit modulo each to find the diagonal it took 342 us for
 // four 4096 x 4096 matrices, now 79.
 __global__ void __launch_bounds__(256)
-split_h_kernel(const float *__restrict__ H, int d_in, __nv_bfloat16 *__restrict__ Hhi, __nv_bfloat16 *__restrict__ Hlo,
-                  float *__restrict__ rdiag)
+split_h_kernel(const float *H, int d_in, __nv_bfloat16 *Hhi, __nv_bfloat16 *Hlo,
+                  float *rdiag)
 {
+    griddep_launch();
+    griddep_wait();
     const int i = static_cast<int>(blockIdx.x);
     const size_t row = static_cast<size_t>(blockIdx.y) * d_in + i;
     const float4 *src = reinterpret_cast<const float4 *>(H + row * d_in);
@@ -103,10 +107,12 @@ split_h_kernel(const float *__restrict__ H, int d_in, __nv_bfloat16 *__restrict_
 
 // Q = Qt^T back to [d_out][d_in] and What = codebook[Q].
 __global__ void __launch_bounds__(256)
-cd_finish_kernel(const float *__restrict__ codebook, const uint8_t *__restrict__ Qt, int d_in, int d_out, int m,
-                 float *__restrict__ What, uint8_t *__restrict__ Q)
+cd_finish_kernel(const float *codebook, const uint8_t *Qt, int d_in, int d_out, int m,
+                 float *What, uint8_t *Q)
 {
     __shared__ uint8_t tq[32][33];
+    griddep_launch();
+    griddep_wait();
     const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
     const int i0 = blockIdx.x * 32, j0 = blockIdx.y * 32;
     for (int r = ty; r < 32; r += 8) {
@@ -264,12 +270,14 @@ cd_block_kernel(const __grid_constant__ CUtensorMap mapH, const __grid_constant_
     auto wait_band = [&](int t) {
         (void)bounded_wait(smem_u32(&bar_h[t % CD_H_BUFS]), static_cast<uint32_t>(t / CD_H_BUFS) & 1u, wc, 21u, blockIdx.x);
     };
+    griddep_launch();
     if (tid == 128) {
         mbar_init(smem_u32(&bar_tiles), 1);
         for (int b = 0; b < CD_H_BUFS; ++b) mbar_init(smem_u32(&bar_h[b]), 1);
         abort_flag = 0u;
         fence_mbar_init();
         fence_proxy_async_smem();
+        griddep_wait();
         load_band(0);
         const uint32_t bar = smem_u32(&bar_tiles);
         mbar_arrive_expect_tx(bar, 3 * CD_TILE_FLOATS * 4);
@@ -278,6 +286,7 @@ cd_block_kernel(const __grid_constant__ CUtensorMap mapH, const __grid_constant_
         tma_load_3d(smem_u32(Ws), &mapW, bar, ch0, p.s0, 0);
         for (int b = 1; b < CD_H_BUFS; ++b) load_band(b);
     }
+    griddep_wait();
     rds[tid] = tid < p.rows ? p.rdiag[static_cast<size_t>(k) * p.d_in + p.s0 + tid] : 0.0f;
     // ---- the channel's levels, sorted (eight threads per channel), and the thresholds between neighbours: their midpoints,
     // lowered by one ulp where the upper level has the smaller given index, so that a tie goes to the smaller index

@@ -10,6 +10,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "gq_ptx.cuh"
+
 namespace gq {
 
 constexpr int CB_MAX_LEVELS = 16;
@@ -18,9 +20,11 @@ constexpr int CB_MAX_LEVELS = 16;
 // coordinates x 64 channels, so that both sides move whole 128-byte segments (one bf16 per lane and 64-byte segments took
 // 57 us for 4096 x 4096 where the bytes need 20).
 __global__ void __launch_bounds__(256)
-cb_transpose_kernel(const float *__restrict__ W, int d_in, int d_out, __nv_bfloat16 *__restrict__ W0, __nv_bfloat16 *__restrict__ W1)
+cb_transpose_kernel(const float *W, int d_in, int d_out, __nv_bfloat16 *W0, __nv_bfloat16 *W1)
 {
     __shared__ float tw[64][33];
+    griddep_launch();
+    griddep_wait();
     const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
     const int i0 = blockIdx.x * 32, j0 = blockIdx.y * 64;
 #pragma unroll
@@ -48,10 +52,12 @@ cb_transpose_kernel(const float *__restrict__ W, int d_in, int d_out, __nv_bfloa
 // regularisation so that the solve always completes.  With one thread per channel and its matrix in local memory 4096
 // channels took 89 us.
 __global__ void __launch_bounds__(128)
-cb_solve_kernel(const double *__restrict__ G, const double *__restrict__ R, int d_out, int m, double lambda,
-                float *__restrict__ codebook)
+cb_solve_kernel(const double *G, const double *R, int d_out, int m, double lambda,
+                float *codebook)
 {
     constexpr int M = CB_MAX_LEVELS;
+    griddep_launch();
+    griddep_wait();
     const int q = threadIdx.x & 15;
     const int jj = blockIdx.x * 8 + (threadIdx.x >> 4);
     const int j = jj < d_out ? jj : d_out - 1;           // all lanes take part in the shuffles
@@ -88,9 +94,11 @@ cb_solve_kernel(const double *__restrict__ G, const double *__restrict__ R, int 
 
 // What[j][i] = codebook[j][Q[j][i]], one block per channel, four codes per thread.  Q 4-byte aligned.
 __global__ void __launch_bounds__(256)
-cb_apply_kernel(const float *__restrict__ codebook, const uint8_t *__restrict__ Q, int d_in, int m, float *__restrict__ What)
+cb_apply_kernel(const float *codebook, const uint8_t *Q, int d_in, int m, float *What)
 {
     __shared__ float cb[CB_MAX_LEVELS];
+    griddep_launch();
+    griddep_wait();
     const size_t j = blockIdx.x;
     if (threadIdx.x < m) cb[threadIdx.x] = codebook[j * m + threadIdx.x];
     __syncthreads();

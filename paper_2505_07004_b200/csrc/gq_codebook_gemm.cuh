@@ -149,6 +149,7 @@ codebook_gemm_kernel(const __grid_constant__ CUtensorMap mapH0, const __grid_con
         prefetch_tensormap(&mapW0);
         prefetch_tensormap(&mapW1);
     }
+    griddep_launch();
     if (warp == 2) {
         tmem_alloc(smem_u32(&tmem_base_smem), TMEM_COLS);
         tmem_relinquish();
@@ -158,6 +159,7 @@ codebook_gemm_kernel(const __grid_constant__ CUtensorMap mapH0, const __grid_con
     tc_fence_after_sync();
     const uint32_t tmem_base = tmem_base_smem;
     const WaitCtx wc{&abort_flag, p.status, p.wait_budget_ns};
+    griddep_wait();
     const int kblocks = (p.d + TILE_K - 1) / TILE_K;
 
     if (warp == 0 && lane == 0) {
@@ -271,7 +273,7 @@ codebook_gemm_kernel(const __grid_constant__ CUtensorMap mapH0, const __grid_con
                 for (int w = 0; w < WORDS; w += 2) {
                     uint2 v = make_uint2(0xffffffffu, 0xffffffffu);
                     if (have && ks < ksteps && row0 + 4 * w < p.d) {
-                        v = __ldg(reinterpret_cast<const uint2 *>(q_row + row0 + 4 * w));
+                        v = ld_u32x2(q_row + row0 + 4 * w);
                         v.x = __vminu4(v.x, top);
                         v.y = __vminu4(v.y, top);
                     }
@@ -368,7 +370,7 @@ codebook_gemm_kernel(const __grid_constant__ CUtensorMap mapH0, const __grid_con
                             const bool in = row < p.d;
 #pragma unroll
                             for (int b = 0; b < 2; ++b) {
-                                code[b][x] = in ? __ldg(reinterpret_cast<const unsigned short *>(qb[b] + row)) : 0u;
+                                code[b][x] = in ? ld_u16(qb[b] + row) : 0u;
                             }
                         }
                         tmem_ld_wait();
@@ -438,7 +440,7 @@ codebook_gemm_kernel(const __grid_constant__ CUtensorMap mapH0, const __grid_con
 #pragma unroll
                     for (int x = 0; x < 4; ++x) {
                         const int row = row0 + n0 + 8 * x;
-                        codes[x] = row < p.d ? __ldg(reinterpret_cast<const uint2 *>(q_row + row)) : make_uint2(0u, 0u);
+                        codes[x] = row < p.d ? ld_u32x2(q_row + row) : make_uint2(0u, 0u);
                     }
                     tmem_ld_wait();
 #pragma unroll

@@ -59,11 +59,15 @@ constexpr int GD_PARTIALS_PER_UNIT = 2 * GD_EPI_WARPS;       // one fp64 per (CT
 constexpr int GD_TARGET_EXP = 14;                            // the largest |delta| * 2^e lies in [2^14, 2^15)
 constexpr int GD_MAX_SHIFT = 100;                            // |e| is kept below this (the scale stays a normal float)
 
+constexpr unsigned DELTA_BLOCK_MAXIMA = 240;      // what the 1 KiB header holds
+
 // Header of the objective workspace, written by the preparation kernels and read by the reduction.
 struct GramDotHeader {
     unsigned int absmax_bits;   // bit pattern of max |W - W_hat| (non-negative floats order like unsigned ints)
     int shift;                  // e: the fp16 matrix holds (W - W_hat) * 2^e
     unsigned int blocks_done;   // groups whose loss has been written (the last one forms the total)
+    unsigned int pad[13];       // the maxima start a 64-byte segment
+    unsigned int block_max[DELTA_BLOCK_MAXIMA];   // bit patterns of the first pass's maxima, if it has that few blocks
 };
 
 struct GramDotParams {
@@ -113,10 +117,14 @@ constexpr int DELTA_VEC_PER_THREAD = 4;      // float4 pairs a thread of the two
 
 // ------------------------------------------------------------------------------------------------
 // max |W - W_hat| over the layer (the differences are formed in fp32, as everywhere in the objective).
-// header->absmax_bits must be 0 before the launch.  One block per 256 * DELTA_VEC_PER_THREAD float4 pairs.
+// One block per 256 * DELTA_VEC_PER_THREAD float4 pairs.  Up to DELTA_BLOCK_MAXIMA blocks leave one maximum each for the
+// second pass to combine; beyond that they meet in header->absmax_bits, which must be 0 before the launch (clearing it is an
+// operation of its own on the stream, which a layer of a few microseconds notices).
 __global__ void __launch_bounds__(256)
 delta_absmax_kernel(const float *__restrict__ W, const float *__restrict__ What, unsigned count4, GramDotHeader *header)
 {
+    griddep_launch();
+    griddep_wait();
     const unsigned base = blockIdx.x * (256u * DELTA_VEC_PER_THREAD) + threadIdx.x;
     float4 w[DELTA_VEC_PER_THREAD], q[DELTA_VEC_PER_THREAD];
 #pragma unroll
@@ -139,7 +147,10 @@ delta_absmax_kernel(const float *__restrict__ W, const float *__restrict__ What,
     if (threadIdx.x == 0) {
         for (int w8 = 1; w8 < 8; ++w8) m = fmaxf(m, red[w8]);
         // NaN never wins fmaxf; an infinite difference gives 0x7f800000 and the shift below saturates
-        if (m > 0.0f) atomicMax(&header->absmax_bits, __float_as_uint(m));
+        if (gridDim.x <= DELTA_BLOCK_MAXIMA)
+            header->block_max[blockIdx.x] = m > 0.0f ? __float_as_uint(m) : 0u;
+        else if (m > 0.0f)
+            atomicMax(&header->absmax_bits, __float_as_uint(m));
     }
 }
 
@@ -161,6 +172,8 @@ __global__ void __launch_bounds__(256)
 delta_half_kernel(const float *__restrict__ W, const float *__restrict__ What, unsigned count4, GramDotHeader *header,
                   __half *__restrict__ out)
 {
+    griddep_launch();
+    griddep_wait();
     const unsigned blk = gridDim.x - 1u - blockIdx.x;
     const unsigned base = blk * (256u * DELTA_VEC_PER_THREAD) + threadIdx.x;
     float4 w[DELTA_VEC_PER_THREAD], q[DELTA_VEC_PER_THREAD];
@@ -171,8 +184,23 @@ delta_half_kernel(const float *__restrict__ W, const float *__restrict__ What, u
         w[t] = in ? ld_f32x4_last_use(reinterpret_cast<const float4 *>(W) + idx) : make_float4(0.f, 0.f, 0.f, 0.f);
         q[t] = in ? ld_f32x4_last_use(reinterpret_cast<const float4 *>(What) + idx) : make_float4(0.f, 0.f, 0.f, 0.f);
     }
-    const int e = gram_dot_shift(header->absmax_bits);
-    if (blockIdx.x == 0 && threadIdx.x == 0) header->shift = e;
+    unsigned int absmax_bits = 0u;
+    if (gridDim.x <= DELTA_BLOCK_MAXIMA) {
+        if (threadIdx.x < gridDim.x) absmax_bits = header->block_max[threadIdx.x];
+        __shared__ unsigned int red[8];
+        absmax_bits = __reduce_max_sync(0xffffffffu, absmax_bits);
+        if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = absmax_bits;
+        __syncthreads();
+#pragma unroll
+        for (int w8 = 0; w8 < 8; ++w8) absmax_bits = max(absmax_bits, red[w8]);
+    } else {
+        absmax_bits = header->absmax_bits;
+    }
+    const int e = gram_dot_shift(absmax_bits);
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        header->shift = e;
+        header->blocks_done = 0u;
+    }
     const float scale = __uint_as_float(static_cast<unsigned int>(127 + e) << 23);
 #pragma unroll
     for (int t = 0; t < DELTA_VEC_PER_THREAD; ++t) {
@@ -189,13 +217,14 @@ delta_half_kernel(const float *__restrict__ W, const float *__restrict__ What, u
 // loss[k] = 2^(-2e) * sum over the group's partial sums (block k), loss[g] = sum_k loss[k] (formed, in group order,
 // by whichever block finishes last).  Every sum is formed in a fixed order (strided per thread, butterfly per warp,
 // warp results in order), so the result does not vary from run to run.  partials: [g][slots][per_unit] (units are
-// numbered group-major).  header->blocks_done must be 0 before the launch.
+// numbered group-major).  header->blocks_done is 0 before the launch (delta_half_kernel).
 __global__ void __launch_bounds__(256)
-gram_dot_reduce_kernel(const double *__restrict__ partials, int slots, int g, int per_unit, GramDotHeader *header,
-                       double *__restrict__ loss)
+gram_dot_reduce_kernel(const double *partials, int slots, int g, int per_unit, GramDotHeader *header, double *loss)
 {
     __shared__ double warp_sum[8];
     __shared__ bool last;
+    griddep_launch();
+    griddep_wait();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int k = blockIdx.x;
     const double *pk = partials + static_cast<size_t>(k) * slots * per_unit;
@@ -275,6 +304,7 @@ gram_dot_kernel(const __grid_constant__ CUtensorMap mapD, const GramDotParams p)
         fence_mbar_init();
         prefetch_tensormap(&mapD);
     }
+    griddep_launch();
     if (warp == 2) {
         tmem_alloc(smem_u32(&tmem_base_smem), TMEM_COLS);
         tmem_relinquish();
@@ -284,6 +314,7 @@ gram_dot_kernel(const __grid_constant__ CUtensorMap mapD, const GramDotParams p)
     tc_fence_after_sync();
     const uint32_t tmem_base = tmem_base_smem;
     const WaitCtx wc{&abort_flag, p.status, p.wait_budget_ns};
+    griddep_wait();
 
     if (warp < 4) {
         // The service warpgroup keeps 40 registers per thread; the rest goes to the epilogue warpgroups.

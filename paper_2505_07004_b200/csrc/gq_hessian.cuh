@@ -57,6 +57,7 @@ constexpr int HS_SET_WARPS = 4;                                // warps per set:
 constexpr int HS_SCALER_WARPS = HS_SETS * HS_SET_WARPS;
 constexpr int HS_EPI_WARPS = 8;
 constexpr int HS_STAGING_BYTES = HS_EPI_WARPS * 4096;          // one 32 x 32 fp32 block per epilogue warp
+constexpr int HS_RING_BLOCKS = HS_STAGES * HS_STAGE_BYTES / (HS_EPI_WARPS * 4096);      // blocks per warp the ring can stage
 constexpr int HS_THREADS = 32 * (4 + HS_SCALER_WARPS + HS_EPI_WARPS);
 constexpr int HS_SMEM_BYTES = HS_STAGES * HS_STAGE_BYTES + HS_STAGING_BYTES + 1024;
 
@@ -134,11 +135,13 @@ __device__ __forceinline__ void st_shared_16(uint32_t addr, const uint4 &v)
 // 2 q + 1 of a token sit side by side, so a scaler thread fetches both with one 8-byte load and does no
 // conversion work in its loop (sixteen threads share a token; converting there would be done sixteen times).
 __global__ void __launch_bounds__(256)
-split_saliency_kernel(const float *__restrict__ s, long long ld_s, int n, int g, uint2 *__restrict__ out);
+split_saliency_kernel(const float *s, long long ld_s, int n, int g, uint2 *out);
 
 __global__ void __launch_bounds__(256)
-split_saliency_kernel(const float *__restrict__ s, long long ld_s, int n, int g, uint2 *__restrict__ out)
+split_saliency_kernel(const float *s, long long ld_s, int n, int g, uint2 *out)
 {
+    griddep_launch();
+    griddep_wait();
     const int slots = (g + 1) / 2;
     const long long total = static_cast<long long>(slots) * n;
     for (long long idx = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x; idx < total;
@@ -228,6 +231,7 @@ hessian_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_constant__
         prefetch_tensormap(&mapX);
         prefetch_tensormap(&mapH);
     }
+    griddep_launch();
     if (warp == 2) {
         tmem_alloc(smem_u32(&tmem_base_smem), TMEM_COLS);
         tmem_relinquish();
@@ -237,6 +241,7 @@ hessian_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_constant__
     tc_fence_after_sync();
     const uint32_t tmem_base = tmem_base_smem;
     const WaitCtx wc{&abort_flag, p.status, p.wait_budget_ns};
+    griddep_wait();
 
     if (warp == 0 && lane == 0) {
         // ------------------------------------------------------------------ TMA producer: raw B columns
@@ -402,14 +407,14 @@ hessian_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_constant__
 #pragma unroll
                     for (int j = 0; j < PASSES; ++j) {
                         buf[j] = ld_stream_16(src + j * step);
-                        sv[j] = __ldg(ssrc + j * TOK_PER_PASS);
+                        sv[j] = ld_u32x2(ssrc + j * TOK_PER_PASS);
                     }
                 } else {
 #pragma unroll
                     for (int j = 0; j < PASSES; ++j) {
                         const bool t_ok = tok0 + j * TOK_PER_PASS < p.n;
                         buf[j] = (f_ok && t_ok) ? ld_stream_16(src + j * step) : make_uint4(0u, 0u, 0u, 0u);
-                        sv[j] = t_ok ? __ldg(ssrc + j * TOK_PER_PASS) : make_uint2(0u, 0u);
+                        sv[j] = t_ok ? ld_u32x2(ssrc + j * TOK_PER_PASS) : make_uint2(0u, 0u);
                     }
                 }
             }
@@ -451,6 +456,12 @@ hessian_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_constant__
             (void)mbar_try_wait(smem_u32(&bar_acc_full), acc_ph);     // every lane observes the completed phase
             tc_fence_after_sync();
             const int row0 = u.ti * TILE_M + static_cast<int>(rank) * CTA_ROWS + q * 32;
+            // After the pair's last item nobody uses the operand ring any more (the accumulators being complete means that
+            // the MMAs have read it): six of a warp's eight blocks are staged there, so that a block does not wait for the
+            // copy engine to have read the one before it (1300 clocks a block, 10 000 an item: the end of every launch).
+            WorkItem w_next;
+            const bool last = !work_item(p.sched, pair, it + 1, w_next);
+            int staged = 0;
             for (int kk = 0; kk < HS_GROUPS; ++kk) {
 #pragma unroll 1
                 for (int c4 = 0; u.use[kk] && c4 < 4; ++c4) {
@@ -462,16 +473,21 @@ hessian_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_constant__
                     tmem_ld_32x32(tmem_base + (static_cast<uint32_t>(q * 32) << 16) +
                                       static_cast<uint32_t>(kk * TILE_N + cc * 32), r);
                     tmem_ld_wait();
-                    if (lane == 0) bulk_wait_group_read0();   // the copy engine has read the previous staging block
+                    const bool in_ring = last && staged < HS_RING_BLOCKS;
+                    const uint32_t block = in_ring ? ring + static_cast<uint32_t>(ew * HS_RING_BLOCKS + staged) * 4096u : stg;
+                    // the copy engine has read what this block's place held before
+                    if (lane == 0 && !in_ring && !(last && staged == HS_RING_BLOCKS)) bulk_wait_group_read0();
+                    if (lane == 0 && last && staged == 0) bulk_wait_group_read0();
+                    ++staged;
                     __syncwarp();
 #pragma unroll
                     for (int v = 0; v < 8; ++v)
-                        st_shared_16(stg + static_cast<uint32_t>(lane * 128 + ((v ^ (lane & 7)) << 4)),
+                        st_shared_16(block + static_cast<uint32_t>(lane * 128 + ((v ^ (lane & 7)) << 4)),
                                      make_uint4(r[v * 4 + 0], r[v * 4 + 1], r[v * 4 + 2], r[v * 4 + 3]));
                     fence_proxy_async_smem();
                     __syncwarp();
                     if (lane == 0) {
-                        tma_reduce_add_3d_hint(&mapH, stg, col0, row0, u.grp[kk], pol_h);
+                        tma_reduce_add_3d_hint(&mapH, block, col0, row0, u.grp[kk], pol_h);
                         bulk_commit_group();
                     }
                 }

@@ -7,6 +7,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "gq_ptx.cuh"
+
 namespace gq {
 
 __device__ __forceinline__ void bf16x8_to_float(const uint4 &v, float (&f)[8])
@@ -124,6 +126,8 @@ __global__ void __launch_bounds__(256)
 saliency_kernel(const __nv_bfloat16 *__restrict__ grad, unsigned n, int m, long long ld_grad, int g, float coef,
                 float *__restrict__ s, long long ld_s, uint32_t *__restrict__ words)
 {
+    griddep_launch();
+    griddep_wait();
     const int lane = threadIdx.x & 31;
     const unsigned seg = blockIdx.x * 8u + (threadIdx.x >> 5);
     if (seg >= n * static_cast<unsigned>(g)) return;
@@ -168,6 +172,8 @@ saliency_strided_kernel(const void *__restrict__ grad, unsigned n, unsigned seq,
 {
     constexpr int PER_VEC = (DTYPE == SAL_FP32) ? 4 : 8;          // values per 16-byte load
     constexpr int ELEM = (DTYPE == SAL_FP32) ? 4 : 2;
+    griddep_launch();
+    griddep_wait();
     const int lane = threadIdx.x & 31;
     const unsigned seg = blockIdx.x * 8u + (threadIdx.x >> 5);
     if (seg >= n * static_cast<unsigned>(g)) return;
@@ -203,6 +209,8 @@ __global__ void __launch_bounds__(256)
 mirror_kernel(float *__restrict__ H, int d)
 {
     __shared__ float tile[MIRROR_TILE][MIRROR_TILE + 1];
+    griddep_launch();
+    griddep_wait();
     int bi, bj;
     {
         const int t = static_cast<int>(blockIdx.x);

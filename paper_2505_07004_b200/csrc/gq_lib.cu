@@ -62,6 +62,24 @@ struct LaunchScope {
     }
 };
 
+// Launch with programmatic stream serialisation (see griddep_wait in gq_ptx.cuh, which every kernel launched here calls).
+// Errors are left for cudaGetLastError, as with <<< >>>.
+template <typename... Params, typename... Args>
+void launch(void (*kernel)(Params...), dim3 grid, int threads, size_t smem, cudaStream_t st, Args &&...args)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(static_cast<unsigned>(threads));
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    (void)cudaLaunchKernelEx(&cfg, kernel, static_cast<Params>(args)...);
+}
+
 // Per-device status word {status, site, block, unit}; written by kernels, read by gq_check().
 __device__ uint32_t g_status_word[4];
 
@@ -328,13 +346,13 @@ size_t hessian_ws_bytes(int64_t n_max, int64_t, int32_t g)
 struct ObjectiveLayout {
     size_t header_off, half_off, partials_off, total;
 };
-// Scratch of gq_objective: a 1 KiB header (largest |delta| and the chosen power-of-two scale), delta as one fp16
+// Scratch of gq_objective: a header (largest |delta| and the chosen power-of-two scale), delta as one fp16
 // matrix, and one fp64 partial sum per (work unit, CTA of the pair, epilogue warp).
 ObjectiveLayout objective_layout(int64_t d_in, int64_t d_out, int32_t g)
 {
     ObjectiveLayout L;
     L.header_off = 0;
-    L.half_off = 1024;
+    L.half_off = round_up(sizeof(gq::GramDotHeader), 1024);
     L.partials_off = L.half_off + round_up(static_cast<size_t>(d_in) * static_cast<size_t>(d_out) * 2, 1024);
     L.total = L.partials_off +
               round_up(static_cast<size_t>(tiles_for(d_in)) * g * gq::GD_PARTIALS_PER_UNIT * sizeof(double), 1024);
@@ -463,7 +481,7 @@ static int32_t saliency_impl(const void *grad, int64_t n, int64_t d_out, int64_t
     const unsigned grid = static_cast<unsigned>((n * g + 7) / 8);            // one warp per (token, group) segment
     {
         LaunchScope scope(GQ_KERNEL_SALIENCY, static_cast<cudaStream_t>(stream));
-        gq::saliency_kernel<<<grid, 256, 0, static_cast<cudaStream_t>(stream)>>>(
+        launch(gq::saliency_kernel, dim3(grid), 256, 0, static_cast<cudaStream_t>(stream), 
             static_cast<const __nv_bfloat16 *>(grad), static_cast<unsigned>(n), m, ld_grad, g, coef, s, ld_s,
             prepare ? static_cast<uint32_t *>(hessian_workspace) : nullptr);
     }
@@ -512,13 +530,13 @@ int32_t gq_saliency_strided(const void *grad, int32_t dtype, int64_t batch, int6
     {
         LaunchScope scope(GQ_KERNEL_SALIENCY, st);
         if (dtype == GQ_DTYPE_BF16)
-            gq::saliency_strided_kernel<gq::SAL_BF16><<<grid, 256, 0, st>>>(grad, static_cast<unsigned>(n), static_cast<unsigned>(seq), m,
+            launch(gq::saliency_strided_kernel<gq::SAL_BF16>, dim3(grid), 256, 0, st, grad, static_cast<unsigned>(n), static_cast<unsigned>(seq), m,
                                                                          stride_b, stride_t, g, coef, s, ld_s);
         else if (dtype == GQ_DTYPE_FP16)
-            gq::saliency_strided_kernel<gq::SAL_FP16><<<grid, 256, 0, st>>>(grad, static_cast<unsigned>(n), static_cast<unsigned>(seq), m,
+            launch(gq::saliency_strided_kernel<gq::SAL_FP16>, dim3(grid), 256, 0, st, grad, static_cast<unsigned>(n), static_cast<unsigned>(seq), m,
                                                                          stride_b, stride_t, g, coef, s, ld_s);
         else
-            gq::saliency_strided_kernel<gq::SAL_FP32><<<grid, 256, 0, st>>>(grad, static_cast<unsigned>(n), static_cast<unsigned>(seq), m,
+            launch(gq::saliency_strided_kernel<gq::SAL_FP32>, dim3(grid), 256, 0, st, grad, static_cast<unsigned>(n), static_cast<unsigned>(seq), m,
                                                                          stride_b, stride_t, g, coef, s, ld_s);
     }
     GQ_CUDA(cudaGetLastError());
@@ -571,7 +589,7 @@ static int32_t hessian_accumulate_impl(const void *X, int64_t n, int64_t d_in, i
         const int grid_s = grid_for(static_cast<long long>((g + 1) / 2) * n, 256, di->sm_count, 4);
         {
             LaunchScope scope(GQ_KERNEL_SPLIT_SALIENCY, st);
-            gq::split_saliency_kernel<<<grid_s, 256, 0, st>>>(s, ld_s, static_cast<int>(n), g,
+            launch(gq::split_saliency_kernel, dim3(grid_s), 256, 0, st, s, ld_s, static_cast<int>(n), g,
                                                              static_cast<uint2 *>(workspace));
         }
         GQ_CUDA(cudaGetLastError());
@@ -613,7 +631,7 @@ static int32_t hessian_accumulate_impl(const void *X, int64_t n, int64_t d_in, i
             const unsigned grid_s = static_cast<unsigned>((static_cast<long long>(ahead->n) * g + 7) / 8);
             {
                 LaunchScope scope(GQ_KERNEL_SALIENCY, st);
-                gq::saliency_kernel<<<grid_s, 256, 0, st>>>(ahead->grad, ahead->n, ahead->m, ahead->ld_grad, g, ahead->coef,
+                launch(gq::saliency_kernel, dim3(grid_s), 256, 0, st, ahead->grad, ahead->n, ahead->m, ahead->ld_grad, g, ahead->coef,
                                                             ahead->s, ahead->ld_s, ahead->words);
             }
             GQ_CUDA(cudaGetLastError());
@@ -621,7 +639,7 @@ static int32_t hessian_accumulate_impl(const void *X, int64_t n, int64_t d_in, i
     }
     {
         LaunchScope scope(GQ_KERNEL_HESSIAN, st);
-        gq::hessian_kernel<<<grid, gq::HS_THREADS, gq::HS_SMEM_BYTES, st>>>(mapX, mapH, p);
+        launch(gq::hessian_kernel, dim3(grid), gq::HS_THREADS, gq::HS_SMEM_BYTES, st, mapX, mapH, p);
     }
     GQ_CUDA(cudaGetLastError());
     return GQ_OK;
@@ -695,7 +713,7 @@ int32_t gq_hessian_finalize(float *H, int64_t d_in, int32_t g, void *stream)
     dim3 grid(nb * (nb + 1) / 2, static_cast<unsigned>(g));
     {
         LaunchScope scope(GQ_KERNEL_MIRROR, static_cast<cudaStream_t>(stream));
-        gq::mirror_kernel<<<grid, 256, 0, static_cast<cudaStream_t>(stream)>>>(H, static_cast<int>(d_in));
+        launch(gq::mirror_kernel, dim3(grid), 256, 0, static_cast<cudaStream_t>(stream), H, static_cast<int>(d_in));
     }
     GQ_CUDA(cudaGetLastError());
     return GQ_OK;
@@ -773,19 +791,19 @@ int32_t gq_objective(const float *W, const float *W_hat, int64_t d_in, int64_t d
     double *partials = reinterpret_cast<double *>(ws + L.partials_off);
     const int64_t m = d_out / g;
     // delta = W - W_hat as one fp16 matrix scaled by a power of two taken from max |delta| (two passes over W, W_hat)
-    GQ_CUDA(cudaMemsetAsync(header, 0, sizeof(gq::GramDotHeader), st));
     {
         const unsigned count4 = static_cast<unsigned>(d_in * d_out / 4);
         const unsigned per_block = 256u * gq::DELTA_VEC_PER_THREAD;
         const unsigned blocks = (count4 + per_block - 1) / per_block;
+        if (blocks > gq::DELTA_BLOCK_MAXIMA) GQ_CUDA(cudaMemsetAsync(&header->absmax_bits, 0, sizeof header->absmax_bits, st));
         {
             LaunchScope scope(GQ_KERNEL_SPLIT_DELTA, st);
-            gq::delta_absmax_kernel<<<blocks, 256, 0, st>>>(W, W_hat, count4, header);
+            launch(gq::delta_absmax_kernel, dim3(blocks), 256, 0, st, W, W_hat, count4, header);
         }
         GQ_CUDA(cudaGetLastError());
         {
             LaunchScope scope(GQ_KERNEL_SPLIT_DELTA, st);
-            gq::delta_half_kernel<<<blocks, 256, 0, st>>>(W, W_hat, count4, header, dh);
+            launch(gq::delta_half_kernel, dim3(blocks), 256, 0, st, W, W_hat, count4, header, dh);
         }
         GQ_CUDA(cudaGetLastError());
     }
@@ -810,12 +828,12 @@ int32_t gq_objective(const float *W, const float *W_hat, int64_t d_in, int64_t d
     p.wait_budget_ns = wait_budget_ns();
     {
         LaunchScope scope(GQ_KERNEL_GRAM_DOT, st);
-        gq::gram_dot_kernel<<<2 * p.sched.pairs, gq::GD_THREADS, gq::GD_SMEM_BYTES, st>>>(mapD, p);
+        launch(gq::gram_dot_kernel, dim3(2 * p.sched.pairs), gq::GD_THREADS, gq::GD_SMEM_BYTES, st, mapD, p);
     }
     GQ_CUDA(cudaGetLastError());
     {
         LaunchScope scope(GQ_KERNEL_REDUCE, st);
-        gq::gram_dot_reduce_kernel<<<static_cast<unsigned>(g), 256, 0, st>>>(partials, slots, g, gq::GD_PARTIALS_PER_UNIT, header, loss_out);
+        launch(gq::gram_dot_reduce_kernel, dim3(static_cast<unsigned>(g)), 256, 0, st, partials, slots, g, gq::GD_PARTIALS_PER_UNIT, header, loss_out);
     }
     GQ_CUDA(cudaGetLastError());
     return GQ_OK;
@@ -929,7 +947,7 @@ static int32_t split_h(const float *H, int64_t d_in, int32_t g, uint8_t *ws, cud
     const dim3 grid(static_cast<unsigned>(d_in), static_cast<unsigned>(g));
     {
         LaunchScope scope(GQ_KERNEL_CD_AUX, st);
-        gq::split_h_kernel<<<grid, 256, 0, st>>>(H, static_cast<int>(d_in), reinterpret_cast<__nv_bfloat16 *>(ws + S.h0),
+        launch(gq::split_h_kernel, dim3(grid), 256, 0, st, H, static_cast<int>(d_in), reinterpret_cast<__nv_bfloat16 *>(ws + S.h0),
                                                  reinterpret_cast<__nv_bfloat16 *>(ws + S.h1), reinterpret_cast<float *>(ws + S.rdiag));
     }
     GQ_CUDA(cudaGetLastError());
@@ -982,7 +1000,7 @@ static int32_t cd_cycles_impl(const float *W, float *W_hat, uint8_t *Q, const fl
     const dim3 tgrid(static_cast<unsigned>((d_in + 31) / 32), static_cast<unsigned>((d_out + 31) / 32));
     {
         LaunchScope scope(GQ_KERNEL_CD_AUX, st);
-        gq::cd_prepare_kernel<<<tgrid, 256, 0, st>>>(W, W_hat, static_cast<int>(d_in), static_cast<int>(d_out), Wt,
+        launch(gq::cd_prepare_kernel, dim3(tgrid), 256, 0, st, W, W_hat, static_cast<int>(d_in), static_cast<int>(d_out), Wt,
                                                      Et, Ehi, Elo);
     }
     GQ_CUDA(cudaGetLastError());
@@ -1035,7 +1053,7 @@ static int32_t cd_cycles_impl(const float *W, float *W_hat, uint8_t *Q, const fl
                 pp.wait_budget_ns = wait_budget_ns();
                 {
                     LaunchScope scope(GQ_KERNEL_CD_PANEL, st);
-                    gq::pair_gemm_kernel<gq::MODE_PANEL><<<2 * pp.sched.pairs, gq::OBJ_THREADS, gq::OBJ_SMEM_BYTES, st>>>(
+                    launch(gq::pair_gemm_kernel<gq::MODE_PANEL>, dim3(2 * pp.sched.pairs), gq::OBJ_THREADS, gq::OBJ_SMEM_BYTES, st, 
                         mapHhi, mapHlo, mapEhi, mapElo, mapEhi, mapElo, pp);
                 }
                 GQ_CUDA(cudaGetLastError());
@@ -1052,14 +1070,14 @@ static int32_t cd_cycles_impl(const float *W, float *W_hat, uint8_t *Q, const fl
                 LaunchScope scope(GQ_KERNEL_CD_BLOCK, st);
                 // fewer levels, fewer compares and selects per coordinate
                 const auto kernel = m <= 4 ? gq::cd_block_kernel<4> : m <= 8 ? gq::cd_block_kernel<8> : gq::cd_block_kernel<16>;
-                kernel<<<g * slices, gq::CD_THREADS, gq::CD_SMEM_BYTES, st>>>(mapHb, mapWb, mapEb, mapPb, bp);
+                launch(kernel, dim3(g * slices), gq::CD_THREADS, gq::CD_SMEM_BYTES, st, mapHb, mapWb, mapEb, mapPb, bp);
             }
             GQ_CUDA(cudaGetLastError());
         }
     }
     {
         LaunchScope scope(GQ_KERNEL_CD_AUX, st);
-        gq::cd_finish_kernel<<<tgrid, 256, 0, st>>>(codebook, Qt, static_cast<int>(d_in), static_cast<int>(d_out), m, W_hat, Q);
+        launch(gq::cd_finish_kernel, dim3(tgrid), 256, 0, st, codebook, Qt, static_cast<int>(d_in), static_cast<int>(d_out), m, W_hat, Q);
     }
     GQ_CUDA(cudaGetLastError());
     return GQ_OK;
@@ -1112,7 +1130,7 @@ static int32_t split_w(const float *W, int64_t d_in, int64_t d_out, uint8_t *ws,
     const dim3 grid(static_cast<unsigned>((d_in + 31) / 32), static_cast<unsigned>((d_out + 63) / 64));
     {
         LaunchScope scope(GQ_KERNEL_CB_AUX, st);
-        gq::cb_transpose_kernel<<<grid, 256, 0, st>>>(W, static_cast<int>(d_in), static_cast<int>(d_out),
+        launch(gq::cb_transpose_kernel, dim3(grid), 256, 0, st, W, static_cast<int>(d_in), static_cast<int>(d_out),
                                                       reinterpret_cast<__nv_bfloat16 *>(ws + L.w0),
                                                       reinterpret_cast<__nv_bfloat16 *>(ws + L.w1));
     }
@@ -1167,18 +1185,18 @@ static int32_t codebook_update_impl(const float *W, const uint8_t *Q, int32_t m,
     {
         LaunchScope scope(GQ_KERNEL_CB_GEMM, st);
         const auto kernel = mp == 4 ? gq::codebook_gemm_kernel<4> : mp == 8 ? gq::codebook_gemm_kernel<8> : gq::codebook_gemm_kernel<16>;
-        kernel<<<2 * p.pairs, gq::CG_THREADS, gq::CG_SMEM_BYTES, st>>>(mH0, mH1, mW0, mW1, p);
+        launch(kernel, dim3(2 * p.pairs), gq::CG_THREADS, gq::CG_SMEM_BYTES, st, mH0, mH1, mW0, mW1, p);
     }
     GQ_CUDA(cudaGetLastError());
     {
         LaunchScope scope(GQ_KERNEL_CB_FOLD, st);
-        gq::cb_solve_kernel<<<static_cast<unsigned>((d_out + 7) / 8), 128, 0, st>>>(Gm, Rv, static_cast<int>(d_out), m,
+        launch(gq::cb_solve_kernel, dim3(static_cast<unsigned>((d_out + 7) / 8)), 128, 0, st, Gm, Rv, static_cast<int>(d_out), m,
                                                                                     lambda, codebook);
     }
     GQ_CUDA(cudaGetLastError());
     if (W_hat) {
         LaunchScope scope(GQ_KERNEL_CB_AUX, st);
-        gq::cb_apply_kernel<<<static_cast<unsigned>(d_out), 256, 0, st>>>(codebook, Q, static_cast<int>(d_in), m, W_hat);
+        launch(gq::cb_apply_kernel, dim3(static_cast<unsigned>(d_out)), 256, 0, st, codebook, Q, static_cast<int>(d_in), m, W_hat);
         GQ_CUDA(cudaGetLastError());
     }
     return GQ_OK;

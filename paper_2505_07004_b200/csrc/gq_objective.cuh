@@ -160,6 +160,7 @@ pair_gemm_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant
         prefetch_tensormap(&map4);
         prefetch_tensormap(&map5);
     }
+    griddep_launch();
     if (warp == 2) {
         tmem_alloc(smem_u32(&tmem_base_smem), TMEM_COLS);
         tmem_relinquish();
@@ -170,6 +171,7 @@ pair_gemm_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant
     const uint32_t tmem_base = tmem_base_smem;
 
     const WaitCtx wc{&abort_flag, p.status, p.wait_budget_ns};
+    griddep_wait();
     const int kblocks = (p.rows + TILE_K - 1) / TILE_K;
 
     if (warp == 0 && lane == 0) {

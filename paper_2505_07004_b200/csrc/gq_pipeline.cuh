@@ -58,8 +58,11 @@ inline Schedule plan_schedule(int units, int ksteps, int pairs, bool balanced)
         p.full_waves = units / pairs;
         p.tail_units = units - p.full_waves * pairs;
         const long long total = static_cast<long long>(p.tail_units) * ksteps;
+        // at least a pair per unit, however short the units (24 units of one k-step each: three pairs took 64 us for what 24
+        // do in 12); at most so many that a piece is worth its epilogue (with 4 k-steps in place of 8 launches of 512 tokens
+        // got 20-30 % longer: every piece adds all of its tile to H)
         long long tp = total / MIN_PIECE_KSTEPS;
-        if (tp < 1) tp = 1;
+        if (tp < p.tail_units) tp = p.tail_units;
         if (tp > pairs) tp = pairs;
         p.tail_pairs = static_cast<int>(tp);
     }

@@ -31,6 +31,36 @@ __device__ __forceinline__ bool elect_one()
     return pred != 0;
 }
 
+// ---------------------------------------------------------------- dependent launches
+// The library's kernels are launched with programmatic stream serialisation: a kernel's blocks may become resident while the
+// kernel before it in the stream is still running, so that its set-up and launch latency overlap the other's tail.  Every
+// thread of every kernel calls griddep_wait() before it touches global memory: it returns when all earlier kernels of the
+// stream have completed and their writes are visible.  griddep_launch() lets the next kernel's blocks be scheduled once
+// every block of this one has reached it.  What an earlier kernel of this library wrote is read with ordinary loads (no
+// __ldg, no const __restrict__ parameters): the compiler may move a read-only load above the wait.
+__device__ __forceinline__ void griddep_wait()
+{
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+__device__ __forceinline__ void griddep_launch()
+{
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
+// Ordinary (coherent) loads that keep their place among the other volatile statements.
+__device__ __forceinline__ uint2 ld_u32x2(const void *p)
+{
+    uint2 v;
+    asm volatile("ld.global.v2.u32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "l"(p) : "memory");
+    return v;
+}
+__device__ __forceinline__ uint32_t ld_u16(const void *p)
+{
+    unsigned short v;
+    asm volatile("ld.global.u16 %0, [%1];" : "=h"(v) : "l"(p) : "memory");
+    return v;
+}
+
 // ---------------------------------------------------------------- cluster of two CTAs
 __device__ __forceinline__ uint32_t cluster_ctarank()
 {
