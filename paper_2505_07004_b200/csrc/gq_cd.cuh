@@ -185,16 +185,18 @@ struct ChainOperands {
     }
 };
 
-// Steps I .. CD_BAND - 1 of a band.  Operands are read two steps ahead (the product warps keep the shared-memory pipe
-// busy, so a read takes longer than a step).  Written as a recursion because the compiler does not unroll the loop, and
-// the sums have to stay in registers.
-template <int LEV, int I>
+// Steps I .. RUN - 1 of a run (a band is CD_BAND / RUN of them).  Bu is a window of 32 sums that starts with the run's rows;
+// every step updates what comes after it in the window.  In the second run of a band the window's upper half lies past the
+// band: those sums are formed from whatever follows in shared memory and never used.  Operands are read two steps ahead (the
+// product warps keep the shared-memory pipe busy, so a read takes longer than a step).  Written as a recursion because the
+// compiler does not unroll the loop, and the sums have to stay in registers.
+template <int LEV, int RUN, int I>
 __device__ __forceinline__ void chain_steps(const ChainOperands &cur, const ChainOperands &nxt, const float *hd, const float *rb,
                                             float *wb, float *eb, float (&Bu)[CD_BAND], const float (&lev)[LEV],
                                             const float (&thr)[LEV])
 {
     ChainOperands after;
-    if constexpr (I + 2 < CD_BAND) after.load<I + 2>(hd, wb, rb);
+    if constexpr (I + 2 < RUN) after.load<I + 2>(hd, wb, rb);
     const float val = nearest_level<LEV>(cur.w - cur.rd * Bu[I], lev, thr);
     const float e_new = val - cur.w;
 #pragma unroll
@@ -204,7 +206,7 @@ __device__ __forceinline__ void chain_steps(const ChainOperands &cur, const Chai
     }
     eb[I * CD_CH] = e_new;
     wb[I * CD_CH] = val;                                 // W_i is not needed any more: What of the block takes its place
-    if constexpr (I + 1 < CD_BAND) chain_steps<LEV, I + 1>(nxt, after, hd, rb, wb, eb, Bu, lev, thr);
+    if constexpr (I + 1 < RUN) chain_steps<LEV, RUN, I + 1>(nxt, after, hd, rb, wb, eb, Bu, lev, thr);
 }
 
 // Where four rows (quad rq of a band) of channel ch stand in a part of the pulled sums, in floats: the swizzle keeps both
@@ -234,7 +236,7 @@ __device__ __forceinline__ int sums_at(int ch, int rq)
 //   loader warp (4)      TMA: the tiles of W, E and P (256 coordinates x 32 channels), and H[all 256][band] (32 KB) per
 //                        band into one of three buffers, two bands ahead.
 // Two named barriers per band: sums ready (products -> chain), band done (chain -> products, loader).
-// Measured for one block of 4096 channels, 16 levels: 42 us (8 levels, 1408 channels: 38); with eight threads per channel
+// Measured for one block of 4096 channels, 16 levels: 35 us (8 levels, 1408 channels: 31); with eight threads per channel
 // that did all updates themselves and two votes and a table read per step it was 81 us (78).
 template <int LEV>
 __global__ void __launch_bounds__(CD_THREADS, 1)
@@ -245,7 +247,8 @@ cd_block_kernel(const __grid_constant__ CUtensorMap mapH, const __grid_constant_
     __shared__ __align__(8) uint64_t bar_tiles;
     __shared__ __align__(8) uint64_t bar_h[CD_H_BUFS];
     __shared__ volatile uint32_t abort_flag;
-    float *Ws = reinterpret_cast<float *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
+    // aligned by an offset: rounding the pointer itself would make every access below a generic one
+    float *Ws = reinterpret_cast<float *>(smem_raw + ((0u - smem_u32(smem_raw)) & 1023u));
     float *Es = Ws + CD_TILE_FLOATS;                     // [256][32] E of the block, updated in place
     float *Ps = Es + CD_TILE_FLOATS;                     // [256][32] P
     float *Hs = Ps + CD_TILE_FLOATS;                     // [CD_H_BUFS][256][32] H[c][rows of a band]
@@ -323,6 +326,9 @@ cd_block_kernel(const __grid_constant__ CUtensorMap mapH, const __grid_constant_
     constexpr int SUMS_THREADS = 7 * 32, BAND_THREADS = CD_THREADS;
     if (warp == 0) {
         // ------------------------------------------------------------------ chain: the coordinates in order
+        // With 16 levels the 32 unrolled steps of a band (30 KB of code) and the products' loops do not fit the instruction
+        // cache together: 39.6 us a block against 34.8 with 16 steps twice.  With 8 they do: 31.4 against 33.2.
+        constexpr int RUN = LEV > 8 ? CD_BAND / 2 : CD_BAND;
         float lev[LEV], thr[LEV];
 #pragma unroll
         for (int q = 0; q < LEV; ++q) {
@@ -351,7 +357,20 @@ cd_block_kernel(const __grid_constant__ CUtensorMap mapH, const __grid_constant_
                 Bu[4 * q + 2] = ((v[0].z + v[1].z) + (v[2].z + v[3].z)) + (v[4].z + v[5].z);
                 Bu[4 * q + 3] = ((v[0].w + v[1].w) + (v[2].w + v[3].w)) + (v[4].w + v[5].w);
             }
-            chain_steps<LEV, 0>(first, second, hd, rb, wb, eb, Bu, lev, thr);
+#pragma unroll 1
+            for (int run = 0; run < CD_BAND / RUN; ++run) {
+                if (run > 0) {
+                    hd += RUN * (CD_BAND + 1);         // the same number of rows and columns on
+                    rb += RUN;
+                    wb += RUN * CD_CH;
+                    eb += RUN * CD_CH;
+                    first.load<0>(hd, wb, rb);
+                    second.load<1>(hd, wb, rb);
+#pragma unroll
+                    for (int r = 0; r + RUN < CD_BAND; ++r) Bu[r] = Bu[r + RUN];
+                }
+                chain_steps<LEV, RUN, 0>(first, second, hd, rb, wb, eb, Bu, lev, thr);
+            }
             if (t + 1 < CD_BANDS) bar_arrive_named(BAR_BAND, BAND_THREADS);
         }
     } else if (warp == 4) {
@@ -392,49 +411,34 @@ cd_block_kernel(const __grid_constant__ CUtensorMap mapH, const __grid_constant_
                 h[4] = hi.x; h[5] = hi.y; h[6] = hi.z; h[7] = hi.w;
             };
             auto load_e = [&](int c) { return *reinterpret_cast<const float4 *>(eb + c * CD_CH); };
-            // `count` (even) coordinates of the block from `first` on, the next one's operands read ahead.  One copy of
-            // this loop serves every use: the chain's unrolled steps already fill most of the instruction cache.
-            auto add_rows = [&](int first, int count) {
-                float ha[8], hb2[8];
-                load_h(first, ha);
-                float4 ea = load_e(first), eb2;
-#pragma unroll 1
-                for (int c = first; c < first + count; c += 2) {
-                    load_h(c + 1, hb2);
-                    eb2 = load_e(c + 1);
-                    add(ha, ea);
-                    const int n = c + 2 < first + count ? c + 2 : first;
-                    load_h(n, ha);
-                    ea = load_e(n);
-                    add(hb2, eb2);
+            // one band for each warp, neither the one the chain is working on (t - 1) nor this one
+            {
+                const int first = (t == 0 ? part + 1 : part >= t - 1 ? part + 2 : part) * CD_BAND;
+#pragma unroll 8
+                for (int c = first; c < first + CD_BAND; ++c) {
+                    float h[8];
+                    load_h(c, h);
+                    add(h, load_e(c));
                 }
-            };
-            // n = 0: one band for each warp, neither the one the chain is working on (t - 1) nor this one; n = 1 (t = 0
-            // only): the one left over, shared by four warps; n = 2: band t - 1 once the chain is through with it, ditto
+            }
+            // bands that all six share, 5 or 6 coordinates each.  n = 0: last cycle's values inside the band, coordinates after
+            // the row only; n = 1 (t = 0 only): the band left over; n = 2: band t - 1 once the chain is through with it.
+            const int k0 = part * CD_BAND / CD_PARTS, k1 = (part + 1) * CD_BAND / CD_PARTS;
 #pragma unroll 1
             for (int n = 0; n < 3; ++n) {
-                int first = (t == 0 ? part + 1 : part >= t - 1 ? part + 2 : part) * CD_BAND, count = CD_BAND;
-                if (n == 1) {
-                    first = 7 * CD_BAND + part * (CD_BAND / 4);
-                    count = t == 0 && part < 4 ? CD_BAND / 4 : 0;
-                    if (part >= 4) {
-                        // last cycle's values inside the band, coordinates after the row only: half a band each
-                        const int k0 = (part - 4) * (CD_BAND / 2);
-#pragma unroll 2
-                        for (int c = k0; c < k0 + CD_BAND / 2; ++c) {
-                            float h[8];
-                            load_h(t * CD_BAND + c, h);
+                if (n == 2 && t > 0) bar_sync_named(BAR_BAND, BAND_THREADS);
+                const int band = n == 0 ? t : n == 1 ? (t == 0 ? 7 : -1) : t - 1;
+                if (band < 0) continue;
 #pragma unroll
-                            for (int a = 0; a < 8; ++a) h[a] = r0 + a < c ? h[a] : 0.0f;
-                            add(h, load_e(t * CD_BAND + c));
-                        }
-                    }
-                } else if (n == 2) {
-                    if (t > 0) bar_sync_named(BAR_BAND, BAND_THREADS);
-                    first = (t - 1) * CD_BAND + part * (CD_BAND / 4);
-                    count = t > 0 && part < 4 ? CD_BAND / 4 : 0;
+                for (int i = 0; i < (CD_BAND + CD_PARTS - 1) / CD_PARTS; ++i) {
+                    const int kc = k0 + i, at = band * CD_BAND + min(kc, CD_BAND - 1);
+                    const int rows = kc >= k1 ? 0 : n == 0 ? kc - r0 : 8;      // of this thread's eight
+                    float h[8];
+                    load_h(at, h);
+#pragma unroll
+                    for (int a = 0; a < 8; ++a) h[a] = a < rows ? h[a] : 0.0f;
+                    add(h, load_e(at));
                 }
-                if (count > 0) add_rows(first, count);
             }
 #pragma unroll
             for (int b = 0; b < 4; ++b)
