@@ -124,12 +124,6 @@ __device__ __forceinline__ uint4 ld_stream_16(const void *p)
     return v;
 }
 
-__device__ __forceinline__ void st_shared_16(uint32_t addr, const uint4 &v)
-{
-    asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w)
-                 : "memory");
-}
-
 // Saliency as the scalers use it.  A value a is carried as two bf16 terms packed in one word: low half
 // hi = bf16(a), high half lo = bf16(a - hi); hi + lo has 16 significant bits.  The words of groups 2 q and
 // 2 q + 1 of a token sit side by side, so a scaler thread fetches both with one 8-byte load and does no

@@ -1010,7 +1010,8 @@ static int32_t cd_cycles_impl(const float *W, float *W_hat, uint8_t *Q, const fl
     if (int32_t rc = make_map(&mapHlo, Hlo, d_in, d_in, g, d_in, d_in * d_in)) return rc;
     if (int32_t rc = make_map(&mapEhi, Ehi, d_out, d_in, 1, d_out, d_in * d_out)) return rc;
     if (int32_t rc = make_map(&mapElo, Elo, d_out, d_in, 1, d_out, d_in * d_out)) return rc;
-    CUtensorMap mapHb, mapWb, mapEb, mapPb;              // fp32 tiles of the block kernel
+    CUtensorMap mapHb, mapWb, mapEb, mapPb, mapPr;       // fp32 tiles of the block kernel; P as the panel product adds to it
+    if (int32_t rc = make_map_f32(&mapPr, P, d_out, gq::CD_BLOCK, 1, 32, CU_TENSOR_MAP_SWIZZLE_128B)) return rc;
     if (int32_t rc = make_map_f32(&mapHb, H, d_in, d_in, g, gq::CD_BLOCK, CU_TENSOR_MAP_SWIZZLE_NONE)) return rc;
     if (int32_t rc = make_map_f32(&mapWb, Wt, d_out, d_in, 1, gq::CD_BLOCK, CU_TENSOR_MAP_SWIZZLE_NONE)) return rc;
     if (int32_t rc = make_map_f32(&mapEb, Et, d_out, d_in, 1, gq::CD_BLOCK, CU_TENSOR_MAP_SWIZZLE_NONE)) return rc;
@@ -1029,11 +1030,6 @@ static int32_t cd_cycles_impl(const float *W, float *W_hat, uint8_t *Q, const fl
                 gq::PairGemmParams pp{};
                 pp.d = static_cast<int>(d_in);
                 pp.g = g;
-                pp.n_terms = 3;                    // Hhi Ehi + Hhi Elo + Hlo Ehi
-                pp.term_a[0] = 0; pp.term_b[0] = 2;
-                pp.term_a[1] = 0; pp.term_b[1] = 3;
-                pp.term_a[2] = 1; pp.term_b[2] = 2;
-                pp.map_grouped[0] = 1; pp.map_grouped[1] = 1; pp.map_grouped[2] = 0; pp.map_grouped[3] = 0;
                 pp.s0 = static_cast<int>(s0);
                 pp.blk_ksteps = blk_ksteps;
                 pp.nk = nk;
@@ -1044,9 +1040,9 @@ static int32_t cd_cycles_impl(const float *W, float *W_hat, uint8_t *Q, const fl
                 const int tiles = g * ch_tiles;
                 int pieces = di->max_pairs / tiles;              // cut the contraction so that every pair has work
                 if (pieces < 1) pieces = 1;
-                if (pieces > 3 * nk) pieces = 3 * nk;
+                if (pieces > nk) pieces = nk;
                 pp.pieces = pieces;
-                const int ksteps = (3 * nk + pieces - 1) / pieces;
+                const int ksteps = (nk + pieces - 1) / pieces;
                 const int units = tiles * pieces;
                 pp.sched = gq::plan_schedule(units, ksteps, units < di->max_pairs ? units : di->max_pairs, false);
                 pp.status = di->status_ptr;
@@ -1054,7 +1050,7 @@ static int32_t cd_cycles_impl(const float *W, float *W_hat, uint8_t *Q, const fl
                 {
                     LaunchScope scope(GQ_KERNEL_CD_PANEL, st);
                     launch(gq::pair_gemm_kernel<gq::MODE_PANEL>, dim3(2 * pp.sched.pairs), gq::OBJ_THREADS, gq::OBJ_SMEM_BYTES, st, 
-                        mapHhi, mapHlo, mapEhi, mapElo, mapEhi, mapElo, pp);
+                        mapHhi, mapHlo, mapEhi, mapElo, mapPr, mapPr, pp);
                 }
                 GQ_CUDA(cudaGetLastError());
             }

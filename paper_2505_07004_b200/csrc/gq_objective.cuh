@@ -22,7 +22,10 @@
 //                  coordinate block: A = H_k (rows = contraction index c, by symmetry H[c][r] = H[r][c]),
 //                  B = E = (What - W)^T (rows = input coordinates c, columns = output channels); work unit =
 //                  (group, tile of 256 channels, piece of the contraction range); the pieces of a tile are
-//                  added into P with red.global.add.
+//                  added into P by TMA reduce-adds out of the ring, which is idle once a pair's only unit is done
+//                  (red.global.add where a pair has several).  A stage holds all four operands of 64 rows,
+//                  [H hi | H lo | E hi | E lo], for three products: 64 KB from L2 per 12 MMAs, where a stage per product
+//                  took 96 (33 us a panel of 4096 x 4096, g = 4; now 25).
 #pragma once
 #include <cuda.h>
 #include <cuda_runtime.h>
@@ -36,6 +39,8 @@ constexpr int OBJ_STAGES = 6;
 constexpr int OBJ_A_BYTES = (CTA_ROWS / BOX_FEATURES) * BOX_BYTES;
 constexpr int OBJ_B_BYTES = (CTA_ROWS / BOX_FEATURES) * BOX_BYTES;
 constexpr int OBJ_STAGE_BYTES = OBJ_A_BYTES + OBJ_B_BYTES;
+constexpr int PANEL_STAGES = 3;                        // of four operand blocks each: the same ring of 192 KB
+constexpr int PANEL_STAGE_BYTES = 2 * OBJ_STAGE_BYTES;
 constexpr int OBJ_THREADS = 256;
 constexpr int OBJ_SMEM_BYTES = OBJ_STAGES * OBJ_STAGE_BYTES + 1024;   // + slack to align the ring to 1024 B
 constexpr int MAX_TERMS = 6;
@@ -51,7 +56,7 @@ struct PairGemmParams {
     int g;                   // groups
     int nj;                  // ceil(d / 256): tile blocks per side
     int raster;              // edge (in tiles) of the super-blocks of the tile order
-    int n_terms;
+    int n_terms;             // MODE_OBJECTIVE
     int term_a[MAX_TERMS];   // which of the six tensor maps feeds A / B in each term
     int term_b[MAX_TERMS];
     int map_grouped[MAX_MAPS];   // 1: the map's third coordinate is the group index; 0: always 0
@@ -62,7 +67,7 @@ struct PairGemmParams {
     // MODE_PANEL
     int s0;                  // first coordinate of the block
     int blk_ksteps;          // 64-row k-steps covered by the block itself (left out of the contraction)
-    int nk;                  // 64-row k-steps outside the block (per term)
+    int nk;                  // 64-row k-steps outside the block
     int ch_tiles;            // tiles of 256 channels per group
     int pieces;              // pieces of the contraction range per (group, channel tile); sched.ksteps each
     int mk;                  // channels per group
@@ -100,23 +105,8 @@ __device__ __forceinline__ bool item_geom(const PairGemmParams &p, const WorkIte
     ge.a0 = p.s0 + static_cast<int>(rank) * CTA_ROWS;
     ge.b0 = ge.k * p.mk + t * TILE_N + static_cast<int>(rank) * CTA_ROWS;
     ge.ks0 = piece * p.sched.ksteps;
-    const int total = p.n_terms * p.nk;
-    ge.ks1 = (ge.ks0 + p.sched.ksteps < total) ? ge.ks0 + p.sched.ksteps : total;
+    ge.ks1 = (ge.ks0 + p.sched.ksteps < p.nk) ? ge.ks0 + p.sched.ksteps : p.nk;
     return ge.ks1 > ge.ks0;          // a piece beyond the end of the range has nothing to do: every role skips it
-}
-
-// Term and first contraction row of flattened k-step ks.
-template <int MODE>
-__device__ __forceinline__ void kstep_coords(const PairGemmParams &p, int ks, int kblocks, int &term, int &row)
-{
-    if (MODE != MODE_PANEL) {
-        term = ks / kblocks;
-        row = (ks - term * kblocks) * TILE_K;
-    } else {
-        term = ks / p.nk;
-        const int kb = ks - term * p.nk;
-        row = (kb < p.s0 / TILE_K ? kb : kb + p.blk_ksteps) * TILE_K;
-    }
 }
 
 template <int MODE>
@@ -126,6 +116,8 @@ pair_gemm_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant
                  const __grid_constant__ CUtensorMap map4, const __grid_constant__ CUtensorMap map5,
                  const PairGemmParams p)
 {
+    constexpr int STAGES = MODE == MODE_PANEL ? PANEL_STAGES : OBJ_STAGES;
+    constexpr int STAGE_BYTES = MODE == MODE_PANEL ? PANEL_STAGE_BYTES : OBJ_STAGE_BYTES;
     extern __shared__ uint8_t smem_raw[];
     __shared__ __align__(8) uint64_t bar_full[OBJ_STAGES];      // used in the pair's first CTA only
     __shared__ __align__(8) uint64_t bar_empty[OBJ_STAGES];     // signalled in both CTAs by the MMA commits
@@ -142,7 +134,7 @@ pair_gemm_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant
     const uint32_t ring = (smem_u32(smem_raw) + 1023u) & ~1023u;
 
     if (threadIdx.x == 0) {
-        for (int s = 0; s < OBJ_STAGES; ++s) {
+        for (int s = 0; s < STAGES; ++s) {
             mbar_init(smem_u32(&bar_full[s]), 1);
             mbar_init(smem_u32(&bar_empty[s]), 1);
         }
@@ -186,35 +178,41 @@ pair_gemm_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant
             if (!item_geom<MODE>(p, w, rank, ge)) continue;
             const void *maps[MAX_MAPS] = {&map0, &map1, &map2, &map3, &map4, &map5};
             for (int ks = ge.ks0; ks < ge.ks1; ++ks) {
-                int term, row;
-                kstep_coords<MODE>(p, ks, kblocks, term, row);
-                const int ma = p.term_a[term], mb = p.term_b[term];
-                const void *amap = maps[ma];
-                const void *bmap = maps[mb];
-                const int ka = p.map_grouped[ma] ? ge.k : 0;
-                const int kb = p.map_grouped[mb] ? ge.k : 0;
                 if (!bounded_wait(smem_u32(&bar_empty[s]), ph ^ 1u, wc, 1u, w.unit)) { ok = false; break; }
                 const uint32_t full_local = smem_u32(&bar_full[s]);
-                if (rank == 0) mbar_arrive_expect_tx(full_local, 2 * OBJ_STAGE_BYTES);   // both CTAs' bytes
+                if (rank == 0) mbar_arrive_expect_tx(full_local, 2 * STAGE_BYTES);   // both CTAs' bytes
                 const uint32_t full = map_to_cta(full_local, 0);
-                const uint32_t sa = ring + s * OBJ_STAGE_BYTES;
-                const uint32_t sb = sa + OBJ_A_BYTES;
+                const uint32_t sa = ring + s * STAGE_BYTES;
+                if (MODE == MODE_PANEL) {
+                    const int row = (ks < p.s0 / TILE_K ? ks : ks + p.blk_ksteps) * TILE_K;
 #pragma unroll
-                for (int q = 0; q < CTA_ROWS / BOX_FEATURES; ++q)
-                    tma_load_3d_pair(sa + q * BOX_BYTES, amap, full, ge.a0 + q * BOX_FEATURES, row, ka);
+                    for (int op = 0; op < 4; ++op)                // H hi, H lo, E hi, E lo
 #pragma unroll
-                for (int q = 0; q < CTA_ROWS / BOX_FEATURES; ++q)
-                    tma_load_3d_pair(sb + q * BOX_BYTES, bmap, full, ge.b0 + q * BOX_FEATURES, row, kb);
+                        for (int q = 0; q < CTA_ROWS / BOX_FEATURES; ++q)
+                            tma_load_3d_pair(sa + op * OBJ_A_BYTES + q * BOX_BYTES, maps[op], full,
+                                             (op < 2 ? ge.a0 : ge.b0) + q * BOX_FEATURES, row, op < 2 ? ge.k : 0);
+                } else {
+                    const int term = ks / kblocks;
+                    const int row = (ks - term * kblocks) * TILE_K;
+                    const int ma = p.term_a[term], mb = p.term_b[term];
+                    const int ka = p.map_grouped[ma] ? ge.k : 0, kb = p.map_grouped[mb] ? ge.k : 0;
+#pragma unroll
+                    for (int q = 0; q < CTA_ROWS / BOX_FEATURES; ++q)
+                        tma_load_3d_pair(sa + q * BOX_BYTES, maps[ma], full, ge.a0 + q * BOX_FEATURES, row, ka);
+#pragma unroll
+                    for (int q = 0; q < CTA_ROWS / BOX_FEATURES; ++q)
+                        tma_load_3d_pair(sa + OBJ_A_BYTES + q * BOX_BYTES, maps[mb], full, ge.b0 + q * BOX_FEATURES, row, kb);
+                }
                 ++issued;
-                if (++s == OBJ_STAGES) { s = 0; ph ^= 1u; }
+                if (++s == STAGES) { s = 0; ph ^= 1u; }
             }
         }
         // Stay until every stage that was filled has been released again: the release is an arrival on
         // this CTA's barriers, which must not come after the CTA has gone.
         // (Stages that were never filled pass at once.)
-        for (int q = 0; ok && issued != 0u && q < OBJ_STAGES; ++q) {
+        for (int q = 0; ok && issued != 0u && q < STAGES; ++q) {
             if (!bounded_wait(smem_u32(&bar_empty[s]), ph ^ 1u, wc, 5u, 0u)) ok = false;
-            if (++s == OBJ_STAGES) { s = 0; ph ^= 1u; }
+            if (++s == STAGES) { s = 0; ph ^= 1u; }
         }
         if (!ok) spin_ns(1000000ull);      // copies already issued land well within this time
     } else if (warp == 1 && lane == 0 && rank == 0) {
@@ -235,16 +233,21 @@ pair_gemm_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant
             for (int ks = ge.ks0; ks < ge.ks1; ++ks) {
                 if (!bounded_wait_hot(smem_u32(&bar_full[s]), ph, wc, 3u, w.unit)) { ok = false; break; }
                 tc_fence_after_sync();
-                const uint32_t sa = ring + s * OBJ_STAGE_BYTES;
-                const uint32_t sb = sa + OBJ_A_BYTES;
+                const uint32_t stage = ring + s * STAGE_BYTES;
+                // products of a stage: one, or hi hi + hi lo + lo hi
 #pragma unroll
-                for (int kk = 0; kk < TILE_K / 16; ++kk) {
-                    const uint64_t adesc = umma_smem_desc_mn_sw128(sa + kk * 16 * 128, BOX_BYTES, 1024);
-                    const uint64_t bdesc = umma_smem_desc_mn_sw128(sb + kk * 16 * 128, BOX_BYTES, 1024);
-                    umma_bf16(d_tmem, adesc, bdesc, idesc, (ks != ge.ks0 || kk != 0) ? 1u : 0u);
+                for (int term = 0; term < (MODE == MODE_PANEL ? 3 : 1); ++term) {
+                    const uint32_t sa = stage + (term == 2 ? OBJ_A_BYTES : 0);
+                    const uint32_t sb = stage + (MODE == MODE_PANEL ? (term == 1 ? 3 : 2) : 1) * OBJ_A_BYTES;
+#pragma unroll
+                    for (int kk = 0; kk < TILE_K / 16; ++kk) {
+                        const uint64_t adesc = umma_smem_desc_mn_sw128(sa + kk * 16 * 128, BOX_BYTES, 1024);
+                        const uint64_t bdesc = umma_smem_desc_mn_sw128(sb + kk * 16 * 128, BOX_BYTES, 1024);
+                        umma_bf16(d_tmem, adesc, bdesc, idesc, (ks != ge.ks0 || kk != 0 || term != 0) ? 1u : 0u);
+                    }
                 }
                 umma_commit_pair(smem_u32(&bar_empty[s]));   // stage reusable in both CTAs once these MMAs have read it
-                if (++s == OBJ_STAGES) { s = 0; ph ^= 1u; }
+                if (++s == STAGES) { s = 0; ph ^= 1u; }
             }
             if (!ok) break;
             umma_commit_pair(smem_u32(&bar_acc_full[buf]));
@@ -335,6 +338,7 @@ pair_gemm_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant
             ok = __all_sync(0xffffffffu, ok);
             if (!ok) break;
             tc_fence_after_sync();
+            const bool only = p.sched.units <= p.sched.pairs;      // the pair's only unit: the ring is idle now
             const int rl = static_cast<int>(rank) * CTA_ROWS + q * 32 + lane;      // row inside the block
             const bool row_ok = p.s0 + rl < p.d;
             const int ch_end = (ge.k + 1) * p.mk;                                  // channels of this group only
@@ -348,6 +352,23 @@ pair_gemm_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant
                 tmem_ld_32x32(tmem_base + (static_cast<uint32_t>(q * 32) << 16) +
                                   static_cast<uint32_t>(buf * TILE_N + cc * 32), r);
                 tmem_ld_wait();
+                if (only) {
+                    // channels past the group's end belong to the next one: zero is added to them; rows past the matrix are zero
+                    const uint32_t block = ring + static_cast<uint32_t>(q * (TILE_N / 32) + cc) * 4096u;
+#pragma unroll
+                    for (int v = 0; v < 8; ++v) {
+                        const bool in = ch0 + v * 4 < ch_end;              // the group's end is a multiple of 8
+                        st_shared_16(block + static_cast<uint32_t>(lane * 128 + ((v ^ (lane & 7)) << 4)),
+                                     in ? make_uint4(r[v * 4 + 0], r[v * 4 + 1], r[v * 4 + 2], r[v * 4 + 3]) : make_uint4(0u, 0u, 0u, 0u));
+                    }
+                    fence_proxy_async_smem();
+                    __syncwarp();
+                    if (lane == 0) {
+                        tma_reduce_add_3d(&map5, block, ch0, rl, 0);
+                        bulk_commit_group();
+                    }
+                    continue;
+                }
                 if (!row_ok) continue;
 #pragma unroll
                 for (int v = 0; v < 8; ++v) {
@@ -362,6 +383,7 @@ pair_gemm_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant
             buf ^= 1;
             if (buf == 0) acc_ph ^= 1u;
         }
+        if (MODE == MODE_PANEL && lane == 0) bulk_wait_group_read0();       // shared memory must outlive the last reduce-add's read
     }
 
     // Both CTAs stay until neither can touch the other's shared memory, barriers or tensor memory any more.

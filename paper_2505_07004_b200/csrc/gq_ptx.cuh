@@ -61,6 +61,12 @@ __device__ __forceinline__ uint32_t ld_u16(const void *p)
     return v;
 }
 
+__device__ __forceinline__ void st_shared_16(uint32_t addr, const uint4 &v)
+{
+    asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w)
+                 : "memory");
+}
+
 // ---------------------------------------------------------------- cluster of two CTAs
 __device__ __forceinline__ uint32_t cluster_ctarank()
 {
