@@ -44,35 +44,37 @@ __device__ __forceinline__ void split_bf16(float v, __nv_bfloat16 &hi, __nv_bflo
     lo = __float2bfloat16_rn(v - __bfloat162float(hi));
 }
 
-// Wt = W^T, E = (What - W)^T (fp32 and as bf16 hi + lo), all [d_in][d_out].  32 x 32 tiles.
+// Wt = W^T, E = (What - W)^T (fp32 and as bf16 hi + lo), all [d_in][d_out].  Tiles of 32 coordinates x 64 channels: whole
+// 128-byte segments on both sides (4096 x 4096: 52 us; one value per
+// lane and 64-byte segments 73).
 __global__ void __launch_bounds__(256)
-cd_prepare_kernel(const float *W, const float *What, int d_in, int d_out,
-                  float *Wt, float *Et,
-                  __nv_bfloat16 *Ehi, __nv_bfloat16 *Elo)
+cd_prepare_kernel(const float *W, const float *What, int d_in, int d_out, float *Wt, float *Et, __nv_bfloat16 *Ehi, __nv_bfloat16 *Elo)
 {
-    __shared__ float tw[32][33], th[32][33];
+    __shared__ float tw[64][33], th[64][33];
     griddep_launch();
     griddep_wait();
     const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
-    const int i0 = blockIdx.x * 32, j0 = blockIdx.y * 32;          // coordinate / channel origin
-    for (int r = ty; r < 32; r += 8) {
-        const int j = j0 + r, i = i0 + tx;
+    const int i0 = blockIdx.x * 32, j0 = blockIdx.y * 64;          // coordinate / channel origin
+#pragma unroll
+    for (int r = 0; r < 64; r += 8) {
+        const int j = j0 + r + ty, i = i0 + tx;
         const bool ok = j < d_out && i < d_in;
-        tw[r][tx] = ok ? W[static_cast<size_t>(j) * d_in + i] : 0.0f;
-        th[r][tx] = ok ? What[static_cast<size_t>(j) * d_in + i] : 0.0f;
+        tw[r + ty][tx] = ok ? W[static_cast<size_t>(j) * d_in + i] : 0.0f;
+        th[r + ty][tx] = ok ? What[static_cast<size_t>(j) * d_in + i] : 0.0f;
     }
     __syncthreads();
-    for (int r = ty; r < 32; r += 8) {
-        const int i = i0 + r, j = j0 + tx;
+#pragma unroll
+    for (int r = 0; r < 32; r += 8) {
+        const int i = i0 + r + ty, j = j0 + 2 * tx;                // d_out is a multiple of 8: pairs are inside or outside
         if (i < d_in && j < d_out) {
-            const float w = tw[tx][r], h = th[tx][r], e = h - w;
+            const float w0 = tw[2 * tx][r + ty], w1 = tw[2 * tx + 1][r + ty];
+            const float e0 = th[2 * tx][r + ty] - w0, e1 = th[2 * tx + 1][r + ty] - w1;
             const size_t o = static_cast<size_t>(i) * d_out + j;
-            Wt[o] = w;
-            Et[o] = e;
-            __nv_bfloat16 hi, lo;
-            split_bf16(e, hi, lo);
-            Ehi[o] = hi;
-            Elo[o] = lo;
+            *reinterpret_cast<float2 *>(Wt + o) = make_float2(w0, w1);
+            *reinterpret_cast<float2 *>(Et + o) = make_float2(e0, e1);
+            const __nv_bfloat162 hi = __floats2bfloat162_rn(e0, e1);
+            *reinterpret_cast<__nv_bfloat162 *>(Ehi + o) = hi;
+            *reinterpret_cast<__nv_bfloat162 *>(Elo + o) = __floats2bfloat162_rn(e0 - __low2float(hi), e1 - __high2float(hi));
         }
     }
 }
@@ -105,27 +107,35 @@ split_h_kernel(const float *H, int d_in, __nv_bfloat16 *Hhi, __nv_bfloat16 *Hlo,
     }
 }
 
-// Q = Qt^T back to [d_out][d_in] and What = codebook[Q].
+// Q = Qt^T back to [d_out][d_in] and What = codebook[Q].  64 x 64 tiles, four codes per thread; `bytes`: Q is not 4-byte
+// aligned and is written byte by byte.  (4096 x 4096: 19 us; 51 with one code per thread, 32-byte segments and W_hat carried through every block.)
 __global__ void __launch_bounds__(256)
-cd_finish_kernel(const float *codebook, const uint8_t *Qt, int d_in, int d_out, int m,
-                 float *What, uint8_t *Q)
+cd_finish_kernel(const float *codebook, const uint8_t *Qt, int d_in, int d_out, int m, float *What, uint8_t *Q, bool bytes)
 {
-    __shared__ uint8_t tq[32][33];
+    __shared__ uint8_t tq[64][68];
     griddep_launch();
     griddep_wait();
-    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
-    const int i0 = blockIdx.x * 32, j0 = blockIdx.y * 32;
-    for (int r = ty; r < 32; r += 8) {
-        const int i = i0 + r, j = j0 + tx;
-        tq[r][tx] = (i < d_in && j < d_out) ? Qt[static_cast<size_t>(i) * d_out + j] : 0;
+    const int c4 = (threadIdx.x & 15) * 4, r0 = threadIdx.x >> 4;
+    const int i0 = blockIdx.x * 64, j0 = blockIdx.y * 64;
+#pragma unroll
+    for (int r = r0; r < 64; r += 16) {                            // d_in and d_out are multiples of 8: fours are inside or outside
+        const int i = i0 + r, j = j0 + c4;
+        *reinterpret_cast<uint32_t *>(&tq[r][c4]) =
+            (i < d_in && j < d_out) ? *reinterpret_cast<const uint32_t *>(Qt + static_cast<size_t>(i) * d_out + j) : 0u;
     }
     __syncthreads();
-    for (int r = ty; r < 32; r += 8) {
-        const int j = j0 + r, i = i0 + tx;
-        if (j < d_out && i < d_in) {
-            const uint8_t code = tq[tx][r];
-            What[static_cast<size_t>(j) * d_in + i] = codebook[static_cast<size_t>(j) * m + code];
-            Q[static_cast<size_t>(j) * d_in + i] = code;
+#pragma unroll
+    for (int r = r0; r < 64; r += 16) {
+        const int j = j0 + r, i = i0 + c4;
+        if (j >= d_out || i >= d_in) continue;
+        const float *cb = codebook + static_cast<size_t>(j) * m;
+        const size_t o = static_cast<size_t>(j) * d_in + i;
+        const uchar4 q = make_uchar4(tq[c4][r], tq[c4 + 1][r], tq[c4 + 2][r], tq[c4 + 3][r]);
+        *reinterpret_cast<float4 *>(What + o) = make_float4(cb[q.x], cb[q.y], cb[q.z], cb[q.w]);
+        if (bytes) {
+            Q[o] = q.x; Q[o + 1] = q.y; Q[o + 2] = q.z; Q[o + 3] = q.w;
+        } else {
+            *reinterpret_cast<uchar4 *>(Q + o) = q;
         }
     }
 }

@@ -59,15 +59,15 @@ constexpr int GD_PARTIALS_PER_UNIT = 2 * GD_EPI_WARPS;       // one fp64 per (CT
 constexpr int GD_TARGET_EXP = 14;                            // the largest |delta| * 2^e lies in [2^14, 2^15)
 constexpr int GD_MAX_SHIFT = 100;                            // |e| is kept below this (the scale stays a normal float)
 
-constexpr unsigned DELTA_BLOCK_MAXIMA = 240;      // what the 1 KiB header holds
+constexpr unsigned DELTA_BLOCK_MAXIMA = 960;      // blocks of the first preparation pass: what the 1 KiB header holds
 
 // Header of the objective workspace, written by the preparation kernels and read by the reduction.
 struct GramDotHeader {
-    unsigned int absmax_bits;   // bit pattern of max |W - W_hat| (non-negative floats order like unsigned ints)
     int shift;                  // e: the fp16 matrix holds (W - W_hat) * 2^e
     unsigned int blocks_done;   // groups whose loss has been written (the last one forms the total)
-    unsigned int pad[13];       // the maxima start a 64-byte segment
-    unsigned int block_max[DELTA_BLOCK_MAXIMA];   // bit patterns of the first pass's maxima, if it has that few blocks
+    unsigned int absmax_bits;   // bit pattern of max |W - W_hat| where the first pass has more blocks than that
+    unsigned int pad[13];       // the exponents start a 64-byte segment
+    uint8_t block_exp[DELTA_BLOCK_MAXIMA];   // biased exponent of each first-pass block's max |W - W_hat|
 };
 
 struct GramDotParams {
@@ -116,10 +116,10 @@ __device__ __forceinline__ float4 ld_f32x4_last_use(const float4 *p)
 constexpr int DELTA_VEC_PER_THREAD = 4;      // float4 pairs a thread of the two preparation kernels handles
 
 // ------------------------------------------------------------------------------------------------
-// max |W - W_hat| over the layer (the differences are formed in fp32, as everywhere in the objective).
-// One block per 256 * DELTA_VEC_PER_THREAD float4 pairs.  Up to DELTA_BLOCK_MAXIMA blocks leave one maximum each for the
-// second pass to combine; beyond that they meet in header->absmax_bits, which must be 0 before the launch (clearing it is an
-// operation of its own on the stream, which a layer of a few microseconds notices).
+// max |W - W_hat| over the layer (the differences are formed in fp32, as everywhere in the objective), one block per
+// 256 * DELTA_VEC_PER_THREAD float4 pairs.  Up to DELTA_BLOCK_MAXIMA blocks leave the exponent of their maximum, all that the
+// scale depends on, in the header; more meet in header->absmax_bits (non-negative floats order like unsigned integers), which
+// must be 0 before the launch.
 __global__ void __launch_bounds__(256)
 delta_absmax_kernel(const float *__restrict__ W, const float *__restrict__ What, unsigned count4, GramDotHeader *header)
 {
@@ -146,19 +146,18 @@ delta_absmax_kernel(const float *__restrict__ W, const float *__restrict__ What,
     __syncthreads();
     if (threadIdx.x == 0) {
         for (int w8 = 1; w8 < 8; ++w8) m = fmaxf(m, red[w8]);
-        // NaN never wins fmaxf; an infinite difference gives 0x7f800000 and the shift below saturates
+        // NaN never wins fmaxf; an infinite difference gives 0xff and the shift below saturates
         if (gridDim.x <= DELTA_BLOCK_MAXIMA)
-            header->block_max[blockIdx.x] = m > 0.0f ? __float_as_uint(m) : 0u;
+            header->block_exp[blockIdx.x] = static_cast<uint8_t>(__float_as_uint(m) >> 23);
         else if (m > 0.0f)
             atomicMax(&header->absmax_bits, __float_as_uint(m));
     }
 }
 
-// The power of two e for a layer whose largest |delta| has the bit pattern `bits`.
-__device__ __forceinline__ int gram_dot_shift(unsigned int bits)
+// The power of two e for a layer whose largest |delta| has the biased exponent `biased` (0: zero or subnormal).
+__device__ __forceinline__ int gram_dot_shift(unsigned int biased)
 {
-    if (bits == 0u) return 0;
-    int k = static_cast<int>((bits >> 23) & 0xffu) - 127;          // floor(log2(max)) for normal values
+    int k = static_cast<int>(biased) - 127;                        // floor(log2(max)) for normal values
     if (k < -126) k = -126;
     int e = GD_TARGET_EXP - k;
     if (e > GD_MAX_SHIFT) e = GD_MAX_SHIFT;
@@ -170,7 +169,7 @@ __device__ __forceinline__ int gram_dot_shift(unsigned int bits)
 // from the END towards the start: what the maximum pass read last is still in L2.
 __global__ void __launch_bounds__(256)
 delta_half_kernel(const float *__restrict__ W, const float *__restrict__ What, unsigned count4, GramDotHeader *header,
-                  __half *__restrict__ out)
+                  unsigned maxima, __half *__restrict__ out)
 {
     griddep_launch();
     griddep_wait();
@@ -184,19 +183,25 @@ delta_half_kernel(const float *__restrict__ W, const float *__restrict__ What, u
         w[t] = in ? ld_f32x4_last_use(reinterpret_cast<const float4 *>(W) + idx) : make_float4(0.f, 0.f, 0.f, 0.f);
         q[t] = in ? ld_f32x4_last_use(reinterpret_cast<const float4 *>(What) + idx) : make_float4(0.f, 0.f, 0.f, 0.f);
     }
-    unsigned int absmax_bits = 0u;
-    if (gridDim.x <= DELTA_BLOCK_MAXIMA) {
-        if (threadIdx.x < gridDim.x) absmax_bits = header->block_max[threadIdx.x];
+    unsigned int biased = 0u;
+    if (maxima == 0u) {                                            // not left block by block
+        biased = *const_cast<volatile unsigned int *>(&header->absmax_bits) >> 23;
+    } else {
+        static_assert(DELTA_BLOCK_MAXIMA <= 4 * 256, "four exponents per thread");
+        if (4u * threadIdx.x < maxima) {
+            const uint32_t four = reinterpret_cast<const volatile uint32_t *>(header->block_exp)[threadIdx.x];
+#pragma unroll
+            for (unsigned b = 0; b < 4; ++b)
+                if (4u * threadIdx.x + b < maxima) biased = max(biased, (four >> (8u * b)) & 0xffu);
+        }
         __shared__ unsigned int red[8];
-        absmax_bits = __reduce_max_sync(0xffffffffu, absmax_bits);
-        if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = absmax_bits;
+        biased = __reduce_max_sync(0xffffffffu, biased);
+        if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = biased;
         __syncthreads();
 #pragma unroll
-        for (int w8 = 0; w8 < 8; ++w8) absmax_bits = max(absmax_bits, red[w8]);
-    } else {
-        absmax_bits = header->absmax_bits;
+        for (int w8 = 0; w8 < 8; ++w8) biased = max(biased, red[w8]);
     }
-    const int e = gram_dot_shift(absmax_bits);
+    const int e = gram_dot_shift(biased);
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         header->shift = e;
         header->blocks_done = 0u;
@@ -218,10 +223,12 @@ delta_half_kernel(const float *__restrict__ W, const float *__restrict__ What, u
 // by whichever block finishes last).  Every sum is formed in a fixed order (strided per thread, butterfly per warp,
 // warp results in order), so the result does not vary from run to run.  partials: [g][slots][per_unit] (units are
 // numbered group-major).  header->blocks_done is 0 before the launch (delta_half_kernel).
-__global__ void __launch_bounds__(256)
+// (1024 threads: two groups of 6441 tiles take 20 us; 256 took 58.)
+constexpr int GD_REDUCE_THREADS = 1024;
+__global__ void __launch_bounds__(GD_REDUCE_THREADS)
 gram_dot_reduce_kernel(const double *partials, int slots, int g, int per_unit, GramDotHeader *header, double *loss)
 {
-    __shared__ double warp_sum[8];
+    __shared__ double warp_sum[GD_REDUCE_THREADS / 32];
     __shared__ bool last;
     griddep_launch();
     griddep_wait();
@@ -231,13 +238,14 @@ gram_dot_reduce_kernel(const double *partials, int slots, int g, int per_unit, G
     const int count = slots * per_unit;
     double acc0 = 0.0, acc1 = 0.0, acc2 = 0.0, acc3 = 0.0;
     int idx = threadIdx.x;
-    for (; idx + 768 < count; idx += 1024) {               // four independent loads in flight
+    constexpr int T = GD_REDUCE_THREADS;
+    for (; idx + 3 * T < count; idx += 4 * T) {            // four independent loads in flight
         acc0 += pk[idx];
-        acc1 += pk[idx + 256];
-        acc2 += pk[idx + 512];
-        acc3 += pk[idx + 768];
+        acc1 += pk[idx + T];
+        acc2 += pk[idx + 2 * T];
+        acc3 += pk[idx + 3 * T];
     }
-    for (; idx < count; idx += 256) acc0 += pk[idx];
+    for (; idx < count; idx += T) acc0 += pk[idx];
     double acc = (acc0 + acc1) + (acc2 + acc3);
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
@@ -245,7 +253,7 @@ gram_dot_reduce_kernel(const double *partials, int slots, int g, int per_unit, G
     __syncthreads();
     if (threadIdx.x == 0) {
         double v = 0.0;
-        for (int w8 = 0; w8 < 8; ++w8) v += warp_sum[w8];
+        for (int w = 0; w < T / 32; ++w) v += warp_sum[w];
         loss[k] = v * ldexp(1.0, -2 * header->shift);
         __threadfence();
         last = atomicAdd(&header->blocks_done, 1u) == static_cast<unsigned int>(g) - 1u;
