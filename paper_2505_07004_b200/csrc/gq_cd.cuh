@@ -130,7 +130,8 @@ cd_finish_kernel(const float *codebook, const uint8_t *Qt, int d_in, int d_out, 
         if (j >= d_out || i >= d_in) continue;
         const float *cb = codebook + static_cast<size_t>(j) * m;
         const size_t o = static_cast<size_t>(j) * d_in + i;
-        const uchar4 q = make_uchar4(tq[c4][r], tq[c4 + 1][r], tq[c4 + 2][r], tq[c4 + 3][r]);
+        const uint8_t top = static_cast<uint8_t>(m - 1);             // no code leads past the channel's levels
+        const uchar4 q = make_uchar4(min(tq[c4][r], top), min(tq[c4 + 1][r], top), min(tq[c4 + 2][r], top), min(tq[c4 + 3][r], top));
         *reinterpret_cast<float4 *>(What + o) = make_float4(cb[q.x], cb[q.y], cb[q.z], cb[q.w]);
         if (bytes) {
             Q[o] = q.x; Q[o + 1] = q.y; Q[o + 2] = q.z; Q[o + 3] = q.w;
@@ -302,18 +303,26 @@ cd_block_kernel(const __grid_constant__ CUtensorMap mapH, const __grid_constant_
     griddep_wait();
     rds[tid] = tid < p.rows ? p.rdiag[static_cast<size_t>(k) * p.d_in + p.s0 + tid] : 0.0f;
     // ---- the channel's levels, sorted (eight threads per channel), and the thresholds between neighbours: their midpoints,
-    // lowered by one ulp where the upper level has the smaller given index, so that a tie goes to the smaller index
+    // lowered by one ulp where the upper level has the smaller given index, so that a tie goes to the smaller index.
+    // Sorted means a total order, so that every position is written: numbers ascending, then NaN, equal ones by index.  A
+    // threshold beside a NaN is a NaN and never exceeded: no target is rounded to it while the channel has a number.  The
+    // positions past the channel's levels hold NaN as well, with the highest indices.
     {
         const int cidx = tid >> 3, l = tid & 7;
         const bool chan = cidx < ch_n;
-        const float v0 = (l < p.m && chan) ? p.codebook[static_cast<size_t>(ch0 + cidx) * p.m + l] : CUDART_INF_F;
-        const float v1 = (l + 8 < p.m && chan) ? p.codebook[static_cast<size_t>(ch0 + cidx) * p.m + l + 8] : CUDART_INF_F;
+        const float v0 = (l < p.m && chan) ? p.codebook[static_cast<size_t>(ch0 + cidx) * p.m + l] : CUDART_NAN_F;
+        const float v1 = (l + 8 < p.m && chan) ? p.codebook[static_cast<size_t>(ch0 + cidx) * p.m + l + 8] : CUDART_NAN_F;
+        auto key = [](float v) {                         // unsigned, ascending with v; -0 as 0, NaN above infinity
+            const uint32_t b = __float_as_uint(v + 0.0f);
+            return isnan(v) ? 0xff800001u : (b ^ (static_cast<uint32_t>(static_cast<int32_t>(b) >> 31) | 0x80000000u));
+        };
+        const uint32_t k0 = key(v0), k1 = key(v1);
         int rank0 = 0, rank1 = 0;                        // positions of (v0, l) and (v1, l + 8) among the 16 pairs
 #pragma unroll
         for (int r = 0; r < CD_MAX_LEVELS; ++r) {
-            const float vr = __shfl_sync(0xffffffffu, r < 8 ? v0 : v1, r & 7, 8);
-            rank0 += (vr < v0 || (vr == v0 && r < l)) ? 1 : 0;
-            rank1 += (vr < v1 || (vr == v1 && r < l + 8)) ? 1 : 0;
+            const uint32_t kr = __shfl_sync(0xffffffffu, r < 8 ? k0 : k1, r & 7, 8);
+            rank0 += kr < k0 + (r < l ? 1u : 0u) ? 1 : 0;
+            rank1 += kr < k1 + (r < l + 8 ? 1u : 0u) ? 1 : 0;
         }
         float *ms = srt + cidx * CD_LEVEL_LD;
         int *mi = sidx + cidx * CD_LEVEL_LD;
@@ -487,7 +496,7 @@ cd_block_kernel(const __grid_constant__ CUtensorMap mapH, const __grid_constant_
 #pragma unroll
             for (int step = LEV / 2; step > 0; step >>= 1)      // one with the smallest given index
                 if (ms[pos + step - 1] < v[b]) pos += step;
-            codes |= static_cast<uint32_t>(sidx[(c + b) * CD_LEVEL_LD + pos]) << (8 * b);
+            codes |= static_cast<uint32_t>(min(sidx[(c + b) * CD_LEVEL_LD + pos], p.m - 1)) << (8 * b);
         }
         *reinterpret_cast<uint32_t *>(p.Qt + o) = codes;
     }

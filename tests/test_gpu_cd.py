@@ -138,6 +138,27 @@ def test_cd_block_edges(dev, seed, d_in, d_out, g, m):
     assert Q_g.max() < m - 1
 
 
+@pytest.mark.parametrize("m", [4, 8, 13, 16])
+def test_cd_levels_that_are_no_numbers(dev, m):
+    """A NaN level is never chosen while its channel has a number: the channel ends where it ends with that level far
+    away.  A channel of NaN only, or with a NaN in W, still gets codes below m, and its neighbours (four channels share a
+    word of codes) the bits they get without it."""
+    W, W0, cb, H = make_problem(40 + m, 264, 64, 2, m)
+    far = cb.copy()
+    far[3, m // 2] = far[9, 0] = far[50, m - 1] = 1e30
+    What_f, Q_f = run_gpu(dev, W, W0, far, H, 2)
+    W_n, cb_n = W.copy(), far.copy()
+    cb_n[far == 1e30] = np.nan
+    cb_n[5] = np.nan
+    W_n[22, 100] = np.nan
+    What_n, Q_n = run_gpu(dev, W_n, W0, cb_n, H, 2)
+    assert Q_n.max() < m
+    assert np.array_equal(What_n, np.take_along_axis(cb_n, Q_n, axis=1), equal_nan=True)
+    assert (Q_n[5] == 0).all()
+    rest = [j for j in range(64) if j not in (5, 22)]
+    assert np.array_equal(Q_n[rest], Q_f[rest]) and np.array_equal(What_n[rest], What_f[rest])
+
+
 def test_cd_errors_and_zero_cycles(dev):
     W, W0, cb, H = make_problem(3, 64, 16, 1, 4)
     Wd, Whd = torch.from_numpy(W).to(dev), torch.from_numpy(W0.copy()).to(dev)

@@ -226,6 +226,21 @@ def test_full_size_layer_sampled_channels(dev):
     assert n_tie <= len(sel) // 2
 
 
+@pytest.mark.parametrize("m", [8, 16])
+def test_gq_lnq_with_a_weight_that_is_no_number(dev, m):
+    """A NaN in one channel's weights makes its codebook NaN; its codes stay below m and the other channels finite."""
+    W, W0, Q0, cb0, H = make_problem(23, 264, 64, 2, m)
+    W[9, 17] = np.nan
+    Wd, Hd = torch.from_numpy(W).to(dev), torch.from_numpy(H).to(dev)
+    ws = libgq.alloc_workspace(libgq.gq_lnq_workspace_bytes(264, 64, 2, m), dev)
+    What, Q, cb = libgq.gq_lnq(Wd, torch.from_numpy(Q0.astype(np.uint8)).to(dev), m, Hd, 1, 2, ws)
+    libgq.gq_check()
+    assert int(Q.max()) < m
+    rest = [j for j in range(64) if j != 9]
+    assert torch.isfinite(What[rest]).all() and torch.isfinite(cb[rest]).all()
+    assert torch.equal(What[rest], torch.gather(cb, 1, Q.long())[rest])
+
+
 def test_gq_lnq_is_the_sequence_of_its_steps(dev):
     """gq_lnq (Algorithm 2 as one call) must give bit for bit what the separate calls give, and land where the
     oracle's LNQ lands (objective per group within 2 %, see test_lnq_loop_descends_like_the_oracle)."""
