@@ -414,14 +414,11 @@ cd_block_kernel(const __grid_constant__ CUtensorMap mapH, const __grid_constant_
                                            : make_float4(0.f, 0.f, 0.f, 0.f);
                 acc[a][0] = v.x; acc[a][1] = v.y; acc[a][2] = v.z; acc[a][3] = v.w;
             }
-            auto add = [&](const float (&h)[8], const float4 &e) {
-#pragma unroll
-                for (int a = 0; a < 8; ++a) {
-                    acc[a][0] = fmaf(h[a], e.x, acc[a][0]);
-                    acc[a][1] = fmaf(h[a], e.y, acc[a][1]);
-                    acc[a][2] = fmaf(h[a], e.z, acc[a][2]);
-                    acc[a][3] = fmaf(h[a], e.w, acc[a][3]);
-                }
+            auto add_row = [&](int a, float h, const float4 &e) {
+                acc[a][0] = fmaf(h, e.x, acc[a][0]);
+                acc[a][1] = fmaf(h, e.y, acc[a][1]);
+                acc[a][2] = fmaf(h, e.z, acc[a][2]);
+                acc[a][3] = fmaf(h, e.w, acc[a][3]);
             };
             auto load_h = [&](int c, float (&h)[8]) {
                 const float4 lo = *reinterpret_cast<const float4 *>(hb + c * CD_BAND);
@@ -437,7 +434,9 @@ cd_block_kernel(const __grid_constant__ CUtensorMap mapH, const __grid_constant_
                 for (int c = first; c < first + CD_BAND; ++c) {
                     float h[8];
                     load_h(c, h);
-                    add(h, load_e(c));
+                    const float4 e = load_e(c);
+#pragma unroll
+                    for (int a = 0; a < 8; ++a) add_row(a, h[a], e);
                 }
             }
             // bands that all six share, 5 or 6 coordinates each.  n = 0: last cycle's values inside the band, coordinates after
@@ -454,9 +453,11 @@ cd_block_kernel(const __grid_constant__ CUtensorMap mapH, const __grid_constant_
                     const int rows = kc >= k1 ? 0 : n == 0 ? kc - r0 : 8;      // of this thread's eight
                     float h[8];
                     load_h(at, h);
+                    const float4 e = load_e(at);
+                    // left out and not multiplied by zero: last cycle's value may be no number
 #pragma unroll
-                    for (int a = 0; a < 8; ++a) h[a] = a < rows ? h[a] : 0.0f;
-                    add(h, load_e(at));
+                    for (int a = 0; a < 8; ++a)
+                        if (a < rows) add_row(a, h[a], e);
                 }
             }
 #pragma unroll

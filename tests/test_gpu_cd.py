@@ -159,6 +159,16 @@ def test_cd_levels_that_are_no_numbers(dev, m):
     assert np.array_equal(Q_n[rest], Q_f[rest]) and np.array_equal(What_n[rest], What_f[rest])
 
 
+@pytest.mark.parametrize("value", [np.nan, np.inf])
+def test_cd_does_not_look_at_the_first_start_value(dev, value):
+    """Coordinate 0 is set before anything reads W_hat[:, 0]: whatever stands there, the result is the same bits."""
+    W, W0, cb, H = make_problem(60, 264, 40, 1, 4)
+    W_any = W0.copy()
+    W_any[:, 0] = value
+    want, got = run_gpu(dev, W, W0, cb, H, 1), run_gpu(dev, W, W_any, cb, H, 1)
+    assert np.array_equal(got[0], want[0]) and np.array_equal(got[1], want[1])
+
+
 def test_cd_errors_and_zero_cycles(dev):
     W, W0, cb, H = make_problem(3, 64, 16, 1, 4)
     Wd, Whd = torch.from_numpy(W).to(dev), torch.from_numpy(W0.copy()).to(dev)
