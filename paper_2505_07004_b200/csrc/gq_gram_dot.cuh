@@ -94,7 +94,7 @@ __host__ __device__ constexpr uint32_t umma_idesc_f16_mn(uint32_t m, uint32_t n)
 // Eight consecutive floats (32 bytes, 32-byte aligned) that are read once: no L1 allocation.
 __device__ __forceinline__ void ld_stream_f32x8(const float *p, float (&v)[8])
 {
-    asm volatile("ld.global.nc.L1::no_allocate.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+    asm volatile("ld.global.L1::no_allocate.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
                  : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]), "=f"(v[4]), "=f"(v[5]), "=f"(v[6]), "=f"(v[7])
                  : "l"(p));
 }
@@ -103,7 +103,7 @@ __device__ __forceinline__ void ld_stream_f32x8(const float *p, float (&v)[8])
 __device__ __forceinline__ float4 ld_f32x4(const float4 *p)
 {
     float4 v;
-    asm volatile("ld.global.nc.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(p));
+    asm volatile("ld.global.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(p));
     return v;
 }
 __device__ __forceinline__ float4 ld_f32x4_last_use(const float4 *p)
@@ -121,7 +121,7 @@ constexpr int DELTA_VEC_PER_THREAD = 4;      // float4 pairs a thread of the two
 // scale depends on, in the header; more meet in header->absmax_bits (non-negative floats order like unsigned integers), which
 // must be 0 before the launch.
 __global__ void __launch_bounds__(256)
-delta_absmax_kernel(const float *__restrict__ W, const float *__restrict__ What, unsigned count4, GramDotHeader *header)
+delta_absmax_kernel(const float *W, const float *What, unsigned count4, GramDotHeader *header)
 {
     griddep_launch();
     griddep_wait();
@@ -168,8 +168,8 @@ __device__ __forceinline__ int gram_dot_shift(unsigned int biased)
 // out = fp16((W - W_hat) * 2^e), round to nearest; the chosen e is stored in the header.  Blocks walk the matrices
 // from the END towards the start: what the maximum pass read last is still in L2.
 __global__ void __launch_bounds__(256)
-delta_half_kernel(const float *__restrict__ W, const float *__restrict__ What, unsigned count4, GramDotHeader *header,
-                  unsigned maxima, __half *__restrict__ out)
+delta_half_kernel(const float *W, const float *What, unsigned count4, GramDotHeader *header,
+                  unsigned maxima, __half *out)
 {
     griddep_launch();
     griddep_wait();

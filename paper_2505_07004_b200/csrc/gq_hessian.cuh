@@ -118,7 +118,7 @@ __device__ __forceinline__ UnitDesc decode_unit(const HessianParams &p, int unit
 __device__ __forceinline__ uint4 ld_stream_16(const void *p)
 {
     uint4 v;
-    asm volatile("ld.global.nc.L1::no_allocate.v4.u32 {%0, %1, %2, %3}, [%4];"
+    asm volatile("ld.global.L1::no_allocate.v4.u32 {%0, %1, %2, %3}, [%4];"
                  : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
                  : "l"(p));
     return v;

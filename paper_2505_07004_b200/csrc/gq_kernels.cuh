@@ -73,7 +73,7 @@ __device__ __forceinline__ float sum_sq_bf16x8(const uint4 &v, float acc)
 // guided-Hessian kernel reads it: [ceil(g / 2)][n] pairs of words, pair q of token i = groups 2q and 2q + 1
 // (the second word of an odd last group is 0).
 // A lane's share of sum_j grad[j]^2 over one segment of `vecs` 16-byte vectors (before the butterfly).
-__device__ __forceinline__ float saliency_lane_sum(const uint4 *__restrict__ src, int vecs, int lane)
+__device__ __forceinline__ float saliency_lane_sum(const uint4 *src, int vecs, int lane)
 {
     float acc[4] = {0.f, 0.f, 0.f, 0.f};
     {
@@ -111,8 +111,8 @@ __device__ __forceinline__ float warp_sum_butterfly(float sum)
 }
 
 // Stores s[k][i] and, if `words` is not null, its packed two-term form (one lane calls this).
-__device__ __forceinline__ void saliency_store(float val, unsigned i, int k, unsigned n, int g, float *__restrict__ s,
-                                               long long ld_s, uint32_t *__restrict__ words)
+__device__ __forceinline__ void saliency_store(float val, unsigned i, int k, unsigned n, int g, float *s,
+                                               long long ld_s, uint32_t *words)
 {
     s[static_cast<long long>(k) * ld_s + i] = val;
     if (words) {
@@ -123,8 +123,8 @@ __device__ __forceinline__ void saliency_store(float val, unsigned i, int k, uns
 }
 
 __global__ void __launch_bounds__(256)
-saliency_kernel(const __nv_bfloat16 *__restrict__ grad, unsigned n, int m, long long ld_grad, int g, float coef,
-                float *__restrict__ s, long long ld_s, uint32_t *__restrict__ words)
+saliency_kernel(const __nv_bfloat16 *grad, unsigned n, int m, long long ld_grad, int g, float coef,
+                float *s, long long ld_s, uint32_t *words)
 {
     griddep_launch();
     griddep_wait();
@@ -167,8 +167,8 @@ __device__ __forceinline__ float sum_sq_vec16(const uint4 &v, float acc)
 
 template <int DTYPE>
 __global__ void __launch_bounds__(256)
-saliency_strided_kernel(const void *__restrict__ grad, unsigned n, unsigned seq, int m, long long stride_b, long long stride_t,
-                        int g, float coef, float *__restrict__ s, long long ld_s)
+saliency_strided_kernel(const void *grad, unsigned n, unsigned seq, int m, long long stride_b, long long stride_t,
+                        int g, float coef, float *s, long long ld_s)
 {
     constexpr int PER_VEC = (DTYPE == SAL_FP32) ? 4 : 8;          // values per 16-byte load
     constexpr int ELEM = (DTYPE == SAL_FP32) ? 4 : 2;
@@ -206,7 +206,7 @@ saliency_strided_kernel(const void *__restrict__ grad, unsigned n, unsigned seq,
 // over the whole square 1517 us = 4.3 TB/s and 56 us.
 constexpr int MIRROR_TILE = 64;
 __global__ void __launch_bounds__(256)
-mirror_kernel(float *__restrict__ H, int d)
+mirror_kernel(float *H, int d)
 {
     __shared__ float tile[MIRROR_TILE][MIRROR_TILE + 1];
     griddep_launch();

@@ -32,12 +32,13 @@ __device__ __forceinline__ bool elect_one()
 }
 
 // ---------------------------------------------------------------- dependent launches
-// The library's kernels are launched with programmatic stream serialisation: a kernel's blocks may become resident while the
-// kernel before it in the stream is still running, so that its set-up and launch latency overlap the other's tail.  Every
-// thread of every kernel calls griddep_wait() before it touches global memory: it returns when all earlier kernels of the
-// stream have completed and their writes are visible.  griddep_launch() lets the next kernel's blocks be scheduled once
-// every block of this one has reached it.  What an earlier kernel of this library wrote is read with ordinary loads (no
-// __ldg, no const __restrict__ parameters): the compiler may move a read-only load above the wait.
+// Kernels started through launch() (gq_lib.cu) may become resident while the kernel before them in the stream is still
+// running, so that set-up and launch latency overlap the other's tail.  Every thread of such a kernel calls griddep_wait()
+// before it touches global memory: it returns when all earlier kernels of the stream have completed and their writes are
+// visible.  griddep_launch() lets the next kernel's blocks be scheduled once every block of this one has reached it.
+// Such a kernel reads nothing through the read-only path (no ld.global.nc, no __ldg, no const __restrict__ parameter): that
+// path asks for data that does not change while the kernel is there, and it is there before the writer is done; and the
+// compiler may move a read-only load above the wait.  Loads in volatile asm stay behind it.
 __device__ __forceinline__ void griddep_wait()
 {
     asm volatile("griddepcontrol.wait;" ::: "memory");

@@ -118,3 +118,39 @@ def test_one_launch_per_chunk_in_a_graph_gives_the_same_bits(dev):
     torch.cuda.synchronize()
     libgq.gq_check()
     assert torch.equal(b[0], ref[0]) and torch.equal(b[4], ref[4])
+
+
+def test_steps_enqueued_without_a_pause_read_what_the_step_before_wrote(dev):
+    """Kernels start before the ones they follow have ended.  Layers small enough for a kernel and the next ones to be on
+    the GPU at the same time: quantiser, objective, Hessian and finalize again and again over the same buffers, without a
+    pause and with one after every call, give the same values."""
+    m, g, d_in, d_out, n = 4, 2, 264, 64, 200
+    gen = torch.Generator(device=dev).manual_seed(3)
+    cases = []
+    for _ in range(3):
+        X = torch.randn(n, d_in, generator=gen, device=dev).to(torch.bfloat16)
+        W = 0.02 * torch.randn(d_out, d_in, generator=gen, device=dev)
+        cb = torch.quantile(W, (torch.arange(m, device=dev) + 0.5) / m, dim=1).T.contiguous()
+        cases.append((X, torch.rand(g, n, generator=gen, device=dev), W, cb))
+
+    def run(pause):
+        H, What = torch.empty(g, d_in, d_in, device=dev), torch.empty(d_out, d_in, device=dev)
+        loss = torch.empty(30, g + 1, dtype=torch.float64, device=dev)
+        hws = libgq.alloc_workspace(libgq.gq_hessian_workspace_bytes(n, d_in, g), dev)
+        cws = libgq.alloc_workspace(libgq.gq_cd_workspace_bytes(d_in, d_out, g), dev)
+        ows = libgq.alloc_workspace(libgq.gq_objective_workspace_bytes(d_in, d_out, g), dev)
+        for i in range(30):
+            X, s, W, cb = cases[i % 3]
+            for step in (lambda: H.zero_(),
+                         lambda: libgq.gq_hessian_accumulate(X, s, H, hws, flags=libgq.GQ_HESSIAN_DETERMINISTIC),
+                         lambda: libgq.gq_hessian_finalize(H),
+                         lambda: What.copy_(cb[:, :1].expand(-1, d_in)),
+                         lambda: libgq.gq_cd_cycles(W, What, cb, H, 1, cws),
+                         lambda: libgq.gq_objective(W, What, H, ows, loss=loss[i])):
+                step()
+                if pause:
+                    torch.cuda.synchronize()
+        libgq.gq_check()
+        return loss
+
+    assert torch.equal(run(False), run(True))
