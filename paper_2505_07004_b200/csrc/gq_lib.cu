@@ -63,9 +63,9 @@ struct LaunchScope {
 };
 
 // Launch with programmatic stream serialisation (see griddep_wait in gq_ptx.cuh, which every kernel launched here calls).
-// Errors are left for cudaGetLastError, as with <<< >>>.
+// Errors are left for cudaGetLastError, as with <<< >>>.  `overlap` = false: the blocks come when the kernel before has ended.
 template <typename... Params, typename... Args>
-void launch(void (*kernel)(Params...), dim3 grid, int threads, size_t smem, cudaStream_t st, Args &&...args)
+void launch_as(bool overlap, void (*kernel)(Params...), dim3 grid, int threads, size_t smem, cudaStream_t st, Args &&...args)
 {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
@@ -76,8 +76,13 @@ void launch(void (*kernel)(Params...), dim3 grid, int threads, size_t smem, cuda
     attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr.val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = &attr;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = overlap ? 1 : 0;
     (void)cudaLaunchKernelEx(&cfg, kernel, static_cast<Params>(args)...);
+}
+template <typename... Params, typename... Args>
+void launch(void (*kernel)(Params...), dim3 grid, int threads, size_t smem, cudaStream_t st, Args &&...args)
+{
+    launch_as(true, kernel, grid, threads, smem, st, static_cast<Args &&>(args)...);
 }
 
 // Per-device status word {status, site, block, unit}; written by kernels, read by gq_check().
@@ -713,7 +718,13 @@ int32_t gq_hessian_finalize(float *H, int64_t d_in, int32_t g, void *stream)
     dim3 grid(nb * (nb + 1) / 2, static_cast<unsigned>(g));
     {
         LaunchScope scope(GQ_KERNEL_MIRROR, static_cast<cudaStream_t>(stream));
-        launch(gq::mirror_kernel, dim3(grid), 256, 0, static_cast<cudaStream_t>(stream), H, static_cast<int>(d_in));
+        // Not overlapped with the kernel before it, which as a rule is the Hessian kernel.  Thousands of blocks that take an
+        // SM over from a kernel with 225 KB of shared memory find the L1 that this left (with a smaller shared-memory
+        // carve-out preferred the loss below is gone for the larger of the two), and so do the kernels that overlap with
+        // them.  Layer of 2360 x 896, 16 groups, 3505 tokens: 540 us, overlapped 571; three batches of 921 tokens at d_in
+        // 1456, one group: 105 us, overlapped 135; d_in 28672, two groups, 4096 tokens: 14.1 ms, overlapped 14.4.  The
+        // smallest layer (256 x 512) takes 46 us either way.
+        launch_as(false, gq::mirror_kernel, dim3(grid), 256, 0, static_cast<cudaStream_t>(stream), H, static_cast<int>(d_in));
     }
     GQ_CUDA(cudaGetLastError());
     return GQ_OK;
