@@ -178,6 +178,19 @@ pair_gemm_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant
             if (!item_geom<MODE>(p, w, rank, ge)) continue;
             const void *maps[MAX_MAPS] = {&map0, &map1, &map2, &map3, &map4, &map5};
             for (int ks = ge.ks0; ks < ge.ks1; ++ks) {
+                // MODE_OBJECTIVE: which operands, looked up while the stage is still in use (after the wait the division
+                // and the table reads are part of every step: a unit of 66 took 1.3 us longer)
+                const void *amap = nullptr, *bmap = nullptr;
+                int term_row = 0, ka = 0, kb = 0;
+                if (MODE == MODE_OBJECTIVE) {
+                    const int term = ks / kblocks;
+                    term_row = (ks - term * kblocks) * TILE_K;
+                    const int ma = p.term_a[term], mb = p.term_b[term];
+                    amap = maps[ma];
+                    bmap = maps[mb];
+                    ka = p.map_grouped[ma] ? ge.k : 0;
+                    kb = p.map_grouped[mb] ? ge.k : 0;
+                }
                 if (!bounded_wait(smem_u32(&bar_empty[s]), ph ^ 1u, wc, 1u, w.unit)) { ok = false; break; }
                 const uint32_t full_local = smem_u32(&bar_full[s]);
                 if (rank == 0) mbar_arrive_expect_tx(full_local, 2 * STAGE_BYTES);   // both CTAs' bytes
@@ -192,16 +205,12 @@ pair_gemm_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant
                             tma_load_3d_pair(sa + op * OBJ_A_BYTES + q * BOX_BYTES, maps[op], full,
                                              (op < 2 ? ge.a0 : ge.b0) + q * BOX_FEATURES, row, op < 2 ? ge.k : 0);
                 } else {
-                    const int term = ks / kblocks;
-                    const int row = (ks - term * kblocks) * TILE_K;
-                    const int ma = p.term_a[term], mb = p.term_b[term];
-                    const int ka = p.map_grouped[ma] ? ge.k : 0, kb = p.map_grouped[mb] ? ge.k : 0;
 #pragma unroll
                     for (int q = 0; q < CTA_ROWS / BOX_FEATURES; ++q)
-                        tma_load_3d_pair(sa + q * BOX_BYTES, maps[ma], full, ge.a0 + q * BOX_FEATURES, row, ka);
+                        tma_load_3d_pair(sa + q * BOX_BYTES, amap, full, ge.a0 + q * BOX_FEATURES, term_row, ka);
 #pragma unroll
                     for (int q = 0; q < CTA_ROWS / BOX_FEATURES; ++q)
-                        tma_load_3d_pair(sa + OBJ_A_BYTES + q * BOX_BYTES, maps[mb], full, ge.b0 + q * BOX_FEATURES, row, kb);
+                        tma_load_3d_pair(sa + OBJ_A_BYTES + q * BOX_BYTES, bmap, full, ge.b0 + q * BOX_FEATURES, term_row, kb);
                 }
                 ++issued;
                 if (++s == STAGES) { s = 0; ph ^= 1u; }
