@@ -110,7 +110,7 @@ __device__ __forceinline__ uint32_t take_bf16x2(float &x, float &y)
 }
 
 // MP: one-hot columns per channel (4, 8 or 16, at least m; columns m .. MP - 1 stay zero).
-// mapH0/1: T as bf16 hi / lo [g][d][d]; mapW0/1: W^T as bf16 hi / lo [d][d_out].
+// mapH0/1: H as bf16 hi / lo [g][d][d]; mapW0/1: W^T as bf16 hi / lo [d][d_out].
 template <int MP>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(CG_THREADS, 1)
 codebook_gemm_kernel(const __grid_constant__ CUtensorMap mapH0, const __grid_constant__ CUtensorMap mapH1,

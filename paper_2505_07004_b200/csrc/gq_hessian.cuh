@@ -129,9 +129,6 @@ __device__ __forceinline__ uint4 ld_stream_16(const void *p)
 // 2 q + 1 of a token sit side by side, so a scaler thread fetches both with one 8-byte load and does no
 // conversion work in its loop (sixteen threads share a token; converting there would be done sixteen times).
 __global__ void __launch_bounds__(256)
-split_saliency_kernel(const float *s, long long ld_s, int n, int g, uint2 *out);
-
-__global__ void __launch_bounds__(256)
 split_saliency_kernel(const float *s, long long ld_s, int n, int g, uint2 *out)
 {
     griddep_launch();

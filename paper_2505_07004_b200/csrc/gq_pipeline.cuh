@@ -1,7 +1,7 @@
-// Shared scaffolding of libgq's two tensor-core kernels (guided Hessian, objective): tile geometry, the
-// distribution of work units over CTA pairs, and bounded mbarrier waits.
+// Shared scaffolding of libgq's tensor-core kernels (guided Hessian, objective, panel product, codebook product): tile
+// geometry, the distribution of work units over CTA pairs, and bounded mbarrier waits.
 //
-// Both kernels run as clusters of two CTAs (one CTA pair per two SMs).  A pair owns one 256 x 256 tile at a
+// The kernels run as clusters of two CTAs (one CTA pair per two SMs).  A pair owns one 256 x 256 tile at a
 // time; each CTA loads 128 of the tile's A rows and 128 of its B columns per 64-row k-step, the first CTA
 // of the pair issues tcgen05.mma.cta_group::2 (M = 256, N = 256, K = 16) for both, and each CTA holds the
 // fp32 accumulator rows of its own 128 rows in its tensor memory.
@@ -69,19 +69,8 @@ inline Schedule plan_schedule(int units, int ksteps, int pairs, bool balanced)
     return p;
 }
 
-// Slot t of the triangular enumeration -> (row block i, column block j) of 256 x 256 tiles with i <= j,
-// column blocks outermost.
-__device__ __forceinline__ void tile_of_slot(int t, int &i, int &j)
-{
-    int jj = static_cast<int>((sqrtf(8.0f * static_cast<float>(t) + 1.0f) - 1.0f) * 0.5f);
-    while (jj * (jj + 1) / 2 > t) --jj;
-    while ((jj + 1) * (jj + 2) / 2 <= t) ++jj;
-    j = jj;
-    i = t - jj * (jj + 1) / 2;
-}
-
-// The same set of tiles in an order that keeps tiles which are worked on at the same time close together in
-// BOTH directions: the upper triangle is cut into super-blocks of R x R tiles (column super-blocks outermost,
+// Slot t -> (row block i, column block j) of the 256 x 256 tiles with i <= j, in an order that keeps tiles which are worked
+// on at the same time close together in BOTH directions: the upper triangle is cut into super-blocks of R x R tiles (column super-blocks outermost,
 // row super-blocks inside, tiles of a super-block row by row), so that a round of P consecutive tiles touches
 // about 2 sqrt(P) row/column blocks of X instead of P + 1.  Every (i <= j) appears exactly once for
 // t in [0, NJ (NJ + 1) / 2).
@@ -133,7 +122,6 @@ __device__ __forceinline__ void colpair_of_slot(int t, int &i, int &q)
 struct WorkItem {
     int unit;      // (tile slot) * g + group
     int ks0, ks1;  // k-step range [ks0, ks1) of the unit's `ksteps`
-    bool piece;    // true: other pairs hold the rest of this unit
 };
 
 // The `it`-th work item of pair `pair`; false when the pair has no more work.  Every role of both CTAs of
@@ -144,7 +132,6 @@ __device__ __forceinline__ bool work_item(const Schedule &p, int pair, int it, W
         w.unit = it * p.pairs + pair;
         w.ks0 = 0;
         w.ks1 = p.ksteps;
-        w.piece = false;
         return w.unit < p.units;
     }
     if (pair >= p.tail_pairs) return false;
@@ -159,7 +146,6 @@ __device__ __forceinline__ bool work_item(const Schedule &p, int pair, int it, W
     w.ks0 = static_cast<int>(cur - static_cast<long long>(tu) * p.ksteps);
     const long long left = end - cur;
     w.ks1 = (left < p.ksteps - w.ks0) ? w.ks0 + static_cast<int>(left) : p.ksteps;
-    w.piece = !(w.ks0 == 0 && w.ks1 == p.ksteps);
     return true;
 }
 

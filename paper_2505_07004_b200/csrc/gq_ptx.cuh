@@ -20,17 +20,6 @@ __device__ __forceinline__ uint64_t global_timer_ns()
     return t;
 }
 
-__device__ __forceinline__ bool elect_one()
-{
-    uint32_t pred;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "elect.sync _|p, 0xffffffff;\n\t"
-        "selp.u32 %0, 1, 0, p;\n\t}"
-        : "=r"(pred));
-    return pred != 0;
-}
-
 // ---------------------------------------------------------------- dependent launches
 // Kernels started through launch() (gq_lib.cu) may become resident while the kernel before them in the stream is still
 // running, so that set-up and launch latency overlap the other's tail.  Every thread of such a kernel calls griddep_wait()
