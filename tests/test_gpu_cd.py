@@ -159,6 +159,14 @@ def test_cd_levels_that_are_no_numbers(dev, m):
     assert np.array_equal(Q_n[rest], Q_f[rest]) and np.array_equal(What_n[rest], What_f[rest])
 
 
+def test_cd_more_panel_tiles_than_pairs(dev):
+    """80 groups of 8 channels: 80 panel units on at most 74 CTA pairs, some pairs take two and add their tiles to P
+    without the staging ring; two ragged panels."""
+    W, W0, cb, H = make_problem(50, 520, 640, 80, 4, n=600)
+    What_g, Q_g = run_gpu(dev, W, W0, cb, H, 1)
+    check_against_oracle(W, W0, cb, H, What_g, Q_g, 1, certify_ties=True)
+
+
 @pytest.mark.parametrize("value", [np.nan, np.inf])
 def test_cd_does_not_look_at_the_first_start_value(dev, value):
     """Coordinate 0 is set before anything reads W_hat[:, 0]: whatever stands there, the result is the same bits."""

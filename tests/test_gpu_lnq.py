@@ -82,21 +82,27 @@ def test_codebook_update_matches_oracle(dev, seed, d_in, d_out, g, m):
 
 @pytest.mark.parametrize("seed,d_in,d_out,g,m", [
     (30, 264, 24, 1, 1),        # one level; a second row block of 8 rows
-    (31, 1288, 40, 1, 3),       # 4 columns per channel, one of them unused; six row blocks: both directions of dealing
+    (31, 1288, 40, 1, 3),       # 4 columns per channel, one of them unused; six row blocks
     (32, 776, 552, 1, 5),       # 8 columns per channel; channel tiles of 256, 256 and 40
     (33, 520, 152, 1, 13),      # 16 columns per channel; the last tile holds 8 channels
     (34, 2056, 72, 3, 16),      # nine row blocks, 24 channels per group
 ])
 def test_codebook_update_tile_edges(dev, seed, d_in, d_out, g, m):
     """Widths of a channel's one-hot columns (4, 8, 16) with levels to spare, ragged row blocks, tiles and groups, and
-    codes at an address that is not a multiple of 8 (same bits as at an aligned one)."""
+    codes at an address that is not a multiple of 8 (the same values as at an aligned one, up to the order in which the
+    fp64 sums are added)."""
     W, W0, Q0, cb0, H = make_problem(seed, d_in, d_out, g, m)
     cb_g, What_g = gpu_codebook(dev, W, Q0, m, H)
     cb_o = cdo.codebook_update(W, Q0, H, m)
     assert np.array_equal(What_g, np.take_along_axis(cb_g, Q0, axis=1))
-    # W enters as two bf16 terms (2^-17 of each weight is dropped), so the error scales with the weights; with many levels
-    # the largest level is of their size, a single level is their mean and may be a hundred times smaller
-    assert (np.abs(cb_g - cb_o) / np.abs(W).max(axis=1, keepdims=True)).max() <= C_RTOL
+    # W enters as two bf16 terms (2^-17 of each weight is dropped), so the error scales with the weights; with several levels
+    # the largest one is of their size, a single level is their mean and may be a hundred times smaller
+    scale = np.abs(W if m == 1 else cb_o).max(axis=1, keepdims=True)
+    assert (np.abs(cb_g - cb_o) / scale).max() <= C_RTOL
+    f_g, f_before = per_channel_objective(W, What_g, H), per_channel_objective(W, W0, H)
+    f_o = per_channel_objective(W, np.take_along_axis(cb_o, Q0, axis=1), H)
+    assert np.all(f_g <= f_o * (1 + F_RTOL))
+    assert np.all(f_g <= f_before * (1 + 1e-6))
     store = torch.zeros(d_out * d_in + 3, dtype=torch.uint8, device=dev)
     Qd = store[3:].view(d_out, d_in)
     Qd.copy_(torch.from_numpy(Q0.astype(np.uint8)))

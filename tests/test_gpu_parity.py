@@ -622,3 +622,24 @@ def test_host_pipeline_matches_device_calls(dev, d_out, g):
     # same kernels, same order; tiles that are cut along tokens are summed with atomics (last-bit freedom)
     assert torch.allclose(H_host, H.cpu(), rtol=1e-5, atol=1e-6 * H.abs().max().item())
     assert torch.allclose(loss_host, loss.cpu(), rtol=1e-6, atol=0.0)
+
+
+@pytest.mark.parametrize("d_in,d_out", [(1280, 3072), (1248, 3152)])      # 960 and 961 blocks of 4096 weights
+def test_objective_scale_where_the_block_maxima_stop_fitting(dev, d_in, d_out):
+    """Up to 960 blocks leave their largest difference in the header one by one, more meet in one word.  The largest
+    difference stands in the last weight, 2^10 above the others: a scale that missed it would take it past fp16's range."""
+    gen = torch.Generator(device=dev).manual_seed(5)
+    A = torch.randn(d_in, d_in, generator=gen, device=dev)
+    H = (A.T @ A).expand(2, d_in, d_in).contiguous()
+    H = ((H + H.transpose(1, 2)) / 2).contiguous()
+    W = 0.02 * torch.randn(d_out, d_in, generator=gen, device=dev)
+    W_hat = W + 0.01 * (torch.rand(d_out, d_in, generator=gen, device=dev) - 0.5)
+    W_hat[-1, -1] = W[-1, -1] + 5.0
+    ows = libgq.alloc_workspace(libgq.gq_objective_workspace_bytes(d_in, d_out, 2), dev)
+    for last in (5.0, -0.005):                           # the second time after a larger one through the same workspace
+        W_hat[-1, -1] = W[-1, -1] + last
+        loss = libgq.gq_objective(W, W_hat, H, ows)
+        libgq.gq_check()
+        delta = (W.double() - W_hat.double()).view(2, -1, d_in)
+        want = torch.stack([((delta[k] @ H[k].double()) * delta[k]).sum() for k in range(2)])
+        assert ((loss[:2] - want).abs() <= 1e-3 * want).all()        # 2^-11 if all roundings of fp16 point one way
