@@ -112,7 +112,7 @@ split_h_kernel(const float *H, int d_in, __nv_bfloat16 *Hhi, __nv_bfloat16 *Hlo,
 __global__ void __launch_bounds__(256)
 cd_finish_kernel(const float *codebook, const uint8_t *Qt, int d_in, int d_out, int m, float *What, uint8_t *Q, bool bytes)
 {
-    __shared__ uint8_t tq[64][68];
+    __shared__ __align__(4) uint8_t tq[64][68];            // stored to in words
     griddep_launch();
     griddep_wait();
     const int c4 = (threadIdx.x & 15) * 4, r0 = threadIdx.x >> 4;
