@@ -45,8 +45,7 @@ __device__ __forceinline__ void split_bf16(float v, __nv_bfloat16 &hi, __nv_bflo
 }
 
 // Wt = W^T, E = (What - W)^T (fp32 and as bf16 hi + lo), all [d_in][d_out].  Tiles of 32 coordinates x 64 channels: whole
-// 128-byte segments on both sides (4096 x 4096: 52 us; one value per
-// lane and 64-byte segments 73).
+// 128-byte segments on both sides (4096 x 4096: 51 us; one value per lane and 64-byte segments 73).
 __global__ void __launch_bounds__(256)
 cd_prepare_kernel(const float *W, const float *What, int d_in, int d_out, float *Wt, float *Et, __nv_bfloat16 *Ehi, __nv_bfloat16 *Elo)
 {
@@ -112,7 +111,7 @@ split_h_kernel(const float *H, int d_in, __nv_bfloat16 *Hhi, __nv_bfloat16 *Hlo,
 __global__ void __launch_bounds__(256)
 cd_finish_kernel(const float *codebook, const uint8_t *Qt, int d_in, int d_out, int m, float *What, uint8_t *Q, bool bytes)
 {
-    __shared__ __align__(4) uint8_t tq[64][68];            // stored to in words
+    __shared__ __align__(4) uint8_t tq[64][68];                    // stored to in words
     griddep_launch();
     griddep_wait();
     const int c4 = (threadIdx.x & 15) * 4, r0 = threadIdx.x >> 4;
@@ -247,8 +246,9 @@ __device__ __forceinline__ int sums_at(int ch, int rq)
 //   loader warp (4)      TMA: the tiles of W, E and P (256 coordinates x 32 channels), and H[all 256][band] (32 KB) per
 //                        band into one of three buffers, two bands ahead.
 // Two named barriers per band: sums ready (products -> chain), band done (chain -> products, loader).
-// Measured for one block of 4096 channels, 16 levels: 35 us (8 levels, 1408 channels: 31); with eight threads per channel
-// that did all updates themselves and two votes and a table read per step it was 81 us (78).
+// Measured for one block of 4096 channels, 16 levels: 33.7 us (8 levels, 1408 channels: 29.8; 34.9 and 31.2 with the excluded
+// coordinates multiplied by zero instead of left out); with eight threads per channel that did all updates themselves and two
+// votes and a table read per step it was 81 us (78).
 template <int LEV>
 __global__ void __launch_bounds__(CD_THREADS, 1)
 cd_block_kernel(const __grid_constant__ CUtensorMap mapH, const __grid_constant__ CUtensorMap mapW,

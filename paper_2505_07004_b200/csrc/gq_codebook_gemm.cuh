@@ -19,7 +19,7 @@
 // descent cycles with them.)
 // Stage: [A | B], 16 KB each per CTA, of which only B comes through the L2.  What bounds the kernel is the tensor core (732
 // clocks a k-step with the one-hot stores left out, 512 at its nominal rate) and shared-memory bandwidth (840 with them).
-// Measured, 4096 x 4096, 4 groups, 16 levels, one update: 3.77 ms = 1280 TFLOP/s.  With the one-hot matrix, H P and H W^T in
+// Measured, 4096 x 4096, 4 groups, 16 levels, one update: 3.73 ms = 1290 TFLOP/s.  With the one-hot matrix, H P and H W^T in
 // global memory it was 0.17 (one-hot) + 2.88 (H P) + 0.40 (H W^T) + 0.55 (sums by level) = 4.00 ms and 0.5 GB of scratch.
 #pragma once
 #include <cuda.h>
