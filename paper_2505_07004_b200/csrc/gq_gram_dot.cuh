@@ -7,9 +7,9 @@
 // matching entries of H_k straight out of tensor memory.
 //
 // Operands.  Delta is prepared once per call as ONE fp16 matrix (delta_half_kernel): delta * 2^e with a single
-// power of two e for the whole layer, chosen from max |delta| (delta_absmax_kernel) so that the largest entry
-// lies in [2^14, 2^15).  fp16 carries 11 significant bits at any magnitude above 2^-14, i.e. down to 2^-28 of
-// the largest entry, and the scaling is undone exactly (2^-2e in the final fp64 reduction).  One product at the
+// power of two e for the whole layer, such that the largest entry lies below 2^15 and, but for the clamps, above 2^11.
+// fp16 carries 11 significant bits at any magnitude above 2^-14, i.e. down to 2^-25 of the largest entry at least, and the
+// scaling is undone exactly (2^-2e in the final fp64 reduction).  One product at the
 // 16-bit rate replaces three bf16 products (hi hi + hi lo + lo hi): the contraction then costs about as much as
 // streaming H from HBM, which is what the kernel below is built around.  Rounding: both factors of every
 // product carry a relative error of at most 2^-12 (round to nearest), unbiased, so the objective is good to
@@ -56,18 +56,16 @@ constexpr int GD_EPI_WARPS = 8;
 constexpr int GD_THREADS = 32 * (4 + GD_EPI_WARPS);
 constexpr int GD_SMEM_BYTES = GD_STAGES * GD_STAGE_BYTES + 1024;
 constexpr int GD_PARTIALS_PER_UNIT = 2 * GD_EPI_WARPS;       // one fp64 per (CTA of the pair, epilogue warp)
-constexpr int GD_TARGET_EXP = 14;                            // the largest |delta| * 2^e lies in [2^14, 2^15)
+constexpr int GD_SAMPLE_EXP = 11;                            // the largest sampled |delta| * 2^e lies in [2^11, 2^12),
+constexpr int GD_LARGEST_EXP = 14;                           // the largest of all has to lie below 2^15; else, with the exact
+                                                             // maximum, in [2^14, 2^15)
 constexpr int GD_MAX_SHIFT = 100;                            // |e| is kept below this (the scale stays a normal float)
-
-constexpr unsigned DELTA_BLOCK_MAXIMA = 960;      // blocks of the first preparation pass: what the 1 KiB header holds
 
 // Header of the objective workspace, written by the preparation kernels and read by the reduction.
 struct GramDotHeader {
+    int guess;                  // e of the first preparation pass
     int shift;                  // e: the fp16 matrix holds (W - W_hat) * 2^e
     unsigned int blocks_done;   // groups whose loss has been written (the last one forms the total)
-    unsigned int absmax_bits;   // bit pattern of max |W - W_hat| where the first pass has more blocks than that
-    unsigned int pad[13];       // the exponents start a 64-byte segment
-    uint8_t block_exp[DELTA_BLOCK_MAXIMA];   // biased exponent of each first-pass block's max |W - W_hat|
 };
 
 struct GramDotParams {
@@ -113,69 +111,65 @@ __device__ __forceinline__ float4 ld_f32x4_last_use(const float4 *p)
     return v;
 }
 
-constexpr int DELTA_VEC_PER_THREAD = 4;      // float4 pairs a thread of the two preparation kernels handles
+constexpr int DELTA_VEC_PER_THREAD = 4;      // float4 pairs a thread of the first preparation kernel handles
+constexpr unsigned DELTA_BLOCK_VECS = 256u * DELTA_VEC_PER_THREAD;
 
-// ------------------------------------------------------------------------------------------------
-// max |W - W_hat| over the layer (the differences are formed in fp32, as everywhere in the objective), one block per
-// 256 * DELTA_VEC_PER_THREAD float4 pairs.  Up to DELTA_BLOCK_MAXIMA blocks leave the exponent of their maximum, all that the
-// scale depends on, in the header; more meet in header->absmax_bits (non-negative floats order like unsigned integers), which
-// must be 0 before the launch.
-__global__ void __launch_bounds__(256)
-delta_absmax_kernel(const float *W, const float *What, unsigned count4, GramDotHeader *header)
+// The power of two that takes a value of biased exponent `biased` (0: zero or subnormal) to [2^target, 2^(target + 1)).
+__device__ __forceinline__ int delta_shift(unsigned int biased, int target)
 {
-    griddep_launch();
-    griddep_wait();
-    const unsigned base = blockIdx.x * (256u * DELTA_VEC_PER_THREAD) + threadIdx.x;
-    float4 w[DELTA_VEC_PER_THREAD], q[DELTA_VEC_PER_THREAD];
-#pragma unroll
-    for (int t = 0; t < DELTA_VEC_PER_THREAD; ++t) {
-        const unsigned idx = base + t * 256u;
-        const bool in = idx < count4;
-        w[t] = in ? ld_f32x4(reinterpret_cast<const float4 *>(W) + idx) : make_float4(0.f, 0.f, 0.f, 0.f);
-        q[t] = in ? ld_f32x4(reinterpret_cast<const float4 *>(What) + idx) : make_float4(0.f, 0.f, 0.f, 0.f);
-    }
-    float m = 0.0f;
-#pragma unroll
-    for (int t = 0; t < DELTA_VEC_PER_THREAD; ++t)
-        m = fmaxf(m, fmaxf(fmaxf(fabsf(w[t].x - q[t].x), fabsf(w[t].y - q[t].y)),
-                           fmaxf(fabsf(w[t].z - q[t].z), fabsf(w[t].w - q[t].w))));
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, off));
-    __shared__ float red[8];
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = m;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        for (int w8 = 1; w8 < 8; ++w8) m = fmaxf(m, red[w8]);
-        // NaN never wins fmaxf; an infinite difference gives 0xff and the shift below saturates
-        if (gridDim.x <= DELTA_BLOCK_MAXIMA)
-            header->block_exp[blockIdx.x] = static_cast<uint8_t>(__float_as_uint(m) >> 23);
-        else if (m > 0.0f)
-            atomicMax(&header->absmax_bits, __float_as_uint(m));
-    }
-}
-
-// The power of two e for a layer whose largest |delta| has the biased exponent `biased` (0: zero or subnormal).
-__device__ __forceinline__ int gram_dot_shift(unsigned int biased)
-{
-    int k = static_cast<int>(biased) - 127;                        // floor(log2(max)) for normal values
+    int k = static_cast<int>(biased) - 127;                        // floor(log2(value)) for normal values
     if (k < -126) k = -126;
-    int e = GD_TARGET_EXP - k;
+    int e = target - k;
     if (e > GD_MAX_SHIFT) e = GD_MAX_SHIFT;
     if (e < -GD_MAX_SHIFT) e = -GD_MAX_SHIFT;
     return e;
 }
-
-// out = fp16((W - W_hat) * 2^e), round to nearest; the chosen e is stored in the header.  Blocks walk the matrices
-// from the END towards the start: what the maximum pass read last is still in L2.
-__global__ void __launch_bounds__(256)
-delta_half_kernel(const float *W, const float *What, unsigned count4, GramDotHeader *header,
-                  unsigned maxima, __half *out)
+__device__ __forceinline__ float delta_scale(int e)
 {
+    return __uint_as_float(static_cast<unsigned int>(127 + e) << 23);
+}
+__device__ __forceinline__ float delta_max(float m, const float4 &w, const float4 &q)      // a NaN never wins fmaxf
+{
+    return fmaxf(m, fmaxf(fmaxf(fabsf(w.x - q.x), fabsf(w.y - q.y)), fmaxf(fabsf(w.z - q.z), fabsf(w.w - q.w))));
+}
+__device__ __forceinline__ uint2 delta_half4(const float4 &w, const float4 &q, float scale)
+{
+    uint2 o;
+    __half2 *h = reinterpret_cast<__half2 *>(&o);
+    h[0] = __floats2half2_rn((w.x - q.x) * scale, (w.y - q.y) * scale);
+    h[1] = __floats2half2_rn((w.z - q.z) * scale, (w.w - q.w) * scale);
+    return o;
+}
+// Maximum over the 256 threads of a block; `red` holds eight words.
+__device__ __forceinline__ unsigned int block_max(unsigned int v, unsigned int *red)
+{
+    v = __reduce_max_sync(0xffffffffu, v);
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
+    __syncthreads();
+#pragma unroll
+    for (int w8 = 0; w8 < 8; ++w8) v = max(v, red[w8]);
+    return v;
+}
+
+// out = fp16((W - W_hat) * 2^e), round to nearest (the differences are formed in fp32, as everywhere in the objective), and
+// the biased exponent of every block's max |W - W_hat| (an infinite difference: 0xff).  e has to be known before the first
+// value is stored and depends on the largest, so it is guessed: every block looks at the same 1024 values, spread over the
+// layer, and leaves room for values 8 times as large.  delta_redo_kernel takes care of layers that need more.
+// HBM-bound: W and W_hat are read once.  Three candidates of a 4096 x 4096 layer, whole calls: 319 us; with a pass over both
+// for the maximum before the pass that converts 352 us (4096 x 11008 layer, one group, all of it: 704 and 760).
+__global__ void __launch_bounds__(256)
+delta_half_kernel(const float *W, const float *What, unsigned count4, GramDotHeader *header, uint8_t *block_exp, __half *out)
+{
+    __shared__ unsigned int red[2][8];
     griddep_launch();
     griddep_wait();
-    const unsigned blk = gridDim.x - 1u - blockIdx.x;
-    const unsigned base = blk * (256u * DELTA_VEC_PER_THREAD) + threadIdx.x;
+    const unsigned base = blockIdx.x * DELTA_BLOCK_VECS + threadIdx.x;
     float4 w[DELTA_VEC_PER_THREAD], q[DELTA_VEC_PER_THREAD];
+    // one pair of float4 per thread, somewhere in the thread's 256th of the layer (the same for every block)
+    const unsigned part = max(count4 / 256u, 1u);
+    const unsigned sidx = min(threadIdx.x * part + __umulhi(threadIdx.x * 2654435761u, part), count4 - 1u);
+    const float4 sw = ld_f32x4(reinterpret_cast<const float4 *>(W) + sidx);
+    const float4 sq = ld_f32x4(reinterpret_cast<const float4 *>(What) + sidx);
 #pragma unroll
     for (int t = 0; t < DELTA_VEC_PER_THREAD; ++t) {
         const unsigned idx = base + t * 256u;
@@ -183,40 +177,50 @@ delta_half_kernel(const float *W, const float *What, unsigned count4, GramDotHea
         w[t] = in ? ld_f32x4_last_use(reinterpret_cast<const float4 *>(W) + idx) : make_float4(0.f, 0.f, 0.f, 0.f);
         q[t] = in ? ld_f32x4_last_use(reinterpret_cast<const float4 *>(What) + idx) : make_float4(0.f, 0.f, 0.f, 0.f);
     }
-    unsigned int biased = 0u;
-    if (maxima == 0u) {                                            // not left block by block
-        biased = *const_cast<volatile unsigned int *>(&header->absmax_bits) >> 23;
-    } else {
-        static_assert(DELTA_BLOCK_MAXIMA <= 4 * 256, "four exponents per thread");
-        if (4u * threadIdx.x < maxima) {
-            const uint32_t four = reinterpret_cast<const volatile uint32_t *>(header->block_exp)[threadIdx.x];
-#pragma unroll
-            for (unsigned b = 0; b < 4; ++b)
-                if (4u * threadIdx.x + b < maxima) biased = max(biased, (four >> (8u * b)) & 0xffu);
-        }
-        __shared__ unsigned int red[8];
-        biased = __reduce_max_sync(0xffffffffu, biased);
-        if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = biased;
-        __syncthreads();
-#pragma unroll
-        for (int w8 = 0; w8 < 8; ++w8) biased = max(biased, red[w8]);
-    }
-    const int e = gram_dot_shift(biased);
+    const int e = delta_shift(block_max(__float_as_uint(delta_max(0.0f, sw, sq)), red[0]) >> 23, GD_SAMPLE_EXP);
     if (blockIdx.x == 0 && threadIdx.x == 0) {
-        header->shift = e;
+        header->guess = e;
         header->blocks_done = 0u;
     }
-    const float scale = __uint_as_float(static_cast<unsigned int>(127 + e) << 23);
+    const float scale = delta_scale(e);
+    float m = 0.0f;
 #pragma unroll
     for (int t = 0; t < DELTA_VEC_PER_THREAD; ++t) {
         const unsigned idx = base + t * 256u;
-        if (idx >= count4) continue;
-        uint2 o;
-        __half2 *h = reinterpret_cast<__half2 *>(&o);
-        h[0] = __floats2half2_rn((w[t].x - q[t].x) * scale, (w[t].y - q[t].y) * scale);
-        h[1] = __floats2half2_rn((w[t].z - q[t].z) * scale, (w[t].w - q[t].w) * scale);
-        reinterpret_cast<uint2 *>(out)[idx] = o;
+        m = delta_max(m, w[t], q[t]);
+        if (idx < count4) reinterpret_cast<uint2 *>(out)[idx] = delta_half4(w[t], q[t], scale);
     }
+    const unsigned int largest = block_max(__float_as_uint(m), red[1]);
+    if (threadIdx.x == 0) block_exp[blockIdx.x] = static_cast<uint8_t>(largest >> 23);
+}
+
+// Decides on e: the guess where the largest |W - W_hat| stays below 2^15 with it (all blocks return at once), else the power
+// of two that takes it to [2^14, 2^15), with which the matrix is written again.  blocks: of delta_half_kernel.
+__global__ void __launch_bounds__(256)
+delta_redo_kernel(const float *W, const float *What, unsigned count4, GramDotHeader *header, const uint8_t *block_exp,
+                  unsigned blocks, __half *out)
+{
+    __shared__ unsigned int red[8];
+    griddep_launch();
+    griddep_wait();
+    unsigned int biased = 0u;
+    const unsigned words = blocks / 16u;
+    for (unsigned i = threadIdx.x; i < words; i += 256u) {         // block_exp is 16-byte aligned
+        const uint4 v = reinterpret_cast<const uint4 *>(block_exp)[i];
+        const uint32_t four = __vmaxu4(__vmaxu4(v.x, v.y), __vmaxu4(v.z, v.w));
+        biased = max(biased, max(max(four & 0xffu, (four >> 8) & 0xffu), max((four >> 16) & 0xffu, four >> 24)));
+    }
+    if (threadIdx.x < blocks % 16u) biased = max(biased, static_cast<unsigned int>(block_exp[words * 16u + threadIdx.x]));
+    biased = block_max(biased, red);
+    const int guess = header->guess, exact = delta_shift(biased, GD_LARGEST_EXP);
+    const bool fits = static_cast<int>(biased) - 127 + guess <= GD_LARGEST_EXP || exact == guess;
+    if (blockIdx.x == 0 && threadIdx.x == 0) header->shift = fits ? guess : exact;
+    if (fits) return;
+    const float scale = delta_scale(exact);
+    const unsigned stride = gridDim.x * 256u;
+    for (unsigned idx = blockIdx.x * 256u + threadIdx.x; idx < count4; idx += stride)
+        reinterpret_cast<uint2 *>(out)[idx] =
+            delta_half4(reinterpret_cast<const float4 *>(W)[idx], reinterpret_cast<const float4 *>(What)[idx], scale);
 }
 
 // loss[k] = 2^(-2e) * sum over the group's partial sums (block k), loss[g] = sum_k loss[k] (formed, in group order,

@@ -351,7 +351,7 @@ size_t hessian_ws_bytes(int64_t n_max, int64_t, int32_t g)
 struct ObjectiveLayout {
     size_t header_off, half_off, partials_off, total;
 };
-// Scratch of gq_objective: a header (largest |delta| and the chosen power-of-two scale), delta as one fp16
+// Scratch of gq_objective: a header (the chosen power-of-two scale), delta as one fp16
 // matrix, and one fp64 partial sum per (work unit, CTA of the pair, epilogue warp).
 ObjectiveLayout objective_layout(int64_t d_in, int64_t d_out, int32_t g)
 {
@@ -359,8 +359,10 @@ ObjectiveLayout objective_layout(int64_t d_in, int64_t d_out, int32_t g)
     L.header_off = 0;
     L.half_off = round_up(sizeof(gq::GramDotHeader), 1024);
     L.partials_off = L.half_off + round_up(static_cast<size_t>(d_in) * static_cast<size_t>(d_out) * 2, 1024);
-    L.total = L.partials_off +
-              round_up(static_cast<size_t>(tiles_for(d_in)) * g * gq::GD_PARTIALS_PER_UNIT * sizeof(double), 1024);
+    size_t tail = static_cast<size_t>(tiles_for(d_in)) * g * gq::GD_PARTIALS_PER_UNIT * sizeof(double);
+    const size_t blocks = (static_cast<size_t>(d_in) * d_out / 4 + gq::DELTA_BLOCK_VECS - 1) / gq::DELTA_BLOCK_VECS;
+    if (tail < blocks) tail = blocks;                              // one byte each, see gq_objective
+    L.total = L.partials_off + round_up(tail, 1024);
     return L;
 }
 
@@ -801,24 +803,21 @@ int32_t gq_objective(const float *W, const float *W_hat, int64_t d_in, int64_t d
     __half *dh = reinterpret_cast<__half *>(ws + L.half_off);
     double *partials = reinterpret_cast<double *>(ws + L.partials_off);
     const int64_t m = d_out / g;
-    // delta = W - W_hat as one fp16 matrix scaled by a power of two taken from max |delta| (two passes over W, W_hat)
+    // delta = W - W_hat as one fp16 matrix scaled by a power of two (gq_gram_dot.cuh); the blocks' maxima stand where the
+    // partial sums come later
     {
         const unsigned count4 = static_cast<unsigned>(d_in * d_out / 4);
-        const unsigned per_block = 256u * gq::DELTA_VEC_PER_THREAD;
-        const unsigned blocks = (count4 + per_block - 1) / per_block;
-        // Few blocks leave their maxima in the header; many meet in an atomic maximum, which has to be cleared first (3 - 6 us
-        // of a call).  Keeping to 960 blocks or 683 of 512 threads instead made the first pass of large layers slower by more
-        // than that (4096 x 11008: 836 us for the whole layer against 799).
-        const bool few = blocks <= gq::DELTA_BLOCK_MAXIMA;
-        if (!few) GQ_CUDA(cudaMemsetAsync(&header->absmax_bits, 0, sizeof header->absmax_bits, st));
+        const unsigned blocks = (count4 + gq::DELTA_BLOCK_VECS - 1) / gq::DELTA_BLOCK_VECS;
+        uint8_t *block_exp = ws + L.partials_off;
         {
             LaunchScope scope(GQ_KERNEL_SPLIT_DELTA, st);
-            launch(gq::delta_absmax_kernel, dim3(blocks), 256, 0, st, W, W_hat, count4, header);
+            launch(gq::delta_half_kernel, dim3(blocks), 256, 0, st, W, W_hat, count4, header, block_exp, dh);
         }
         GQ_CUDA(cudaGetLastError());
         {
             LaunchScope scope(GQ_KERNEL_SPLIT_DELTA, st);
-            launch(gq::delta_half_kernel, dim3(blocks), 256, 0, st, W, W_hat, count4, header, few ? blocks : 0u, dh);
+            const int grid = grid_for(count4, 256, di->sm_count, 4);
+            launch(gq::delta_redo_kernel, dim3(grid), 256, 0, st, W, W_hat, count4, header, block_exp, blocks, dh);
         }
         GQ_CUDA(cudaGetLastError());
     }

@@ -1,0 +1,83 @@
+"""The objective (Eq. 7) where the scale of its fp16 operand takes another branch, against the oracle.
+
+The tolerance is the objective's 1e-3: both factors of every product carry one fp16 rounding of at most 2^-12, so 2^-11 =
+4.9e-4 where all errors align.
+"""
+import numpy as np
+import pytest
+import torch
+
+from oracle import gq_oracle as orc
+from paper_2505_07004_b200 import api as libgq
+
+pytestmark = pytest.mark.gpu
+
+L_RTOL = 1e-3
+
+
+@pytest.fixture(scope="module")
+def dev():
+    assert torch.cuda.is_available()
+    torch.cuda.set_device(0)
+    return torch.device("cuda:0")
+
+
+def problem(d_in, d_out, g):
+    rng = np.random.default_rng(d_in + 3 * d_out + g)
+    X = rng.standard_normal((64, d_in)) * np.exp(rng.standard_normal(d_in))
+    H = np.stack([(X * rng.random((64, 1))).T @ X for _ in range(g)]).astype(np.float32)
+    H = (H + H.transpose(0, 2, 1)) / 2
+    W = (0.02 * rng.standard_normal((d_out, d_in))).astype(np.float32)
+    return H, W, rng
+
+
+def run(dev, W, W_hat, H):
+    """Two calls on a scratch full of ones: nothing in it is read before it is written, the order of every sum is fixed."""
+    ws = libgq.alloc_workspace(libgq.gq_objective_workspace_bytes(H.shape[1], W.shape[0], H.shape[0]), dev)
+    ws.fill_(0xFF)
+    args = [torch.from_numpy(a).to(dev) for a in (W, W_hat, H)]
+    first, second = (libgq.gq_objective(*args, ws).cpu().numpy() for _ in range(2))
+    libgq.gq_check()
+    assert np.array_equal(first, second, equal_nan=True)
+    return first
+
+
+def check(loss, ref):
+    assert np.all(np.abs(loss - ref) <= L_RTOL * np.abs(ref)), "relative error %s" % (np.abs(loss - ref) / np.abs(ref))
+
+
+# Factors around the room that the guess of the scale leaves (8 is inside whatever the sample, 16 is not), and far past it
+@pytest.mark.parametrize("factor", [8.0, 16.0, 1e3, 1e6])
+@pytest.mark.parametrize("at", [0, 5, -1])
+def test_scale_of_outliers(dev, factor, at):
+    d_in, d_out, g = 264, 1024, 2
+    H, W, rng = problem(d_in, d_out, g)
+    delta = (rng.integers(0, 2, W.shape) * 2 - 1) * 0.001 * (1 + 0.4 * rng.random(W.shape))
+    delta.reshape(-1)[at] = 0.001 * factor
+    W_hat = (W + delta).astype(np.float32)
+    check(run(dev, W, W_hat, H), orc.objective(W, W_hat, H, impl="numpy"))
+
+
+def test_scale_of_a_single_difference(dev):
+    """Every sample is zero; magnitudes from the smallest that the scale reaches to large ones."""
+    d_in, d_out, g = 128, 4096, 1
+    H, W, _ = problem(d_in, d_out, g)
+    W[:] = 0
+    for mag in (1e-25, 1e-6, 1.0, 1e15):
+        W_hat = W.copy()
+        W_hat[1234, 77] = mag
+        loss = run(dev, W, W_hat, H)
+        ref = float(np.float32(mag)) ** 2 * float(H[0, 77, 77])
+        assert abs(loss[0] - ref) <= L_RTOL * ref and loss[1] == loss[0]
+    assert not run(dev, W, W.copy(), H).any()
+
+
+def test_differences_that_are_not_finite(dev):
+    """An infinite or undefined difference gives a loss that is not finite, for its group only."""
+    d_in, d_out, g = 264, 1024, 2
+    H, W, rng = problem(d_in, d_out, g)
+    for bad in (np.inf, -np.inf, np.nan):
+        W_hat = (W + 0.003 * rng.standard_normal(W.shape)).astype(np.float32)
+        W_hat[700, 100] = bad
+        loss = run(dev, W, W_hat, H)
+        assert np.isfinite(loss[0]) and not np.isfinite(loss[1]) and not np.isfinite(loss[2])
