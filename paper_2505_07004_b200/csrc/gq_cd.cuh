@@ -29,14 +29,17 @@ namespace gq {
 constexpr int CD_BLOCK = 256;           // coordinates per block
 constexpr int CD_BAND = 32;             // coordinates whose running sums one chain thread holds
 constexpr int CD_BANDS = CD_BLOCK / CD_BAND;
-constexpr int CD_CH = 32;               // channels per CTA of the block kernel: one lane of the chain warp each
 constexpr int CD_THREADS = 256;
 constexpr int CD_MAX_LEVELS = 16;       // codebook entries per channel (m = 2^b, b <= 4)
 constexpr int CD_LEVEL_LD = CD_MAX_LEVELS + 1;   // padded per-channel rows of the level tables
 constexpr int CD_H_BUFS = 3;
-constexpr int CD_TILE_FLOATS = CD_BLOCK * CD_CH;         // one [256][32] tile: 32 KB
-constexpr int CD_PARTS = 6;             // pieces of the contraction range of a band's pulled sums: one per product warp
-constexpr int CD_SMEM_BYTES = ((3 + CD_H_BUFS) * CD_TILE_FLOATS + CD_PARTS * CD_BAND * CD_CH + CD_BLOCK + 3 * CD_CH * CD_LEVEL_LD) * 4 + 1024;
+constexpr int CD_H_FLOATS = CD_BLOCK * CD_BAND;          // one [256][32] tile of H: 32 KB
+constexpr int CD_PARTS = 6;             // pieces of the contraction range of a band's pulled sums
+// CH: channels per CTA of the block kernel, 32 or 16; a lane of the chain warp each
+constexpr int cd_smem_bytes(int CH)
+{
+    return (3 * CD_BLOCK * CH + CD_H_BUFS * CD_H_FLOATS + CD_PARTS * CD_BAND * CH + CD_BLOCK + 3 * CH * CD_LEVEL_LD) * 4 + 1024;
+}
 
 __device__ __forceinline__ void split_bf16(float v, __nv_bfloat16 &hi, __nv_bfloat16 &lo)
 {
@@ -150,7 +153,7 @@ struct CdBlockParams {
     int d_in, d_out, g, mk, m;
     int s0;                  // first coordinate of the block
     int rows;                // coordinates in the block (<= CD_BLOCK)
-    int slices;              // ceil(mk / CD_CH): CTAs per group
+    int slices;              // ceil(mk / CH): CTAs per group
     bool last_cycle;         // write the codes
     uint32_t *status;
     unsigned long long wait_budget_ns;
@@ -185,12 +188,12 @@ __device__ __forceinline__ float nearest_level(float target, const float (&lev)[
 struct ChainOperands {
     float4 h[CD_BAND / 4];
     float w, rd;
-    template <int I>
+    template <int I, int CH>
     __device__ __forceinline__ void load(const float *hd, const float *wb, const float *rb)
     {
 #pragma unroll
         for (int q = (I + 1) / 4; q < CD_BAND / 4; ++q) h[q] = *reinterpret_cast<const float4 *>(hd + I * CD_BAND + 4 * q);
-        w = wb[I * CD_CH];
+        w = wb[I * CH];
         rd = rb[I];
     }
 };
@@ -200,13 +203,13 @@ struct ChainOperands {
 // band: those sums are formed from whatever follows in shared memory and never used.  Operands are read two steps ahead (the
 // product warps keep the shared-memory pipe busy, so a read takes longer than a step).  Written as a recursion because the
 // compiler does not unroll the loop, and the sums have to stay in registers.
-template <int LEV, int RUN, int I>
+template <int LEV, int CH, int RUN, int I>
 __device__ __forceinline__ void chain_steps(const ChainOperands &cur, const ChainOperands &nxt, const float *hd, const float *rb,
                                             float *wb, float *eb, float (&Bu)[CD_BAND], const float (&lev)[LEV],
                                             const float (&thr)[LEV])
 {
     ChainOperands after;
-    if constexpr (I + 2 < RUN) after.load<I + 2>(hd, wb, rb);
+    if constexpr (I + 2 < RUN) after.load<I + 2, CH>(hd, wb, rb);
     const float val = nearest_level<LEV>(cur.w - cur.rd * Bu[I], lev, thr);
     const float e_new = val - cur.w;
 #pragma unroll
@@ -214,9 +217,9 @@ __device__ __forceinline__ void chain_steps(const ChainOperands &cur, const Chai
         const float4 hq = cur.h[r >> 2];
         Bu[r] = fmaf((r & 3) == 0 ? hq.x : (r & 3) == 1 ? hq.y : (r & 3) == 2 ? hq.z : hq.w, e_new, Bu[r]);
     }
-    eb[I * CD_CH] = e_new;
-    wb[I * CD_CH] = val;                                 // W_i is not needed any more: What of the block takes its place
-    if constexpr (I + 1 < RUN) chain_steps<LEV, RUN, I + 1>(nxt, after, hd, rb, wb, eb, Bu, lev, thr);
+    eb[I * CH] = e_new;
+    wb[I * CH] = val;                                 // W_i is not needed any more: What of the block takes its place
+    if constexpr (I + 1 < RUN) chain_steps<LEV, CH, RUN, I + 1>(nxt, after, hd, rb, wb, eb, Bu, lev, thr);
 }
 
 // Where four rows (quad rq of a band) of channel ch stand in a part of the pulled sums, in floats: the swizzle keeps both
@@ -227,7 +230,7 @@ __device__ __forceinline__ int sums_at(int ch, int rq)
     return ch * CD_BAND + ((rq ^ (ch >> 2) ^ ch) & 7) * 4;
 }
 
-// One block of coordinates for CD_CH channels of one group.
+// One block of coordinates for CH channels of one group.
 //
 // The running sums  Bu[r] = sum_{c != r} H[r][c] E_c  (current E: this cycle's values for c < r, last cycle's for c > r)
 // are needed one coordinate after the other, each after a rounding decision on the one before it: 256 dependent steps.
@@ -249,7 +252,7 @@ __device__ __forceinline__ int sums_at(int ch, int rq)
 // Measured for one block of 4096 channels, 16 levels: 33.7 us (8 levels, 1408 channels: 29.8; 34.9 and 31.2 with the excluded
 // coordinates multiplied by zero instead of left out); with eight threads per channel that did all updates themselves and two
 // votes and a table read per step it was 81 us (78).
-template <int LEV>
+template <int LEV, int CH>
 __global__ void __launch_bounds__(CD_THREADS, 1)
 cd_block_kernel(const __grid_constant__ CUtensorMap mapH, const __grid_constant__ CUtensorMap mapW,
                 const __grid_constant__ CUtensorMap mapE, const __grid_constant__ CUtensorMap mapP, const CdBlockParams p)
@@ -260,25 +263,25 @@ cd_block_kernel(const __grid_constant__ CUtensorMap mapH, const __grid_constant_
     __shared__ volatile uint32_t abort_flag;
     // aligned by an offset: rounding the pointer itself would make every access below a generic one
     float *Ws = reinterpret_cast<float *>(smem_raw + ((0u - smem_u32(smem_raw)) & 1023u));
-    float *Es = Ws + CD_TILE_FLOATS;                     // [256][32] E of the block, updated in place
-    float *Ps = Es + CD_TILE_FLOATS;                     // [256][32] P
-    float *Hs = Ps + CD_TILE_FLOATS;                     // [CD_H_BUFS][256][32] H[c][rows of a band]
-    float *Ss = Hs + CD_H_BUFS * CD_TILE_FLOATS;         // [CD_PARTS][32 ch][32 rows] pulled sums of a band (sums_at)
-    float *rds = Ss + CD_PARTS * CD_BAND * CD_CH;        // [256]
-    float *srt = rds + CD_BLOCK;                         // [32][CD_LEVEL_LD] sorted levels
-    float *thr_s = srt + CD_CH * CD_LEVEL_LD;            // [32][CD_LEVEL_LD] thresholds between neighbours
-    int *sidx = reinterpret_cast<int *>(thr_s + CD_CH * CD_LEVEL_LD);   // [32][CD_LEVEL_LD] given index by sorted position
+    float *Es = Ws + CD_BLOCK * CH;                      // [256][CH] E of the block, updated in place
+    float *Ps = Es + CD_BLOCK * CH;                      // [256][CH] P
+    float *Hs = Ps + CD_BLOCK * CH;                      // [CD_H_BUFS][256][32] H[c][rows of a band]
+    float *Ss = Hs + CD_H_BUFS * CD_H_FLOATS;            // [CD_PARTS][CH][32 rows] pulled sums of a band (sums_at)
+    float *rds = Ss + CD_PARTS * CD_BAND * CH;           // [256]
+    float *srt = rds + CD_BLOCK;                         // [CH][CD_LEVEL_LD] sorted levels
+    float *thr_s = srt + CH * CD_LEVEL_LD;               // [CH][CD_LEVEL_LD] thresholds between neighbours
+    int *sidx = reinterpret_cast<int *>(thr_s + CH * CD_LEVEL_LD);      // [CH][CD_LEVEL_LD] given index by sorted position
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int k = blockIdx.x / p.slices;
-    const int ch0 = k * p.mk + (blockIdx.x % p.slices) * CD_CH;          // first channel of this CTA
-    const int ch_n = min(CD_CH, (k + 1) * p.mk - ch0);                   // valid channels (a multiple of 8)
+    const int ch0 = k * p.mk + (blockIdx.x % p.slices) * CH;             // first channel of this CTA
+    const int ch_n = min(CH, (k + 1) * p.mk - ch0);                   // valid channels (a multiple of 8)
     const WaitCtx wc{&abort_flag, p.status, p.wait_budget_ns};
 
     auto load_band = [&](int t) {                        // H[block coordinates][band t] (zero outside the matrix)
         const uint32_t bar = smem_u32(&bar_h[t % CD_H_BUFS]);
-        mbar_arrive_expect_tx(bar, CD_TILE_FLOATS * 4);
-        tma_load_3d(smem_u32(Hs + (t % CD_H_BUFS) * CD_TILE_FLOATS), &mapH, bar, p.s0 + t * CD_BAND, p.s0, k);
+        mbar_arrive_expect_tx(bar, CD_H_FLOATS * 4);
+        tma_load_3d(smem_u32(Hs + (t % CD_H_BUFS) * CD_H_FLOATS), &mapH, bar, p.s0 + t * CD_BAND, p.s0, k);
     };
     // A wait that ran out is recorded; the warps go on (with wrong values) so that every barrier completes.
     auto wait_band = [&](int t) {
@@ -294,7 +297,7 @@ cd_block_kernel(const __grid_constant__ CUtensorMap mapH, const __grid_constant_
         griddep_wait();
         load_band(0);
         const uint32_t bar = smem_u32(&bar_tiles);
-        mbar_arrive_expect_tx(bar, 3 * CD_TILE_FLOATS * 4);
+        mbar_arrive_expect_tx(bar, 3 * CD_BLOCK * CH * 4);
         tma_load_3d(smem_u32(Es), &mapE, bar, ch0, p.s0, 0);
         tma_load_3d(smem_u32(Ps), &mapP, bar, ch0, 0, 0);
         tma_load_3d(smem_u32(Ws), &mapW, bar, ch0, p.s0, 0);
@@ -307,7 +310,7 @@ cd_block_kernel(const __grid_constant__ CUtensorMap mapH, const __grid_constant_
     // Sorted means a total order, so that every position is written: numbers ascending, then NaN, equal ones by index.  A
     // threshold beside a NaN is a NaN and never exceeded: no target is rounded to it while the channel has a number.  The
     // positions past the channel's levels hold NaN as well, with the highest indices.
-    {
+    if (tid < 8 * CH) {
         const int cidx = tid >> 3, l = tid & 7;
         const bool chan = cidx < ch_n;
         const float v0 = (l < p.m && chan) ? p.codebook[static_cast<size_t>(ch0 + cidx) * p.m + l] : CUDART_NAN_F;
@@ -342,35 +345,38 @@ cd_block_kernel(const __grid_constant__ CUtensorMap mapH, const __grid_constant_
     (void)bounded_wait(smem_u32(&bar_tiles), 0u, wc, 20u, blockIdx.x);
 
     constexpr int BAR_SUMS = 1, BAR_BAND = 2;
-    constexpr int SUMS_THREADS = 7 * 32, BAND_THREADS = CD_THREADS;
+    constexpr int SHARE = 32 / CH;                       // parts a product warp forms, CH lanes each
+    constexpr int PRODUCTS = CD_PARTS / SHARE;           // product warps: 1 .. 3 and, with CH = 32, 5 .. 7
+    constexpr int SUMS_THREADS = (1 + PRODUCTS) * 32, BAND_THREADS = SUMS_THREADS + 32;
     if (warp == 0) {
         // ------------------------------------------------------------------ chain: the coordinates in order
         // With 16 levels the 32 unrolled steps of a band (30 KB of code) and the products' loops do not fit the instruction
         // cache together: 39.6 us a block against 34.8 with 16 steps twice.  With 8 they do: 31.4 against 33.2.
         constexpr int RUN = LEV > 8 ? CD_BAND / 2 : CD_BAND;
+        const int ch = lane % CH;                        // further lanes do the same as the first CH
         float lev[LEV], thr[LEV];
 #pragma unroll
         for (int q = 0; q < LEV; ++q) {
-            lev[q] = srt[lane * CD_LEVEL_LD + q];
-            thr[q] = thr_s[lane * CD_LEVEL_LD + q];
+            lev[q] = srt[ch * CD_LEVEL_LD + q];
+            thr[q] = thr_s[ch * CD_LEVEL_LD + q];
         }
 #pragma unroll 1
         for (int t = 0; t < CD_BANDS; ++t) {
             wait_band(t);
-            const float *hd = Hs + (t % CD_H_BUFS) * CD_TILE_FLOATS + t * CD_BAND * CD_BAND;      // H[band][band]
-            float *wb = Ws + t * CD_BAND * CD_CH + lane, *eb = Es + t * CD_BAND * CD_CH + lane;
+            const float *hd = Hs + (t % CD_H_BUFS) * CD_H_FLOATS + t * CD_BAND * CD_BAND;      // H[band][band]
+            float *wb = Ws + t * CD_BAND * CH + ch, *eb = Es + t * CD_BAND * CH + ch;
             const float *rb = rds + t * CD_BAND;
             ChainOperands first, second;                 // not written by the products: read while the sums are awaited
-            first.load<0>(hd, wb, rb);
-            second.load<1>(hd, wb, rb);
+            first.load<0, CH>(hd, wb, rb);
+            second.load<1, CH>(hd, wb, rb);
             bar_sync_named(BAR_SUMS, SUMS_THREADS);
             float Bu[CD_BAND];
 #pragma unroll
             for (int q = 0; q < CD_BAND / 4; ++q) {
-                const float *sp = Ss + sums_at(lane, q);
+                const float *sp = Ss + sums_at(ch, q);
                 float4 v[CD_PARTS];
 #pragma unroll
-                for (int n = 0; n < CD_PARTS; ++n) v[n] = *reinterpret_cast<const float4 *>(sp + n * CD_BAND * CD_CH);
+                for (int n = 0; n < CD_PARTS; ++n) v[n] = *reinterpret_cast<const float4 *>(sp + n * CD_BAND * CH);
                 Bu[4 * q + 0] = ((v[0].x + v[1].x) + (v[2].x + v[3].x)) + (v[4].x + v[5].x);
                 Bu[4 * q + 1] = ((v[0].y + v[1].y) + (v[2].y + v[3].y)) + (v[4].y + v[5].y);
                 Bu[4 * q + 2] = ((v[0].z + v[1].z) + (v[2].z + v[3].z)) + (v[4].z + v[5].z);
@@ -381,14 +387,14 @@ cd_block_kernel(const __grid_constant__ CUtensorMap mapH, const __grid_constant_
                 if (run > 0) {
                     hd += RUN * (CD_BAND + 1);         // the same number of rows and columns on
                     rb += RUN;
-                    wb += RUN * CD_CH;
-                    eb += RUN * CD_CH;
-                    first.load<0>(hd, wb, rb);
-                    second.load<1>(hd, wb, rb);
+                    wb += RUN * CH;
+                    eb += RUN * CH;
+                    first.load<0, CH>(hd, wb, rb);
+                    second.load<1, CH>(hd, wb, rb);
 #pragma unroll
                     for (int r = 0; r + RUN < CD_BAND; ++r) Bu[r] = Bu[r + RUN];
                 }
-                chain_steps<LEV, RUN, 0>(first, second, hd, rb, wb, eb, Bu, lev, thr);
+                chain_steps<LEV, CH, RUN, 0>(first, second, hd, rb, wb, eb, Bu, lev, thr);
             }
             if (t + 1 < CD_BANDS) bar_arrive_named(BAR_BAND, BAND_THREADS);
         }
@@ -398,19 +404,19 @@ cd_block_kernel(const __grid_constant__ CUtensorMap mapH, const __grid_constant_
             bar_sync_named(BAR_BAND, BAND_THREADS);      // band t's buffer is free
             if (lane == 0 && t + CD_H_BUFS < CD_BANDS) load_band(t + CD_H_BUFS);
         }
-    } else {
+    } else if ((warp < 4 ? warp - 1 : warp - 2) < PRODUCTS) {
         // ------------------------------------------------------------------ products: sums of band t
-        const int part = warp < 4 ? warp - 1 : warp - 2;                       // 0..5
-        const int r0 = (lane >> 3) * 8, c0 = (lane & 7) * 4;                   // 8 rows x 4 channels
+        const int part = (warp < 4 ? warp - 1 : warp - 2) * SHARE + lane / CH;                 // 0..5
+        const int r0 = (lane % CH) / (CH / 4) * 8, c0 = (lane % (CH / 4)) * 4;                 // 8 rows x 4 channels
 #pragma unroll 1
         for (int t = 0; t < CD_BANDS; ++t) {
             wait_band(t);
-            const float *hb = Hs + (t % CD_H_BUFS) * CD_TILE_FLOATS + r0;
+            const float *hb = Hs + (t % CD_H_BUFS) * CD_H_FLOATS + r0;
             const float *eb = Es + c0;
             float acc[8][4];
 #pragma unroll
             for (int a = 0; a < 8; ++a) {
-                const float4 v = part == 0 ? *reinterpret_cast<const float4 *>(Ps + (t * CD_BAND + r0 + a) * CD_CH + c0)
+                const float4 v = part == 0 ? *reinterpret_cast<const float4 *>(Ps + (t * CD_BAND + r0 + a) * CH + c0)
                                            : make_float4(0.f, 0.f, 0.f, 0.f);
                 acc[a][0] = v.x; acc[a][1] = v.y; acc[a][2] = v.z; acc[a][3] = v.w;
             }
@@ -426,7 +432,7 @@ cd_block_kernel(const __grid_constant__ CUtensorMap mapH, const __grid_constant_
                 h[0] = lo.x; h[1] = lo.y; h[2] = lo.z; h[3] = lo.w;
                 h[4] = hi.x; h[5] = hi.y; h[6] = hi.z; h[7] = hi.w;
             };
-            auto load_e = [&](int c) { return *reinterpret_cast<const float4 *>(eb + c * CD_CH); };
+            auto load_e = [&](int c) { return *reinterpret_cast<const float4 *>(eb + c * CH); };
             // one band for each warp, neither the one the chain is working on (t - 1) nor this one
             {
                 const int first = (t == 0 ? part + 1 : part >= t - 1 ? part + 2 : part) * CD_BAND;
@@ -464,7 +470,7 @@ cd_block_kernel(const __grid_constant__ CUtensorMap mapH, const __grid_constant_
             for (int b = 0; b < 4; ++b)
 #pragma unroll
                 for (int q = 0; q < 2; ++q)
-                    *reinterpret_cast<float4 *>(Ss + part * CD_BAND * CD_CH + sums_at(c0 + b, r0 / 4 + q)) =
+                    *reinterpret_cast<float4 *>(Ss + part * CD_BAND * CH + sums_at(c0 + b, r0 / 4 + q)) =
                         make_float4(acc[4 * q][b], acc[4 * q + 1][b], acc[4 * q + 2][b], acc[4 * q + 3][b]);
             bar_arrive_named(BAR_SUMS, SUMS_THREADS);
         }
@@ -472,13 +478,13 @@ cd_block_kernel(const __grid_constant__ CUtensorMap mapH, const __grid_constant_
     __syncthreads();
 
     // ---- tiles out, four channels per thread; P is left zero for the next block's panel product
-    for (int idx = tid; idx < CD_BLOCK * CD_CH / 4; idx += CD_THREADS) {
-        const int r = idx >> 3, c = (idx & 7) * 4;
+    for (int idx = tid; idx < CD_BLOCK * CH / 4; idx += CD_THREADS) {
+        const int r = idx / (CH / 4), c = idx % (CH / 4) * 4;
         if (c >= ch_n) continue;
         *reinterpret_cast<float4 *>(p.P + static_cast<size_t>(r) * p.d_out + ch0 + c) = make_float4(0.f, 0.f, 0.f, 0.f);
         if (r >= p.rows) continue;
         const size_t o = static_cast<size_t>(p.s0 + r) * p.d_out + ch0 + c;
-        const float4 e4 = *reinterpret_cast<const float4 *>(Es + r * CD_CH + c);
+        const float4 e4 = *reinterpret_cast<const float4 *>(Es + r * CH + c);
         const float e[4] = {e4.x, e4.y, e4.z, e4.w};
         __align__(8) __nv_bfloat16 hi[4], lo[4];
 #pragma unroll
@@ -487,7 +493,7 @@ cd_block_kernel(const __grid_constant__ CUtensorMap mapH, const __grid_constant_
         *reinterpret_cast<uint2 *>(p.Ehi + o) = *reinterpret_cast<uint2 *>(hi);
         *reinterpret_cast<uint2 *>(p.Elo + o) = *reinterpret_cast<uint2 *>(lo);
         if (!p.last_cycle) continue;                     // the codes of earlier cycles are never read
-        const float4 v4 = *reinterpret_cast<const float4 *>(Ws + r * CD_CH + c);
+        const float4 v4 = *reinterpret_cast<const float4 *>(Ws + r * CH + c);
         const float v[4] = {v4.x, v4.y, v4.z, v4.w};
         uint32_t codes = 0;
 #pragma unroll

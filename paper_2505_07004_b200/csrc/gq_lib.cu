@@ -163,9 +163,12 @@ int32_t device_info(DeviceInfo **out)
         GQ_CUDA(cudaFuncSetAttribute(gq::codebook_gemm_kernel<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, gq::CG_SMEM_BYTES));
         GQ_CUDA(cudaFuncSetAttribute(gq::codebook_gemm_kernel<16>, cudaFuncAttributeMaxDynamicSharedMemorySize, gq::CG_SMEM_BYTES));
         GQ_CUDA(cudaFuncSetAttribute(gq::gram_dot_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, gq::GD_SMEM_BYTES));
-        GQ_CUDA(cudaFuncSetAttribute(gq::cd_block_kernel<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, gq::CD_SMEM_BYTES));
-        GQ_CUDA(cudaFuncSetAttribute(gq::cd_block_kernel<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, gq::CD_SMEM_BYTES));
-        GQ_CUDA(cudaFuncSetAttribute(gq::cd_block_kernel<16>, cudaFuncAttributeMaxDynamicSharedMemorySize, gq::CD_SMEM_BYTES));
+        GQ_CUDA(cudaFuncSetAttribute(gq::cd_block_kernel<4, 32>, cudaFuncAttributeMaxDynamicSharedMemorySize, gq::cd_smem_bytes(32)));
+        GQ_CUDA(cudaFuncSetAttribute(gq::cd_block_kernel<4, 16>, cudaFuncAttributeMaxDynamicSharedMemorySize, gq::cd_smem_bytes(16)));
+        GQ_CUDA(cudaFuncSetAttribute(gq::cd_block_kernel<8, 32>, cudaFuncAttributeMaxDynamicSharedMemorySize, gq::cd_smem_bytes(32)));
+        GQ_CUDA(cudaFuncSetAttribute(gq::cd_block_kernel<8, 16>, cudaFuncAttributeMaxDynamicSharedMemorySize, gq::cd_smem_bytes(16)));
+        GQ_CUDA(cudaFuncSetAttribute(gq::cd_block_kernel<16, 32>, cudaFuncAttributeMaxDynamicSharedMemorySize, gq::cd_smem_bytes(32)));
+        GQ_CUDA(cudaFuncSetAttribute(gq::cd_block_kernel<16, 16>, cudaFuncAttributeMaxDynamicSharedMemorySize, gq::cd_smem_bytes(16)));
         GQ_CUDA(cudaFuncSetAttribute(gq::hessian_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                      gq::HS_SMEM_BYTES));
         {
@@ -238,13 +241,13 @@ int32_t make_map(CUtensorMap *map, const void *base, int64_t features, int64_t r
     return GQ_OK;
 }
 
-// fp32 tensor [groups][rows][cols] as a TMA map with boxes of 32 columns x `box_rows` rows.
+// fp32 tensor [groups][rows][cols] as a TMA map with boxes of `box_cols` columns x `box_rows` rows.
 int32_t make_map_f32(CUtensorMap *map, const float *base, int64_t cols, int64_t rows, int64_t groups, int box_rows,
-                     CUtensorMapSwizzle swizzle)
+                     CUtensorMapSwizzle swizzle, int box_cols = 32)
 {
     cuuint64_t dims[3] = {static_cast<cuuint64_t>(cols), static_cast<cuuint64_t>(rows), static_cast<cuuint64_t>(groups)};
     cuuint64_t strides[2] = {static_cast<cuuint64_t>(cols) * 4, static_cast<cuuint64_t>(cols) * static_cast<cuuint64_t>(rows) * 4};
-    cuuint32_t box[3] = {32, static_cast<cuuint32_t>(box_rows), 1};
+    cuuint32_t box[3] = {static_cast<cuuint32_t>(box_cols), static_cast<cuuint32_t>(box_rows), 1};
     cuuint32_t estr[3] = {1, 1, 1};
     CUresult r = g_encode(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, const_cast<float *>(base), dims, strides, box, estr,
                           CU_TENSOR_MAP_INTERLEAVE_NONE, swizzle, CU_TENSOR_MAP_L2_PROMOTION_NONE,
@@ -1025,16 +1028,19 @@ static int32_t cd_cycles_impl(const float *W, float *W_hat, uint8_t *Q, const fl
     if (int32_t rc = make_map(&mapHlo, Hlo, d_in, d_in, g, d_in, d_in * d_in)) return rc;
     if (int32_t rc = make_map(&mapEhi, Ehi, d_out, d_in, 1, d_out, d_in * d_out)) return rc;
     if (int32_t rc = make_map(&mapElo, Elo, d_out, d_in, 1, d_out, d_in * d_out)) return rc;
+    // Channels per CTA of the block kernel: 16 where that leaves no SM with two CTAs.  A step of the chain takes as long for 16
+    // channels as for 32, but the sums around it take half.
+    const int ch = g * ((mk + 15) / 16) <= di->sm_count ? 16 : 32;
     CUtensorMap mapHb, mapWb, mapEb, mapPb, mapPr;       // fp32 tiles of the block kernel; P as the panel product adds to it
     if (int32_t rc = make_map_f32(&mapPr, P, d_out, gq::CD_BLOCK, 1, 32, CU_TENSOR_MAP_SWIZZLE_128B)) return rc;
     if (int32_t rc = make_map_f32(&mapHb, H, d_in, d_in, g, gq::CD_BLOCK, CU_TENSOR_MAP_SWIZZLE_NONE)) return rc;
-    if (int32_t rc = make_map_f32(&mapWb, Wt, d_out, d_in, 1, gq::CD_BLOCK, CU_TENSOR_MAP_SWIZZLE_NONE)) return rc;
-    if (int32_t rc = make_map_f32(&mapEb, Et, d_out, d_in, 1, gq::CD_BLOCK, CU_TENSOR_MAP_SWIZZLE_NONE)) return rc;
-    if (int32_t rc = make_map_f32(&mapPb, P, d_out, gq::CD_BLOCK, 1, gq::CD_BLOCK, CU_TENSOR_MAP_SWIZZLE_NONE)) return rc;
+    if (int32_t rc = make_map_f32(&mapWb, Wt, d_out, d_in, 1, gq::CD_BLOCK, CU_TENSOR_MAP_SWIZZLE_NONE, ch)) return rc;
+    if (int32_t rc = make_map_f32(&mapEb, Et, d_out, d_in, 1, gq::CD_BLOCK, CU_TENSOR_MAP_SWIZZLE_NONE, ch)) return rc;
+    if (int32_t rc = make_map_f32(&mapPb, P, d_out, gq::CD_BLOCK, 1, gq::CD_BLOCK, CU_TENSOR_MAP_SWIZZLE_NONE, ch)) return rc;
     GQ_CUDA(cudaMemsetAsync(P, 0, static_cast<size_t>(gq::CD_BLOCK) * d_out * sizeof(float), st));   // the block kernel leaves it zero
     const int kblocks = static_cast<int>((d_in + gq::TILE_K - 1) / gq::TILE_K);
     const int ch_tiles = static_cast<int>((mk + gq::TILE_N - 1) / gq::TILE_N);
-    const int slices = static_cast<int>((mk + gq::CD_CH - 1) / gq::CD_CH);
+    const int slices = static_cast<int>((mk + ch - 1) / ch);
 
     for (int32_t cyc = 0; cyc < cycles; ++cyc) {
         for (int64_t s0 = 0; s0 < d_in; s0 += gq::CD_BLOCK) {
@@ -1080,8 +1086,9 @@ static int32_t cd_cycles_impl(const float *W, float *W_hat, uint8_t *Q, const fl
             {
                 LaunchScope scope(GQ_KERNEL_CD_BLOCK, st);
                 // fewer levels, fewer compares and selects per coordinate
-                const auto kernel = m <= 4 ? gq::cd_block_kernel<4> : m <= 8 ? gq::cd_block_kernel<8> : gq::cd_block_kernel<16>;
-                launch(kernel, dim3(g * slices), gq::CD_THREADS, gq::CD_SMEM_BYTES, st, mapHb, mapWb, mapEb, mapPb, bp);
+                const auto narrow = m <= 4 ? gq::cd_block_kernel<4, 16> : m <= 8 ? gq::cd_block_kernel<8, 16> : gq::cd_block_kernel<16, 16>;
+                const auto wide = m <= 4 ? gq::cd_block_kernel<4, 32> : m <= 8 ? gq::cd_block_kernel<8, 32> : gq::cd_block_kernel<16, 32>;
+                launch(ch == 16 ? narrow : wide, dim3(g * slices), gq::CD_THREADS, gq::cd_smem_bytes(ch), st, mapHb, mapWb, mapEb, mapPb, bp);
             }
             GQ_CUDA(cudaGetLastError());
         }
