@@ -441,17 +441,17 @@ hessian_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_constant__
         WorkItem w;
         for (int it = 0; ok && work_item(p.sched, pair, it, w); ++it) {
             const UnitDesc u = decode_unit(p, w.unit);
+            // After the pair's last item nobody uses the operand ring any more (the accumulators being complete means that
+            // the MMAs have read it): six of a warp's eight blocks are staged there, so that a block does not wait for the
+            // copy engine to have read the one before it (1300 clocks a block, 10 000 an item: the end of every launch).
+            WorkItem w_next;
+            const bool last = !work_item(p.sched, pair, it + 1, w_next);
             if (lane == 0) ok = bounded_wait(smem_u32(&bar_acc_full), acc_ph, wc, 4u, w.unit);
             ok = __shfl_sync(0xffffffffu, ok, 0);
             if (!ok) break;
             (void)mbar_try_wait(smem_u32(&bar_acc_full), acc_ph);     // every lane observes the completed phase
             tc_fence_after_sync();
             const int row0 = u.ti * TILE_M + static_cast<int>(rank) * CTA_ROWS + q * 32;
-            // After the pair's last item nobody uses the operand ring any more (the accumulators being complete means that
-            // the MMAs have read it): six of a warp's eight blocks are staged there, so that a block does not wait for the
-            // copy engine to have read the one before it (1300 clocks a block, 10 000 an item: the end of every launch).
-            WorkItem w_next;
-            const bool last = !work_item(p.sched, pair, it + 1, w_next);
             int staged = 0;
             for (int kk = 0; kk < HS_GROUPS; ++kk) {
 #pragma unroll 1

@@ -42,6 +42,7 @@ struct Schedule {
     int full_waves;          // rounds of whole units dealt round-robin
     int tail_units;          // units after the full rounds (0 <= tail_units < pairs), cut into pieces
     int tail_pairs;          // pairs that take a piece of the tail
+    unsigned tail_share, tail_rest;      // tail_units * ksteps = tail_share * tail_pairs + tail_rest
 };
 
 // Host side: fills the distribution fields.  `balanced` cuts the last, incomplete round into pieces.
@@ -54,6 +55,7 @@ inline Schedule plan_schedule(int units, int ksteps, int pairs, bool balanced)
     p.full_waves = (units + pairs - 1) / pairs;
     p.tail_units = 0;
     p.tail_pairs = 0;
+    p.tail_share = p.tail_rest = 0;
     if (balanced && units % pairs != 0) {
         p.full_waves = units / pairs;
         p.tail_units = units - p.full_waves * pairs;
@@ -65,6 +67,8 @@ inline Schedule plan_schedule(int units, int ksteps, int pairs, bool balanced)
         if (tp < p.tail_units) tp = p.tail_units;
         if (tp > pairs) tp = pairs;
         p.tail_pairs = static_cast<int>(tp);
+        p.tail_share = static_cast<unsigned>(total / tp);
+        p.tail_rest = static_cast<unsigned>(total % tp);
     }
     return p;
 }
@@ -125,7 +129,9 @@ struct WorkItem {
 };
 
 // The `it`-th work item of pair `pair`; false when the pair has no more work.  Every role of both CTAs of
-// a pair walks the same list.
+// a pair walks the same list, several of them before they can start: a pair's share of the tail, [total pair / tail_pairs,
+// total (pair + 1) / tail_pairs) of total = tail_units * ksteps < 2^32, is formed without 64-bit divisions (with three of them
+// the first k-step came 1.5 us later, and so did the first read-out).
 __device__ __forceinline__ bool work_item(const Schedule &p, int pair, int it, WorkItem &w)
 {
     if (it < p.full_waves) {
@@ -135,17 +141,16 @@ __device__ __forceinline__ bool work_item(const Schedule &p, int pair, int it, W
         return w.unit < p.units;
     }
     if (pair >= p.tail_pairs) return false;
-    const long long total = static_cast<long long>(p.tail_units) * p.ksteps;
-    const long long begin = total * pair / p.tail_pairs;
-    const long long end = total * (pair + 1) / p.tail_pairs;
-    long long cur = begin;
-    for (int q = p.full_waves; q < it && cur < end; ++q) cur = (cur / p.ksteps + 1) * p.ksteps;
+    const unsigned tp = static_cast<unsigned>(p.tail_pairs), pr = static_cast<unsigned>(pair), ksteps = static_cast<unsigned>(p.ksteps);
+    unsigned cur = p.tail_share * pr + p.tail_rest * pr / tp;
+    const unsigned end = p.tail_share * (pr + 1) + p.tail_rest * (pr + 1) / tp;
+    unsigned tu = cur / ksteps;
+    for (int q = p.full_waves; q < it && cur < end; ++q) cur = ++tu * ksteps;
     if (cur >= end) return false;
-    const int tu = static_cast<int>(cur / p.ksteps);
-    w.unit = p.full_waves * p.pairs + tu;
-    w.ks0 = static_cast<int>(cur - static_cast<long long>(tu) * p.ksteps);
-    const long long left = end - cur;
-    w.ks1 = (left < p.ksteps - w.ks0) ? w.ks0 + static_cast<int>(left) : p.ksteps;
+    w.unit = p.full_waves * p.pairs + static_cast<int>(tu);
+    w.ks0 = static_cast<int>(cur - tu * ksteps);
+    const unsigned left = end - cur;
+    w.ks1 = (left < ksteps - static_cast<unsigned>(w.ks0)) ? w.ks0 + static_cast<int>(left) : p.ksteps;
     return true;
 }
 
