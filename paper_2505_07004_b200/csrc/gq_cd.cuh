@@ -351,8 +351,10 @@ cd_block_kernel(const __grid_constant__ CUtensorMap mapH, const __grid_constant_
     if (warp == 0) {
         // ------------------------------------------------------------------ chain: the coordinates in order
         // With 16 levels the 32 unrolled steps of a band (30 KB of code) and the products' loops do not fit the instruction
-        // cache together: 39.6 us a block against 34.8 with 16 steps twice.  With 8 they do: 31.4 against 33.2.
-        constexpr int RUN = LEV > 8 ? CD_BAND / 2 : CD_BAND;
+        // cache together: 39.6 us a block against 34.8 with 16 steps twice.  With 8 they do (31.4 against 33.2), but where a
+        // block is short the first band, which fetches all code, counts for more: with 16 channels 1181 against 1191 us for the
+        // descent named below.  With 4 levels 32 steps stay the better (2320 x 2032, two cycles: 740 against 747).
+        constexpr int RUN = LEV > 8 || (LEV == 8 && CH == 16) ? CD_BAND / 2 : CD_BAND;
         const int ch = lane % CH;                        // further lanes do the same as the first CH
         float lev[LEV], thr[LEV];
 #pragma unroll
@@ -433,10 +435,13 @@ cd_block_kernel(const __grid_constant__ CUtensorMap mapH, const __grid_constant_
                 h[4] = hi.x; h[5] = hi.y; h[6] = hi.z; h[7] = hi.w;
             };
             auto load_e = [&](int c) { return *reinterpret_cast<const float4 *>(eb + c * CH); };
-            // one band for each warp, neither the one the chain is working on (t - 1) nor this one
+            // (coordinates at a time: four with 16 channels, 1250 -> 1191 us for 2056 x 1408, 8 levels, four cycles; two 1238; with 32
+            // channels eight, 1275 against 1280 for 1400 x 2480, 16 levels, two rounds)
+            constexpr int UNROLL = CH == 16 ? 4 : 8;
+            // one band for each part, neither the one the chain is working on (t - 1) nor this one
             {
                 const int first = (t == 0 ? part + 1 : part >= t - 1 ? part + 2 : part) * CD_BAND;
-#pragma unroll 8
+#pragma unroll UNROLL
                 for (int c = first; c < first + CD_BAND; ++c) {
                     float h[8];
                     load_h(c, h);

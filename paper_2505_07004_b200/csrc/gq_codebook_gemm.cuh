@@ -198,8 +198,10 @@ codebook_gemm_kernel(const __grid_constant__ CUtensorMap mapH0, const __grid_con
             if (++s == CG_STAGES) { s = 0; ph ^= 1u; }
         }
         if (!ok) spin_ns(1000000ull);
-    } else if (warp == 1 && lane == 0 && rank == 0) {
+    } else if (warp == 3 && lane == 0 && rank == 0) {
         // ------------------------------------------------------------------ MMA issuer (first CTA)
+        // Warp 3: what this thread does between two k-steps the tensor core waits for, and warps 4 w + 1 on its scheduler include
+        // two of the one-hot warps, warps 4 w + 3 one.  4096 x 4096, 16 levels, one round: 9.83 -> 9.48 ms with warp 1 -> 3.
         constexpr uint32_t idesc = umma_idesc_bf16_mn(TILE_M, TILE_N);
         int s = 0;
         uint32_t ph = 0;
