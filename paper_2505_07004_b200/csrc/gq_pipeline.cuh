@@ -8,7 +8,7 @@
 //
 // Work distribution: units are dealt round-robin to the pairs for `full_waves` rounds, so that pairs that
 // run at the same time work on neighbouring tiles and share operands in L2; what is left (fewer units than
-// pairs) can be cut along the contraction index into equal pieces, one per pair.
+// pairs) can be cut along the contraction index into pieces for all pairs.
 //
 // Every wait on an mbarrier is bounded by a time budget; when it runs out the kernel records
 // STATUS_TIMEOUT in the status word, all roles of that CTA leave their loops (the peer CTA's own waits
@@ -30,7 +30,9 @@ constexpr int TILE_K = 64;
 constexpr int BOX_FEATURES = 64;                       // 128 bytes of bf16
 constexpr int BOX_BYTES = TILE_K * 128;                // one TMA box: 64 rows x 128 B
 constexpr uint32_t TMEM_COLS = 512;
-constexpr int MIN_PIECE_KSTEPS = 8;                    // smallest k-range worth an epilogue of its own
+constexpr int MIN_PIECE_KSTEPS = 8;                    // smallest k-range worth an epilogue of its own, where a pair may get two
+constexpr int MIN_EVEN_PIECE_KSTEPS = 2;               // and where it gets one
+constexpr int EPILOGUE_KSTEPS = 8;                     // k-steps that take as long as an epilogue
 
 constexpr uint32_t STATUS_TIMEOUT = 6;   // stored in the status word; the host maps it to GQ_ERR_TIMEOUT
 
@@ -60,12 +62,21 @@ inline Schedule plan_schedule(int units, int ksteps, int pairs, bool balanced)
         p.full_waves = units / pairs;
         p.tail_units = units - p.full_waves * pairs;
         const long long total = static_cast<long long>(p.tail_units) * ksteps;
-        // at least a pair per unit, however short the units (24 units of one k-step each: three pairs took 64 us for what 24
-        // do in 12); at most so many that a piece is worth its epilogue (with 4 k-steps in place of 8 launches of 512 tokens
-        // got 20-30 % longer: every piece adds all of its tile to H)
+        // Across units: equal shares for as many pairs as there are, so that most pairs end up with pieces of two units.  At least
+        // a pair per unit, however short the units (24 units of one k-step each: three pairs took 64 us for what 24 do in 12); at
+        // most so many that a piece is worth its epilogue (with 4 k-steps in place of 8 launches of 512 tokens got 20-30 % longer).
         long long tp = total / MIN_PIECE_KSTEPS;
         if (tp < p.tail_units) tp = p.tail_units;
         if (tp > pairs) tp = pairs;
+        // Evenly: every unit into the same number of pieces, a pair each, so that no pair has a second epilogue to go through and
+        // less is added to H.  The shorter of the two by the k-steps and epilogues of a pair; for long units across is (a third
+        // of the pairs idle for 64 k-steps cost more than an epilogue), for launches of a few thousand tokens and less evenly.
+        // d_in, tokens, groups: across / evenly in us: 1456, 921, 1: 22.9 / 13.7; 1032, 2048, 3: 27.6 / 23.8; 256, 2048, 4 (whose
+        // two units went to eight pairs, now to 32): 15.5 / 11.8; 4096, 2048, 1: 38.0 / 33.1; the smallest pieces 4 k-steps long
+        // instead of 2: 13.7 -> 14.3, 11.8 -> 12.8.
+        int cut = pairs / p.tail_units;
+        if (cut > ksteps / MIN_EVEN_PIECE_KSTEPS) cut = ksteps >= MIN_EVEN_PIECE_KSTEPS ? ksteps / MIN_EVEN_PIECE_KSTEPS : 1;
+        if (ksteps / cut + EPILOGUE_KSTEPS <= total / tp + 2 * EPILOGUE_KSTEPS) tp = static_cast<long long>(cut) * p.tail_units;
         p.tail_pairs = static_cast<int>(tp);
         p.tail_share = static_cast<unsigned>(total / tp);
         p.tail_rest = static_cast<unsigned>(total % tp);
