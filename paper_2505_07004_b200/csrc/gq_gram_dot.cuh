@@ -7,8 +7,9 @@
 // matching entries of H_k straight out of tensor memory.
 //
 // Operands.  Delta is prepared once per call as ONE fp16 matrix (delta_half_kernel): delta * 2^e with a single
-// power of two e for the whole layer, such that the largest entry lies below 2^15 and, but for the clamps, above 2^11.
-// fp16 carries 11 significant bits at any magnitude above 2^-14, i.e. down to 2^-25 of the largest entry at least, and the
+// power of two e for the whole layer, such that the largest entry lies below 2^16 and, but for the clamps, above 2^12.
+// fp16 carries 11 significant bits at any magnitude above 2^-14, i.e. down to 2^-26 of the largest entry at least (what is
+// smaller is off by at most 2^-37 of the largest, 2^-25 of the error that the largest may have), and the
 // scaling is undone exactly (2^-2e in the final fp64 reduction).  One product at the
 // 16-bit rate replaces three bf16 products (hi hi + hi lo + lo hi): the contraction then costs about as much as
 // streaming H from HBM, which is what the kernel below is built around.  Rounding: both factors of every
@@ -56,9 +57,10 @@ constexpr int GD_EPI_WARPS = 8;
 constexpr int GD_THREADS = 32 * (4 + GD_EPI_WARPS);
 constexpr int GD_SMEM_BYTES = GD_STAGES * GD_STAGE_BYTES + 1024;
 constexpr int GD_PARTIALS_PER_UNIT = 2 * GD_EPI_WARPS;       // one fp64 per (CTA of the pair, epilogue warp)
-constexpr int GD_SAMPLE_EXP = 11;                            // the largest sampled |delta| * 2^e lies in [2^11, 2^12),
-constexpr int GD_LARGEST_EXP = 14;                           // the largest of all has to lie below 2^15; else, with the exact
-                                                             // maximum, in [2^14, 2^15)
+constexpr int GD_SAMPLE_EXP = 12;                            // the largest sampled |delta| * 2^e lies in [2^12, 2^13);
+constexpr int GD_LARGEST_EXP = 14;                           // the largest of all, if known first, in [2^14, 2^15)
+constexpr int GD_FITS_EXP = 15;                              // it has to round to a finite value, 65504 at most
+constexpr unsigned int GD_FITS_ROUND = 0x1000;               // carries into the exponent what fp16 rounds up to 2^16: 65520 on
 constexpr int GD_MAX_SHIFT = 100;                            // |e| is kept below this (the scale stays a normal float)
 
 // Header of the objective workspace, written by the preparation kernels and read by the reduction.
@@ -152,9 +154,10 @@ __device__ __forceinline__ unsigned int block_max(unsigned int v, unsigned int *
 }
 
 // out = fp16((W - W_hat) * 2^e), round to nearest (the differences are formed in fp32, as everywhere in the objective), and
-// the biased exponent of every block's max |W - W_hat| (an infinite difference: 0xff).  e has to be known before the first
+// the biased exponent of every block's max |W - W_hat| (one more where fp16 would round it up to the next power of two; an
+// infinite difference: 0xff).  e has to be known before the first
 // value is stored and depends on the largest, so it is guessed: every block looks at the same 1024 values, spread over the
-// layer, and leaves room for values 8 times as large.  delta_redo_kernel takes care of layers that need more.
+// layer, and leaves room for values 7.9 times as large.  delta_redo_kernel takes care of layers that need more.
 // HBM-bound: W and W_hat are read once.  Three candidates of a 4096 x 4096 layer, whole calls: 319 us; with a pass over both
 // for the maximum before the pass that converts 352 us (4096 x 11008 layer, one group, all of it: 704 and 760).
 __global__ void __launch_bounds__(256)
@@ -191,11 +194,11 @@ delta_half_kernel(const float *W, const float *What, unsigned count4, GramDotHea
         if (idx < count4) reinterpret_cast<uint2 *>(out)[idx] = delta_half4(w[t], q[t], scale);
     }
     const unsigned int largest = block_max(__float_as_uint(m), red[1]);
-    if (threadIdx.x == 0) block_exp[blockIdx.x] = static_cast<uint8_t>(largest >> 23);
+    if (threadIdx.x == 0) block_exp[blockIdx.x] = static_cast<uint8_t>((largest + GD_FITS_ROUND) >> 23);
 }
 
-// Decides on e: the guess where the largest |W - W_hat| stays below 2^15 with it (all blocks return at once), else the power
-// of two that takes it to [2^14, 2^15), with which the matrix is written again.  blocks: of delta_half_kernel.
+// Decides on e: the guess where the largest |W - W_hat| is a finite fp16 with it (all blocks return at once), else the power
+// of two that takes it to [2^14, 2^15) (one less where it rounds up), with which the matrix is written again.  blocks: of delta_half_kernel.
 __global__ void __launch_bounds__(256)
 delta_redo_kernel(const float *W, const float *What, unsigned count4, GramDotHeader *header, const uint8_t *block_exp,
                   unsigned blocks, __half *out)
@@ -213,7 +216,7 @@ delta_redo_kernel(const float *W, const float *What, unsigned count4, GramDotHea
     if (threadIdx.x < blocks % 16u) biased = max(biased, static_cast<unsigned int>(block_exp[words * 16u + threadIdx.x]));
     biased = block_max(biased, red);
     const int guess = header->guess, exact = delta_shift(biased, GD_LARGEST_EXP);
-    const bool fits = static_cast<int>(biased) - 127 + guess <= GD_LARGEST_EXP || exact == guess;
+    const bool fits = static_cast<int>(biased) - 127 + guess <= GD_FITS_EXP || exact == guess;
     if (blockIdx.x == 0 && threadIdx.x == 0) header->shift = fits ? guess : exact;
     if (fits) return;
     const float scale = delta_scale(exact);

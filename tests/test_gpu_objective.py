@@ -46,8 +46,8 @@ def check(loss, ref):
     assert np.all(np.abs(loss - ref) <= L_RTOL * np.abs(ref)), "relative error %s" % (np.abs(loss - ref) / np.abs(ref))
 
 
-# Factors around the room that the guess of the scale leaves (8 is inside whatever the sample, 16 is not), and far past it
-@pytest.mark.parametrize("factor", [8.0, 16.0, 1e3, 1e6])
+# Factors around the room that the guess of the scale leaves (8 is inside whatever the sample, 32 is not), and far past it
+@pytest.mark.parametrize("factor", [8.0, 16.0, 32.0, 1e6])
 @pytest.mark.parametrize("at", [0, 5, -1])
 def test_scale_of_outliers(dev, factor, at):
     d_in, d_out, g = 264, 1024, 2
@@ -81,3 +81,14 @@ def test_differences_that_are_not_finite(dev):
         W_hat[700, 100] = bad
         loss = run(dev, W, W_hat, H)
         assert np.isfinite(loss[0]) and not np.isfinite(loss[1]) and not np.isfinite(loss[2])
+
+
+@pytest.mark.parametrize("mantissa", [65503.0, 65504.0, 65519.9, 65520.0, 65535.0, 65536.0])
+def test_scale_where_fp16_ends(dev, mantissa):
+    """The largest difference lands, with the guessed scale, on either side of what fp16 can hold."""
+    d_in, d_out, g = 64, 1024, 1
+    H, W, _ = problem(d_in, d_out, g)
+    W[:] = 0
+    delta = np.full(W.shape, 4096.0 / 65536.0, dtype=np.float32)      # every sample: 2^12 with the guessed scale
+    delta[5, 7] = mantissa / 65536.0
+    check(run(dev, W, delta, H), orc.objective(W, delta, H, impl="numpy"))
