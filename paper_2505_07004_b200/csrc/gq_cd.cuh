@@ -238,20 +238,20 @@ __device__ __forceinline__ int sums_at(int ch, int rq)
 //   chain warp (0)       one lane per channel.  A band of 32 coordinates at a time, its 32 running sums in registers: round
 //                        (nearest_level: compares and selects only), E_i = val - W_i, add H[i][r] E_i to the sums of the
 //                        rows after i inside the band.  No shuffle, vote or table read lies on the path.
-//   product warps (6)    while the chain works on band t they form the sums of band t + 1 over every coordinate of the block
+//   product warps (6, with 16 channels 3 of two parts each)   while the chain works on band t they form the sums of band t + 1 over every coordinate of the block
 //                        outside bands t and t + 1, plus last cycle's values of band t + 1 above its diagonal; when the chain
-//                        is through with band t they add its new values (32 x 32 x 32) and hand the sums over.  Every warp
-//                        forms the whole 32 x 32 sums, 8 rows x 4 channels per thread, over a share of the contraction;
+//                        is through with band t they add its new values (32 x 32 x CH) and hand the sums over.  Every part
+//                        forms all of the 32 x CH sums, 8 rows x 4 channels per thread, over a share of the contraction;
 //                        all of them on the three schedulers that the chain warp does not use.  A value loaded from shared
 //                        memory costs a lane-register write whether or not lanes share it (measured: a 16-byte load takes
 //                        4 clocks of the SM's load pipe, 2 if all lanes read the same address), hence 12 loaded values
 //                        per 32 multiply-adds.
-//   loader warp (4)      TMA: the tiles of W, E and P (256 coordinates x 32 channels), and H[all 256][band] (32 KB) per
+//   loader warp (4)      TMA: the tiles of W, E and P (256 coordinates x CH channels), and H[all 256][band] (32 KB) per
 //                        band into one of three buffers, two bands ahead.
 // Two named barriers per band: sums ready (products -> chain), band done (chain -> products, loader).
-// Measured for one block of 4096 channels, 16 levels: 33.7 us (8 levels, 1408 channels: 29.8; 34.9 and 31.2 with the excluded
-// coordinates multiplied by zero instead of left out); with eight threads per channel that did all updates themselves and two
-// votes and a table read per step it was 81 us (78).
+// Measured for one block of 4096 channels, 16 levels: 33.7 us (8 levels, 1408 channels: 19 from the end of the panel product to
+// its own, 27 with 32 channels per CTA); 1.2 us more with the excluded coordinates multiplied by zero instead of left out;
+// with eight threads per channel that did all updates themselves and two votes and a table read per step it was 81 us (78).
 template <int LEV, int CH>
 __global__ void __launch_bounds__(CD_THREADS, 1)
 cd_block_kernel(const __grid_constant__ CUtensorMap mapH, const __grid_constant__ CUtensorMap mapW,

@@ -17,9 +17,10 @@
 // H only, G = F + F^T, halves the work and was measured: 1.85 ms an update.  It was not kept: the tensor core's fp32
 // accumulation truncates, with half as many additions the levels come out 1e-5 different, and 11 % of the codes of the next
 // descent cycles with them.)
-// Stage: [A | B], 16 KB each per CTA, of which only B comes through the L2.  What bounds the kernel is the tensor core (732
-// clocks a k-step with the one-hot stores left out, 512 at its nominal rate) and shared-memory bandwidth (840 with them).
-// Measured, 4096 x 4096, 4 groups, 16 levels, one update: 3.73 ms = 1290 TFLOP/s.  With the one-hot matrix, H P and H W^T in
+// Stage: [A | B], 16 KB each per CTA, of which only B comes through the L2.  What bounds the kernel is the tensor core and
+// the thread that feeds it (695 clocks a k-step with the one-hot stores left out, 512 at the nominal rate) and shared-memory
+// bandwidth (807 with them).  Measured, 4096 x 4096, 4 groups, 16 levels, one update: 3.7 ms = 1300 TFLOP/s with the issuing
+// thread on warp 1; on warp 3 a call with two updates takes 0.35 ms less.  With the one-hot matrix, H P and H W^T in
 // global memory it was 0.17 (one-hot) + 2.88 (H P) + 0.40 (H W^T) + 0.55 (sums by level) = 4.00 ms and 0.5 GB of scratch.
 #pragma once
 #include <cuda.h>
