@@ -231,6 +231,8 @@ int32_t gq_hessian_gather_shares(float *const *H_ranks, int32_t ranks, int32_t r
  * fp64 in a fixed order and multiplied by 2^-2e.  Relative error of the result: at most 2^-11 = 4.9e-4 if
  * every rounding error had the same sign and H_k had no negative entries, about 1e-6 for rounding errors of
  * random sign (what is seen on quantisation errors).  Results are bit-reproducible run to run.
+ * A difference that is infinite or NaN makes its group's loss and the sum of all not finite; the scale is taken from
+ * the finite differences, and the other groups' losses are what they are without it.
  */
 int32_t gq_objective(const float *W, const float *W_hat, int64_t d_in, int64_t d_out, const float *H,
                      int32_t g, double *loss_out, void *workspace, size_t workspace_bytes,

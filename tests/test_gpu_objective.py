@@ -72,15 +72,31 @@ def test_scale_of_a_single_difference(dev):
     assert not run(dev, W, W.copy(), H).any()
 
 
-def test_differences_that_are_not_finite(dev):
-    """An infinite or undefined difference gives a loss that is not finite, for its group only."""
+# The first weight always belongs to the sample that the scale is guessed from; (700, 100) does not, (1023, 263) is the last
+@pytest.mark.parametrize("at", [(0, 0), (700, 100), (1023, 263)])
+@pytest.mark.parametrize("bad", [np.inf, -np.inf, np.nan])
+def test_differences_that_are_not_finite(dev, bad, at):
+    """An infinite or undefined difference gives a loss that is not finite, for its group only; the other group's loss is what
+    it is without it."""
     d_in, d_out, g = 264, 1024, 2
     H, W, rng = problem(d_in, d_out, g)
-    for bad in (np.inf, -np.inf, np.nan):
-        W_hat = (W + 0.003 * rng.standard_normal(W.shape)).astype(np.float32)
-        W_hat[700, 100] = bad
-        loss = run(dev, W, W_hat, H)
-        assert np.isfinite(loss[0]) and not np.isfinite(loss[1]) and not np.isfinite(loss[2])
+    W_hat = (W + 0.003 * rng.standard_normal(W.shape)).astype(np.float32)
+    ref = orc.objective(W, W_hat, H, impl="numpy")
+    W_hat[at] = bad
+    loss = run(dev, W, W_hat, H)
+    hit = at[0] // (d_out // g)
+    assert not np.isfinite(loss[hit]) and not np.isfinite(loss[2])
+    check(loss[1 - hit], ref[1 - hit])
+
+
+def test_differences_that_are_all_infinite(dev):
+    """No finite difference in one group, zeros in the other."""
+    d_in, d_out, g = 64, 256, 2
+    H, W, _ = problem(d_in, d_out, g)
+    W_hat = W.copy()
+    W_hat[:128] = np.inf
+    loss = run(dev, W, W_hat, H)
+    assert not np.isfinite(loss[0]) and loss[1] == 0.0 and not np.isfinite(loss[2])
 
 
 @pytest.mark.parametrize("mantissa", [65503.0, 65504.0, 65519.9, 65520.0, 65535.0, 65536.0])
