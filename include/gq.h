@@ -223,9 +223,9 @@ int32_t gq_hessian_gather_shares(float *const *H_ranks, int32_t ranks, int32_t r
  *              1024-byte aligned
  * Same shape rules as above (d_in % 8 == 0, d_out % g == 0, (d_out / g) % 8 == 0).
  * Arithmetic: delta = W - W_hat in fp32, written to the workspace as ONE fp16 matrix delta * 2^e.  e is guessed
- * from 1024 values spread over the layer so that the largest of them lies in [2^12, 2^13); where an entry turns out
- * to be 8 to 16 times as large, the matrix is written again with the largest of all in [2^14, 2^15).  Either way 11
- * significant bits for every entry down to 2^-26 of the largest; round to nearest, no bias.  The Gram
+ * from 1024 values spread over the layer so that the largest of them lies in [2^14, 2^15); where an entry turns out to
+ * be 2 to 4 times as large, the matrix is written again with the largest of all in [2^14, 2^15).  Either way 11
+ * significant bits for every entry down to 2^-28 of the largest; round to nearest, no bias.  The Gram
  * matrices Delta_k^T Delta_k are formed on the tensor cores (fp16 operands, fp32 accumulation) two 256-column
  * tiles at a time and contracted with H_k (fp32) straight out of tensor memory; partial sums are reduced in
  * fp64 in a fixed order and multiplied by 2^-2e.  Relative error of the result: at most 2^-11 = 4.9e-4 if

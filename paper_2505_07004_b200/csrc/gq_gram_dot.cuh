@@ -7,9 +7,9 @@
 // matching entries of H_k straight out of tensor memory.
 //
 // Operands.  Delta is prepared once per call as ONE fp16 matrix (delta_half_kernel): delta * 2^e with a single
-// power of two e for the whole layer, such that the largest entry lies below 2^16 and, but for the clamps, above 2^12.
-// fp16 carries 11 significant bits at any magnitude above 2^-14, i.e. down to 2^-26 of the largest entry at least (what is
-// smaller is off by at most 2^-37 of the largest, 2^-25 of the error that the largest may have), and the
+// power of two e for the whole layer, such that the largest finite entry lies below 2^16 and, but for the clamps, not below 2^14.
+// fp16 carries 11 significant bits at any magnitude above 2^-14, i.e. down to 2^-28 of the largest entry at least (what is
+// smaller is off by at most 2^-39 of the largest), and the
 // scaling is undone exactly (2^-2e in the final fp64 reduction).  One product at the
 // 16-bit rate replaces three bf16 products (hi hi + hi lo + lo hi): the contraction then costs about as much as
 // streaming H from HBM, which is what the kernel below is built around.  Rounding: both factors of every
@@ -58,7 +58,7 @@ constexpr int GD_EPI_WARPS = 8;
 constexpr int GD_THREADS = 32 * (4 + GD_EPI_WARPS);
 constexpr int GD_SMEM_BYTES = GD_STAGES * GD_STAGE_BYTES + 1024;
 constexpr int GD_PARTIALS_PER_UNIT = 2 * GD_EPI_WARPS;       // one fp64 per (CTA of the pair, epilogue warp)
-constexpr int GD_SAMPLE_EXP = 12;                            // the largest sampled |delta| * 2^e lies in [2^12, 2^13);
+constexpr int GD_SAMPLE_EXP = 14;                            // the largest sampled |delta| * 2^e lies in [2^14, 2^15);
 constexpr int GD_LARGEST_EXP = 14;                           // the largest of all, if known first, in [2^14, 2^15)
 constexpr int GD_FITS_EXP = 15;                              // it has to round to a finite value, 65504 at most
 constexpr unsigned int GD_FITS_ROUND = 0x1000;               // carries into the exponent what fp16 rounds up to 2^16: 65520 on
@@ -166,7 +166,7 @@ __device__ __forceinline__ unsigned int block_max(unsigned int v, unsigned int *
 // the biased exponent of every block's largest finite |W - W_hat| (one more where fp16 would round it up to the next power of
 // two).  e has to be known before the first
 // value is stored and depends on the largest, so it is guessed: every block looks at the same 1024 values, spread over the
-// layer, and leaves room for values 7.9 times as large.  delta_redo_kernel takes care of layers that need more.
+// layer, and leaves room for values 1.9 to 4 times as large.  delta_redo_kernel takes care of layers that need more.
 // HBM-bound: W and W_hat are read once.  Three candidates of a 4096 x 4096 layer, whole calls: 319 us; with a pass over both
 // for the maximum before the pass that converts 352 us (4096 x 11008 layer, one group, all of it: 704 and 760).
 __global__ void __launch_bounds__(256)
