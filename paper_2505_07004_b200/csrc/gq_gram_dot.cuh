@@ -116,6 +116,7 @@ __device__ __forceinline__ float4 ld_f32x4_last_use(const float4 *p)
 
 constexpr int DELTA_VEC_PER_THREAD = 4;      // float4 pairs a thread of the first preparation kernel handles
 constexpr unsigned DELTA_BLOCK_VECS = 256u * DELTA_VEC_PER_THREAD;
+constexpr unsigned DELTA_REDO_VECS = 256u * DELTA_VEC_PER_THREAD;      // of eight fp16 values, a block of the second one at a time
 
 // The power of two that takes a value of biased exponent `biased` (0: zero or subnormal) to [2^target, 2^(target + 1)).
 __device__ __forceinline__ int delta_shift(unsigned int biased, int target)
@@ -211,8 +212,32 @@ delta_half_kernel(const float *W, const float *What, unsigned count4, GramDotHea
     if (threadIdx.x == 0) block_exp[blockIdx.x] = static_cast<uint8_t>((largest + GD_FITS_ROUND) >> 23);
 }
 
-// Decides on e: the guess where the largest finite |W - W_hat| is a finite fp16 with it (all blocks return at once), else the power
-// of two that takes it to [2^14, 2^15) (one less where it rounds up), with which the matrix is written again.  blocks: of delta_half_kernel.
+// Eight fp16 values of scale 2^guess at the scale 2^(guess - down), in place.  Where the results are normal, or zero to begin with,
+// that is `down` less in their exponents: the bits that rounding at the smaller scale gives.  False where a value is not finite
+// or would lose bits that it has.
+__host__ __device__ __forceinline__ bool delta_lower(uint4 &v, unsigned down)
+{
+    const unsigned least = down < 30u ? (down + 1u) << 10 : 0x7c00u, span = 0x7c00u - least;      // magnitudes in [least, 0x7c00)
+    bool ok = true;
+    auto two = [&](uint32_t &w) {
+        const unsigned lo = w & 0x7fffu, hi = (w >> 16) & 0x7fffu;
+        ok = ok && (lo == 0u || lo - least < span) && (hi == 0u || hi - least < span);
+        w -= (lo ? down << 10 : 0u) + (hi ? down << 26 : 0u);
+    };
+    two(v.x);
+    two(v.y);
+    two(v.z);
+    two(v.w);
+    return ok;
+}
+
+// Decides on e: the guess where the largest finite |W - W_hat| is a finite fp16 with it (all blocks return at once), else the
+// power of two that takes it to [2^14, 2^15) (one less where it rounds up), to which the matrix is then brought: the values that
+// have their bits by lowering the exponent, a quarter of the bytes of W and W_hat and most of them in the L2, the others (among
+// them what has overflowed) from W and W_hat.  blocks: of delta_half_kernel.
+// One row 20 times as wide as the others, a call: 113 us for 4096 x 4096 and 250 for 4096 x 11008 with one group; 131 and 294 with
+// all values from W and W_hat again, 123 and 273 with a pass over both for the maximum before one that converts.  A million
+// times as wide, where 3 % of the threads' values are formed again: 115 and 258, 131 and 292, 121 and 271.
 __global__ void __launch_bounds__(256)
 delta_redo_kernel(const float *W, const float *What, unsigned count4, GramDotHeader *header, const uint8_t *block_exp,
                   unsigned blocks, __half *out)
@@ -234,10 +259,30 @@ delta_redo_kernel(const float *W, const float *What, unsigned count4, GramDotHea
     if (blockIdx.x == 0 && threadIdx.x == 0) header->shift = fits ? guess : exact;
     if (fits) return;
     const float scale = delta_scale(exact);
-    const unsigned stride = gridDim.x * 256u;
-    for (unsigned idx = blockIdx.x * 256u + threadIdx.x; idx < count4; idx += stride)
-        reinterpret_cast<uint2 *>(out)[idx] =
-            delta_half4(reinterpret_cast<const float4 *>(W)[idx], reinterpret_cast<const float4 *>(What)[idx], scale);
+    const unsigned down = static_cast<unsigned>(guess - exact);    // positive: what does not fit is too large
+    const unsigned count8 = count4 / 2u, stride = gridDim.x * DELTA_REDO_VECS;
+    uint4 *o = reinterpret_cast<uint4 *>(out);
+    // from the end: what delta_half_kernel has written last is still in the L2
+    for (unsigned base = blockIdx.x * DELTA_REDO_VECS + threadIdx.x; base < count8; base += stride) {
+        uint4 v[DELTA_VEC_PER_THREAD];
+#pragma unroll
+        for (int t = 0; t < DELTA_VEC_PER_THREAD; ++t) {
+            const unsigned idx = base + t * 256u;
+            v[t] = idx < count8 ? o[count8 - 1u - idx] : make_uint4(0u, 0u, 0u, 0u);
+        }
+#pragma unroll
+        for (int t = 0; t < DELTA_VEC_PER_THREAD; ++t) {
+            const unsigned idx = base + t * 256u, at = count8 - 1u - idx;
+            if (idx >= count8) continue;
+            if (!delta_lower(v[t], down)) {
+                const float4 *w = reinterpret_cast<const float4 *>(W) + 2 * static_cast<size_t>(at);
+                const float4 *q = reinterpret_cast<const float4 *>(What) + 2 * static_cast<size_t>(at);
+                const uint2 a = delta_half4(ld_f32x4(w), ld_f32x4(q), scale), b = delta_half4(ld_f32x4(w + 1), ld_f32x4(q + 1), scale);
+                v[t] = make_uint4(a.x, a.y, b.x, b.y);
+            }
+            o[at] = v[t];
+        }
+    }
 }
 
 // loss[k] = 2^(-2e) * sum over the group's partial sums (block k), loss[g] = sum_k loss[k] (formed, in group order,

@@ -819,7 +819,7 @@ int32_t gq_objective(const float *W, const float *W_hat, int64_t d_in, int64_t d
         GQ_CUDA(cudaGetLastError());
         {
             LaunchScope scope(GQ_KERNEL_SPLIT_DELTA, st);
-            const int grid = grid_for(count4, 256, di->sm_count, 4);
+            const int grid = grid_for(count4 / 2, gq::DELTA_REDO_VECS, di->sm_count, 4);
             launch(gq::delta_redo_kernel, dim3(grid), 256, 0, st, W, W_hat, count4, header, block_exp, blocks, dh);
         }
         GQ_CUDA(cudaGetLastError());

@@ -58,6 +58,17 @@ def test_scale_of_outliers(dev, factor, at):
     check(run(dev, W, W_hat, H), orc.objective(W, W_hat, H, impl="numpy"))
 
 
+def test_scale_of_an_outlier_row(dev):
+    """A row 300 times as wide as the others (every value of it overflows with the guessed scale, a few others are lowered into
+    the subnormal range), in a layer that the second preparation kernel goes over twice."""
+    d_in, d_out, g = 2312, 2320, 1
+    H, W, rng = problem(d_in, d_out, g)
+    delta = 0.001 * rng.standard_normal(W.shape)
+    delta[1234] *= 300
+    W_hat = (W + delta).astype(np.float32)
+    check(run(dev, W, W_hat, H), orc.objective(W, W_hat, H, impl="numpy"))
+
+
 def test_scale_of_a_single_difference(dev):
     """Every sample is zero; magnitudes from the smallest that the scale reaches to large ones."""
     d_in, d_out, g = 128, 4096, 1
