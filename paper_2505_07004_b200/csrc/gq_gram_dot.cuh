@@ -168,8 +168,10 @@ __device__ __forceinline__ unsigned int block_max(unsigned int v, unsigned int *
 // two).  e has to be known before the first
 // value is stored and depends on the largest, so it is guessed: every block looks at the same 1024 values, spread over the
 // layer, and leaves room for values 1.9 to 4 times as large.  delta_redo_kernel takes care of layers that need more.
-// HBM-bound: W and W_hat are read once.  Three candidates of a 4096 x 4096 layer, whole calls: 319 us; with a pass over both
-// for the maximum before the pass that converts 352 us (4096 x 11008 layer, one group, all of it: 704 and 760).
+// HBM-bound: W and W_hat are read once.  The sample is 64 runs of 64 bytes and not 256 of 16, each a request of its own in every
+// block.  Three candidates of a 4096 x 4096 layer, whole calls: 324 us, with a pass over both matrices for the maximum before the
+// pass that converts 371; with the sample of 256 places 348 and 380 in another run.  Two candidates of 3152 x 296, where all is in
+// the L2: 4 % slower than two passes with 256 places, layers of 0.2 to 2 million weights with 64 none.
 __global__ void __launch_bounds__(256)
 delta_half_kernel(const float *W, const float *What, unsigned count4, GramDotHeader *header, uint8_t *block_exp, __half *out)
 {
@@ -178,9 +180,9 @@ delta_half_kernel(const float *W, const float *What, unsigned count4, GramDotHea
     griddep_wait();
     const unsigned base = blockIdx.x * DELTA_BLOCK_VECS + threadIdx.x;
     float4 w[DELTA_VEC_PER_THREAD], q[DELTA_VEC_PER_THREAD];
-    // one pair of float4 per thread, somewhere in the thread's 256th of the layer (the same for every block)
-    const unsigned part = max(count4 / 256u, 1u);
-    const unsigned sidx = min(threadIdx.x * part + __umulhi(threadIdx.x * 2654435761u, part), count4 - 1u);
+    // four pairs of float4 side by side, somewhere in each 64th of the layer (the same for every block)
+    const unsigned part = max(count4 / 64u, 4u), spot = threadIdx.x / 4u;
+    const unsigned sidx = min(((spot * part + __umulhi(spot * 2654435761u, part)) & ~3u) + threadIdx.x % 4u, count4 - 1u);
     const float4 sw = ld_f32x4(reinterpret_cast<const float4 *>(W) + sidx);
     const float4 sq = ld_f32x4(reinterpret_cast<const float4 *>(What) + sidx);
 #pragma unroll
