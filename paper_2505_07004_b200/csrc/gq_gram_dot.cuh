@@ -168,6 +168,7 @@ __device__ __forceinline__ unsigned int block_max(unsigned int v, unsigned int *
 // two).  e has to be known before the first
 // value is stored and depends on the largest, so it is guessed: every block looks at the same 1024 values, spread over the
 // layer, and leaves room for values 1.9 to 4 times as large.  delta_redo_kernel takes care of layers that need more.
+// A block goes over DELTA_BLOCK_VECS pairs of float4, or several times as many where there is no room for a byte from each.
 // HBM-bound: W and W_hat are read once.  The sample is 64 runs of 64 bytes and not 256 of 16, each a request of its own in every
 // block.  Three candidates of a 4096 x 4096 layer, whole calls: 324 us, with a pass over both matrices for the maximum before the
 // pass that converts 371; with the sample of 256 places 348 and 380 in another run.  Two candidates of 3152 x 296, where all is in
@@ -178,40 +179,50 @@ delta_half_kernel(const float *W, const float *What, unsigned count4, GramDotHea
     __shared__ unsigned int red[2][8];
     griddep_launch();
     griddep_wait();
-    const unsigned base = blockIdx.x * DELTA_BLOCK_VECS + threadIdx.x;
+    unsigned base = blockIdx.x * DELTA_BLOCK_VECS + threadIdx.x;
     float4 w[DELTA_VEC_PER_THREAD], q[DELTA_VEC_PER_THREAD];
     // four pairs of float4 side by side, somewhere in each 64th of the layer (the same for every block)
     const unsigned part = max(count4 / 64u, 4u), spot = threadIdx.x / 4u;
     const unsigned sidx = min(((spot * part + __umulhi(spot * 2654435761u, part)) & ~3u) + threadIdx.x % 4u, count4 - 1u);
     const float4 sw = ld_f32x4(reinterpret_cast<const float4 *>(W) + sidx);
     const float4 sq = ld_f32x4(reinterpret_cast<const float4 *>(What) + sidx);
+    auto load = [&] {
 #pragma unroll
-    for (int t = 0; t < DELTA_VEC_PER_THREAD; ++t) {
-        const unsigned idx = base + t * 256u;
-        const bool in = idx < count4;
-        w[t] = in ? ld_f32x4_last_use(reinterpret_cast<const float4 *>(W) + idx) : make_float4(0.f, 0.f, 0.f, 0.f);
-        q[t] = in ? ld_f32x4_last_use(reinterpret_cast<const float4 *>(What) + idx) : make_float4(0.f, 0.f, 0.f, 0.f);
-    }
+        for (int t = 0; t < DELTA_VEC_PER_THREAD; ++t) {
+            const unsigned idx = base + t * 256u;
+            const bool in = idx < count4;
+            w[t] = in ? ld_f32x4_last_use(reinterpret_cast<const float4 *>(W) + idx) : make_float4(0.f, 0.f, 0.f, 0.f);
+            q[t] = in ? ld_f32x4_last_use(reinterpret_cast<const float4 *>(What) + idx) : make_float4(0.f, 0.f, 0.f, 0.f);
+        }
+    };
+    load();
     const int e = delta_shift(block_max(__float_as_uint(delta_max_finite(0.0f, sw, sq)), red[0]) >> 23, GD_SAMPLE_EXP);
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         header->guess = e;
         header->blocks_done = 0u;
     }
     const float scale = delta_scale(e);
-    float m = 0.0f;
+    float largest = 0.0f;
+    for (;;) {
+        float m = 0.0f;
 #pragma unroll
-    for (int t = 0; t < DELTA_VEC_PER_THREAD; ++t) {
-        const unsigned idx = base + t * 256u;
-        m = delta_max(m, w[t], q[t]);
-        if (idx < count4) reinterpret_cast<uint2 *>(out)[idx] = delta_half4(w[t], q[t], scale);
-    }
-    if (!(m < CUDART_INF_F)) {
-        m = 0.0f;
+        for (int t = 0; t < DELTA_VEC_PER_THREAD; ++t) {
+            const unsigned idx = base + t * 256u;
+            m = delta_max(m, w[t], q[t]);
+            if (idx < count4) reinterpret_cast<uint2 *>(out)[idx] = delta_half4(w[t], q[t], scale);
+        }
+        if (!(m < CUDART_INF_F)) {
+            m = 0.0f;
 #pragma unroll
-        for (int t = 0; t < DELTA_VEC_PER_THREAD; ++t) m = delta_max_finite(m, w[t], q[t]);
+            for (int t = 0; t < DELTA_VEC_PER_THREAD; ++t) m = delta_max_finite(m, w[t], q[t]);
+        }
+        largest = fmaxf(largest, m);
+        base += gridDim.x * DELTA_BLOCK_VECS;
+        if (base - threadIdx.x >= count4) break;
+        load();
     }
-    const unsigned int largest = block_max(__float_as_uint(m), red[1]);
-    if (threadIdx.x == 0) block_exp[blockIdx.x] = static_cast<uint8_t>((largest + GD_FITS_ROUND) >> 23);
+    const unsigned int bits = block_max(__float_as_uint(largest), red[1]);
+    if (threadIdx.x == 0) block_exp[blockIdx.x] = static_cast<uint8_t>((bits + GD_FITS_ROUND) >> 23);
 }
 
 // Eight fp16 values of scale 2^guess at the scale 2^(guess - down), in place.  Where the results are normal, or zero to begin with,

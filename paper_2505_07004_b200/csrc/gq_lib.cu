@@ -362,10 +362,8 @@ ObjectiveLayout objective_layout(int64_t d_in, int64_t d_out, int32_t g)
     L.header_off = 0;
     L.half_off = round_up(sizeof(gq::GramDotHeader), 1024);
     L.partials_off = L.half_off + round_up(static_cast<size_t>(d_in) * static_cast<size_t>(d_out) * 2, 1024);
-    size_t tail = static_cast<size_t>(tiles_for(d_in)) * g * gq::GD_PARTIALS_PER_UNIT * sizeof(double);
-    const size_t blocks = (static_cast<size_t>(d_in) * d_out / 4 + gq::DELTA_BLOCK_VECS - 1) / gq::DELTA_BLOCK_VECS;
-    if (tail < blocks) tail = blocks;                              // one byte each, see gq_objective
-    L.total = L.partials_off + round_up(tail, 1024);
+    L.total = L.partials_off +
+              round_up(static_cast<size_t>(tiles_for(d_in)) * g * gq::GD_PARTIALS_PER_UNIT * sizeof(double), 1024);
     return L;
 }
 
@@ -806,11 +804,13 @@ int32_t gq_objective(const float *W, const float *W_hat, int64_t d_in, int64_t d
     __half *dh = reinterpret_cast<__half *>(ws + L.half_off);
     double *partials = reinterpret_cast<double *>(ws + L.partials_off);
     const int64_t m = d_out / g;
-    // delta = W - W_hat as one fp16 matrix scaled by a power of two (gq_gram_dot.cuh); the blocks' maxima stand where the
-    // partial sums come later
+    // delta = W - W_hat as one fp16 matrix scaled by a power of two (gq_gram_dot.cuh); the blocks' maxima, a byte each, stand
+    // where the partial sums come later: at least a thousand, for small d_in not as many as the layer would have blocks
     {
         const unsigned count4 = static_cast<unsigned>(d_in * d_out / 4);
-        const unsigned blocks = (count4 + gq::DELTA_BLOCK_VECS - 1) / gq::DELTA_BLOCK_VECS;
+        const size_t room = L.total - L.partials_off;
+        unsigned blocks = (count4 + gq::DELTA_BLOCK_VECS - 1) / gq::DELTA_BLOCK_VECS;
+        if (blocks > room) blocks = static_cast<unsigned>(room);
         uint8_t *block_exp = ws + L.partials_off;
         {
             LaunchScope scope(GQ_KERNEL_SPLIT_DELTA, st);

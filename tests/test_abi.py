@@ -52,6 +52,7 @@ def test_workspace_sizes(L):
     # objective: a 1 KiB header, delta as one fp16 matrix, 16 fp64 partial sums per (upper-triangular 256 x 256 tile, group)
     nj = 4096 // 256
     assert L.gq_objective_workspace_bytes(4096, 4096, 4) == 1024 + 4096 * 4096 * 2 + (nj * (nj + 1) // 2) * 4 * 16 * 8
+    assert L.gq_objective_workspace_bytes(128, 65536, 1) == 1024 + 128 * 65536 * 2 + 1024      # few tiles, many channels
     assert L.gq_objective_workspace_bytes(4096, 4096, 3) == 0          # d_out % g != 0
     assert L.gq_objective_workspace_bytes(4096, 24, 6) == 0            # (d_out / g) % 8 != 0
     assert L.gq_layer_host_arena_bytes(0, 4096, 4096, 4) == 0

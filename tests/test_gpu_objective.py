@@ -69,6 +69,18 @@ def test_scale_of_an_outlier_row(dev):
     check(run(dev, W, W_hat, H), orc.objective(W, W_hat, H, impl="numpy"))
 
 
+@pytest.mark.parametrize("at", [(5, 3), (60000, 40), (120007, 71)])
+def test_scale_where_blocks_share_a_byte(dev, at):
+    """Few features and many channels: the scratch has no room for as many maxima as the layer has blocks, so that a block goes
+    over several pieces.  The largest difference stands in a first piece, in a further one, and in the last, a partial one."""
+    d_in, d_out, g = 72, 120008, 1
+    H, W, rng = problem(d_in, d_out, g)
+    delta = 0.001 * rng.random(W.shape)
+    delta[at] = 1.0
+    W_hat = (W + delta).astype(np.float32)
+    check(run(dev, W, W_hat, H), orc.objective(W, W_hat, H, impl="numpy"))
+
+
 def test_scale_of_a_single_difference(dev):
     """Every sample is zero; magnitudes from the smallest that the scale reaches to large ones."""
     d_in, d_out, g = 128, 4096, 1
