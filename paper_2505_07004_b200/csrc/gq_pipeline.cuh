@@ -32,6 +32,7 @@ constexpr int BOX_BYTES = TILE_K * 128;                // one TMA box: 64 rows x
 constexpr uint32_t TMEM_COLS = 512;
 constexpr int MIN_PIECE_KSTEPS = 8;                    // smallest k-range worth an epilogue of its own, where a pair may get two
 constexpr int MIN_EVEN_PIECE_KSTEPS = 2;               // and where it gets one
+constexpr int MAX_EVEN_PIECE_KSTEPS = 16;              // largest there: 1024 tokens
 constexpr int EPILOGUE_KSTEPS = 8;                     // k-steps that take as long as an epilogue
 
 constexpr uint32_t STATUS_TIMEOUT = 6;   // stored in the status word; the host maps it to GQ_ERR_TIMEOUT
@@ -69,14 +70,19 @@ inline Schedule plan_schedule(int units, int ksteps, int pairs, bool balanced)
         if (tp < p.tail_units) tp = p.tail_units;
         if (tp > pairs) tp = pairs;
         // Evenly: every unit into the same number of pieces, a pair each, so that no pair has a second epilogue to go through and
-        // less is added to H.  The shorter of the two by the k-steps and epilogues of a pair; for long units across is (a third
-        // of the pairs idle for 64 k-steps cost more than an epilogue), for launches of a few thousand tokens and less evenly.
+        // less is added to H.  The shorter of the two by the k-steps and epilogues of a pair, for launches of few thousand tokens.
         // d_in, tokens, groups: across / evenly in us: 1456, 921, 1: 22.9 / 13.7; 1032, 2048, 3: 27.6 / 23.8; 256, 2048, 4 (whose
-        // two units went to eight pairs, now to 32): 15.5 / 11.8; 4096, 2048, 1: 38.0 / 33.1; the smallest pieces 4 k-steps long
-        // instead of 2: 13.7 -> 14.3, 11.8 -> 12.8.
+        // two units went to eight pairs, now to 32): 15.5 / 11.8; the smallest pieces 4 k-steps long instead of 2: 13.7 -> 14.3,
+        // 11.8 -> 12.8.
+        // Longer pieces stay with the cut across, although 72 whole units of 32 k-steps take 33.1 us instead of 38.0 and of 256
+        // 201 instead of 220: the tensor core truncates as it accumulates, and across most units are summed in two shorter runs.
+        // Error of H against 64 bits, evenly over across: 1.18 at worst with runs of 256 k-steps, 1.05 with 120, 1.009 with 32;
+        // up to 16, 40 shapes with four inputs each, 1.0001 in the mean and 1.005 at most, 0.997 at least.
         int cut = pairs / p.tail_units;
         if (cut > ksteps / MIN_EVEN_PIECE_KSTEPS) cut = ksteps >= MIN_EVEN_PIECE_KSTEPS ? ksteps / MIN_EVEN_PIECE_KSTEPS : 1;
-        if (ksteps / cut + EPILOGUE_KSTEPS <= total / tp + 2 * EPILOGUE_KSTEPS) tp = static_cast<long long>(cut) * p.tail_units;
+        const int longest = (ksteps + cut - 1) / cut;
+        if (longest <= MAX_EVEN_PIECE_KSTEPS && ksteps / cut + EPILOGUE_KSTEPS <= total / tp + 2 * EPILOGUE_KSTEPS)
+            tp = static_cast<long long>(cut) * p.tail_units;
         p.tail_pairs = static_cast<int>(tp);
         p.tail_share = static_cast<unsigned>(total / tp);
         p.tail_rest = static_cast<unsigned>(total % tp);
@@ -143,7 +149,7 @@ struct WorkItem {
 // a pair walks the same list, several of them before they can start: a pair's share of the tail, [total pair / tail_pairs,
 // total (pair + 1) / tail_pairs) of total = tail_units * ksteps < 2^32, is formed without 64-bit divisions (with three of them
 // the first k-step came 1.5 us later, and so did the first read-out).
-__device__ __forceinline__ bool work_item(const Schedule &p, int pair, int it, WorkItem &w)
+__host__ __device__ __forceinline__ bool work_item(const Schedule &p, int pair, int it, WorkItem &w)
 {
     if (it < p.full_waves) {
         w.unit = it * p.pairs + pair;

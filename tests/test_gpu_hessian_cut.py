@@ -21,3 +21,18 @@ def test_cut_last_round(dev, d_in, n, g):  # noqa: F811
     s = torch.rand(g, n, generator=gen, device=dev) + 0.1
     H = gpu_hessian([X, X], [s, s], d_in, g, dev)                     # twice: pieces add to what is there
     check_H(H, 2 * orc.hessian(synth.bf16_bits(X), s.cpu().numpy().astype(np.float64)))
+
+
+def test_error_of_a_long_launch(dev):  # noqa: F811
+    """16384 tokens of 4096 features, one group: 72 units for (at most) 74 pairs.  Accumulated in two shorter runs each, as most
+    of them are where the units are cut across the pairs, H is 2.36e-4 from 64 bits; in one run of 256 k-steps each, whose
+    truncated additions weigh more, 2.79e-4.  (The rest is the one bf16 rounding of every product, the same either way.)"""
+    d_in, n = 4096, 16384
+    syn = synth.LayerSynth(synth.LayerConfig("long", n, n, d_in, 512, (1,), "lognormal", 0.01, 20.0), dev, 2)
+    X = syn.x_chunk(0)
+    gen = torch.Generator(device=dev).manual_seed(7)
+    s = torch.exp(2 * torch.randn(1, n, generator=gen, device=dev))
+    H = gpu_hessian([X], [s], d_in, 1, dev)
+    exact = (X.double() * s[0, :, None].double()).T @ X.double()
+    error = float((H[0].double() - exact).norm() / exact.norm())
+    assert error <= 2.55e-4, "error against 64 bits %.3e" % error
