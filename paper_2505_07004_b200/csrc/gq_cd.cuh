@@ -355,7 +355,7 @@ cd_block_kernel(const __grid_constant__ CUtensorMap mapH, const __grid_constant_
         // block is short the first band, which fetches all code, counts for more: with 16 channels 1181 against 1191 us for the
         // descent named below.  With 4 levels 32 steps stay the better (2320 x 2032, two cycles: 740 against 747).
         constexpr int RUN = LEV > 8 || (LEV == 8 && CH == 16) ? CD_BAND / 2 : CD_BAND;
-        const int ch = lane % CH;                        // further lanes do the same as the first CH
+        const int ch = lane % CH;                        // lanes past the channels read along until the steps begin
         float lev[LEV], thr[LEV];
 #pragma unroll
         for (int q = 0; q < LEV; ++q) {
@@ -372,32 +372,35 @@ cd_block_kernel(const __grid_constant__ CUtensorMap mapH, const __grid_constant_
             first.load<0, CH>(hd, wb, rb);
             second.load<1, CH>(hd, wb, rb);
             bar_sync_named(BAR_SUMS, SUMS_THREADS);
-            float Bu[CD_BAND];
+            if (lane < CH) {                             // one lane per channel, or two would share its words of W and E
+                float Bu[CD_BAND];
 #pragma unroll
-            for (int q = 0; q < CD_BAND / 4; ++q) {
-                const float *sp = Ss + sums_at(ch, q);
-                float4 v[CD_PARTS];
+                for (int q = 0; q < CD_BAND / 4; ++q) {
+                    const float *sp = Ss + sums_at(ch, q);
+                    float4 v[CD_PARTS];
 #pragma unroll
-                for (int n = 0; n < CD_PARTS; ++n) v[n] = *reinterpret_cast<const float4 *>(sp + n * CD_BAND * CH);
-                Bu[4 * q + 0] = ((v[0].x + v[1].x) + (v[2].x + v[3].x)) + (v[4].x + v[5].x);
-                Bu[4 * q + 1] = ((v[0].y + v[1].y) + (v[2].y + v[3].y)) + (v[4].y + v[5].y);
-                Bu[4 * q + 2] = ((v[0].z + v[1].z) + (v[2].z + v[3].z)) + (v[4].z + v[5].z);
-                Bu[4 * q + 3] = ((v[0].w + v[1].w) + (v[2].w + v[3].w)) + (v[4].w + v[5].w);
-            }
-#pragma unroll 1
-            for (int run = 0; run < CD_BAND / RUN; ++run) {
-                if (run > 0) {
-                    hd += RUN * (CD_BAND + 1);         // the same number of rows and columns on
-                    rb += RUN;
-                    wb += RUN * CH;
-                    eb += RUN * CH;
-                    first.load<0, CH>(hd, wb, rb);
-                    second.load<1, CH>(hd, wb, rb);
-#pragma unroll
-                    for (int r = 0; r + RUN < CD_BAND; ++r) Bu[r] = Bu[r + RUN];
+                    for (int n = 0; n < CD_PARTS; ++n) v[n] = *reinterpret_cast<const float4 *>(sp + n * CD_BAND * CH);
+                    Bu[4 * q + 0] = ((v[0].x + v[1].x) + (v[2].x + v[3].x)) + (v[4].x + v[5].x);
+                    Bu[4 * q + 1] = ((v[0].y + v[1].y) + (v[2].y + v[3].y)) + (v[4].y + v[5].y);
+                    Bu[4 * q + 2] = ((v[0].z + v[1].z) + (v[2].z + v[3].z)) + (v[4].z + v[5].z);
+                    Bu[4 * q + 3] = ((v[0].w + v[1].w) + (v[2].w + v[3].w)) + (v[4].w + v[5].w);
                 }
-                chain_steps<LEV, CH, RUN, 0>(first, second, hd, rb, wb, eb, Bu, lev, thr);
+#pragma unroll 1
+                for (int run = 0; run < CD_BAND / RUN; ++run) {
+                    if (run > 0) {
+                        hd += RUN * (CD_BAND + 1);         // the same number of rows and columns on
+                        rb += RUN;
+                        wb += RUN * CH;
+                        eb += RUN * CH;
+                        first.load<0, CH>(hd, wb, rb);
+                        second.load<1, CH>(hd, wb, rb);
+#pragma unroll
+                        for (int r = 0; r + RUN < CD_BAND; ++r) Bu[r] = Bu[r + RUN];
+                    }
+                    chain_steps<LEV, CH, RUN, 0>(first, second, hd, rb, wb, eb, Bu, lev, thr);
+                }
             }
+            __syncwarp();
             if (t + 1 < CD_BANDS) bar_arrive_named(BAR_BAND, BAND_THREADS);
         }
     } else if (warp == 4) {
