@@ -10,6 +10,7 @@ import subprocess
 import pytest
 
 from paper_2505_07004_b200 import build as gq_build
+from test_gpu_hessian_cut import ACROSS, EVENLY
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 PAIRS = 74                       # of a GPU with 148 SMs
@@ -74,3 +75,27 @@ def test_runs_are_not_longer_than_across_units(items):
         else:
             assert longest <= min(ksteps, -(-total // across))
     assert kinds == {True, False}
+
+
+def hessian_launch(d_in, n, g):
+    """(units, k-steps) of a Hessian launch: 256 x 256 tiles on the upper triangle for every two groups, and for an odd last
+    group the pairs of neighbouring column tiles by row tile."""
+    nj = -(-d_in // 256)
+    slots = nj // 2 * (nj // 2 + 1) + (nj if nj % 2 else 0)
+    return nj * (nj + 1) // 2 * (g // 2) + (slots if g % 2 else 0), -(-n // 64)
+
+
+def test_ways_of_the_launches_that_run_on_the_gpu(items):
+    """What tests/test_gpu_hessian_cut.py says about its launches."""
+    plans = items([hessian_launch(*shape) + (PAIRS, 1) for shape in EVENLY + ACROSS])
+    for shape, ((full, tail_units, tail_pairs), work) in zip(EVENLY + ACROSS, plans):
+        units, ksteps = hessian_launch(*shape)
+        tail = [w for w in work if w[1] >= full * PAIRS]
+        of_pair = [len([w for w in tail if w[0] == p]) for p in range(tail_pairs)]
+        lengths = {w[3] - w[2] for w in tail}
+        if shape in EVENLY:
+            assert tail_pairs % tail_units == 0 and set(of_pair) == {1}
+        else:
+            assert tail_pairs == PAIRS and max(of_pair) == 2 and len(lengths) > 2 and tail_units * ksteps % PAIRS != 0
+            assert shape[1] % 64 != 0
+    assert {p[0][0] for p in plans} == {0, 1}                         # with and without a whole round before
