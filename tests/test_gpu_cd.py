@@ -89,7 +89,7 @@ def check_against_oracle(W, W0, cb, H, What_g, Q_g, cycles, certify_ties):
 @pytest.mark.parametrize("seed,d_in,d_out,g,m", [
     (0, 128, 64, 2, 4),         # one block, no panel product
     (1, 328, 96, 3, 8),         # two blocks, the second ragged (72 coordinates); 32 channels per group
-    (2, 520, 48, 2, 16),        # three blocks; 24 channels per group (a partly filled channel slice)
+    (2, 520, 48, 2, 16),        # three blocks; 24 channels per group (a half filled slice of 16 channels)
     (3, 1032, 256, 1, 2),       # five blocks, one group, binary codebooks
     (4, 768, 1024, 2, 4),       # two channel tiles of 256 per group
 ])
@@ -122,7 +122,7 @@ def test_cd_llama_shaped_group(dev):
 
 
 @pytest.mark.parametrize("seed,d_in,d_out,g,m", [
-    (20, 296, 88, 1, 3),        # channel slices of 32, 32 and 24; second block of 40 coordinates: a band and a quarter
+    (20, 296, 88, 1, 3),        # five channel slices of 16 and one of 8; second block of 40 coordinates: a band and a quarter
     (21, 512, 40, 1, 5),        # whole blocks
     (22, 264, 72, 3, 13),       # second block of 8 coordinates
 ])
@@ -138,12 +138,14 @@ def test_cd_block_edges(dev, seed, d_in, d_out, g, m):
     assert Q_g.max() < m - 1
 
 
-@pytest.mark.parametrize("m", [4, 8, 13, 16])
-def test_cd_levels_that_are_no_numbers(dev, m):
+# narrow layers (16 channels per CTA); and one of 32 per CTA, the last slice of a group with 8, in one block of coordinates
+@pytest.mark.parametrize("m,d_in,d_out,g", [(4, 264, 64, 2), (8, 264, 64, 2), (13, 264, 64, 2), (16, 264, 64, 2), (3, 256, 2424, 3),
+                                            (8, 256, 2424, 3), (16, 256, 2424, 3)])
+def test_cd_levels_that_are_no_numbers(dev, m, d_in, d_out, g):
     """A NaN level is never chosen while its channel has a number: the channel ends where it ends with that level far
     away.  A channel of NaN only, or with a NaN in W, still gets codes below m, and its neighbours (four channels share a
     word of codes) the bits they get without it."""
-    W, W0, cb, H = make_problem(40 + m, 264, 64, 2, m)
+    W, W0, cb, H = make_problem(40 + m, d_in, d_out, g, m)
     far = cb.copy()
     far[3, m // 2] = far[9, 0] = far[50, m - 1] = 1e30
     What_f, Q_f = run_gpu(dev, W, W0, far, H, 2)
@@ -155,7 +157,7 @@ def test_cd_levels_that_are_no_numbers(dev, m):
     assert Q_n.max() < m
     assert np.array_equal(What_n, np.take_along_axis(cb_n, Q_n, axis=1), equal_nan=True)
     assert (Q_n[5] == 0).all()
-    rest = [j for j in range(64) if j not in (5, 22)]
+    rest = [j for j in range(d_out) if j not in (5, 22)]
     assert np.array_equal(Q_n[rest], Q_f[rest]) and np.array_equal(What_n[rest], What_f[rest])
 
 
