@@ -127,8 +127,9 @@ int32_t gq_saliency_strided(const void *grad, int32_t dtype, int64_t batch, int6
  * (s_k[i] X[i][a]) * X[i][b] are accumulated in fp32 in tensor memory (two groups per pass over X), and
  * each call adds its fp32 tile sums to H with reduce-add transactions, so H is never read by the SMs.
  * Work is dealt to the SM pairs in whole 256 x 256 tiles of two groups; with flags == 0 the last,
- * incomplete round of tiles is cut along the token axis so that every SM pair gets the same amount of
- * work, and the pieces of such a tile reach H in no fixed order: those entries can differ in the last
+ * incomplete round of tiles is cut along the token axis, every tile into the same number of pieces of at most
+ * 1024 tokens or all of them into equal shares for all SM pairs.  Launches of one tile and 256 tokens are cut
+ * already.  The pieces of a tile reach H in no fixed order: those entries can differ in the last
  * bit from run to run.  With GQ_HESSIAN_DETERMINISTIC every element of H receives exactly one add per
  * call and results are bit-reproducible run to run, at the price of an idle tail in the last round.
  */
@@ -226,8 +227,8 @@ int32_t gq_hessian_gather_shares(float *const *H_ranks, int32_t ranks, int32_t r
  * from 1024 values spread over the layer so that the largest of them lies in [2^14, 2^15); where an entry turns out to
  * be 2 to 4 times as large, the matrix is written again with the largest of all in [2^14, 2^15).  Either way 11
  * significant bits for every entry down to 2^-28 of the largest; round to nearest, no bias.  The Gram
- * matrices Delta_k^T Delta_k are formed on the tensor cores (fp16 operands, fp32 accumulation) two 256-column
- * tiles at a time and contracted with H_k (fp32) straight out of tensor memory; partial sums are reduced in
+ * matrices Delta_k^T Delta_k are formed on the tensor cores (fp16 operands, fp32 accumulation) in 256 x 256
+ * tiles and contracted with H_k (fp32) straight out of tensor memory; partial sums are reduced in
  * fp64 in a fixed order and multiplied by 2^-2e.  Relative error of the result: at most 2^-11 = 4.9e-4 if
  * every rounding error had the same sign and H_k had no negative entries, about 1e-6 for rounding errors of
  * random sign (what is seen on quantisation errors).  Results are bit-reproducible run to run.
@@ -405,7 +406,7 @@ enum gq_kernel_id {
     GQ_KERNEL_SALIENCY = 0,    /* Algorithm 1, saliency step                                    */
     GQ_KERNEL_HESSIAN = 1,     /* tensor-core H += X^T Diag(s_k) X, scaling fused (Algorithm 1, Hessian step) */
     GQ_KERNEL_MIRROR = 2,      /* gq_hessian_finalize                                    */
-    GQ_KERNEL_SPLIT_DELTA = 3, /* W - W_hat -> fp16 (maximum pass + conversion pass)     */
+    GQ_KERNEL_SPLIT_DELTA = 3, /* W - W_hat -> fp16 (conversion, and check of its scale)  */
     GQ_KERNEL_GRAM_DOT = 4,    /* tensor-core Delta_k^T Delta_k contracted with H_k (Eq. 7) */
     GQ_KERNEL_REDUCE = 5,      /* fp64 reduction of the partial sums                     */
     GQ_KERNEL_SPLIT_SALIENCY = 6, /* s -> pairs of bf16 terms for the Hessian kernel's scalers */

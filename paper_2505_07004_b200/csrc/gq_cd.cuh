@@ -249,8 +249,9 @@ __device__ __forceinline__ int sums_at(int ch, int rq)
 //   loader warp (4)      TMA: the tiles of W, E and P (256 coordinates x CH channels), and H[all 256][band] (32 KB) per
 //                        band into one of three buffers, two bands ahead.
 // Two named barriers per band: sums ready (products -> chain), band done (chain -> products, loader).
-// Measured for one block of 4096 channels, 16 levels: 33.7 us (8 levels, 1408 channels: 19 from the end of the panel product to
-// its own, 27 with 32 channels per CTA); 1.2 us more with the excluded coordinates multiplied by zero instead of left out;
+// Measured for one block of 4096 channels, 16 levels: 33.9 us (8 levels, 1408 channels: 22.8 by itself, 19 from the end of the
+// panel product to its own, 27 with 32 channels per CTA); 1.2 us more with the excluded coordinates multiplied by zero instead of
+// left out;
 // with eight threads per channel that did all updates themselves and two votes and a table read per step it was 81 us (78).
 template <int LEV, int CH>
 __global__ void __launch_bounds__(CD_THREADS, 1)

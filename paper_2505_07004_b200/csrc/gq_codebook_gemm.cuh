@@ -20,7 +20,7 @@
 // Stage: [A | B], 16 KB each per CTA, of which only B comes through the L2.  What bounds the kernel is the tensor core and
 // the thread that feeds it (695 clocks a k-step with the one-hot stores left out, 512 at the nominal rate) and shared-memory
 // bandwidth (807 with them).  Measured, 4096 x 4096, 4 groups, 16 levels, one update: 3.7 ms = 1300 TFLOP/s with the issuing
-// thread on warp 1; on warp 3 a call with two updates takes 0.35 ms less.  With the one-hot matrix, H P and H W^T in
+// thread on warp 1, a tenth of a millisecond less on warp 3.  With the one-hot matrix, H P and H W^T in
 // global memory it was 0.17 (one-hot) + 2.88 (H P) + 0.40 (H W^T) + 0.55 (sums by level) = 4.00 ms and 0.5 GB of scratch.
 #pragma once
 #include <cuda.h>
@@ -202,7 +202,8 @@ codebook_gemm_kernel(const __grid_constant__ CUtensorMap mapH0, const __grid_con
     } else if (warp == 3 && lane == 0 && rank == 0) {
         // ------------------------------------------------------------------ MMA issuer (first CTA)
         // Warp 3: what this thread does between two k-steps the tensor core waits for, and warps 4 w + 1 on its scheduler include
-        // two of the one-hot warps, warps 4 w + 3 one.  4096 x 4096, 16 levels, one round: 9.83 -> 9.48 ms with warp 1 -> 3.
+        // two of the one-hot warps, warps 4 w + 3 one.  gq_lnq with two updates, 4096 x 4096, 16 levels: 10.11 -> 9.89 ms with
+        // warp 1 -> 3, both sides in turn; six other layers 0 to 2.4 % faster.
         constexpr uint32_t idesc = umma_idesc_bf16_mn(TILE_M, TILE_N);
         int s = 0;
         uint32_t ph = 0;

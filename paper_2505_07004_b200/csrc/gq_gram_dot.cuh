@@ -167,7 +167,7 @@ __device__ __forceinline__ unsigned int block_max(unsigned int v, unsigned int *
 // the biased exponent of every block's largest finite |W - W_hat| (one more where fp16 would round it up to the next power of
 // two).  e has to be known before the first
 // value is stored and depends on the largest, so it is guessed: every block looks at the same 1024 values, spread over the
-// layer, and leaves room for values 1.9 to 4 times as large.  delta_redo_kernel takes care of layers that need more.
+// layer, and leaves room for values 2 to 4 times as large.  delta_redo_kernel takes care of layers that need more.
 // A block goes over DELTA_BLOCK_VECS pairs of float4, or several times as many where there is no room for a byte from each.
 // HBM-bound: W and W_hat are read once.  The sample is 64 runs of 64 bytes and not 256 of 16, each a request of its own in every
 // block.  Three candidates of a 4096 x 4096 layer, whole calls: 324 us, with a pass over both matrices for the maximum before the

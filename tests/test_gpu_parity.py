@@ -626,8 +626,8 @@ def test_host_pipeline_matches_device_calls(dev, d_out, g):
 
 @pytest.mark.parametrize("d_in,d_out", [(1280, 3072), (1248, 3152)])      # 960 and 961 blocks of 4096 weights
 def test_objective_scale_where_the_block_maxima_stop_fitting(dev, d_in, d_out):
-    """Up to 960 blocks leave their largest difference in the header one by one, more meet in one word.  The largest
-    difference stands in the last weight, 2^10 above the others: a scale that missed it would take it past fp16's range."""
+    """Every block of the preparation leaves its largest difference; here the last block's is the layer's.  It stands in the
+    last weight, 2^10 above the others: a scale that missed it would take it past fp16's range."""
     gen = torch.Generator(device=dev).manual_seed(5)
     A = torch.randn(d_in, d_in, generator=gen, device=dev)
     H = (A.T @ A).expand(2, d_in, d_in).contiguous()
