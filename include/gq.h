@@ -225,7 +225,7 @@ int32_t gq_hessian_gather_shares(float *const *H_ranks, int32_t ranks, int32_t r
  * Same shape rules as above (d_in % 8 == 0, d_out % g == 0, (d_out / g) % 8 == 0).
  * Arithmetic: delta = W - W_hat in fp32, written to the workspace as ONE fp16 matrix delta * 2^e.  e is guessed
  * from 1024 values spread over the layer so that the largest of them lies in [2^14, 2^15); where an entry turns out to
- * be 2 to 4 times as large, the matrix is written again with the largest of all in [2^14, 2^15).  Either way 11
+ * be 2 to 4 times as large, the matrix is brought to the scale where the largest of all rounds to [2^15, 2^16).  Either way 11
  * significant bits for every entry down to 2^-28 of the largest; round to nearest, no bias.  The Gram
  * matrices Delta_k^T Delta_k are formed on the tensor cores (fp16 operands, fp32 accumulation) in 256 x 256
  * tiles and contracted with H_k (fp32) straight out of tensor memory; partial sums are reduced in

@@ -7,7 +7,7 @@
 // matching entries of H_k straight out of tensor memory.
 //
 // Operands.  Delta is prepared once per call as ONE fp16 matrix (delta_half_kernel): delta * 2^e with a single
-// power of two e for the whole layer, such that the largest finite entry lies below 2^16 and, but for the clamps, not below 2^14.
+// power of two e for the whole layer, such that the largest finite entry rounds to [2^14, 2^16), but for the clamps.
 // fp16 carries 11 significant bits at any magnitude above 2^-14, i.e. down to 2^-28 of the largest entry at least (what is
 // smaller is off by at most 2^-39 of the largest), and the
 // scaling is undone exactly (2^-2e in the final fp64 reduction).  One product at the
@@ -59,8 +59,7 @@ constexpr int GD_THREADS = 32 * (4 + GD_EPI_WARPS);
 constexpr int GD_SMEM_BYTES = GD_STAGES * GD_STAGE_BYTES + 1024;
 constexpr int GD_PARTIALS_PER_UNIT = 2 * GD_EPI_WARPS;       // one fp64 per (CTA of the pair, epilogue warp)
 constexpr int GD_SAMPLE_EXP = 14;                            // the largest sampled |delta| * 2^e lies in [2^14, 2^15);
-constexpr int GD_LARGEST_EXP = 14;                           // the largest of all, if known first, in [2^14, 2^15)
-constexpr int GD_FITS_EXP = 15;                              // it has to round to a finite value, 65504 at most
+constexpr int GD_FITS_EXP = 15;                              // the largest of all has to round to a finite value, 65504 at most
 constexpr unsigned int GD_FITS_ROUND = 0x1000;               // carries into the exponent what fp16 rounds up to 2^16: 65520 on
 constexpr int GD_MAX_SHIFT = 100;                            // |e| is kept below this (the scale stays a normal float)
 
@@ -245,9 +244,9 @@ __host__ __device__ __forceinline__ bool delta_lower(uint4 &v, unsigned down)
 }
 
 // Decides on e: the guess where the largest finite |W - W_hat| is a finite fp16 with it (all blocks return at once), else the
-// power of two that takes it to [2^14, 2^15) (one less where it rounds up), to which the matrix is then brought: the values that
-// have their bits by lowering the exponent, a quarter of the bytes of W and W_hat and most of them in the L2, the others (among
-// them what has overflowed) from W and W_hat.  blocks: of delta_half_kernel.
+// power of two that takes it to [2^15, 65520), or just below where it rounds up to 2^15, to which the matrix is then brought:
+// the values that have their bits by lowering the exponent, a quarter of the bytes of W and W_hat and most of them in the L2,
+// the others (among them what has overflowed) from W and W_hat.  blocks: of delta_half_kernel.
 // One row 20 times as wide as the others, a call: 113 us for 4096 x 4096 and 250 for 4096 x 11008 with one group; 131 and 294 with
 // all values from W and W_hat again, 123 and 273 with a pass over both for the maximum before one that converts.  A million
 // times as wide, where 3 % of the threads' values are formed again: 115 and 258, 131 and 292, 121 and 271.
@@ -267,7 +266,7 @@ delta_redo_kernel(const float *W, const float *What, unsigned count4, GramDotHea
     }
     if (threadIdx.x < blocks % 16u) biased = max(biased, static_cast<unsigned int>(block_exp[words * 16u + threadIdx.x]));
     biased = block_max(biased, red);
-    const int guess = header->guess, exact = delta_shift(biased, GD_LARGEST_EXP);
+    const int guess = header->guess, exact = delta_shift(biased, GD_FITS_EXP);
     const bool fits = static_cast<int>(biased) - 127 + guess <= GD_FITS_EXP || exact == guess;
     if (blockIdx.x == 0 && threadIdx.x == 0) header->shift = fits ? guess : exact;
     if (fits) return;

@@ -9,7 +9,7 @@ import pytest
 from paper_2505_07004_b200 import build as gq_build
 
 HERE = os.path.dirname(os.path.abspath(__file__))
-DOWN = (2, 3, 5, 10, 14, 24, 28, 29, 30, 31, 100, 200)
+DOWN = (1, 2, 3, 5, 10, 14, 24, 28, 29, 30, 31, 100, 200)
 
 
 @pytest.fixture(scope="module")

@@ -133,12 +133,14 @@ def test_scale_where_fp16_ends(dev, mantissa):
     check(run(dev, W, delta, H), orc.objective(W, delta, H, impl="numpy"))
 
 
-@pytest.mark.parametrize("outlier", [1.0, 3.0, 100.0])
+# The last one rounds up to 2^7 in fp16
+@pytest.mark.parametrize("outlier", [1.0, 3.0, 100.0, 127.99])
 def test_small_group_keeps_its_bits(dev, outlier):
     """Differences 2^-28 of the layer's largest keep 11 significant bits, wherever the largest stands.
 
-    All of the group's are equal, so every rounding error has the same sign: 2^-28 (1 + 2^-9) of the largest is 2^-14 (1 + 2^-9)
-    or more in fp16, exact; a quarter of that has two bits less there, loses the 2^-9 and gives a loss 2^-8 = 3.9e-3 too small.
+    All of the group's are equal, so every rounding error has the same sign: 2^-28 (1 + 2^-10) of the largest's power of two is
+    2^-14 (1 + 2^-10) or more in fp16, exact; half of that has a bit less there, loses the 2^-10 and gives a loss 2^-9 = 1.95e-3
+    too small.
     """
     d_in, d_out, g = 64, 1024, 2
     H, W, _ = problem(d_in, d_out, g)
@@ -146,5 +148,5 @@ def test_small_group_keeps_its_bits(dev, outlier):
     W[:] = 0
     delta = np.full(W.shape, 1.0, dtype=np.float32)
     delta[5, 7] = outlier                                              # not in the sample
-    delta[d_out // 2:] = 2.0 ** -28 * 2.0 ** np.floor(np.log2(outlier)) * (1 + 2.0 ** -9)
+    delta[d_out // 2:] = 2.0 ** -28 * 2.0 ** np.floor(np.log2(outlier)) * (1 + 2.0 ** -10)
     check(run(dev, W, delta, H), orc.objective(W, delta, H, impl="numpy"))
