@@ -412,7 +412,7 @@ gram_dot_kernel(const __grid_constant__ CUtensorMap mapD, const GramDotParams p)
             uint32_t issued = 0;
             bool ok = true;
             WorkItem w;
-            for (int it = 0; ok && work_item(p.sched, pair, it, w); ++it) {
+            for (int it = 0; ok && whole_unit(p.sched, pair, it, w); ++it) {
                 const GramUnit u = gram_unit(p, w.unit);
                 const int a0 = u.ti * TILE_M + static_cast<int>(rank) * CTA_ROWS;
                 const int b0 = u.tj * TILE_N + static_cast<int>(rank) * CTA_ROWS;
@@ -447,7 +447,7 @@ gram_dot_kernel(const __grid_constant__ CUtensorMap mapD, const GramDotParams p)
             uint32_t acc_ph[2] = {0u, 0u};
             bool ok = true;
             WorkItem w;
-            for (int it = 0; ok && work_item(p.sched, pair, it, w); ++it) {
+            for (int it = 0; ok && whole_unit(p.sched, pair, it, w); ++it) {
                 const int buf = it & 1;
                 // the accumulator of unit it - 2 must have been read out
                 if (!bounded_wait_hot(smem_u32(&bar_acc_empty[buf]), acc_ph[buf] ^ 1u, wc, 2u, w.unit)) { ok = false; break; }
@@ -487,7 +487,7 @@ gram_dot_kernel(const __grid_constant__ CUtensorMap mapD, const GramDotParams p)
         uint32_t full_ph[2] = {0u, 0u};
         bool ok = true;
         WorkItem w;
-        for (int it = 0; ok && work_item(p.sched, pair, it, w); ++it) {
+        for (int it = 0; ok && whole_unit(p.sched, pair, it, w); ++it) {
             const int buf = it & 1;
             const GramUnit u = gram_unit(p, w.unit);
             const int row0 = u.ti * TILE_M + static_cast<int>(rank) * CTA_ROWS + q * 32;

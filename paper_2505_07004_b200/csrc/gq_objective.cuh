@@ -173,7 +173,7 @@ pair_gemm_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant
         uint32_t issued = 0;
         bool ok = true;
         WorkItem w;
-        for (int it = 0; ok && work_item(p.sched, pair, it, w); ++it) {
+        for (int it = 0; ok && whole_unit(p.sched, pair, it, w); ++it) {
             ItemGeom ge;
             if (!item_geom<MODE>(p, w, rank, ge)) continue;
             const void *maps[MAX_MAPS] = {&map0, &map1, &map2, &map3, &map4, &map5};
@@ -233,7 +233,7 @@ pair_gemm_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant
         uint32_t acc_ph = 0;
         bool ok = true;
         WorkItem w;
-        for (int it = 0; ok && work_item(p.sched, pair, it, w); ++it) {
+        for (int it = 0; ok && whole_unit(p.sched, pair, it, w); ++it) {
             ItemGeom ge;
             if (!item_geom<MODE>(p, w, rank, ge)) continue;
             if (!bounded_wait_hot(smem_u32(&bar_acc_empty[buf]), acc_ph ^ 1u, wc, 2u, w.unit)) { ok = false; break; }
@@ -276,7 +276,7 @@ pair_gemm_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant
         uint32_t acc_ph = 0;
         bool ok = true;
         WorkItem w;
-        for (int it = 0; ok && work_item(p.sched, pair, it, w); ++it) {
+        for (int it = 0; ok && whole_unit(p.sched, pair, it, w); ++it) {
             ItemGeom ge;
             if (!item_geom<MODE>(p, w, rank, ge)) continue;
             if (MODE == MODE_OBJECTIVE) {
